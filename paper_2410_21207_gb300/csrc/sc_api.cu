@@ -114,13 +114,12 @@ struct Workspace {
   DevBuf<int32_t> enl_log;       // sc_enlarge: the k seams, the carved copy, the widening bitmap
   DevBuf<uint8_t> enl_tmp;
   DevBuf<uint32_t> enl_bits;
-  DevBuf<uint32_t> Mmulti;
   DevBuf<DpArgs> dargs;
   bool flags_zeroed = false;
   void release_all() {
     img.release(); img2.release(); Mrow.release();
     E.release(); seam.release(); lists.release(); hin.release(); hout.release(); flags.release();
-    Emulti.release(); Mmulti.release(); dargs.release(); gates.release(); wdirs.release(); wanc.release();
+    Emulti.release(); dargs.release(); gates.release(); wdirs.release(); wanc.release();
     enl_log.release(); enl_tmp.release(); enl_bits.release();
     flags_zeroed = false;
   }
@@ -449,15 +448,13 @@ int sc_find_seam_multi(const uint16_t *const *energies, int n, int H, int W, int
   std::lock_guard<std::mutex> lk(ws.mu);
   if ((rc = ensure_flags(ws, st))) return rc;
   const int pe = pitch_e_for(W);
-  const int S = (H + KS - 1) / KS;
-  const size_t e_per = (size_t)H * pe, m_per = (size_t)(S + 1) * pe;
+  const size_t e_per = (size_t)H * pe;
   // a map is read in place when its rows are 16-byte aligned (W a multiple of 8, aligned base);
   // any other map is first copied into a padded workspace
   auto in_place = [&](int k) { return (W % 8) == 0 && ((uintptr_t)energies[k] & 15u) == 0; };
   int ncopy = 0;
   for (int k = 0; k < n; ++k) ncopy += !in_place(k);
   if (ncopy) SC_CUDA(ws.Emulti.ensure(e_per * ncopy));
-  SC_CUDA(ws.Mmulti.ensure(m_per * n));
   SC_CUDA(ws.dargs.ensure((size_t)n));
   SC_CUDA(ws.gates.ensure((size_t)n));
   if ((rc = ensure_wide(ws, H, W, n))) return rc;
@@ -477,8 +474,6 @@ int sc_find_seam_multi(const uint16_t *const *energies, int n, int H, int W, int
     }
     a.H = H;
     a.W = W;
-    a.Mrow = ws.Mmulti.p + m_per * k + E_PADL;
-    a.pitch_m = pe;
     a.seam = seams_out + (size_t)k * H;
     a.seam_log = nullptr;
     a.cost = costs_out ? costs_out + k : nullptr;

@@ -65,7 +65,6 @@ __device__ void batch_seam_pass(const BatchItem &it, uint32_t *words, int rows, 
     a.pitch_e = it.pe;
     a.H = rows;
     a.W = w;
-    a.Mrow = it.Mrow + E_PADL;
     a.seam = it.seam;
     a.seam_log = log ? log + (size_t)t * rows : nullptr;
     a.cost = costs ? costs + t : nullptr;

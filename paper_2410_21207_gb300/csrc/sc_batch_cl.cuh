@@ -46,7 +46,6 @@ __device__ void clb_seam_pass(const BatchItem &it, uint32_t *words, int rows, in
     a.pitch_e = it.pe;
     a.H = rows;
     a.W = w;
-    a.Mrow = it.Mrow + E_PADL;
     a.seam = it.seam;
     a.seam_log = log ? log + (size_t)t * rows : nullptr;
     a.cost = costs ? costs + t : nullptr;

@@ -49,7 +49,6 @@ __global__ void __launch_bounds__(Geo<NW, KT, true>::THREADS, 1) k_dp(DpArgs p) 
   a.pitch_e = p.pitch_e;
   a.H = p.H;
   a.W = p.W;
-  a.Mrow = p.Mrow;
   a.seam = p.seam;
   a.seam_log = p.seam_log;
   a.cost = p.cost;

@@ -33,13 +33,11 @@ __global__ void __launch_bounds__(Geo<NW, KT, true>::THREADS, NW == 8 ? 2 : 4) k
   a.pitch_e = p.pitch_e;
   a.H = p.H;
   a.W = p.W;
-  a.Mrow = p.Mrow;
   a.seam = p.seam;
   a.seam_log = p.seam_log;
   a.cost = p.cost;
   a.err = p.err;
   a.gated = (p.gate != nullptr) && (*p.gate & ERR_ENERGY_RANGE);
-  a.pitch_m = p.pitch_m;
   a.gate = p.gate;
   SearchState st;
   seam_search<NW, KT, true, MULTI_FILL_WARPS, false, KS, true>(a, smem, S, st);

@@ -52,7 +52,7 @@ struct DpArgs {
   const uint16_t *E;   // row 0, column 0 (already offset by E_PADL)
   int pitch_e;
   int H, W;
-  uint32_t *Mrow;      // super-tile boundary rows, row s at Mrow + s*pitch_m (offset by E_PADL)
+  uint32_t *Mrow;      // super-tile boundary rows, row s at Mrow + s*pitch_e (offset by E_PADL)
   int32_t *seam;       // out [H]
   int32_t *seam_log;   // nullable, out [H]
   int64_t *cost;       // nullable, out [1]
@@ -60,7 +60,6 @@ struct DpArgs {
   int *gate;           // nullable: with ERR_ENERGY_RANGE set the 24-bit search skips the map and the
                        // wide-cost search takes it (the multi-map search also sets it itself)
   int64_t pstride = 0; // forward energy: elements between the CU, DL, DR planes (0: the e1 map)
-  int pitch_m = 0;     // row stride of Mrow (0: pitch_e)
 };
 
 // Launchers (enqueue on `st`; return cudaError_t of the launch).

@@ -126,7 +126,6 @@ extern "C" int sc_find_seam_static(const uint16_t *energy, int H, int W, int32_t
   a.pitch_e = pe;
   a.H = H;
   a.W = W;
-  a.Mrow = reinterpret_cast<uint32_t *>(base + off_M) + E_PADL;
   a.seam = seam_out;
   a.seam_log = nullptr;
   a.cost = cost_out;
