@@ -101,12 +101,12 @@ struct DevBuf {
 
 struct Workspace {
   std::mutex mu;
-  DevBuf<uint32_t> img, img2, Mrow;
+  DevBuf<uint32_t> img, img2, scratch;
   DevBuf<uint16_t> E;
   DevBuf<int32_t> seam;
   DevBuf<int16_t> lists;          // two generations of pending-removal lists
   DevBuf<uint8_t> hin, hout;     // staging for the host-pointer entry point
-  DevBuf<int> flags;             // [0] error word, [1] energy-range gate
+  DevBuf<int> flags;             // [0] error word, [1] energy-range gate, [2] the search's arrival counter
   DevBuf<int> gates;             // one energy-range gate per map of sc_find_seam_multi
   DevBuf<uint32_t> wdirs;        // wide-cost search: directions and ancestors (per map)
   DevBuf<uint16_t> wanc;
@@ -117,7 +117,7 @@ struct Workspace {
   DevBuf<DpArgs> dargs;
   bool flags_zeroed = false;
   void release_all() {
-    img.release(); img2.release(); Mrow.release();
+    img.release(); img2.release(); scratch.release();
     E.release(); seam.release(); lists.release(); hin.release(); hout.release(); flags.release();
     Emulti.release(); dargs.release(); gates.release(); wdirs.release(); wanc.release();
     enl_log.release(); enl_tmp.release(); enl_bits.release();
@@ -175,7 +175,7 @@ static int ensure_carve_buffers(Workspace &ws, int H, int W) {
   const int pe = pitch_e_for(R);
   SC_CUDA(ws.E.ensure((size_t)R * pe));
   const int S = (R + KS - 1) / KS;
-  SC_CUDA(ws.Mrow.ensure((size_t)(S + 1) * pe));
+  SC_CUDA(ws.scratch.ensure((size_t)(S + 1) * pe));
   SC_CUDA(ws.seam.ensure((size_t)R));
   SC_CUDA(ws.lists.ensure((size_t)2 * R * RPEND));
   return SC_OK;
@@ -199,7 +199,8 @@ static int launch_search(Workspace &ws, uint16_t *Ebase, int pe, int H, int W, i
   a.pitch_e = pe;
   a.H = H;
   a.W = W;
-  a.Mrow = ws.Mrow.p + E_PADL;
+  a.scratch = ws.scratch.p;
+  a.sync = ws.flags.p + 2;
   a.seam = seam;
   a.seam_log = seam_log;
   a.cost = cost;
@@ -233,7 +234,8 @@ static int carve_pass_plain(Workspace &ws, uint32_t *img, int pitch, int H, int 
     a.pitch_e = pe;
     a.H = H;
     a.W = w;
-    a.Mrow = ws.Mrow.p + E_PADL;
+    a.scratch = ws.scratch.p;
+    a.sync = ws.flags.p + 2;
     a.seam = ws.seam.p;
     a.seam_log = seam_log ? seam_log + (size_t)t * H : nullptr;
     a.cost = cost_log ? cost_log + t : nullptr;
@@ -427,7 +429,7 @@ int sc_find_seam(const uint16_t *energy, int H, int W, int32_t *seam_out, int64_
   if ((rc = ensure_flags(ws, st))) return rc;
   const int pe = pitch_e_for(W);
   SC_CUDA(ws.E.ensure((size_t)H * pe));
-  SC_CUDA(ws.Mrow.ensure((size_t)((H + KS - 1) / KS + 1) * pe));
+  SC_CUDA(ws.scratch.ensure((size_t)((H + KS - 1) / KS + 1) * pe));
   if ((rc = ensure_wide(ws, H, W, 1))) return rc;
   SC_CUDA(cudaMemsetAsync(ws.flags.p + 1, 0, sizeof(int), st));
   SC_CUDA(launch_copy_energy(energy, H, W, ws.E.p + E_PADL, pe, ws.flags.p + 1, st));
@@ -546,7 +548,7 @@ int sc_find_seam_forward(const uint16_t *cu, const uint16_t *dl, const uint16_t 
   const int pe = pitch_e_for(W);
   const int64_t pstride = (int64_t)H * pe;
   SC_CUDA(ws.E.ensure((size_t)3 * H * pe));
-  SC_CUDA(ws.Mrow.ensure((size_t)((H + KS - 1) / KS + 1) * pe));
+  SC_CUDA(ws.scratch.ensure((size_t)((H + KS - 1) / KS + 1) * pe));
   if ((rc = ensure_wide(ws, H, W, 1))) return rc;
   SC_CUDA(cudaMemsetAsync(ws.flags.p + 1, 0, sizeof(int), st));
   SC_CUDA(launch_copy_planes(cu, dl, dr, H, W, ws.E.p + E_PADL, pe, pstride, ws.flags.p + 1, st));

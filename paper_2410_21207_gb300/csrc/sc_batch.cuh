@@ -15,8 +15,6 @@ namespace sc {
 // up to 64 * (NW + 1) rows); their direction rows share the idle staging ring.
 __host__ __device__ constexpr int batch_fill_warps(int nw, int kt) { return 16; }
 
-__device__ __forceinline__ void fence_proxy_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
-
 // rows x cols word image -> its transpose (cols x rows), 32x32 tiles staged in shared memory; `tile`
 // holds `ntw` warps' 32x33 tiles.
 __device__ inline void cta_transpose(const uint32_t *src, int ps, int rows, int cols, uint32_t *dst, int pd,
@@ -154,7 +152,7 @@ __global__ void __launch_bounds__(Geo<NW, KT, false>::THREADS, 1)
   // the current image's descriptor lives in shared memory and its fields are read where they are
   // used, so they do not occupy registers across the seam loop
   __shared__ BatchItem cur;
-  search_init<NW, KT, false, batch_fill_warps(NW, KT)>(smem, Smax);
+  search_init<NW>(smem, search_plan<NW, KT, false, batch_fill_warps(NW, KT)>(Smax));
   __syncthreads();
   SearchState st;
   for (;;) {

@@ -20,8 +20,6 @@
 
 namespace sc {
 
-__device__ __forceinline__ void fence_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
-
 // (count) vertical seams of a rows x cols word image whose energy is in it.E
 template <int NW, int KT, int FWM>
 __device__ void clb_seam_pass(const BatchItem &it, uint32_t *words, int rows, int cols, int count, int32_t *log,
@@ -67,7 +65,7 @@ __device__ void clb_seam_pass(const BatchItem &it, uint32_t *words, int rows, in
                           reinterpret_cast<uint32_t *>(sbuf + (size_t)warp * sbuf_elems), sbuf_elems / 2);
       m = 0;
     }
-    fence_async_global();   // the next search stages the compacted energy rows with TMA
+    fence_proxy_async_global();   // the next search stages the compacted energy rows with TMA
     cl.sync();
   }
   if (m > 0) {
@@ -82,7 +80,7 @@ __device__ inline void clb_energy(const uint32_t *words, int pitch, int rows, in
   for (int i = rank; i < rows; i += cs)
     for (int j = threadIdx.x; j < cols; j += blockDim.x)
       E[(int64_t)i * pe + j] = (uint16_t)energy_at(words, pitch, rows, cols, i, j);
-  fence_async_global();
+  fence_proxy_async_global();
   cg::this_cluster().sync();
 }
 
@@ -158,7 +156,7 @@ __global__ void __launch_bounds__(Geo<NW, KT, true, FWM>::THREADS, 1)
   pdl_launch_dependents();
   cg::cluster_group cl = cg::this_cluster();
   const int rank = (int)cl.block_rank(), cs = (int)cl.num_blocks();
-  search_init<NW, KT, true, FWM>(smem, Smax);
+  search_init<NW>(smem, search_plan<NW, KT, true, FWM>(Smax));
   cl.sync();
   SearchState st;
   for (;;) {

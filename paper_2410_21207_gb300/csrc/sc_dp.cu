@@ -1,5 +1,6 @@
-// One seam search per launch on one thread-block cluster (the plain per-seam path and
-// sc_find_seam). The search itself is seam_search in sc_search.cuh.
+// One seam search per launch (the per-seam path of the carve and sc_find_seam): maps of at least
+// TWO_MIN_ROWS rows from both ends by two thread-block clusters (k_dp_two), shorter ones and forward
+// energy by one cluster (k_dp, seam_search in sc_search.cuh).
 #include "sc_search.cuh"
 
 namespace sc {
@@ -38,7 +39,7 @@ __global__ void __launch_bounds__(Geo<NW, KT, true>::THREADS, 1) k_dp(DpArgs p) 
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int KSS = dp_super_rows<NW, KT, FWD>();
   const int S = (p.H + KSS - 1) / KSS;
-  search_init<NW, KT, true, FILL_WARPS_MAX, FWD, KSS>(smem, S);
+  search_init<NW>(smem, search_plan<NW, KT, true, FILL_WARPS_MAX, FWD, KSS>(S));
   // neighbours push into each other's halo buffers: every CTA's barriers must be initialised first
   cg::this_cluster().sync();
   // the set-up above overlaps the previous kernel of the seam loop; its results are read below
@@ -59,6 +60,26 @@ __global__ void __launch_bounds__(Geo<NW, KT, true>::THREADS, 1) k_dp(DpArgs p) 
   seam_search<NW, KT, true, FILL_WARPS_MAX, FWD, KSS>(a, smem, S, st);
 }
 
+// one or two clusters of cs CTAs; a programmatic dependent (may start before its predecessor ends)
+static cudaError_t launch_dp_cluster(void (*kernel)(DpArgs), int grid, int cs, int threads, size_t smem,
+                                     cudaStream_t st, const DpArgs &a) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = cs;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, kernel, a);
+}
+
 template <int NW, int KT, bool FWD = false>
 static cudaError_t launch_dp_shape(const DpArgs &a, int cs, cudaStream_t st) {
   constexpr int KSS = dp_super_rows<NW, KT, FWD>();
@@ -72,21 +93,249 @@ static cudaError_t launch_dp_shape(const DpArgs &a, int cs, cudaStream_t st) {
     configured = true;
   }
   if (smem > 232448) return cudaErrorInvalidValue;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(cs);
-  cfg.blockDim = dim3(Geo<NW, KT, true>::THREADS);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute at[2];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = cs;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // may start before its predecessor ends
-  at[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, k_dp<NW, KT, FWD>, a);
+  return launch_dp_cluster(k_dp<NW, KT, FWD>, cs, cs, Geo<NW, KT, true>::THREADS, smem, st, a);
+}
+
+// ---- the two-ended search ----
+// The search of one map is a chain of dependent rows. The seam is the leftmost of all optimal paths
+// (the pointwise minimum of two optimal paths is again an optimal path: where they cross without
+// sharing a cell they can be exchanged), which does not depend on the direction it is computed from.
+// So one cluster sweeps the upper half downwards from row 0 and a second one the lower half upwards
+// from the bottom row (the same sweep with a negative row pitch), and the chain is half as long:
+//   * with D(j) the cost of the best path from row 0 to column j of the upper half's last row and
+//     U(j) that from the bottom row to column j of the row below it, the seam costs the minimum of
+//     D(j) + min(U(j-1), U(j), U(j+1)); its columns in those two rows are the leftmost j and the
+//     leftmost of the three that reach it;
+//   * each half's ancestors give the seam's columns at its super-tile boundaries, towards row 0 and
+//     towards the bottom row: two chains that one warp follows side by side, half as many hops each;
+//   * the super-tiles of both halves are then backtracked in parallel as in seam_search.
+// No cluster waits for the other: both leave their last cost row and their ancestor table in
+// global memory, count themselves in, and the cluster that holds the last CTA to arrive does the rest
+// while the other one leaves. (The two need not be resident together, so the launch cannot
+// deadlock beside other work.)
+//
+// Scratch, in p.scratch: the two cost rows (gw uint32 each), then the ancestor tables (gw bytes per
+// super-tile, upper half first), gw = the columns the cluster covers. It fits (S + 1) rows of pitch_e
+// words, S = ceil(H / 32), for H >= 64: 8 gw + (S + 1) gw <= 4 (S + 1) pitch_e.
+//
+// Bound by latency: the chain of H / 2 rows (about 54 cycles a row with the tile boundaries), then
+// the hand-over, chain and fill. 1920x1080 carve 24.5 -> 17.7 ms, 3840x2160 carve 183.9 -> 106.8 ms,
+// 1279x853 -> 1021x701 18.5 -> 13.5 ms. The hand-over costs a few microseconds, so short maps keep the
+// one-ended search: one launch takes 16.5 / 16.6 us (two-ended / one-ended) at 128 rows, 18.5 / 17.2 at
+// 160, 18.5 / 18.7 at 192, 18.7 / 20.8 at 256, 22.8 / 28.9 at 512 (1000 columns; the same line at 64 to
+// 3840 columns).
+constexpr int TWO_MIN_ROWS = 192;
+
+template <int NW, int KT>
+struct Two {
+  static constexpr int KSS = dp_super_rows<NW, KT, false>();
+  using G = Geo<NW, KT, true, FILL_WARPS_MAX, KSS>;
+  int H0, H1, S0, S1, gw;
+  size_t tab_bytes;      // both tables
+  bool tab_smem;         // rank 0 of the finishing cluster copies them into its staging ring's place
+  SearchPlan plan;       // jb holds both halves' columns: S0 + 1, then S1 + 1
+  size_t tbar;           // mbarrier of that copy
+
+  __host__ __device__ Two(int H, int cs) {
+    H0 = (H + 1) / 2;
+    H1 = H - H0;
+    S0 = (H0 + KSS - 1) / KSS;
+    S1 = (H1 + KSS - 1) / KSS;
+    gw = cs * G::OWC;
+    tab_bytes = (size_t)(S0 + S1) * gw;
+    layout(true);
+    if (plan.total > SEARCH_SMEM_LIMIT) layout(false);
+  }
+  __host__ __device__ void layout(bool tab) {
+    tab_smem = tab;
+    size_t o = 0;
+    auto take = [&](size_t bytes) { const size_t at = o; o = (o + bytes + 15) & ~(size_t)15; return at; };
+    plan.bnd = take((size_t)2 * G::BW * 4);
+    plan.hbuf = take((size_t)2 * 2 * K2 * 4);
+    plan.wmin = 0;
+    plan.cmin = take((size_t)MAX_CLUSTER * (NW + 1) * 8);   // every warp's minimum, pushed to rank 0
+    plan.jb = take((size_t)(S0 + S1 + 2) * 4);
+    plan.misc = take(16);   // [0] this cluster arrived last, [1] path cost sum (rank 0), [2] chain found
+    plan.anc = plan.emx = plan.gat = 0;
+    plan.gw = 0;
+    plan.bars = take((size_t)(2 * NSLOT + 3) * 8);
+    tbar = plan.bars + (size_t)(2 * NSLOT + 2) * 8;
+    // the staging ring; after the sweep its place holds the tables, then the fills' directions
+    size_t r = (size_t)NSLOT * KT * G::BW * 2;
+    const size_t fd = (size_t)G::FW * KSS * G::FILLW;
+    r = r > fd ? r : fd;
+    if (tab && tab_bytes > r) r = tab_bytes;
+    plan.ring = plan.fdir = take(r);
+    plan.total = o;
+  }
+};
+
+template <int NW, int KT>
+__global__ void __launch_bounds__(Geo<NW, KT, true>::THREADS, 1) k_dp_two(DpArgs p) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  using T = Two<NW, KT>;
+  using G = typename T::G;
+  constexpr int KSS = T::KSS;
+  cg::cluster_group cl = cg::this_cluster();
+  const int cs = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+  const int half = (int)blockIdx.x / cs;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const T g(p.H, cs);
+  const SearchPlan &plan = g.plan;
+  int *jb = reinterpret_cast<int *>(smem + plan.jb);
+  int *misc = reinterpret_cast<int *>(smem + plan.misc);
+  uint64_t *tbar = reinterpret_cast<uint64_t *>(smem + g.tbar);
+  search_init<NW>(smem, plan);
+  if (threadIdx.x == 0) {
+    mbar_init(tbar, 1);
+    fence_mbar_init();
+    misc[0] = 0;
+  }
+  // neighbours push into each other's halo buffers: every CTA's barriers must be initialised first
+  cl.sync();
+  // the set-up above overlaps the previous kernel of the seam loop; its results are read below
+  pdl_launch_dependents();
+  pdl_wait_prerequisites();
+  if (p.gate && (*p.gate & ERR_ENERGY_RANGE)) return;   // left to the wide-cost search
+  uint32_t *const end0 = p.scratch, *const end1 = end0 + g.gw;
+  uint8_t *const tab = reinterpret_cast<uint8_t *>(end1 + g.gw);
+  const uint16_t *const E1 = p.E + (ptrdiff_t)(p.H - 1) * p.pitch_e;
+  {
+    SearchArgs a;
+    a.E = half ? E1 : p.E;
+    a.pitch_e = half ? -p.pitch_e : p.pitch_e;
+    a.H = half ? g.H1 : g.H0;
+    a.W = p.W;
+    a.err = p.err;
+    a.gated = false;
+    a.pstride = 0;
+    a.gtab = tab + (half ? (size_t)g.S0 * g.gw : 0);
+    a.gw = g.gw;
+    a.endrow = half ? end1 : end0;
+    SearchState st;
+    seam_sweep<NW, KT, true, FILL_WARPS_MAX, false, KSS, false, true>(a, smem, plan, st);
+  }
+  // ---- count this CTA in; the cluster of the last one goes on ----
+  fence_proxy_async_global();   // the tables are read by a bulk copy below
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    if (atomicAdd(p.sync, 1) == 2 * cs - 1) {
+      __threadfence();
+      *p.sync = 0;   // for the next launch
+      for (int r = 0; r < cs; ++r) cl.map_shared_rank(misc, r)[0] = 1;
+    }
+  }
+  cl.sync();
+  if (misc[0] == 0) return;
+
+  // ---- the seam's cost and its columns in the two middle rows ----
+  unsigned char *const stab = smem + plan.ring;
+  if (rank == 0 && warp == NW && g.tab_smem) {
+    // rank 0 fetches both ancestor tables meanwhile
+    fence_proxy_async_global();
+    fence_proxy_async_smem();   // the ring's last reads come first
+    if (lane == 0) mbar_arrive_expect_tx(tbar, (uint32_t)g.tab_bytes);
+    __syncwarp();
+    for (int s = lane; s < g.S0 + g.S1; s += 32) bulk_g2s(stab + (size_t)s * g.gw, tab + (size_t)s * g.gw, g.gw, tbar);
+  }
+  unsigned long long best = ~0ull;   // cost << 32 | upper column << 2 | step to the lower column
+  const int jend = min(p.W, (rank + 1) * G::OWC);
+  for (int j = rank * G::OWC + threadIdx.x; j < jend; j += G::THREADS) {
+    const uint32_t d = __ldcg(end0 + j);
+    const uint32_t u0 = j > 0 ? __ldcg(end1 + j - 1) : SENT, u1 = __ldcg(end1 + j),
+                   u2 = j + 1 < p.W ? __ldcg(end1 + j + 1) : SENT;
+    const uint32_t m = min3u(u0, u1, u2);
+    const uint32_t st = m == u0 ? 0u : (m == u1 ? 1u : 2u);
+    const unsigned long long k = ((unsigned long long)(d + m) << 32) | ((uint32_t)j << 2) | st;
+    best = k < best ? k : best;
+  }
+  auto warp_min = [](unsigned long long v) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      const unsigned long long o = __shfl_xor_sync(0xffffffffu, v, off);
+      v = o < v ? o : v;
+    }
+    return v;
+  };
+  best = warp_min(best);
+  unsigned long long *cmin = reinterpret_cast<unsigned long long *>(smem + plan.cmin);
+  if (lane == 0) cl.map_shared_rank(cmin, 0)[rank * (NW + 1) + warp] = best;
+  cl.sync();
+
+  // ---- ancestor chains (rank 0): lane 0 towards row 0, lane 1 towards the bottom row ----
+  if (rank == 0 && warp == 0) {
+    best = ~0ull;
+    for (int q = lane; q < cs * (NW + 1); q += 32) best = cmin[q] < best ? cmin[q] : best;
+    best = warp_min(best);
+    bool bad = false;
+    if (g.tab_smem && !mbar_wait_bounded(tbar, 0u, WAIT_TIMEOUT_NS)) {
+      if (lane == 0) atomicOr(p.err, ERR_TIMEOUT);
+      bad = true;
+    }
+    if (lane < 2) {
+      const int Sh = lane ? g.S1 : g.S0;
+      const size_t t0 = lane ? (size_t)g.S0 * g.gw : 0;
+      int *jh = jb + (lane ? g.S0 + 1 : 0);
+      int j = (int)((uint32_t)best >> 2) + (lane ? (int)(best & 3u) - 1 : 0);
+      // a column outside the map is clamped (every read stays inside the table) and recorded
+      auto keep = [&](int c) { bad |= (unsigned)c >= (unsigned)p.W; return min(max(c, 0), p.W - 1); };
+      j = keep(j);
+      for (int s = Sh - 1; s >= 0; --s) {
+        jh[s] = j;
+        const size_t at = t0 + (size_t)s * g.gw + j;
+        j = keep(j + (g.tab_smem ? (int)stab[at] : (int)__ldcg(tab + at)) - 128);
+      }
+      jh[Sh] = j;
+      if (bad) atomicOr(p.err, ERR_BAD_SEAM);
+    }
+    bad = __any_sync(0xffffffffu, bad);
+    if (lane == 0) {
+      misc[1] = 0;
+      if (!bad && p.cost) *p.cost = (int64_t)(best >> 32);
+    }
+    __syncwarp();
+    // every CTA gets the columns
+    for (int q = lane; q < g.S0 + g.S1 + 2; q += 32) {
+      const int v = jb[q];
+      for (int r = 1; r < cs; ++r) cl.map_shared_rank(jb, r)[q] = v;
+    }
+    if (lane < cs) cl.map_shared_rank(misc, lane)[2] = bad ? 0 : 1;
+  }
+  cl.sync();
+
+  // ---- the super-tiles of both halves, the lower half's from the last warp on ----
+  if (misc[2] == 0) return;   // recorded; nothing refers to another CTA's shared memory any more
+  if (warp < G::FW) {
+    uint32_t *const csum = reinterpret_cast<uint32_t *>(cl.map_shared_rank(misc, 0) + 1);
+    const int Wa = (p.W + 7) & ~7;
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {
+      const int last = h ? p.H - 1 : 0;
+      const FillCtx f{h ? E1 : p.E, h ? jb + g.S0 + 1 : jb, smem + plan.fdir, csum, p.seam + last,
+                      p.seam_log ? p.seam_log + last : nullptr, p.err, 0, h ? -p.pitch_e : p.pitch_e,
+                      h ? g.H1 : g.H0, p.W, Wa, h ? g.S1 : g.S0, cs, h ? -1 : 1};
+      backtrack_fill<NW, KT, true, FILL_WARPS_MAX, false, KSS, false, 16>(
+          f, (h ? G::FW - 1 - warp : warp) * cs + rank, warp, lane);
+    }
+  }
+  cl.sync();   // rank 0's sum is complete
+  if (rank == 0 && threadIdx.x == 0 && (uint32_t)misc[1] != (uint32_t)(best >> 32)) atomicOr(p.err, ERR_COST_MISMATCH);
+}
+
+template <int NW, int KT>
+static cudaError_t launch_dp_two(const DpArgs &a, int cs, cudaStream_t st) {
+  const size_t smem = Two<NW, KT>(a.H, cs).plan.total;
+  static bool configured = false;
+  if (!configured) {
+    cudaError_t e = cudaFuncSetAttribute(k_dp_two<NW, KT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(k_dp_two<NW, KT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    configured = true;
+  }
+  if (smem > SEARCH_SMEM_LIMIT) return cudaErrorInvalidValue;
+  return launch_dp_cluster(k_dp_two<NW, KT>, 2 * cs, cs, Geo<NW, KT, true>::THREADS, smem, st, a);
 }
 
 // forward energy stages three planes per row: one shape, 4 warps x 16-row tiles (W <= 4096)
@@ -100,6 +349,11 @@ cudaError_t launch_dp(const DpArgs &a, cudaStream_t st) {
   }
   const DpShape s = dp_shape_for(a.W);
   if (s.cs > MAX_CLUSTER) return cudaErrorInvalidValue;
+  if (a.H >= TWO_MIN_ROWS) {
+    if (s.nw == 4 && s.kt == 32) return launch_dp_two<4, 32>(a, s.cs, st);
+    if (s.nw == 8 && s.kt == 32) return launch_dp_two<8, 32>(a, s.cs, st);
+    return launch_dp_two<8, 16>(a, s.cs, st);
+  }
   if (s.nw == 4 && s.kt == 32) return launch_dp_shape<4, 32>(a, s.cs, st);
   if (s.nw == 8 && s.kt == 32) return launch_dp_shape<8, 32>(a, s.cs, st);
   return launch_dp_shape<8, 16>(a, s.cs, st);

@@ -6,7 +6,7 @@
 //   E     : uint16 energy, H rows x pitch_e elements; column j of row i lives at
 //           E + i*pitch_e + E_PADL + j. The pads keep every window load of the seam search in
 //           bounds; their contents are never used for a result.
-//   Mrow  : uint32 cost-table rows saved at super-tile boundaries (see sc_dp.cu), same padding.
+//   scratch: what the two-ended search's clusters leave for each other (see sc_dp.cu).
 //   seam  : int32[H]; patch: uint32[H] (the two refreshed energies of a row, low/high half).
 #pragma once
 #include <cstdint>
@@ -14,7 +14,7 @@
 
 namespace sc {
 
-constexpr int E_PADL = 256;    // left pad (elements) of E and Mrow rows
+constexpr int E_PADL = 256;    // left pad (elements) of E rows
 constexpr int E_PADR = 1024;   // right pad (elements)
 
 // Seam-search geometry (sc_search.cuh). A lane owns V consecutive columns; a warp's window is
@@ -52,7 +52,8 @@ struct DpArgs {
   const uint16_t *E;   // row 0, column 0 (already offset by E_PADL)
   int pitch_e;
   int H, W;
-  uint32_t *Mrow;      // super-tile boundary rows, row s at Mrow + s*pitch_e (offset by E_PADL)
+  uint32_t *scratch;   // two-ended search: cost rows and ancestor tables, (ceil(H/KS) + 1) * pitch_e words
+  int *sync;           // two-ended search: arrival counter, 0 between launches
   int32_t *seam;       // out [H]
   int32_t *seam_log;   // nullable, out [H]
   int64_t *cost;       // nullable, out [1]

@@ -5,8 +5,8 @@
 // back. cudaMalloc/cudaFree can synchronise the whole device and take an unpredictable time, which
 // a latency-critical frame loop cannot afford, and hosts that account for every device byte through
 // their own allocator or a fixed memory budget forbid allocations they do not control. Such callers
-// pass their own input and output buffers; the scratch (a padded copy of the energy map, the cost
-// rows saved for the backtrack, the wide-cost search's directions and ancestors, three status
+// pass their own input and output buffers; the scratch (a padded copy of the energy map, the
+// search's cost rows and ancestor tables, the wide-cost search's directions and ancestors, three status
 // words) comes from the array below.
 #include <cstdio>
 #include <mutex>
@@ -26,8 +26,9 @@ static __device__ __align__(256) unsigned char g_static_scratch[STATIC_SCRATCH_B
 //   [0] the errors of the call in flight (cleared by each call),
 //   [1] the call's energy-range gate (cleared by each call),
 //   [2] errors not yet reported: every call's errors are added here, and sc_check reads and
-//       clears it.
-constexpr int ST_CALL_ERR = 0, ST_GATE = 1, ST_PENDING = 2;
+//       clears it,
+//   [3] the search's arrival counter (zero between calls).
+constexpr int ST_CALL_ERR = 0, ST_GATE = 1, ST_PENDING = 2, ST_SYNC = 3;
 
 // Host code cannot use the name g_static_scratch as a device address: it is a host-side stand-in.
 // The device address is looked up once per device with cudaGetSymbolAddress.
@@ -131,6 +132,8 @@ extern "C" int sc_find_seam_static(const uint16_t *energy, int H, int W, int32_t
   a.cost = cost_out;
   a.err = words + ST_CALL_ERR;
   a.gate = words + ST_GATE;
+  a.scratch = reinterpret_cast<uint32_t *>(base + off_M);
+  a.sync = words + ST_SYNC;
   SC_STATIC_CUDA(launch_dp(a, st));
   SC_STATIC_CUDA(launch_dp_wide(a, reinterpret_cast<uint32_t *>(base + off_D), reinterpret_cast<uint16_t *>(base + off_A),
                                 st));

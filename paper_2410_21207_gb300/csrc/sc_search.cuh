@@ -125,6 +125,11 @@ struct SearchArgs {
   int *err;            // device error word
   bool gated;          // skip the search (energy range failure)
   int64_t pstride;     // forward energy: elements from one cost plane (CU, DL, DR) to the next
+  // half of a two-ended search: the ancestor table (row stride gw) and the last row's costs, in
+  // global memory (pitch_e is negative where the rows are swept from the bottom of the map)
+  uint8_t *gtab = nullptr;
+  int gw = 0;
+  uint32_t *endrow = nullptr;
 };
 
 // Running counters of the mbarrier phases, identical in every thread of the CTA.
@@ -142,20 +147,24 @@ __device__ __forceinline__ uint32_t hi8(uint32_t x) { return __byte_perm(x, 0u, 
 // Bookkeeping after row i (keys k of this lane's V columns, warp frame base fb):
 //  - bottom of a super-tile: record the ancestors of the CTA-own columns (one byte: a - col + 128),
 //    in rank 0's gathered table (row stride gw) when there is one, else in this CTA's table;
-//  - last row of the image: fold the lane's (M << 32 | column) minimum.
-template <int KSS>
+//  - last row of the image: fold the lane's (M << 32 | column) minimum, or, where the sweep ends in
+//    the middle of the map (TWO), store the cost row.
+template <int KSS, bool TWO>
 __device__ __forceinline__ void row_events(int i, const uint32_t (&k)[V], int H, int W, int c0, int fb, bool cta_own,
                                            int A, uint8_t *__restrict__ ancT, int OWC, uint8_t *gat, int gw,
-                                           unsigned long long &lastmin) {
+                                           unsigned long long &lastmin, uint32_t *endrow) {
   if (!cta_own) return;
   if (((i + 1) % KSS == 0) || (i == H - 1)) {
     const uint32_t d = (uint32_t)(fb - c0 + 128);
     const uint32_t a = ((k[0] + d) & 0xFFu) | (((k[1] + d - 1u) & 0xFFu) << 8) | (((k[2] + d - 2u) & 0xFFu) << 16) |
                        (((k[3] + d - 3u) & 0xFFu) << 24);
-    if (gw) *reinterpret_cast<uint32_t *>(gat + (size_t)(i / KSS) * gw + c0) = a;
+    if (TWO || gw) *reinterpret_cast<uint32_t *>(gat + (size_t)(i / KSS) * gw + c0) = a;
     else *reinterpret_cast<uint32_t *>(ancT + (size_t)(i / KSS) * OWC + (c0 - A)) = a;
   }
-  if (i == H - 1) {
+  if (TWO) {
+    if (i == H - 1)
+      *reinterpret_cast<uint4 *>(endrow + c0) = make_uint4(k[0] >> 8, k[1] >> 8, k[2] >> 8, k[3] >> 8);
+  } else if (i == H - 1) {
 #pragma unroll
     for (int u = 0; u < V; ++u) {
       if (c0 + u < W) {
@@ -288,9 +297,8 @@ __device__ __forceinline__ void dp_rows_n_fwd(uint32_t (&k)[V], const uint16_t *
 
 // Initialise the staging and halo mbarriers (thread 0; the caller then synchronises the CTA, and
 // the cluster when CL).
-template <int NW, int KT, bool CL, int FWM = FILL_WARPS_MAX, bool FWD = false, int KSS = KS, bool DIRECT = false>
-__device__ inline void search_init(unsigned char *smem, int S) {
-  const SearchPlan plan = search_plan<NW, KT, CL, FWM, FWD, KSS, DIRECT>(S);
+template <int NW>
+__device__ inline void search_init(unsigned char *smem, const SearchPlan &plan) {
   uint64_t *full = reinterpret_cast<uint64_t *>(smem + plan.bars);
   uint64_t *empty = full + NSLOT;
   uint64_t *hbar = empty + NSLOT;
@@ -311,7 +319,7 @@ __device__ __forceinline__ void group_sync() {
 }
 
 // The parallel backtrack of seam_search: each fill warp walks its super-tiles (rows s*KSS ..
-// s*KSS+KSS-1, s = warp*cs + rank, + FW*cs, ...). The ancestor chain has fixed both ends of the
+// s*KSS+KSS-1, s = s_first, s_first + FW*cs, ...). The ancestor chain has fixed both ends of the
 // seam inside a super-tile: column jb[s] in its bottom row and column jb[s-1] in the row above it
 // (row 0's column for s = 0), and the seam between them is the leftmost cheapest path from one to
 // the other. So the fill is a small search of its own: costs start at 0 in the upper end and at
@@ -340,11 +348,12 @@ struct FillCtx {
   int32_t *seam, *seam_log;
   int *err;
   int64_t pstride;
-  int pitch_e, H, W, Wa, S, rank, cs;
+  int pitch_e, H, W, Wa, S, cs;
+  int step = 1;        // seam entries from one row to the next (-1: the map is swept from its bottom row)
 };
 
 template <int NW, int KT, bool CL, int FWM, bool FWD, int KSS, bool DIRECT, int CH>
-__device__ __forceinline__ void backtrack_fill(const FillCtx &f, int warp, int lane) {
+__device__ __forceinline__ void backtrack_fill(const FillCtx &f, int s_first, int warp, int lane) {
   using G = Geo<NW, KT, CL, FWM, KSS>;
   constexpr int NP = FWD ? 3 : 1;   // cost planes per row
   constexpr int FV = G::FV, FILLW = G::FILLW;
@@ -357,7 +366,7 @@ __device__ __forceinline__ void backtrack_fill(const FillCtx &f, int warp, int l
   int *const errw = f.err;
   const int *const jb0 = f.jb0;
   const int64_t pstride = f.pstride;
-  const int pitch_e = f.pitch_e, H = f.H, W = f.W, Wa = f.Wa, S = f.S, rank = f.rank, cs = f.cs;
+  const int pitch_e = f.pitch_e, H = f.H, W = f.W, Wa = f.Wa, S = f.S, cs = f.cs;
   // the energies of a super-tile's diamond (KSS rows, two rows per lane at most) are prefetched
   // into L2 one super-tile ahead: the map may have left L2 since the DP pass read it. The
   // prefetch starts on a 16-byte boundary and covers the diamond.
@@ -385,7 +394,7 @@ __device__ __forceinline__ void backtrack_fill(const FillCtx &f, int warp, int l
       x[2 * q + 1] = (w[q] >> 16) << 2;
     }
   };
-  for (int s = warp * cs + rank; s < S; s += G::FW * cs) {
+  for (int s = s_first; s < S; s += G::FW * cs) {
     prefetch_window(s + G::FW * cs);
     const int jbs = jb0[s];
     const int jprev = (s > 0) ? jb0[s - 1] : jb0[S];
@@ -481,8 +490,8 @@ __device__ __forceinline__ void backtrack_fill(const FillCtx &f, int warp, int l
     __syncwarp();
     for (int i = first + lane; i < re; i += 32) {
       const int j = x0 + (int)*reinterpret_cast<const uint32_t *>(fd + (i - rs) * FILLW);
-      seam_out[i] = j;
-      if (seam_log) seam_log[i] = j;
+      seam_out[i * f.step] = j;
+      if (seam_log) seam_log[i * f.step] = j;
     }
     if (s == 0 && lane == 0) {
       seam_out[0] = jprev;
@@ -496,14 +505,17 @@ __device__ __forceinline__ void backtrack_fill(const FillCtx &f, int warp, int l
 // the one-CTA batched kernel, whose 512 threads have at most 128 registers each, can load deeper
 // energy chunks
 template <int NW, int KT, bool CL, int FWM, bool FWD, int KSS, bool DIRECT, int CH>
-static __device__ __noinline__ void backtrack_fill_call(FillCtx f, int warp, int lane) {
-  backtrack_fill<NW, KT, CL, FWM, FWD, KSS, DIRECT, CH>(f, warp, lane);
+static __device__ __noinline__ void backtrack_fill_call(FillCtx f, int s_first, int warp, int lane) {
+  backtrack_fill<NW, KT, CL, FWM, FWD, KSS, DIRECT, CH>(f, s_first, warp, lane);
 }
 
-// The search. Every thread of the CTA (of every CTA of the cluster when CL) calls it with the same
-// arguments; `Smax` is the super-tile count the shared-memory plan was sized for.
-template <int NW, int KT, bool CL, int FWM = FILL_WARPS_MAX, bool FWD = false, int KSS = KS, bool DIRECT = false>
-__device__ void seam_search(const SearchArgs &p, unsigned char *smem, int Smax, SearchState &st) {
+// The row loop: every thread of the CTA (of every CTA of the cluster when CL) calls it with the same
+// arguments; `plan` is the shared-memory plan. Returns the thread's minimum of the last row
+// (M << 32 | column). With TWO (half of a two-ended search) the ancestors go to the global table
+// p.gtab (row stride p.gw) and the last row's costs to p.endrow instead.
+template <int NW, int KT, bool CL, int FWM, bool FWD, int KSS, bool DIRECT, bool TWO>
+__device__ __forceinline__ unsigned long long seam_sweep(const SearchArgs &p, unsigned char *smem, const SearchPlan &plan,
+                                                         SearchState &st) {
   static_assert(!DIRECT || (CL && !FWD), "the in-place form is built for the cluster search of e1 maps");
   constexpr int NP = FWD ? 3 : 1;   // cost planes staged per row
   // the single-map search: one cluster, a CTA per SM, every compute warp alone on its SM
@@ -516,24 +528,16 @@ __device__ void seam_search(const SearchArgs &p, unsigned char *smem, int Smax, 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const bool producer = (warp == NW);
   const int H = p.H, W = p.W;
-  const int S = (H + KSS - 1) / KSS;
-  const SearchPlan plan = search_plan<NW, KT, CL, FWM, FWD, KSS, DIRECT>(Smax);
   uint32_t *bnd = reinterpret_cast<uint32_t *>(smem + plan.bnd);
   uint32_t *hbuf = reinterpret_cast<uint32_t *>(smem + plan.hbuf);
   uint8_t *ancT = reinterpret_cast<uint8_t *>(smem + plan.anc);
-  unsigned long long *wmin = reinterpret_cast<unsigned long long *>(smem + plan.wmin);
-  unsigned long long *cmin = reinterpret_cast<unsigned long long *>(smem + plan.cmin);
-  int *jb = reinterpret_cast<int *>(smem + plan.jb);
-  int *misc = reinterpret_cast<int *>(smem + plan.misc);
   uint32_t *emx = reinterpret_cast<uint32_t *>(smem + plan.emx);   // DIRECT: [NW + 1] per warp, then per CTA
-  uint8_t *fdir = smem + plan.fdir;
   uint16_t *ring = reinterpret_cast<uint16_t *>(smem + plan.ring);
   uint64_t *full = reinterpret_cast<uint64_t *>(smem + plan.bars);
   uint64_t *empty = full + NSLOT;
   uint64_t *hbar = empty + NSLOT;
-  const int gw = plan.gw;
-  uint8_t *const gat = smem + plan.gat;
-  uint8_t *const gat0 = (CL && gw) ? cg::this_cluster().map_shared_rank(gat, 0) : gat;
+  const int gw = TWO ? p.gw : plan.gw;
+  uint8_t *const gat0 = TWO ? p.gtab : ((CL && gw) ? cg::this_cluster().map_shared_rank(smem + plan.gat, 0) : smem + plan.gat);
 
   // geometry
   const int A = rank * OWC, B = A + OWC;
@@ -584,7 +588,7 @@ __device__ void seam_search(const SearchArgs &p, unsigned char *smem, int Smax, 
 #pragma unroll
         for (int pl = 0; pl < NP; ++pl)
           bulk_g2s(ring + (size_t)((slot * NP + pl) * KT + lane) * BW + (clo - cbeg),
-                   Estage + pl * pstride + (size_t)(rbeg + lane) * pitch_e + (clo - cbeg), COPY_BYTES, &full[slot]);
+                   Estage + pl * pstride + (ptrdiff_t)(rbeg + lane) * pitch_e + (clo - cbeg), COPY_BYTES, &full[slot]);
       }
     }
   } else if (!active) {
@@ -638,7 +642,8 @@ __device__ void seam_search(const SearchArgs &p, unsigned char *smem, int Smax, 
           __syncwarp();
           if (lane == 0) mbar_arrive(&empty[slot]);   // this warp is done with the staged rows
           if (((r0 + KT) % KSS) == 0 || r0 + KT == H)
-            row_events<KSS>(r0 + KT - 1, k, H, W, c0, frame_base, cta_own, A, ancT, OWC, gat0, gw, lastmin);
+            row_events<KSS, TWO>(r0 + KT - 1, k, H, W, c0, frame_base, cta_own, A, ancT, OWC, gat0, gw,
+                                 lastmin, p.endrow);
         } else {
           // first tile (row 0 has no predecessor) or a ragged last tile. Neither holds a row with
           // bookkeeping except the image's last row and the first tile's last row when KSS = KT:
@@ -658,7 +663,8 @@ __device__ void seam_search(const SearchArgs &p, unsigned char *smem, int Smax, 
           __syncwarp();
           if (lane == 0) mbar_arrive(&empty[slot]);
           if (((r0 + n) % KSS) == 0 || r0 + n == H)
-            row_events<KSS>(r0 + n - 1, k, H, W, c0, frame_base, cta_own, A, ancT, OWC, gat0, gw, lastmin);
+            row_events<KSS, TWO>(r0 + n - 1, k, H, W, c0, frame_base, cta_own, A, ancT, OWC, gat0, gw,
+                                 lastmin, p.endrow);
         }
         if (more) {
           const bool exch = CL && ((r0 + KT) % K2 == 0) && cs > 1;
@@ -705,6 +711,33 @@ __device__ void seam_search(const SearchArgs &p, unsigned char *smem, int Smax, 
   if (DIRECT && lane == 0 && (producer || !active)) emx[warp] = 0u;
   st.tiles += (uint32_t)nt;
   if (CL && nt > 0) st.exch += (uint32_t)((cs > 1) ? ((H - 1) / K2) : 0);
+  return lastmin;
+}
+
+// The search. Every thread of the CTA (of every CTA of the cluster when CL) calls it with the same
+// arguments; `Smax` is the super-tile count the shared-memory plan was sized for.
+template <int NW, int KT, bool CL, int FWM = FILL_WARPS_MAX, bool FWD = false, int KSS = KS, bool DIRECT = false>
+__device__ void seam_search(const SearchArgs &p, unsigned char *smem, int Smax, SearchState &st) {
+  using G = Geo<NW, KT, CL, FWM, KSS>;
+  constexpr int OWC = G::OWC;
+  const int rank = CL ? (int)cg::this_cluster().block_rank() : 0;
+  const int cs = CL ? (int)cg::this_cluster().num_blocks() : 1;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int H = p.H, W = p.W, Wa = (W + 7) & ~7;
+  const int S = (H + KSS - 1) / KSS;
+  const SearchPlan plan = search_plan<NW, KT, CL, FWM, FWD, KSS, DIRECT>(Smax);
+  uint8_t *ancT = reinterpret_cast<uint8_t *>(smem + plan.anc);
+  unsigned long long *wmin = reinterpret_cast<unsigned long long *>(smem + plan.wmin);
+  unsigned long long *cmin = reinterpret_cast<unsigned long long *>(smem + plan.cmin);
+  int *jb = reinterpret_cast<int *>(smem + plan.jb);
+  int *misc = reinterpret_cast<int *>(smem + plan.misc);
+  uint32_t *emx = reinterpret_cast<uint32_t *>(smem + plan.emx);   // DIRECT: [NW + 1] per warp, then per CTA
+  uint8_t *fdir = smem + plan.fdir;
+  const int gw = plan.gw;
+  uint8_t *const gat = smem + plan.gat;
+  const int64_t pstride = FWD ? p.pstride : 0;
+
+  unsigned long long lastmin = seam_sweep<NW, KT, CL, FWM, FWD, KSS, DIRECT, false>(p, smem, plan, st);
 
   // ---- last-row argmin: the leftmost minimum (min of (M << 32) | column) ----
 #pragma unroll
@@ -779,17 +812,17 @@ __device__ void seam_search(const SearchArgs &p, unsigned char *smem, int Smax, 
   const int ok = misc0[0];
   if (ok && warp < G::FW) {
     const FillCtx f{p.E, jb0, fdir, const_cast<uint32_t *>(reinterpret_cast<const uint32_t *>(misc0 + 1)), p.seam,
-                    p.seam_log, p.err, pstride, pitch_e, H, W, Wa, S, rank, cs};
+                    p.seam_log, p.err, pstride, p.pitch_e, H, W, Wa, S, cs};
     // energy chunks: the single-map search (all fill warps, one CTA per SM, latency-bound) has
     // registers to spare and keeps 32 rows of loads in flight; the multi-map and cluster batched
     // kernels, whose latency other CTAs hide and whose registers are capped, use 8-row chunks; the
     // one-CTA batched kernel calls the fill as a function of its own (the same call in the cluster
     // batched kernel was slower, so that one stays inline).
     if constexpr (!CL && !FWD) {
-      backtrack_fill_call<NW, KT, CL, FWM, FWD, KSS, DIRECT, 8>(f, warp, lane);
+      backtrack_fill_call<NW, KT, CL, FWM, FWD, KSS, DIRECT, 8>(f, warp * cs + rank, warp, lane);
     } else {
       constexpr int CH = FWD ? 4 : ((CL && FWM >= FILL_WARPS_MAX) ? 16 : 8);
-      backtrack_fill<NW, KT, CL, FWM, FWD, KSS, DIRECT, CH>(f, warp, lane);
+      backtrack_fill<NW, KT, CL, FWM, FWD, KSS, DIRECT, CH>(f, warp * cs + rank, warp, lane);
     }
   }
   group_sync<CL>();   // rank 0's shared memory is read above; the seam is complete after this
