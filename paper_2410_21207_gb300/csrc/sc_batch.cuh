@@ -152,7 +152,7 @@ __global__ void __launch_bounds__(Geo<NW, KT, false>::THREADS, 1)
   // the current image's descriptor lives in shared memory and its fields are read where they are
   // used, so they do not occupy registers across the seam loop
   __shared__ BatchItem cur;
-  search_init<NW>(smem, search_plan<NW, KT, false, batch_fill_warps(NW, KT)>(Smax));
+  search_init(smem, search_plan<NW, KT, false, batch_fill_warps(NW, KT)>(Smax));
   __syncthreads();
   SearchState st;
   for (;;) {

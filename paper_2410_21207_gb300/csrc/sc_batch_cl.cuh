@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(Geo<NW, KT, true, FWM>::THREADS, 1)
   pdl_launch_dependents();
   cg::cluster_group cl = cg::this_cluster();
   const int rank = (int)cl.block_rank(), cs = (int)cl.num_blocks();
-  search_init<NW>(smem, search_plan<NW, KT, true, FWM>(Smax));
+  search_init(smem, search_plan<NW, KT, true, FWM>(Smax));
   cl.sync();
   SearchState st;
   for (;;) {

@@ -1,6 +1,11 @@
 // One seam search per launch (the per-seam path of the carve and sc_find_seam): maps of at least
 // TWO_MIN_ROWS rows from both ends by two thread-block clusters (k_dp_two), shorter ones and forward
 // energy by one cluster (k_dp, seam_search in sc_search.cuh).
+#include <atomic>
+
+#include <cuda.h>
+#include <cudaTypedefs.h>
+
 #include "sc_search.cuh"
 
 namespace sc {
@@ -35,11 +40,12 @@ template <int NW, int KT, bool FWD>
 __host__ __device__ constexpr int dp_super_rows() { return (NW == 4 && KT == 32 && !FWD) ? KS : KS_WIDE; }
 
 template <int NW, int KT, bool FWD = false>
-__global__ void __launch_bounds__(Geo<NW, KT, true>::THREADS, 1) k_dp(DpArgs p) {
-  extern __shared__ __align__(16) unsigned char smem[];
+__global__ void __launch_bounds__(Geo<NW, KT, true>::THREADS, 1)
+    k_dp(DpArgs p, const __grid_constant__ CUtensorMap tmap) {
+  extern __shared__ __align__(128) unsigned char smem[];
   constexpr int KSS = dp_super_rows<NW, KT, FWD>();
   const int S = (p.H + KSS - 1) / KSS;
-  search_init<NW>(smem, search_plan<NW, KT, true, FILL_WARPS_MAX, FWD, KSS>(S));
+  search_init(smem, search_plan<NW, KT, true, FILL_WARPS_MAX, FWD, KSS>(S));
   // neighbours push into each other's halo buffers: every CTA's barriers must be initialised first
   cg::this_cluster().sync();
   // the set-up above overlaps the previous kernel of the seam loop; its results are read below
@@ -56,13 +62,16 @@ __global__ void __launch_bounds__(Geo<NW, KT, true>::THREADS, 1) k_dp(DpArgs p) 
   a.err = p.err;
   a.gated = (p.gate != nullptr) && (*p.gate & ERR_ENERGY_RANGE);
   a.pstride = p.pstride;
+  a.tmap = &tmap;
+  a.plane_rows = FWD ? (int)(p.pstride / p.pitch_e) : 0;
   SearchState st;
-  seam_search<NW, KT, true, FILL_WARPS_MAX, FWD, KSS>(a, smem, S, st);
+  seam_search<NW, KT, true, FILL_WARPS_MAX, FWD, KSS, false, true>(a, smem, S, st);
 }
 
 // one or two clusters of cs CTAs; a programmatic dependent (may start before its predecessor ends)
-static cudaError_t launch_dp_cluster(void (*kernel)(DpArgs), int grid, int cs, int threads, size_t smem,
-                                     cudaStream_t st, const DpArgs &a) {
+template <typename... KArgs, typename... Args>
+static cudaError_t launch_dp_cluster(void (*kernel)(KArgs...), int grid, int cs, int threads, size_t smem,
+                                     cudaStream_t st, const Args &...args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(threads);
@@ -77,7 +86,29 @@ static cudaError_t launch_dp_cluster(void (*kernel)(DpArgs), int grid, int cs, i
   at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, kernel, a);
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+// Tensor map of `rows` rows of pitch elements (base: 16-byte aligned), copied in boxes of KT rows, BW
+// columns split into equal parts of at most 256. The driver's encoder is looked up once.
+static cudaError_t energy_tensor_map(CUtensorMap *m, const uint16_t *base, int pitch, int rows, int BW, int KT) {
+  static std::atomic<PFN_cuTensorMapEncodeTiled_v12000> encode{nullptr};
+  PFN_cuTensorMapEncodeTiled_v12000 fn = encode.load();
+  if (!fn) {
+    void *ptr = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    const cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &ptr, 12000, cudaEnableDefault, &q);
+    if (e != cudaSuccess) return e;
+    if (q != cudaDriverEntryPointSuccess || !ptr) return cudaErrorNotSupported;
+    fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(ptr);
+    encode.store(fn);
+  }
+  const cuuint64_t dims[2] = {(cuuint64_t)pitch, (cuuint64_t)rows}, strides[1] = {(cuuint64_t)pitch * 2};
+  const cuuint32_t box[2] = {(cuuint32_t)(BW / ((BW + 255) / 256)), (cuuint32_t)KT}, es[2] = {1, 1};
+  const CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_UINT16, 2, const_cast<uint16_t *>(base), dims, strides, box, es,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
 template <int NW, int KT, bool FWD = false>
@@ -93,7 +124,11 @@ static cudaError_t launch_dp_shape(const DpArgs &a, int cs, cudaStream_t st) {
     configured = true;
   }
   if (smem > 232448) return cudaErrorInvalidValue;
-  return launch_dp_cluster(k_dp<NW, KT, FWD>, cs, cs, Geo<NW, KT, true>::THREADS, smem, st, a);
+  CUtensorMap tmap;
+  const int rows = a.H + (FWD ? (int)(2 * a.pstride / a.pitch_e) : 0);   // the three planes in a row
+  const cudaError_t e = energy_tensor_map(&tmap, a.E - E_PADL, a.pitch_e, rows, Geo<NW, KT, true>::BW, KT);
+  if (e != cudaSuccess) return e;
+  return launch_dp_cluster(k_dp<NW, KT, FWD>, cs, cs, Geo<NW, KT, true>::THREADS, smem, st, a, tmap);
 }
 
 // ---- the two-ended search ----
@@ -106,8 +141,8 @@ static cudaError_t launch_dp_shape(const DpArgs &a, int cs, cudaStream_t st) {
 //     U(j) that from the bottom row to column j of the row below it, the seam costs the minimum of
 //     D(j) + min(U(j-1), U(j), U(j+1)); its columns in those two rows are the leftmost j and the
 //     leftmost of the three that reach it;
-//   * each half's ancestors give the seam's columns at its super-tile boundaries, towards row 0 and
-//     towards the bottom row: two chains that one warp follows side by side, half as many hops each;
+//   * each half's ancestors give the seam's columns at its super-tile boundaries, towards the top and
+//     towards the bottom: two chains that one warp follows side by side, half as many hops each;
 //   * the super-tiles of both halves are then backtracked in parallel as in seam_search.
 // No cluster waits for the other: both leave their last cost row and their ancestor table in
 // global memory, count themselves in, and the cluster that holds the last CTA to arrive does the rest
@@ -137,7 +172,9 @@ struct Two {
   size_t tbar;           // mbarrier of that copy
 
   __host__ __device__ Two(int H, int cs) {
-    H0 = (H + 1) / 2;
+    // a whole number of tiles in the upper half where there is a choice: only one half then ends on a
+    // ragged tile
+    H0 = ((H + 1) / 2 + KT - 1) / KT * KT;
     H1 = H - H0;
     S0 = (H0 + KSS - 1) / KSS;
     S1 = (H1 + KSS - 1) / KSS;
@@ -158,21 +195,23 @@ struct Two {
     plan.misc = take(16);   // [0] this cluster arrived last, [1] path cost sum (rank 0), [2] chain found
     plan.anc = plan.emx = plan.gat = 0;
     plan.gw = 0;
-    plan.bars = take((size_t)(2 * NSLOT + 3) * 8);
-    tbar = plan.bars + (size_t)(2 * NSLOT + 2) * 8;
+    plan.bars = take((size_t)(NSLOT + 3) * 8);
+    tbar = plan.bars + (size_t)(NSLOT + 2) * 8;
     // the staging ring; after the sweep its place holds the tables, then the fills' directions
     size_t r = (size_t)NSLOT * KT * G::BW * 2;
     const size_t fd = (size_t)G::FW * KSS * G::FILLW;
     r = r > fd ? r : fd;
     if (tab && tab_bytes > r) r = tab_bytes;
+    o = (o + 127) & ~(size_t)127;
     plan.ring = plan.fdir = take(r);
     plan.total = o;
   }
 };
 
 template <int NW, int KT>
-__global__ void __launch_bounds__(Geo<NW, KT, true>::THREADS, 1) k_dp_two(DpArgs p) {
-  extern __shared__ __align__(16) unsigned char smem[];
+__global__ void __launch_bounds__(Geo<NW, KT, true>::THREADS, 1)
+    k_dp_two(DpArgs p, const __grid_constant__ CUtensorMap tmap) {
+  extern __shared__ __align__(128) unsigned char smem[];
   using T = Two<NW, KT>;
   using G = typename T::G;
   constexpr int KSS = T::KSS;
@@ -185,11 +224,12 @@ __global__ void __launch_bounds__(Geo<NW, KT, true>::THREADS, 1) k_dp_two(DpArgs
   int *jb = reinterpret_cast<int *>(smem + plan.jb);
   int *misc = reinterpret_cast<int *>(smem + plan.misc);
   uint64_t *tbar = reinterpret_cast<uint64_t *>(smem + g.tbar);
-  search_init<NW>(smem, plan);
+  search_init(smem, plan);
   if (threadIdx.x == 0) {
     mbar_init(tbar, 1);
     fence_mbar_init();
     misc[0] = 0;
+    prefetch_tensormap(&tmap);
   }
   // neighbours push into each other's halo buffers: every CTA's barriers must be initialised first
   cl.sync();
@@ -212,8 +252,11 @@ __global__ void __launch_bounds__(Geo<NW, KT, true>::THREADS, 1) k_dp_two(DpArgs
     a.gtab = tab + (half ? (size_t)g.S0 * g.gw : 0);
     a.gw = g.gw;
     a.endrow = half ? end1 : end0;
+    a.tmap = &tmap;
+    a.y0 = half ? p.H - 1 : 0;
     SearchState st;
-    seam_sweep<NW, KT, true, FILL_WARPS_MAX, false, KSS, false, true>(a, smem, plan, st);
+    if (half) seam_sweep<NW, KT, true, FILL_WARPS_MAX, false, KSS, false, true, true, true>(a, smem, plan, st);
+    else seam_sweep<NW, KT, true, FILL_WARPS_MAX, false, KSS, false, true, true, false>(a, smem, plan, st);
   }
   // ---- count this CTA in; the cluster of the last one goes on ----
   fence_proxy_async_global();   // the tables are read by a bulk copy below
@@ -335,7 +378,10 @@ static cudaError_t launch_dp_two(const DpArgs &a, int cs, cudaStream_t st) {
     configured = true;
   }
   if (smem > SEARCH_SMEM_LIMIT) return cudaErrorInvalidValue;
-  return launch_dp_cluster(k_dp_two<NW, KT>, 2 * cs, cs, Geo<NW, KT, true>::THREADS, smem, st, a);
+  CUtensorMap tmap;
+  const cudaError_t e = energy_tensor_map(&tmap, a.E - E_PADL, a.pitch_e, a.H, Geo<NW, KT, true>::BW, KT);
+  if (e != cudaSuccess) return e;
+  return launch_dp_cluster(k_dp_two<NW, KT>, 2 * cs, cs, Geo<NW, KT, true>::THREADS, smem, st, a, tmap);
 }
 
 // forward energy stages three planes per row: one shape, 4 warps x 16-row tiles (W <= 4096)

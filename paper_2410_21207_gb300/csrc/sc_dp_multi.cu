@@ -26,7 +26,7 @@ __global__ void __launch_bounds__(Geo<NW, KT, true>::THREADS, NW == 8 ? 2 : 4) k
   const int img = blockIdx.x / cg::this_cluster().num_blocks();
   const DpArgs p = ps ? ps[img] : inl.a[img];
   const int S = (p.H + KS - 1) / KS;
-  search_init<NW>(smem, search_plan<NW, KT, true, MULTI_FILL_WARPS, false, KS, true>(S));
+  search_init(smem, search_plan<NW, KT, true, MULTI_FILL_WARPS, false, KS, true>(S));
   cg::this_cluster().sync();
   SearchArgs a;
   a.E = p.E;

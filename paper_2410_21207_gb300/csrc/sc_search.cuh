@@ -26,11 +26,12 @@
 //     between its two boundary columns in a 2*KSS-column window (KSS/16 columns per lane) with
 //     explicit directions.
 //   * Energies are staged in shared memory by TMA: a producer warp issues one bulk copy per row
-//     (one row per lane) into an NSLOT-slot ring, gated by full/empty mbarriers; a lane reads its 4
-//     energies of a row with one 8-byte shared-memory load.
-//   * The rows of a tile are branch-free (row 0 initialises from its energies; a ragged last tile
-//     runs a counted loop), and per-super-tile bookkeeping runs after the tile, on its last row
-//     (the only row of a tile where it can occur, since KSS is a multiple of KT).
+//     (one row per lane) into an NSLOT-slot ring, waits for the next tile to land and joins the CTA
+//     barrier that ends the current one, which also frees its slot; a lane reads its 4 energies of a
+//     row with one 8-byte shared-memory load.
+//   * The rows of a tile are branch-free (the map has an added row of cost 0 above row 0), and
+//     per-super-tile bookkeeping runs after the tile, on its last row (the only row of a tile where
+//     it can occur, since KSS is a multiple of KT).
 // The result is Algorithm 3's seam exactly (leftmost ties, leftmost last-row minimum).
 // With DIRECT the map is the caller's own H x W array (any row pitch that is a multiple of 8
 // elements, 16-byte aligned rows), read in place: the row copies are clipped to the map's columns,
@@ -96,9 +97,10 @@ __host__ __device__ inline SearchPlan search_plan(int S) {
   // staged tile has been consumed before the argmin), unless the ring is the smaller of the two
   const size_t fdir_sz = (size_t)G::FW * KSS * G::FILLW, ring_sz = (size_t)NSLOT * (FWD ? 3 : 1) * KT * G::BW * 2;
   if (fdir_sz > ring_sz) { p.fdir = o; o += fdir_sz;  o = (o + 15) & ~(size_t)15; }
+  o = (o + 127) & ~(size_t)127;   // (tensor copies: 128-byte aligned)
   p.ring = o; o += ring_sz;  o = (o + 15) & ~(size_t)15;
   if (fdir_sz <= ring_sz) p.fdir = p.ring;
-  p.bars = o; o += (size_t)(2 * NSLOT + 2) * 8;   // full[NSLOT], empty[NSLOT], halo[2]
+  p.bars = o; o += (size_t)(NSLOT + 2) * 8;   // full[NSLOT], halo[2]
   o = (o + 15) & ~(size_t)15;
   // single-map cluster search: every CTA writes its super-tile ancestors straight into rank 0's
   // table (remote stores during the row loop), so the chain after the argmin is all local loads;
@@ -130,6 +132,8 @@ struct SearchArgs {
   uint8_t *gtab = nullptr;
   int gw = 0;
   uint32_t *endrow = nullptr;
+  const void *tmap = nullptr;   // tensor map of the energy buffer (rows of pitch_e elements)
+  int y0 = 0, plane_rows = 0;   // its row of this half's row 0; rows from one cost plane to the next
 };
 
 // Running counters of the mbarrier phases, identical in every thread of the CTA.
@@ -144,35 +148,12 @@ __device__ __forceinline__ uint32_t min3u(uint32_t a, uint32_t b, uint32_t c) { 
 __device__ __forceinline__ uint32_t lo8(uint32_t x) { return __byte_perm(x, 0u, 0x4104); }
 __device__ __forceinline__ uint32_t hi8(uint32_t x) { return __byte_perm(x, 0u, 0x4324); }
 
-// Bookkeeping after row i (keys k of this lane's V columns, warp frame base fb):
-//  - bottom of a super-tile: record the ancestors of the CTA-own columns (one byte: a - col + 128),
-//    in rank 0's gathered table (row stride gw) when there is one, else in this CTA's table;
-//  - last row of the image: fold the lane's (M << 32 | column) minimum, or, where the sweep ends in
-//    the middle of the map (TWO), store the cost row.
-template <int KSS, bool TWO>
-__device__ __forceinline__ void row_events(int i, const uint32_t (&k)[V], int H, int W, int c0, int fb, bool cta_own,
-                                           int A, uint8_t *__restrict__ ancT, int OWC, uint8_t *gat, int gw,
-                                           unsigned long long &lastmin, uint32_t *endrow) {
-  if (!cta_own) return;
-  if (((i + 1) % KSS == 0) || (i == H - 1)) {
-    const uint32_t d = (uint32_t)(fb - c0 + 128);
-    const uint32_t a = ((k[0] + d) & 0xFFu) | (((k[1] + d - 1u) & 0xFFu) << 8) | (((k[2] + d - 2u) & 0xFFu) << 16) |
-                       (((k[3] + d - 3u) & 0xFFu) << 24);
-    if (TWO || gw) *reinterpret_cast<uint32_t *>(gat + (size_t)(i / KSS) * gw + c0) = a;
-    else *reinterpret_cast<uint32_t *>(ancT + (size_t)(i / KSS) * OWC + (c0 - A)) = a;
-  }
-  if (TWO) {
-    if (i == H - 1)
-      *reinterpret_cast<uint4 *>(endrow + c0) = make_uint4(k[0] >> 8, k[1] >> 8, k[2] >> 8, k[3] >> 8);
-  } else if (i == H - 1) {
-#pragma unroll
-    for (int u = 0; u < V; ++u) {
-      if (c0 + u < W) {
-        const unsigned long long c = ((unsigned long long)(k[u] >> 8) << 32) | (unsigned)(c0 + u);
-        lastmin = c < lastmin ? c : lastmin;
-      }
-    }
-  }
+// The ancestors of this lane's V columns (one byte each: a - column + 128) from its keys; c0: the
+// lane's first column, fb: the warp's frame base.
+__device__ __forceinline__ uint32_t pack_ancestors(const uint32_t (&k)[V], int c0, int fb) {
+  const uint32_t d = (uint32_t)(fb - c0 + 128);
+  return ((k[0] + d) & 0xFFu) | (((k[1] + d - 1u) & 0xFFu) << 8) | (((k[2] + d - 2u) & 0xFFu) << 16) |
+         ((k[3] + d - 3u) << 24);
 }
 
 // key + energy, forced to SENT where the mask is SENT (outside the image). max(x + e, mask) equals
@@ -220,37 +201,45 @@ __device__ __forceinline__ void emax_acc(uint32_t &acc, uint2 ev, uint2 cm) {
   if (CHK) acc = __vimax3_u16x2(acc, MASK ? (ev.x & cm.x) : ev.x, MASK ? (ev.y & cm.y) : ev.y);
 }
 
-// KT rows of a full tile from the staged energies er (row stride BW); MASK applies oobm.
-template <int KT, int BW, bool MASK, bool LAT = false, bool CHK = false>
-__device__ __forceinline__ void dp_rows(uint32_t (&k)[V], const uint16_t *er, const uint32_t (&oobm)[V],
+// n rows (n <= KT) of a tile from the staged energies er (row stride BW; REV: upwards), the energies
+// loaded two rows ahead of the row that needs them, off the dependent chain: in blocks of U unrolled
+// rows, and the last n % U rows of a ragged tile in blocks of 8 and then one by one. MASK applies
+// oobm. The latency-bound search unrolls whole tiles (33 cycles a row at 4 warps; 37.6 in blocks of
+// 8), the batched and multi-map kernels blocks of 8 (several warps hide the loop).
+template <int U, int BW, bool MASK, bool LAT = false, bool CHK = false, bool REV = false>
+__device__ __forceinline__ void dp_rows(uint32_t (&k)[V], const uint16_t *er, const uint32_t (&oobm)[V], int n,
                                         uint32_t &acc, uint2 cm) {
-  uint2 a = *reinterpret_cast<const uint2 *>(er);
-  uint2 b = *reinterpret_cast<const uint2 *>(er + BW);
+  constexpr int RS = REV ? -BW : BW;
+  auto row = [&](int r) { return *reinterpret_cast<const uint2 *>(er + r * RS); };
+  if (n >= U) {
+    uint2 a = row(0), b = row(1);
+    auto block = [&](auto more) {
 #pragma unroll
-  for (int r = 0; r < KT; ++r) {
-    const uint2 ev = a;
-    a = b;
-    if (r + 2 < KT) b = *reinterpret_cast<const uint2 *>(er + (r + 2) * BW);
-    dp_row<MASK, LAT>(k, ev, oobm);
-    emax_acc<CHK, MASK>(acc, ev, cm);
+      for (int r = 0; r < U; ++r) {
+        const uint2 ev = a;
+        a = b;
+        if (decltype(more)::value || r + 2 < U) b = row(r + 2);
+        dp_row<MASK, LAT>(k, ev, oobm);
+        emax_acc<CHK, MASK>(acc, ev, cm);
+      }
+      er += U * RS;
+      n -= U;
+    };
+    if (U == 8) {
+#pragma unroll 1
+      while (n >= 2 * U) block(std::true_type());
+    }
+    block(std::false_type());
   }
-}
-
-// Rows rb .. n-1 (n <= KT) of a tile: the first tile (rb = 1, row 0 initialises) or a ragged
-// last tile, at the pace of a full tile.
-template <int KT, int BW, bool MASK, bool LAT = false, bool CHK = false>
-__device__ __forceinline__ void dp_rows_n(uint32_t (&k)[V], const uint16_t *er, const uint32_t (&oobm)[V], int rb,
-                                          int n, uint32_t &acc, uint2 cm) {
-  uint2 a = *reinterpret_cast<const uint2 *>(er + rb * BW);
-  uint2 b = a;
-  if (rb + 1 < n) b = *reinterpret_cast<const uint2 *>(er + (rb + 1) * BW);
-#pragma unroll 2
-  for (int r = rb; r < n; ++r) {
-    const uint2 ev = a;
-    a = b;
-    if (r + 2 < n) b = *reinterpret_cast<const uint2 *>(er + (r + 2) * BW);
-    dp_row<MASK, LAT>(k, ev, oobm);
-    emax_acc<CHK, MASK>(acc, ev, cm);
+  if (U > 8) {
+    if (n > 0) dp_rows<8, BW, MASK, LAT, CHK, REV>(k, er, oobm, n, acc, cm);
+  } else {
+#pragma unroll 1
+    for (int r = 0; r < n; ++r) {
+      const uint2 ev = row(r);
+      dp_row<MASK, LAT>(k, ev, oobm);
+      emax_acc<CHK, MASK>(acc, ev, cm);
+    }
   }
 }
 
@@ -266,10 +255,10 @@ __device__ __forceinline__ void dp_row_fwd(uint32_t (&k)[V], uint2 cu, uint2 dl,
   k[0] = n0; k[1] = n1; k[2] = n2; k[3] = n3;
 }
 
-// KT forward-energy rows of a full tile; the three planes are KT rows apart in the staging ring.
-template <int KT, int BW, bool MASK>
+// KT forward-energy rows of a full tile (row stride BW); the three planes are PL elements apart in
+// the staging ring.
+template <int KT, int BW, int PL, bool MASK>
 __device__ __forceinline__ void dp_rows_fwd(uint32_t (&k)[V], const uint16_t *er, const uint32_t (&oobm)[V]) {
-  constexpr int PL = KT * BW;
   uint2 a0 = *reinterpret_cast<const uint2 *>(er), a1 = *reinterpret_cast<const uint2 *>(er + PL),
         a2 = *reinterpret_cast<const uint2 *>(er + 2 * PL);
 #pragma unroll
@@ -284,12 +273,10 @@ __device__ __forceinline__ void dp_rows_fwd(uint32_t (&k)[V], const uint16_t *er
   }
 }
 
-// Forward-energy rows rb .. n-1 (n <= KT) of a first or ragged last tile.
-template <int KT, int BW, bool MASK>
-__device__ __forceinline__ void dp_rows_n_fwd(uint32_t (&k)[V], const uint16_t *er, const uint32_t (&oobm)[V], int rb,
-                                              int n) {
-  constexpr int PL = KT * BW;
-  for (int r = rb; r < n; ++r)
+// n (n < KT) forward-energy rows of a ragged last tile.
+template <int BW, int PL, bool MASK>
+__device__ __forceinline__ void dp_rows_n_fwd(uint32_t (&k)[V], const uint16_t *er, const uint32_t (&oobm)[V], int n) {
+  for (int r = 0; r < n; ++r)
     dp_row_fwd<MASK>(k, *reinterpret_cast<const uint2 *>(er + r * BW),
                      *reinterpret_cast<const uint2 *>(er + PL + r * BW),
                      *reinterpret_cast<const uint2 *>(er + 2 * PL + r * BW), oobm);
@@ -297,16 +284,11 @@ __device__ __forceinline__ void dp_rows_n_fwd(uint32_t (&k)[V], const uint16_t *
 
 // Initialise the staging and halo mbarriers (thread 0; the caller then synchronises the CTA, and
 // the cluster when CL).
-template <int NW>
 __device__ inline void search_init(unsigned char *smem, const SearchPlan &plan) {
   uint64_t *full = reinterpret_cast<uint64_t *>(smem + plan.bars);
-  uint64_t *empty = full + NSLOT;
-  uint64_t *hbar = empty + NSLOT;
+  uint64_t *hbar = full + NSLOT;
   if (threadIdx.x == 0) {
-    for (int q = 0; q < NSLOT; ++q) {
-      mbar_init(&full[q], 1);
-      mbar_init(&empty[q], NW);
-    }
+    for (int q = 0; q < NSLOT; ++q) mbar_init(&full[q], 1);
     mbar_init(&hbar[0], 1);
     mbar_init(&hbar[1], 1);
     fence_mbar_init();
@@ -321,7 +303,7 @@ __device__ __forceinline__ void group_sync() {
 // The parallel backtrack of seam_search: each fill warp walks its super-tiles (rows s*KSS ..
 // s*KSS+KSS-1, s = s_first, s_first + FW*cs, ...). The ancestor chain has fixed both ends of the
 // seam inside a super-tile: column jb[s] in its bottom row and column jb[s-1] in the row above it
-// (row 0's column for s = 0), and the seam between them is the leftmost cheapest path from one to
+// (jb[S] in the added row above row 0 for s = 0), and the seam between them is the leftmost cheapest path from one to
 // the other. So the fill is a small search of its own: costs start at 0 in the upper end and at
 // infinity everywhere else, and only the cells within r columns of the upper end and n - r of the
 // lower end can be on the path (n rows, r of them down), a diamond at most n + 1 columns wide around
@@ -401,7 +383,6 @@ __device__ __forceinline__ void backtrack_fill(const FillCtx &f, int s_first, in
     const int x0 = (((jprev + jbs) >> 1) - FILLW / 2) & ~(FV - 1);
     const int xc = x0 + lane * FV;
     const int rs = s * KSS, re = (rs + KSS < H) ? rs + KSS : H;
-    const int first = (s == 0) ? 1 : rs;
     uint32_t m[FV], oob[FV];
 #pragma unroll
     for (int u = 0; u < FV; ++u) {
@@ -410,8 +391,7 @@ __device__ __forceinline__ void backtrack_fill(const FillCtx &f, int s_first, in
     }
     // DIRECT: a lane's FV columns lie wholly inside or wholly outside the caller's [0, Wa)
     const bool xin = !DIRECT || (xc >= 0 && xc + FV <= Wa);
-    if (s == 0 && xc <= jprev && jprev < xc + FV) atomicAdd(f.csum, (uint32_t)Ef[jprev]);   // row 0's cell
-    // rows first..re-1 in chunks of CH rows, the next chunk's energies loaded ahead
+    // rows rs..re-1 in chunks of CH rows, the next chunk's energies loaded ahead
     EVec eb0[NP][CH], eb1[NP][CH];
     auto load_chunk = [&](EVec (&eb)[NP][CH], int rbeg) {
 #pragma unroll
@@ -455,7 +435,7 @@ __device__ __forceinline__ void backtrack_fill(const FillCtx &f, int s_first, in
         *reinterpret_cast<DirT *>(fd + (i - rs) * FILLW + lane * FV) = (DirT)dirs;
       }
     };
-    int rb = first;
+    int rb = rs;
     load_chunk(eb0, rb);
     while (rb < re) {
       if (rb + CH < re) load_chunk(eb1, rb + CH);
@@ -479,7 +459,7 @@ __device__ __forceinline__ void backtrack_fill(const FillCtx &f, int s_first, in
       // a step leaving the window is clamped (every read stays in this warp's rows) and recorded as
       // a failure
       uint8_t *fb = fd + (re - 1 - rs) * FILLW;
-      for (int i = re - 1; i >= first; --i, fb -= FILLW) {
+      for (int i = re - 1; i >= rs; --i, fb -= FILLW) {
         const int nr = rel + (int)fb[rel] - 1;
         *reinterpret_cast<uint32_t *>(fb) = (uint32_t)rel;
         okp &= (unsigned)nr < (unsigned)FILLW;
@@ -488,14 +468,10 @@ __device__ __forceinline__ void backtrack_fill(const FillCtx &f, int s_first, in
       if (!okp || x0 + rel != jprev) atomicOr(errw, ERR_FILL_MISMATCH);
     }
     __syncwarp();
-    for (int i = first + lane; i < re; i += 32) {
+    for (int i = rs + lane; i < re; i += 32) {
       const int j = x0 + (int)*reinterpret_cast<const uint32_t *>(fd + (i - rs) * FILLW);
       seam_out[i * f.step] = j;
       if (seam_log) seam_log[i * f.step] = j;
-    }
-    if (s == 0 && lane == 0) {
-      seam_out[0] = jprev;
-      if (seam_log) seam_log[0] = jprev;
     }
     __syncwarp();
   }
@@ -513,7 +489,14 @@ static __device__ __noinline__ void backtrack_fill_call(FillCtx f, int s_first, 
 // arguments; `plan` is the shared-memory plan. Returns the thread's minimum of the last row
 // (M << 32 | column). With TWO (half of a two-ended search) the ancestors go to the global table
 // p.gtab (row stride p.gw) and the last row's costs to p.endrow instead.
-template <int NW, int KT, bool CL, int FWM, bool FWD, int KSS, bool DIRECT, bool TWO>
+// TM stages a tile's rows with tensor copies of p.tmap, NBOX boxes of KT rows side by side (a
+// row-by-row copy costs its warp about 65 cycles, 2,100 per 32-row tile: more than the tile's rows
+// take, so the producer paced the sweep); the box rows of the half swept upwards (REV) lie in reverse
+// order. Half a 1920x1080 map: 40,000 -> 29,700 cycles; 3840x2160: 88,500 -> 73,500; a forward-energy
+// carve at 1920x1080 (three planes: 48 row copies per 16-row tile) 60.3 -> 34.9 ms. The batched and
+// multi-map kernels keep the row copies: their maps have no tensor maps (a caller's, or one of a
+// batch's many), and several warps per SM sub-partition need longer for a tile than its copies.
+template <int NW, int KT, bool CL, int FWM, bool FWD, int KSS, bool DIRECT, bool TM, bool TWO = false, bool REV = false>
 __device__ __forceinline__ unsigned long long seam_sweep(const SearchArgs &p, unsigned char *smem, const SearchPlan &plan,
                                                          SearchState &st) {
   static_assert(!DIRECT || (CL && !FWD), "the in-place form is built for the cluster search of e1 maps");
@@ -534,8 +517,7 @@ __device__ __forceinline__ unsigned long long seam_sweep(const SearchArgs &p, un
   uint32_t *emx = reinterpret_cast<uint32_t *>(smem + plan.emx);   // DIRECT: [NW + 1] per warp, then per CTA
   uint16_t *ring = reinterpret_cast<uint16_t *>(smem + plan.ring);
   uint64_t *full = reinterpret_cast<uint64_t *>(smem + plan.bars);
-  uint64_t *empty = full + NSLOT;
-  uint64_t *hbar = empty + NSLOT;
+  uint64_t *hbar = full + NSLOT;
   const int gw = TWO ? p.gw : plan.gw;
   uint8_t *const gat0 = TWO ? p.gtab : ((CL && gw) ? cg::this_cluster().map_shared_rank(smem + plan.gat, 0) : smem + plan.gat);
 
@@ -552,7 +534,9 @@ __device__ __forceinline__ unsigned long long seam_sweep(const SearchArgs &p, un
   for (int u = 0; u < V; ++u) oobm[u] = (c0 + u < 0 || c0 + u >= W) ? SENT : 0u;
   const bool edge = __any_sync(0xffffffffu, (oobm[0] | oobm[V - 1]) != 0u);
   const int bidx0 = c0 - (ext0 - KT);           // index of c0 in bnd and in a staged energy row
-
+  constexpr int NBOX = TM ? (BW + 255) / 256 : 1;   // a tensor copy's rows hold at most 256 elements
+  constexpr int BWB = BW / NBOX;                     // staged row stride
+  static_assert(BWB * NBOX == BW && BWB % 8 == 0 && (KT * BWB * 2) % 128 == 0, "tensor box");
   unsigned long long lastmin = ~0ull;
   const int nt = p.gated ? 0 : (H + KT - 1) / KT;
   // single CTA: only the warps whose strips reach into [0, W) compute, and only their columns are
@@ -574,13 +558,22 @@ __device__ __forceinline__ unsigned long long seam_sweep(const SearchArgs &p, un
   if (producer) {
     // ---- energy staging: rows of columns [ext0 - KT, ext0 - KT + BW), one bulk copy per lane ----
     const uint16_t *Estage = p.E + (ext0 - KT);
-    for (int tt = 0; tt < nt; ++tt) {
-      const uint32_t g = st.tiles + tt;
-      const int slot = (int)(g % NSLOT);
-      if (g >= NSLOT && !mbar_wait_bounded(&empty[slot], ((g / NSLOT) - 1) & 1u, WAIT_TIMEOUT_NS)) {
-        if (lane == 0) atomicOr(p.err, ERR_TIMEOUT);
-      }
+    auto issue = [&](int tt) {
+      const int slot = (int)((st.tiles + tt) % NSLOT);
       const int rbeg = tt * KT;
+      if constexpr (TM) {
+        if (lane == 0) {
+          mbar_arrive_expect_tx(&full[slot], (uint32_t)(NP * KT * BW * 2));
+          const int y = REV ? p.y0 - rbeg - (KT - 1) : p.y0 + rbeg;
+#pragma unroll
+          for (int pl = 0; pl < NP; ++pl)
+#pragma unroll
+            for (int b = 0; b < NBOX; ++b)
+              tensor_g2s_2d(ring + (size_t)((slot * NP + pl) * NBOX + b) * KT * BWB, p.tmap, E_PADL + cbeg + b * BWB,
+                            y + pl * p.plane_rows, &full[slot]);
+        }
+        return;
+      }
       const int nrows = (H - rbeg < KT) ? H - rbeg : KT;
       if (lane == 0) mbar_arrive_expect_tx(&full[slot], (uint32_t)(NP * nrows) * COPY_BYTES);
       __syncwarp();
@@ -590,42 +583,82 @@ __device__ __forceinline__ unsigned long long seam_sweep(const SearchArgs &p, un
           bulk_g2s(ring + (size_t)((slot * NP + pl) * KT + lane) * BW + (clo - cbeg),
                    Estage + pl * pstride + (ptrdiff_t)(rbeg + lane) * pitch_e + (clo - cbeg), COPY_BYTES, &full[slot]);
       }
+    };
+    fence_proxy_async_smem();   // the ring's place may have held other data before this search
+    for (int tt = 0; tt < NSLOT && tt < nt; ++tt) issue(tt);
+    // The barrier that ends tile t has every warp's word that it has read the tile's slot, and this
+    // warp's that the next tile has landed: the compute warps never wait on a staging barrier
+    // after the first tile.
+    for (int t = 0; t + 1 < nt; ++t) {
+      const uint32_t g = st.tiles + t + 1;
+      if (!mbar_wait_bounded(&full[g % NSLOT], (g / NSLOT) & 1u, WAIT_TIMEOUT_NS)) {
+        if (lane == 0) atomicOr(p.err, ERR_TIMEOUT);
+      }
+      named_bar_sync(G::THREADS);
+      if (t + NSLOT < nt) issue(t + NSLOT);
     }
   } else if (!active) {
-    // outside the image: release every slot at once and keep the barrier count
-    for (int t = 0; t < nt; ++t) {
-      const uint32_t g = st.tiles + t;
-      if (lane == 0) mbar_arrive(&empty[g % NSLOT]);
-      if (t * KT + KT < H) named_bar_sync(NW * 32);
-    }
+    // outside the image: keep the barrier count
+    for (int t = 0; t + 1 < nt; ++t) named_bar_sync(G::THREADS);
   } else {
-    uint32_t k[V] = {0u, 0u, 0u, 0u};
+    const uint32_t own_a = (uint32_t)(c0 - frame_base);   // this lane's first column, warp frame
     uint32_t emax = 0u;   // DIRECT: running maximum of this lane's in-map energies (two uint16 halves)
     const uint2 cm = make_uint2((oobm[0] ? 0u : 0xFFFFu) | (oobm[1] ? 0u : 0xFFFF0000u),
                                 (oobm[2] ? 0u : 0xFFFFu) | (oobm[3] ? 0u : 0xFFFF0000u));
+    // the neighbour's halo buffer that this lane's own columns go to at an exchange: the first K2 own
+    // columns are the left neighbour's right halo, the last K2 the right neighbour's left halo
+    static_assert(!CL || OWC >= 2 * K2, "a column is pushed to one neighbour");
+    uint32_t push = 0u, push_bar = 0u;
+    if constexpr (CL) {
+      const bool tl = cta_own && rank > 0 && c0 < A + K2, tr = cta_own && rank < cs - 1 && c0 >= B - K2;
+      if (tl || tr) {
+        push = mapa_u32(hbuf + (tl ? K2 + (c0 - A) : c0 - (B - K2)), tl ? rank - 1 : rank + 1);
+        push_bar = mapa_u32(hbar, tl ? rank - 1 : rank + 1);
+      }
+    }
+    uint8_t *anc_out = TWO ? gat0 + c0 : nullptr;   // where this lane's ancestors of the current super-tile go
+    // this lane's place in the halo buffer where its columns are a neighbour's (-1: this CTA's)
+    int hoff = -1;
+    if (CL && rank > 0 && c0 >= A - K2 && c0 < A) hoff = c0 - (A - K2);
+    if (CL && rank < cs - 1 && c0 >= B && c0 < B + K2) hoff = K2 + (c0 - B);
+    const bool hneed = CL && __any_sync(0xffffffffu, hoff >= 0);
+    // with one tile per super-tile every boundary starts new ancestors, and only costs cross it
+    constexpr bool FRESH = KSS == KT;
+    const int er0 = TM ? (bidx0 / BWB) * KT * BWB + bidx0 % BWB + (REV ? (KT - 1) * BWB : 0) : bidx0;
     // The tile loop, compiled twice: EDGE warps hold columns outside the image and apply the
     // exclusion mask on every row; the others never test it.
     auto tiles = [&](auto edge_tag) {
       constexpr bool EDGE = decltype(edge_tag)::value;
-      const uint32_t own_a = (uint32_t)(c0 - frame_base);   // this lane's first column, warp frame
+      // the row above row 0: cost 0 in every column, each its own ancestor (row 0 then costs its
+      // energies; the leftmost optimal path of the extended map is the seam below a column of the
+      // added row, so no tile is special)
+      uint32_t k[V];
+#pragma unroll
+      for (int u = 0; u < V; ++u) k[u] = (own_a + u) | (EDGE ? oobm[u] : 0u);
+      if (nt > 0 && !mbar_wait_bounded(&full[st.tiles % NSLOT], (st.tiles / NSLOT) & 1u, WAIT_TIMEOUT_NS)) {
+        if (lane == 0) atomicOr(p.err, ERR_TIMEOUT);
+      }
       for (int t = 0; t < nt; ++t) {
         const int r0 = t * KT;
-        const bool more = r0 + KT < H;
+        const int n = (H - r0 < KT) ? H - r0 : KT;
+        const bool more = t + 1 < nt;
         const uint32_t g = st.tiles + t;
-        const int slot = (int)(g % NSLOT);
-        // one barrier test per tile: the tile was issued NSLOT - 1 tiles ago and has landed by now
-        // (an earlier test of the next tile, overlapped with this tile's rows, found it still in
-        // flight every time and cost more than it saved)
-        if (!mbar_wait_bounded(&full[slot], (g / NSLOT) & 1u, WAIT_TIMEOUT_NS)) {
-          if (lane == 0) atomicOr(p.err, ERR_TIMEOUT);
-        }
-        const uint16_t *er = ring + (size_t)slot * NP * KT * BW + bidx0;
+        const uint16_t *er = ring + (size_t)(g % NSLOT) * NP * KT * BW + er0;
         if (t > 0) {
-          // window of the previous row from the boundary buffer (relative ancestors -> warp frame).
-          // At a new super-tile every cell becomes its own ancestor; the old ancestor field is
-          // dropped without arithmetic (it may lie outside this warp's frame).
-          const uint4 v = *reinterpret_cast<const uint4 *>(bnd + ((t - 1) & 1) * BW + bidx0);
-          const bool fresh = (r0 % KSS) == 0;
+          // window of the previous row from the boundary buffer, or from the halo buffer for a
+          // neighbour's columns after an exchange (relative ancestors -> warp frame). At a new
+          // super-tile every cell becomes its own ancestor; the old ancestor field is dropped
+          // without arithmetic (it may lie outside this warp's frame).
+          const uint32_t *src = bnd + ((t - 1) & 1) * BW + bidx0;
+          if (CL && hneed && cs > 1 && (r0 % K2) == 0) {
+            const uint32_t xg = st.exch + (uint32_t)(r0 / K2 - 1);
+            if (!mbar_wait_bounded(&hbar[xg & 1], (xg >> 1) & 1u, WAIT_TIMEOUT_NS)) {
+              if (lane == 0) atomicOr(p.err, ERR_TIMEOUT);
+            }
+            if (hoff >= 0) src = hbuf + (int)(xg & 1) * 2 * K2 + hoff;
+          }
+          const uint4 v = *reinterpret_cast<const uint4 *>(src);
+          const bool fresh = FRESH || (r0 % KSS) == 0;
           const uint32_t d = own_a - 128u;
           k[0] = fresh ? ((v.x & ~0xFFu) | own_a) : (v.x + d);
           k[1] = fresh ? ((v.y & ~0xFFu) | (own_a + 1u)) : (v.y + d + 1u);
@@ -633,71 +666,48 @@ __device__ __forceinline__ unsigned long long seam_sweep(const SearchArgs &p, un
           k[3] = fresh ? ((v.w & ~0xFFu) | (own_a + 3u)) : (v.w + d + 3u);
           if (EDGE) { k[0] |= oobm[0]; k[1] |= oobm[1]; k[2] |= oobm[2]; k[3] |= oobm[3]; }
         }
-        if (t > 0 && r0 + KT <= H) {
-          // full tile: KT branch-free rows (the energies of the next rows are loaded ahead of
-          // the row that needs them, off the dependent chain); bookkeeping only where a
-          // super-tile or the image ends on its last row
-          if (FWD) dp_rows_fwd<KT, BW, EDGE>(k, er, oobm);
-          else dp_rows<KT, BW, EDGE, LAT, DIRECT>(k, er, oobm, emax, cm);
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&empty[slot]);   // this warp is done with the staged rows
-          if (((r0 + KT) % KSS) == 0 || r0 + KT == H)
-            row_events<KSS, TWO>(r0 + KT - 1, k, H, W, c0, frame_base, cta_own, A, ancT, OWC, gat0, gw,
-                                 lastmin, p.endrow);
+        if (FWD) {
+          if (n == KT) dp_rows_fwd<KT, BWB, KT * BW, EDGE>(k, er, oobm);
+          else dp_rows_n_fwd<BWB, KT * BW, EDGE>(k, er, oobm, n);
         } else {
-          // first tile (row 0 has no predecessor) or a ragged last tile. Neither holds a row with
-          // bookkeeping except the image's last row and the first tile's last row when KSS = KT:
-          // a super-tile ends on a multiple of KSS (a multiple of KT), which is never inside
-          // these tiles' rows 0 .. n-2
-          const int n = (H - r0 < KT) ? H - r0 : KT;
-          if (t == 0) {
-            const uint2 ev = *reinterpret_cast<const uint2 *>(er);   // CU with FWD
-            k[0] = (lo8(ev.x) | own_a) | oobm[0];
-            k[1] = (hi8(ev.x) | (own_a + 1u)) | oobm[1];
-            k[2] = (lo8(ev.y) | (own_a + 2u)) | oobm[2];
-            k[3] = (hi8(ev.y) | (own_a + 3u)) | oobm[3];
-            emax_acc<DIRECT, EDGE>(emax, ev, cm);
-          }
-          if (FWD) dp_rows_n_fwd<KT, BW, EDGE>(k, er, oobm, t == 0 ? 1 : 0, n);
-          else dp_rows_n<KT, BW, EDGE, LAT, DIRECT>(k, er, oobm, t == 0 ? 1 : 0, n, emax, cm);
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&empty[slot]);
-          if (((r0 + n) % KSS) == 0 || r0 + n == H)
-            row_events<KSS, TWO>(r0 + n - 1, k, H, W, c0, frame_base, cta_own, A, ancT, OWC, gat0, gw,
-                                 lastmin, p.endrow);
+          dp_rows<(TM ? KT : 8), BWB, EDGE, LAT, DIRECT, REV>(k, er, oobm, n, emax, cm);
         }
-        if (more) {
-          const bool exch = CL && ((r0 + KT) % K2 == 0) && cs > 1;
-          const uint32_t d = own_a - 128u;
-          uint4 v;
-          v.x = k[0] - d; v.y = k[1] - d - 1u; v.z = k[2] - d - 2u; v.w = k[3] - d - 3u;
-          // publish this warp's strip (relative ancestor encoding); at an exchange the CTA's halo
-          // columns come from the neighbours instead
-          if (strip_lane && (!exch || (c0 >= A && c0 < B)))
-            *reinterpret_cast<uint4 *>(bnd + (t & 1) * BW + bidx0) = v;
-          if constexpr (CL) if (exch) {
-            const uint32_t xg = st.exch + (uint32_t)((r0 + KT) / K2 - 1);
-            const int par = (int)(xg & 1);
-            // my first K2 own columns are the left neighbour's right halo, my last K2 the right's left
-            if (strip_lane && rank > 0 && c0 >= A && c0 < A + K2)
-              st_async_v4(mapa_u32(hbuf + par * 2 * K2 + K2 + (c0 - A), rank - 1), v, mapa_u32(&hbar[par], rank - 1));
-            if (strip_lane && rank < cs - 1 && c0 >= B - K2 && c0 < B)
-              st_async_v4(mapa_u32(hbuf + par * 2 * K2 + (c0 - (B - K2)), rank + 1), v, mapa_u32(&hbar[par], rank + 1));
-            if (threadIdx.x == 0)
-              mbar_arrive_expect_tx(&hbar[par], (uint32_t)(((rank > 0) + (rank < cs - 1)) * K2 * 4));
-            if (!mbar_wait_bounded(&hbar[par], (xg >> 1) & 1u, WAIT_TIMEOUT_NS)) {
-              if (lane == 0) atomicOr(p.err, ERR_TIMEOUT);
-            }
-            uint32_t *mine = bnd + (t & 1) * BW;
-            for (int q = threadIdx.x; q < 2 * K2; q += NW * 32) {
-              if (q < K2) {
-                if (rank > 0) mine[(A - K2 + q) - (ext0 - KT)] = hbuf[par * 2 * K2 + q];
-              } else {
-                if (rank < cs - 1) mine[(B + (q - K2)) - (ext0 - KT)] = hbuf[par * 2 * K2 + q];
+        // bookkeeping on the tile's last row, the only one where a super-tile (KSS is a multiple
+        // of KT) or the image can end: the ancestors of the CTA-own columns (in rank 0's gathered
+        // table, the global one or this CTA's), and below the last row its costs
+        if (cta_own && (FRESH || ((r0 + n) % KSS) == 0 || !more)) {
+          const uint32_t anc = pack_ancestors(k, c0, frame_base);
+          const size_t sup = (size_t)((r0 + n - 1) / KSS);
+          if (TWO) {
+            *reinterpret_cast<uint32_t *>(anc_out) = anc;
+            anc_out += gw;
+            if (!more) *reinterpret_cast<uint4 *>(p.endrow + c0) = make_uint4(k[0] >> 8, k[1] >> 8, k[2] >> 8, k[3] >> 8);
+          } else {
+            *reinterpret_cast<uint32_t *>(gw ? gat0 + sup * gw + c0 : ancT + sup * OWC + (c0 - A)) = anc;
+#pragma unroll
+            for (int u = 0; u < V; ++u) {
+              if (!more && c0 + u < W) {
+                const unsigned long long c = ((unsigned long long)(k[u] >> 8) << 32) | (unsigned)(c0 + u);
+                lastmin = c < lastmin ? c : lastmin;
               }
             }
           }
-          named_bar_sync(NW * 32);
+        }
+        if (more) {
+          const bool exch = CL && ((r0 + KT) % K2 == 0) && cs > 1;
+          // publish this warp's strip (relative ancestor encoding)
+          const uint32_t d = FRESH ? 0u : own_a - 128u, du = FRESH ? 0u : 1u;
+          uint4 v;
+          v.x = k[0] - d; v.y = k[1] - d - du; v.z = k[2] - d - 2 * du; v.w = k[3] - d - 3 * du;
+          if constexpr (CL) if (exch) {
+            // read there at the start of the next tile
+            const uint32_t par = (st.exch + (uint32_t)((r0 + KT) / K2 - 1)) & 1u;
+            if (push) st_async_v4(push + par * (2 * K2 * 4), v, push_bar + par * 8);
+            if (threadIdx.x == 0)
+              mbar_arrive_expect_tx(&hbar[par], (uint32_t)(((rank > 0) + (rank < cs - 1)) * K2 * 4));
+          }
+          if (strip_lane) *reinterpret_cast<uint4 *>(bnd + (t & 1) * BW + bidx0) = v;
+          named_bar_sync(G::THREADS);
         }
       }
     };
@@ -716,7 +726,8 @@ __device__ __forceinline__ unsigned long long seam_sweep(const SearchArgs &p, un
 
 // The search. Every thread of the CTA (of every CTA of the cluster when CL) calls it with the same
 // arguments; `Smax` is the super-tile count the shared-memory plan was sized for.
-template <int NW, int KT, bool CL, int FWM = FILL_WARPS_MAX, bool FWD = false, int KSS = KS, bool DIRECT = false>
+template <int NW, int KT, bool CL, int FWM = FILL_WARPS_MAX, bool FWD = false, int KSS = KS, bool DIRECT = false,
+          bool TM = false>
 __device__ void seam_search(const SearchArgs &p, unsigned char *smem, int Smax, SearchState &st) {
   using G = Geo<NW, KT, CL, FWM, KSS>;
   constexpr int OWC = G::OWC;
@@ -737,7 +748,7 @@ __device__ void seam_search(const SearchArgs &p, unsigned char *smem, int Smax, 
   uint8_t *const gat = smem + plan.gat;
   const int64_t pstride = FWD ? p.pstride : 0;
 
-  unsigned long long lastmin = seam_sweep<NW, KT, CL, FWM, FWD, KSS, DIRECT, false>(p, smem, plan, st);
+  unsigned long long lastmin = seam_sweep<NW, KT, CL, FWM, FWD, KSS, DIRECT, TM>(p, smem, plan, st);
 
   // ---- last-row argmin: the leftmost minimum (min of (M << 32) | column) ----
 #pragma unroll
@@ -798,7 +809,7 @@ __device__ void seam_search(const SearchArgs &p, unsigned char *smem, int Smax, 
       j = j + (int)ra[(size_t)s * OWC + (j - c * OWC)] - 128;
       if (j < 0 || j >= W) { ok = 0; atomicOr(p.err, ERR_BAD_SEAM); }
     }
-    jb[S] = j;          // the seam's column in row 0
+    jb[S] = j;          // the seam's column in the added row above row 0
     misc[0] = ok;
     best_m = (uint32_t)(best >> 32);
     misc[1] = 0;   // the fills add their path costs here
