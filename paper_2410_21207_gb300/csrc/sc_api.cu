@@ -106,7 +106,7 @@ struct Workspace {
   DevBuf<int32_t> seam;
   DevBuf<int16_t> lists;          // two generations of pending-removal lists
   DevBuf<uint8_t> hin, hout;     // staging for the host-pointer entry point
-  DevBuf<int> flags;             // [0] error word, [1] energy-range gate, [2] the search's arrival counter
+  DevBuf<int> flags;             // [0] error word, [1] energy-range gate, [2], [3] the search's sync words
   DevBuf<int> gates;             // one energy-range gate per map of sc_find_seam_multi
   DevBuf<uint32_t> wdirs;        // wide-cost search: directions and ancestors (per map)
   DevBuf<uint16_t> wanc;
@@ -327,10 +327,11 @@ int sc_check(void *stream) {
   // a stream with no earlier work has fresh (uninitialised) flag words: they start at zero
   if ((rc = ensure_flags(ws, st))) return rc;
   SC_CUDA(cudaStreamSynchronize(st));
-  int h[2] = {0, 0};
-  SC_CUDA(cudaMemcpy(h, ws.flags.p, 2 * sizeof(int), cudaMemcpyDeviceToHost));
-  SC_CUDA(cudaMemset(ws.flags.p, 0, 2 * sizeof(int)));
+  int h[4] = {0, 0, 0, 0};
+  SC_CUDA(cudaMemcpy(h, ws.flags.p, 4 * sizeof(int), cudaMemcpyDeviceToHost));
+  SC_CUDA(cudaMemset(ws.flags.p, 0, 4 * sizeof(int)));
   int e = h[0];
+  if (h[3] != 0) e |= ERR_COST_MISMATCH;   // some search's path costs did not add up to its cost
   if (int *ge = device_error_word()) {
     int g = 0;
     SC_CUDA(cudaMemcpy(&g, ge, sizeof(int), cudaMemcpyDeviceToHost));

@@ -145,9 +145,13 @@ static cudaError_t launch_dp_shape(const DpArgs &a, int cs, cudaStream_t st) {
 //     towards the bottom: two chains that one warp follows side by side, half as many hops each;
 //   * the super-tiles of both halves are then backtracked in parallel as in seam_search.
 // No cluster waits for the other: both leave their last cost row and their ancestor table in
-// global memory, count themselves in, and the cluster that holds the last CTA to arrive does the rest
-// while the other one leaves. (The two need not be resident together, so the launch cannot
-// deadlock beside other work.)
+// global memory and every CTA counts itself in. The last CTA to arrive joins the halves and follows the
+// chains on its own (a second pass over 2 x 4 bytes a column is cheaper than the cluster barriers
+// that would split it), then hands the columns to its cluster, which backtracks while the other
+// cluster leaves. (The two need not be resident together, so the launch cannot deadlock beside
+// other work.)
+// The cost self-check needs no barrier either: a launch adds its cost to sync[1] and the super-tiles
+// subtract their path costs, so the word is 0 whenever the stream is idle (sc_check looks).
 //
 // Scratch, in p.scratch: the two cost rows (gw uint32 each), then the ancestor tables (gw bytes per
 // super-tile, upper half first), gw = the columns the cluster covers. It fits (S + 1) rows of pitch_e
@@ -165,13 +169,13 @@ template <int NW, int KT>
 struct Two {
   static constexpr int KSS = dp_super_rows<NW, KT, false>();
   using G = Geo<NW, KT, true, FILL_WARPS_MAX, KSS>;
-  int H0, H1, S0, S1, gw;
+  int H0, H1, S0, S1, cs, gw;
   size_t tab_bytes;      // both tables
   bool tab_smem;         // rank 0 of the finishing cluster copies them into its staging ring's place
   SearchPlan plan;       // jb holds both halves' columns: S0 + 1, then S1 + 1
   size_t tbar;           // mbarrier of that copy
 
-  __host__ __device__ Two(int H, int cs) {
+  __host__ __device__ Two(int H, int ctas) : cs(ctas) {
     // a whole number of tiles in the upper half where there is a choice: only one half then ends on a
     // ragged tile
     H0 = ((H + 1) / 2 + KT - 1) / KT * KT;
@@ -190,20 +194,20 @@ struct Two {
     plan.bnd = take((size_t)2 * G::BW * 4);
     plan.hbuf = take((size_t)2 * 2 * K2 * 4);
     plan.wmin = 0;
-    plan.cmin = take((size_t)MAX_CLUSTER * (NW + 1) * 8);   // every warp's minimum, pushed to rank 0
+    plan.cmin = take((size_t)(NW + 1 + (S0 + S1 + cs - 1) / cs) * 8);   // warps' minima, then super-tiles' ends
     plan.jb = take((size_t)(S0 + S1 + 2) * 4);
-    plan.misc = take(16);   // [0] this cluster arrived last, [1] path cost sum (rank 0), [2] chain found
+    plan.misc = take(16);   // [0] this CTA arrived last, [1] its cluster goes on with the ends in cmin
     plan.anc = plan.emx = plan.gat = 0;
     plan.gw = 0;
     plan.bars = take((size_t)(NSLOT + 3) * 8);
     tbar = plan.bars + (size_t)(NSLOT + 2) * 8;
-    // the staging ring; after the sweep its place holds the tables, then the fills' directions
+    // the staging ring; after the sweep its place holds the tables, then the fills' rows
     size_t r = (size_t)NSLOT * KT * G::BW * 2;
-    const size_t fd = (size_t)G::FW * KSS * G::FILLW;
-    r = r > fd ? r : fd;
+    const size_t fb = (size_t)G::FW * G::fill_bytes(false);
+    r = r > fb ? r : fb;
     if (tab && tab_bytes > r) r = tab_bytes;
     o = (o + 127) & ~(size_t)127;
-    plan.ring = plan.fdir = take(r);
+    plan.ring = plan.fill = take(r);
     plan.total = o;
   }
 };
@@ -228,7 +232,7 @@ __global__ void __launch_bounds__(Geo<NW, KT, true>::THREADS, 1)
   if (threadIdx.x == 0) {
     mbar_init(tbar, 1);
     fence_mbar_init();
-    misc[0] = 0;
+    misc[0] = misc[1] = 0;
     prefetch_tensormap(&tmap);
   }
   // neighbours push into each other's halo buffers: every CTA's barriers must be initialised first
@@ -258,112 +262,109 @@ __global__ void __launch_bounds__(Geo<NW, KT, true>::THREADS, 1)
     if (half) seam_sweep<NW, KT, true, FILL_WARPS_MAX, false, KSS, false, true, true, true>(a, smem, plan, st);
     else seam_sweep<NW, KT, true, FILL_WARPS_MAX, false, KSS, false, true, true, false>(a, smem, plan, st);
   }
-  // ---- count this CTA in; the cluster of the last one goes on ----
+  // ---- count this CTA in ----
   fence_proxy_async_global();   // the tables are read by a bulk copy below
   __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    if (atomicAdd(p.sync, 1) == 2 * cs - 1) {
-      __threadfence();
-      *p.sync = 0;   // for the next launch
-      for (int r = 0; r < cs; ++r) cl.map_shared_rank(misc, r)[0] = 1;
+  if (threadIdx.x == 0 && atomic_add_acq_rel(p.sync, 1) == 2 * cs - 1) {
+    *p.sync = 0;   // for the next launch
+    misc[0] = 1;
+  }
+  __syncthreads();
+  if (misc[0]) {
+    // ---- the last CTA: the seam's cost and its columns in the two middle rows ----
+    unsigned char *const stab = smem + plan.ring;
+    if (warp == NW && g.tab_smem) {
+      // both ancestor tables arrive meanwhile, in a few large copies
+      fence_proxy_async_global();
+      fence_proxy_async_smem();   // the ring's last reads come first
+      if (lane == 0) mbar_arrive_expect_tx(tbar, (uint32_t)g.tab_bytes);
+      __syncwarp();
+      constexpr uint32_t PIECE = 8192;
+      for (uint32_t o = lane * PIECE; o < (uint32_t)g.tab_bytes; o += 32 * PIECE)
+        bulk_g2s(stab + o, tab + o, min(PIECE, (uint32_t)g.tab_bytes - o), tbar);
     }
-  }
-  cl.sync();
-  if (misc[0] == 0) return;
-
-  // ---- the seam's cost and its columns in the two middle rows ----
-  unsigned char *const stab = smem + plan.ring;
-  if (rank == 0 && warp == NW && g.tab_smem) {
-    // rank 0 fetches both ancestor tables meanwhile
-    fence_proxy_async_global();
-    fence_proxy_async_smem();   // the ring's last reads come first
-    if (lane == 0) mbar_arrive_expect_tx(tbar, (uint32_t)g.tab_bytes);
-    __syncwarp();
-    for (int s = lane; s < g.S0 + g.S1; s += 32) bulk_g2s(stab + (size_t)s * g.gw, tab + (size_t)s * g.gw, g.gw, tbar);
-  }
-  unsigned long long best = ~0ull;   // cost << 32 | upper column << 2 | step to the lower column
-  const int jend = min(p.W, (rank + 1) * G::OWC);
-  for (int j = rank * G::OWC + threadIdx.x; j < jend; j += G::THREADS) {
-    const uint32_t d = __ldcg(end0 + j);
-    const uint32_t u0 = j > 0 ? __ldcg(end1 + j - 1) : SENT, u1 = __ldcg(end1 + j),
-                   u2 = j + 1 < p.W ? __ldcg(end1 + j + 1) : SENT;
-    const uint32_t m = min3u(u0, u1, u2);
-    const uint32_t st = m == u0 ? 0u : (m == u1 ? 1u : 2u);
-    const unsigned long long k = ((unsigned long long)(d + m) << 32) | ((uint32_t)j << 2) | st;
-    best = k < best ? k : best;
-  }
-  auto warp_min = [](unsigned long long v) {
+    uint32_t best = SENT, where = SENT;   // cost; upper column << 2 | step to the lower column
+#pragma unroll 4
+    for (int q = threadIdx.x; q < (p.W + 3) / 4; q += G::THREADS) {
+      const int j0 = 4 * q;
+      const uint4 d = __ldcg(reinterpret_cast<const uint4 *>(end0) + q), u = __ldcg(reinterpret_cast<const uint4 *>(end1) + q);
+      const uint32_t ul = j0 > 0 ? __ldcg(end1 + j0 - 1) : SENT, ur = j0 + 4 < p.W ? __ldcg(end1 + j0 + 4) : SENT;
+      const uint32_t dv[4] = {d.x, d.y, d.z, d.w}, uv[6] = {ul, u.x, u.y, u.z, u.w, ur};
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      const unsigned long long o = __shfl_xor_sync(0xffffffffu, v, off);
-      v = o < v ? o : v;
-    }
-    return v;
-  };
-  best = warp_min(best);
-  unsigned long long *cmin = reinterpret_cast<unsigned long long *>(smem + plan.cmin);
-  if (lane == 0) cl.map_shared_rank(cmin, 0)[rank * (NW + 1) + warp] = best;
-  cl.sync();
-
-  // ---- ancestor chains (rank 0): lane 0 towards row 0, lane 1 towards the bottom row ----
-  if (rank == 0 && warp == 0) {
-    best = ~0ull;
-    for (int q = lane; q < cs * (NW + 1); q += 32) best = cmin[q] < best ? cmin[q] : best;
-    best = warp_min(best);
-    bool bad = false;
-    if (g.tab_smem && !mbar_wait_bounded(tbar, 0u, WAIT_TIMEOUT_NS)) {
-      if (lane == 0) atomicOr(p.err, ERR_TIMEOUT);
-      bad = true;
-    }
-    if (lane < 2) {
-      const int Sh = lane ? g.S1 : g.S0;
-      const size_t t0 = lane ? (size_t)g.S0 * g.gw : 0;
-      int *jh = jb + (lane ? g.S0 + 1 : 0);
-      int j = (int)((uint32_t)best >> 2) + (lane ? (int)(best & 3u) - 1 : 0);
-      // a column outside the map is clamped (every read stays inside the table) and recorded
-      auto keep = [&](int c) { bad |= (unsigned)c >= (unsigned)p.W; return min(max(c, 0), p.W - 1); };
-      j = keep(j);
-      for (int s = Sh - 1; s >= 0; --s) {
-        jh[s] = j;
-        const size_t at = t0 + (size_t)s * g.gw + j;
-        j = keep(j + (g.tab_smem ? (int)stab[at] : (int)__ldcg(tab + at)) - 128);
+      for (int c = 0; c < 4; ++c) {
+        const int j = j0 + c;
+        const uint32_t right = j + 1 < p.W ? uv[c + 2] : SENT;
+        const uint32_t m = min3u(uv[c], uv[c + 1], right), sum = dv[c] + m;
+        if (j < p.W && sum < best) {   // columns come in ascending order: ties keep the left one
+          best = sum;
+          where = ((uint32_t)j << 2) | (m == uv[c] ? 0u : (m == uv[c + 1] ? 1u : 2u));
+        }
       }
-      jh[Sh] = j;
-      if (bad) atomicOr(p.err, ERR_BAD_SEAM);
     }
-    bad = __any_sync(0xffffffffu, bad);
-    if (lane == 0) {
-      misc[1] = 0;
-      if (!bad && p.cost) *p.cost = (int64_t)(best >> 32);
+    const uint32_t wb = __reduce_min_sync(0xffffffffu, best);
+    const uint32_t ww = __reduce_min_sync(0xffffffffu, best == wb ? where : SENT);
+    uint2 *const cmin = reinterpret_cast<uint2 *>(smem + plan.cmin);
+    if (lane == 0) cmin[warp] = make_uint2(wb, ww);
+    __syncthreads();
+    if (warp == 0) {
+      const uint2 v = lane <= NW ? cmin[lane] : make_uint2(SENT, SENT);
+      best = __reduce_min_sync(0xffffffffu, v.x);
+      where = __reduce_min_sync(0xffffffffu, v.x == best ? v.y : SENT);
+      // ---- ancestor chains: lane 0 towards the top, lane 1 towards the bottom ----
+      bool bad = false;
+      if (g.tab_smem && !mbar_wait_bounded(tbar, 0u, WAIT_TIMEOUT_NS)) {
+        if (lane == 0) atomicOr(p.err, ERR_TIMEOUT);
+        bad = true;
+      }
+      if (lane < 2) {
+        const int Sh = lane ? g.S1 : g.S0;
+        int *jh = jb + (lane ? g.S0 + 1 : 0);
+        int j = (int)(where >> 2) + (lane ? (int)(where & 3u) - 1 : 0);
+        // a column outside the map is clamped (every read stays inside the table) and recorded
+        auto keep = [&](int c) { bad |= (unsigned)c >= (unsigned)p.W; return min(max(c, 0), p.W - 1); };
+        j = keep(j);
+        size_t at = (size_t)(Sh - 1 + (lane ? g.S0 : 0)) * g.gw;
+        for (int s = Sh - 1; s >= 0; --s, at -= g.gw) {
+          jh[s] = j;
+          j = keep(j + (g.tab_smem ? (int)stab[at + j] : (int)__ldcg(tab + at + j)) - 128);
+        }
+        jh[Sh] = j;
+        if (bad) atomicOr(p.err, ERR_BAD_SEAM);
+      }
+      bad = __any_sync(0xffffffffu, bad);
+      if (lane == 0 && !bad) {
+        if (p.cost) *p.cost = (int64_t)best;
+        atomicAdd(reinterpret_cast<uint32_t *>(p.sync + 1), best);
+      }
+      __syncwarp();
+      // CTA r of the cluster gets the ends of super-tiles r, r + cs, ... (the upper half's first)
+      for (int r = lane; r < cs; r += 32) {
+        int2 *dst = reinterpret_cast<int2 *>(cl.map_shared_rank(smem + plan.cmin, r));
+        for (int q = r; q < g.S0 + g.S1; q += cs) {
+          const int *jh = q < g.S0 ? jb : jb + g.S0 + 1;
+          const int s = q < g.S0 ? q : q - g.S0, Sh = q < g.S0 ? g.S0 : g.S1;
+          *dst++ = make_int2(s > 0 ? jh[s - 1] : jh[Sh], jh[s]);
+        }
+        cl.map_shared_rank(misc, r)[1] = bad ? 0 : 1;
+      }
     }
-    __syncwarp();
-    // every CTA gets the columns
-    for (int q = lane; q < g.S0 + g.S1 + 2; q += 32) {
-      const int v = jb[q];
-      for (int r = 1; r < cs; ++r) cl.map_shared_rank(jb, r)[q] = v;
-    }
-    if (lane < cs) cl.map_shared_rank(misc, lane)[2] = bad ? 0 : 1;
   }
   cl.sync();
 
-  // ---- the super-tiles of both halves, the lower half's from the last warp on ----
-  if (misc[2] == 0) return;   // recorded; nothing refers to another CTA's shared memory any more
-  if (warp < G::FW) {
-    uint32_t *const csum = reinterpret_cast<uint32_t *>(cl.map_shared_rank(misc, 0) + 1);
-    const int Wa = (p.W + 7) & ~7;
+  // ---- the super-tiles of both halves ----
+  if (misc[1] == 0) return;   // the other cluster goes on (or a recorded failure)
+  const int2 *const ends = reinterpret_cast<const int2 *>(smem + plan.cmin);
 #pragma unroll 1
-    for (int h = 0; h < 2; ++h) {
-      const int last = h ? p.H - 1 : 0;
-      const FillCtx f{h ? E1 : p.E, h ? jb + g.S0 + 1 : jb, smem + plan.fdir, csum, p.seam + last,
-                      p.seam_log ? p.seam_log + last : nullptr, p.err, 0, h ? -p.pitch_e : p.pitch_e,
-                      h ? g.H1 : g.H0, p.W, Wa, h ? g.S1 : g.S0, cs, h ? -1 : 1};
-      backtrack_fill<NW, KT, true, FILL_WARPS_MAX, false, KSS, false, 16>(
-          f, (h ? G::FW - 1 - warp : warp) * cs + rank, warp, lane);
-    }
+  for (int k = warp; k * cs + rank < g.S0 + g.S1; k += G::FW) {
+    if (warp >= G::FW) break;
+    const int q = k * cs + rank;
+    const bool low = q >= g.S0;
+    const int last = low ? p.H - 1 : 0;
+    const FillCtx f{low ? E1 : p.E, smem + plan.fill, reinterpret_cast<uint32_t *>(p.sync + 1), 0xFFFFFFFFu, p.seam + last,
+                    p.seam_log ? p.seam_log + last : nullptr, p.err, 0, low ? -p.pitch_e : p.pitch_e,
+                    low ? g.H1 : g.H0, p.W, 0, low ? -1 : 1};
+    fill_super_tile<G, false, KSS, false>(f, low ? q - g.S0 : q, ends[k].x, ends[k].y, warp, lane);
   }
-  cl.sync();   // rank 0's sum is complete
-  if (rank == 0 && threadIdx.x == 0 && (uint32_t)misc[1] != (uint32_t)(best >> 32)) atomicOr(p.err, ERR_COST_MISMATCH);
 }
 
 template <int NW, int KT>

@@ -53,7 +53,7 @@ struct DpArgs {
   int pitch_e;
   int H, W;
   uint32_t *scratch;   // two-ended search: cost rows and ancestor tables, (ceil(H/KS) + 1) * pitch_e words
-  int *sync;           // two-ended search: arrival counter, 0 between launches
+  int *sync;           // two-ended search: [0] arrival counter, [1] cost check sum; 0 between launches
   int32_t *seam;       // out [H]
   int32_t *seam_log;   // nullable, out [H]
   int64_t *cost;       // nullable, out [1]

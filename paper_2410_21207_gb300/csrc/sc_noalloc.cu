@@ -27,7 +27,7 @@ static __device__ __align__(256) unsigned char g_static_scratch[STATIC_SCRATCH_B
 //   [1] the call's energy-range gate (cleared by each call),
 //   [2] errors not yet reported: every call's errors are added here, and sc_check reads and
 //       clears it,
-//   [3] the search's arrival counter (zero between calls).
+//   [3], [4] the search's sync words (zero between calls; cleared by each call all the same).
 constexpr int ST_CALL_ERR = 0, ST_GATE = 1, ST_PENDING = 2, ST_SYNC = 3;
 
 // Host code cannot use the name g_static_scratch as a device address: it is a host-side stand-in.
@@ -56,7 +56,7 @@ static int static_base(unsigned char **out, bool lookup) {
 // The last step of every static call: the call's error bits join the pending word, and a call
 // that recorded any reports it through its outputs too (every seam entry and the cost set to -1).
 __global__ void k_static_finish(int H, int32_t *seam, int64_t *cost, int *words) {
-  const int e = words[ST_CALL_ERR];
+  const int e = words[ST_CALL_ERR] | (words[ST_SYNC + 1] != 0 ? ERR_COST_MISMATCH : 0);
   if (e == 0) return;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     atomicOr(&words[ST_PENDING], e);
@@ -121,6 +121,7 @@ extern "C" int sc_find_seam_static(const uint16_t *energy, int H, int W, int32_t
   uint16_t *E = reinterpret_cast<uint16_t *>(base + off_E);
   // the array keeps the previous call's contents: this call's error word and gate start at zero
   SC_STATIC_CUDA(cudaMemsetAsync(words, 0, 2 * sizeof(int), st));
+  SC_STATIC_CUDA(cudaMemsetAsync(words + ST_SYNC, 0, 2 * sizeof(int), st));
   SC_STATIC_CUDA(launch_copy_energy(energy, H, W, E + E_PADL, pe, words + ST_GATE, st));
   DpArgs a;
   a.E = E + E_PADL;

@@ -113,6 +113,14 @@ __device__ __forceinline__ void st_async_v4(uint32_t remote_addr, uint4 v, uint3
                : "memory");
 }
 
+// atomic addition that publishes this thread's (and, after a CTA barrier, its CTA's) earlier writes and
+// sees what the earlier additions published
+__device__ __forceinline__ int atomic_add_acq_rel(int *p, int v) {
+  int old;
+  asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
+  return old;
+}
+
 // 16-byte asynchronous copy global -> shared (both 16-byte aligned), completed by cp_async_wait_all
 __device__ __forceinline__ void cp_async16(void *dst_smem, const void *src_gmem) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst_smem)), "l"(src_gmem) : "memory");

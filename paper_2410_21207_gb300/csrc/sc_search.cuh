@@ -68,6 +68,12 @@ struct Geo {
   static constexpr int THREADS = (NW + 1) * 32;          // compute warps + the producer warp
   static constexpr int FV = KSS / 16;                    // backtrack-fill columns per lane
   static constexpr int FILLW = 32 * FV;                  // backtrack-fill window (2 * KSS columns)
+  // rows whose energies a fill warp holds in shared memory at a time: the whole super-tile in the
+  // single-map search of e1 maps up to 32 rows, else half of it or a quarter
+  static constexpr int fill_rows(bool fwd) { return FWM >= FILL_WARPS_MAX && !fwd && CL ? 32 : 16; }
+  static constexpr size_t fill_bytes(bool fwd) {         // per fill warp: directions, energies
+    return (size_t)KSS * FILLW + (size_t)fill_rows(fwd) * FILLW * 2 * (fwd ? 3 : 1);
+  }
   static_assert(Q > 0 && KSS % KT == 0 && K2 % KT == 0, "tile geometry");
   static_assert(KSS == 32 || KSS == 64, "super-tile height");
   static_assert(Q + 2 * KSS <= 256, "the ancestor frame must fit 8 bits");
@@ -75,7 +81,7 @@ struct Geo {
 
 // offsets of the dynamic shared-memory regions used by seam_search
 struct SearchPlan {
-  size_t bnd, hbuf, anc, wmin, cmin, jb, misc, emx, fdir, ring, bars, gat, total;
+  size_t bnd, hbuf, anc, wmin, cmin, jb, misc, emx, fill, ring, bars, gat, total;
   int gw;   // row stride (bytes) of the gathered ancestor table in rank 0; 0: not gathered
 };
 
@@ -93,13 +99,11 @@ __host__ __device__ inline SearchPlan search_plan(int S) {
   p.misc = o; o += 16;
   p.emx = o;  o += DIRECT ? (size_t)(NW + 1 + MAX_CLUSTER) * 4 : 0;   // energy maxima: per warp, per CTA
   o = (o + 15) & ~(size_t)15;
-  // the backtrack fill's direction rows live in the staging ring, which is idle by then (every
-  // staged tile has been consumed before the argmin), unless the ring is the smaller of the two
-  const size_t fdir_sz = (size_t)G::FW * KSS * G::FILLW, ring_sz = (size_t)NSLOT * (FWD ? 3 : 1) * KT * G::BW * 2;
-  if (fdir_sz > ring_sz) { p.fdir = o; o += fdir_sz;  o = (o + 15) & ~(size_t)15; }
+  // the backtrack fill works in the staging ring's place, which is idle by then (every staged tile
+  // has been consumed before the argmin)
+  const size_t fill_sz = (size_t)G::FW * G::fill_bytes(FWD), ring_sz = (size_t)NSLOT * (FWD ? 3 : 1) * KT * G::BW * 2;
   o = (o + 127) & ~(size_t)127;   // (tensor copies: 128-byte aligned)
-  p.ring = o; o += ring_sz;  o = (o + 15) & ~(size_t)15;
-  if (fdir_sz <= ring_sz) p.fdir = p.ring;
+  p.ring = p.fill = o; o += fill_sz > ring_sz ? fill_sz : ring_sz;  o = (o + 15) & ~(size_t)15;
   p.bars = o; o += (size_t)(NSLOT + 2) * 8;   // full[NSLOT], halo[2]
   o = (o + 15) & ~(size_t)15;
   // single-map cluster search: every CTA writes its super-tile ancestors straight into rank 0's
@@ -300,189 +304,278 @@ __device__ __forceinline__ void group_sync() {
   if (CL) cg::this_cluster().sync(); else __syncthreads();
 }
 
-// The parallel backtrack of seam_search: each fill warp walks its super-tiles (rows s*KSS ..
-// s*KSS+KSS-1, s = s_first, s_first + FW*cs, ...). The ancestor chain has fixed both ends of the
-// seam inside a super-tile: column jb[s] in its bottom row and column jb[s-1] in the row above it
-// (jb[S] in the added row above row 0 for s = 0), and the seam between them is the leftmost cheapest path from one to
-// the other. So the fill is a small search of its own: costs start at 0 in the upper end and at
-// infinity everywhere else, and only the cells within r columns of the upper end and n - r of the
-// lower end can be on the path (n rows, r of them down), a diamond at most n + 1 columns wide around
-// the middle of the two. A window of FILLW = 2*KSS columns centred there (FV = KSS/16 per lane) keeps
-// the shuffles' wrap-around at its edges, which spreads one column per row, out of the diamond. No
-// cost row has to be saved for the fill by the row loop.
-// A path cell's predecessor q is the leftmost minimum of the full costs, and its own path runs
-// through the upper end; another candidate left of q has a larger full cost, so its cost from the
-// upper end is larger too, and one right of q cannot be smaller: the restricted search takes q.
-// Costs are kept times 4 with the direction (0: from j-1, 1: from j, 2: from j+1) in the low bits
-// of each candidate, so one 3-input minimum yields the cost and the leftmost direction.
-// Energies are read in chunks of CH rows, the next chunk loaded ahead of the current one's rows.
-// Latency-bound: a chain of KSS rows (shuffle, minimum, add) and one of KSS shared-memory loads.
-// Against the form that recomputed full costs in a 4*KSS-column window from a saved cost row with
-// explicit comparisons: 1920x1080 carve 25.01 -> 24.52 ms, 3840x2160 carve 190.5 -> 183.9 ms, forward
-// energy at 1920x1080 62.2 -> 57.7 ms, a batch of 256 images (240..1280 columns) 44.5 -> 40.7 ms.
-constexpr uint32_t FILL_INF = 0x80000000u;   // above every path's 4 * cost (64 rows * 2 * 65535 * 4 < 2^25)
+// The parallel backtrack of seam_search, one warp per super-tile (rows rs .. rs+n-1, n <= KSS). The
+// ancestor chain has fixed both ends of the seam inside a super-tile: column jbs in its bottom row
+// and column jprev in the row above it (in the added row above row 0 for the first one), and the
+// seam between them is the leftmost cheapest path from one to the other: another candidate left of a
+// path cell's predecessor has a larger full cost, so a larger cost from the upper end too. So the fill
+// is a small search of its own, and like the search it runs from both ends at once: the upper nt rows
+// downwards from jprev (cost 0 there, infinity everywhere else), the lower nb rows upwards from jbs,
+// two independent chains in the same instructions; where they meet, the leftmost column of the cheapest
+// join continues both ways, and two lanes walk the directions to the two ends.
+// Only cells within r columns of an end, r rows from it, can be on the path: a diamond at most n + 1
+// columns wide around the middle of the two. A window of FILLW = 2*KSS columns centred there
+// (FV = KSS/16 per lane) keeps the shuffles' wrap-around at its edges, which spreads one column per
+// row, out of the diamond.
+// Costs are kept times 256 with the direction (0: from j-1, 1: from j, 2: from j+1) in the low byte of
+// each candidate, so two add-minima yield the cost and the leftmost direction.
+// Energies are read in chunks of fill_rows() rows, half of them from either end, every load of a chunk
+// in flight at once, and held in shared memory, so that the row loop stays a loop: the code runs
+// once per search and warp, from a cold instruction cache, where unrolled rows cost more to fetch
+// than to execute.
+// Latency-bound: loads ~1,100 cycles, rows and walk of half a super-tile each. Steps (1920x1080 carve):
+// full costs recomputed in a 4*KSS window from saved cost rows 25.0 ms, between the two ends 24.5 ms (a
+// batch of 256 images 44.5 -> 40.7 ms).
+constexpr uint32_t FILL_INF = 0x80000000u;   // above every path's 256 * cost (64 rows * 2 * 65535 * 256 < 2^31)
 
 struct FillCtx {
   const uint16_t *E;
-  const int *jb0;      // the chain's columns (rank 0's jb)
-  uint8_t *fdir;       // direction rows of the fill warps, a byte per column
-  uint32_t *csum;      // rank 0's sum of the recomputed path costs
+  unsigned char *fill; // the fill warps' shared memory
+  uint32_t *csum;      // receives the recomputed path costs ...
+  uint32_t csign;      // ... times this (1 or -1)
   int32_t *seam, *seam_log;
   int *err;
   int64_t pstride;
-  int pitch_e, H, W, Wa, S, cs;
+  int pitch_e, H, W, Wa;
   int step = 1;        // seam entries from one row to the next (-1: the map is swept from its bottom row)
 };
 
-template <int NW, int KT, bool CL, int FWM, bool FWD, int KSS, bool DIRECT, int CH>
-__device__ __forceinline__ void backtrack_fill(const FillCtx &f, int s_first, int warp, int lane) {
-  using G = Geo<NW, KT, CL, FWM, KSS>;
+// L2 prefetch of a super-tile's diamond (KSS rows, two rows per lane at most; from a 16-byte boundary)
+template <int KSS, bool FWD, bool DIRECT>
+__device__ __forceinline__ void fill_prefetch(const FillCtx &f, int s, int jprev, int jbs, int lane) {
+  int x0 = (((jprev + jbs) >> 1) - KSS / 2 - 1) & ~7;
+  int x1 = x0 + KSS + 16;
+  if (DIRECT) {   // only the caller's columns
+    x0 = max(x0, 0);
+    x1 = min(x1, f.Wa);
+    if (x1 <= x0) return;
+  }
+  for (int i = s * KSS + lane; i < s * KSS + KSS && i < f.H; i += 32)
+#pragma unroll
+    for (int pl = 0; pl < (FWD ? 3 : 1); ++pl)
+      bulk_prefetch_l2(f.E + pl * f.pstride + (ptrdiff_t)i * f.pitch_e + x0, (uint32_t)(x1 - x0) * 2);
+}
+
+// super-tile s between columns jprev and jbs, by one warp
+template <typename G, bool FWD, int KSS, bool DIRECT>
+__device__ __forceinline__ void fill_super_tile(const FillCtx &f, int s, int jprev, int jbs, int warp, int lane) {
   constexpr int NP = FWD ? 3 : 1;   // cost planes per row
-  constexpr int FV = G::FV, FILLW = G::FILLW;
+  constexpr int FV = G::FV, FILLW = G::FILLW, CR = G::fill_rows(FWD), HC = CR / 2;
   using DirT = typename std::conditional<FV == 4, uint32_t, uint16_t>::type;   // a byte per column
   using EVec = typename std::conditional<FV == 4, uint2, uint32_t>::type;      // FV uint16 energies
-  uint8_t *const fd = f.fdir + (size_t)warp * KSS * FILLW;
-  const uint16_t *const Ef = f.E;
-  int32_t *const seam_out = f.seam;
-  int32_t *const seam_log = f.seam_log;
-  int *const errw = f.err;
-  const int *const jb0 = f.jb0;
-  const int64_t pstride = f.pstride;
-  const int pitch_e = f.pitch_e, H = f.H, W = f.W, Wa = f.Wa, S = f.S, cs = f.cs;
-  // the energies of a super-tile's diamond (KSS rows, two rows per lane at most) are prefetched
-  // into L2 one super-tile ahead: the map may have left L2 since the DP pass read it. The
-  // prefetch starts on a 16-byte boundary and covers the diamond.
-  auto prefetch_window = [&](int s) {
-    if (s >= S) return;
-    const int mid = (jb0[s] + (s > 0 ? jb0[s - 1] : jb0[S])) >> 1;
-    int x0 = (mid - KSS / 2 - 1) & ~7;
-    int x1 = x0 + KSS + 16;
-    if (DIRECT) {   // only the caller's columns
-      x0 = max(x0, 0);
-      x1 = min(x1, Wa);
-      if (x1 <= x0) return;
-    }
-    for (int i = s * KSS + lane; i < s * KSS + KSS && i < H; i += 32)
+  unsigned char *const wmem = f.fill + (size_t)warp * G::fill_bytes(FWD);
+  EVec *const est = reinterpret_cast<EVec *>(wmem) + lane;   // this lane's energies: plane, end, row
+  uint8_t *const fd = wmem + CR * FILLW * 2 * NP;            // direction rows
+  const int x0 = (((jprev + jbs) >> 1) - FILLW / 2) & ~(FV - 1);
+  const int xc = x0 + lane * FV;
+  const int rs = s * KSS, n = min(KSS, f.H - rs);
+  // the upper nt rows and the lower nb; after the bottom row, which only holds the path's end, and the
+  // top row where nt = nb, both chains have T more rows to run together
+  const int nt = n >> 1, nb = n - nt, T = nb - 1, lead = nt - T;   // lead: 0 or 1
+  uint32_t m[FV], w[FV], wl[FV], wr[FV], oob[FV];   // costs from above, from below (FWD: plus DL, DR of their row)
 #pragma unroll
-      for (int pl = 0; pl < NP; ++pl)
-        bulk_prefetch_l2(Ef + pl * pstride + (ptrdiff_t)i * pitch_e + x0, (uint32_t)(x1 - x0) * 2);
-  };
-  // 4 * energy of the lane's columns
+  for (int u = 0; u < FV; ++u) {
+    oob[u] = (xc + u < 0 || xc + u >= f.W) ? FILL_INF : 0u;
+    m[u] = (xc + u == jprev) ? 0u : FILL_INF;
+  }
+  // 256 * energy of the lane's columns
   auto unpack = [](const EVec &v, uint32_t (&x)[FV]) {
-    const uint32_t *w = reinterpret_cast<const uint32_t *>(&v);
+    const uint32_t *p = reinterpret_cast<const uint32_t *>(&v);
 #pragma unroll
     for (int q = 0; q < FV / 2; ++q) {
-      x[2 * q] = (w[q] & 0xFFFFu) << 2;
-      x[2 * q + 1] = (w[q] >> 16) << 2;
+      x[2 * q] = lo8(p[q]);
+      x[2 * q + 1] = hi8(p[q]);
     }
   };
-  for (int s = s_first; s < S; s += G::FW * cs) {
-    prefetch_window(s + G::FW * cs);
-    const int jbs = jb0[s];
-    const int jprev = (s > 0) ? jb0[s - 1] : jb0[S];
-    const int x0 = (((jprev + jbs) >> 1) - FILLW / 2) & ~(FV - 1);
-    const int xc = x0 + lane * FV;
-    const int rs = s * KSS, re = (rs + KSS < H) ? rs + KSS : H;
-    uint32_t m[FV], oob[FV];
+  // one row: costs m (candidates from the left l, from the right r) -> new costs plus energies e, and
+  // the directions in the low bytes of the candidates' minima
+  auto step_row = [&](const uint32_t (&l)[FV], const uint32_t (&c)[FV], const uint32_t (&r)[FV], const uint32_t (&e)[FV],
+                      uint32_t (&out)[FV], uint8_t *dst) {
+    uint32_t mn[FV];
 #pragma unroll
     for (int u = 0; u < FV; ++u) {
-      oob[u] = (xc + u < 0 || xc + u >= W) ? FILL_INF : 0u;
-      m[u] = (xc + u == jprev) ? 0u : FILL_INF;
+      mn[u] = __viaddmin_u32(r[u], 2u, __viaddmin_u32(c[u], 1u, l[u]));
+      out[u] = __viaddmax_u32(mn[u] & ~0xFFu, e[u], oob[u]);
     }
-    // DIRECT: a lane's FV columns lie wholly inside or wholly outside the caller's [0, Wa)
-    const bool xin = !DIRECT || (xc >= 0 && xc + FV <= Wa);
-    // rows rs..re-1 in chunks of CH rows, the next chunk's energies loaded ahead
-    EVec eb0[NP][CH], eb1[NP][CH];
-    auto load_chunk = [&](EVec (&eb)[NP][CH], int rbeg) {
+    uint32_t d = __byte_perm(mn[0], mn[1], 0x0040);
+    if (FV == 4) d = __byte_perm(d, __byte_perm(mn[FV - 2], mn[FV - 1], 0x0040), 0x5410);
+    *reinterpret_cast<DirT *>(dst) = (DirT)d;
+  };
+  // DIRECT: a lane's FV columns lie wholly inside or wholly outside the caller's [0, Wa)
+  const bool xin = !DIRECT || (xc >= 0 && xc + FV <= f.Wa);
+  // chunk q0: the rows q0, q0 + 1, ... after the top row(s) led by, and before the bottom row
+  EVec eb[NP][CR];
+  auto load_chunk = [&](int q0) {
 #pragma unroll
-      for (int r = 0; r < CH; ++r) {
-        const int i = rbeg + r;
+    for (int pl = 0; pl < NP; ++pl) {
+      const uint16_t *top = f.E + pl * f.pstride + (ptrdiff_t)(rs + lead + q0) * f.pitch_e + xc;
+      const uint16_t *bot = f.E + pl * f.pstride + (ptrdiff_t)(rs + n - 2 - q0) * f.pitch_e + xc;
 #pragma unroll
-        for (int pl = 0; pl < NP; ++pl)
-          if (i < re) {
-            if (xin) eb[pl][r] = *reinterpret_cast<const EVec *>(Ef + pl * pstride + (ptrdiff_t)i * pitch_e + xc);
-            else eb[pl][r] = EVec{};
-          }
-      }
-    };
-    auto run_chunk = [&](const EVec (&eb)[NP][CH], int rbeg) {
-#pragma unroll
-      for (int r = 0; r < CH; ++r) {
-        const int i = rbeg + r;
-        if (i >= re) break;
-        uint32_t ee[FV], dl[FV], dr[FV];
-#pragma unroll
-        for (int u = 0; u < FV; ++u) dl[u] = dr[u] = 0u;
-        unpack(eb[0][r], ee);
-        if (FWD) {
-          unpack(eb[NP > 1 ? 1 : 0][r], dl);
-          unpack(eb[NP > 2 ? 2 : 0][r], dr);
+      for (int r = 0; r < HC; ++r, top += f.pitch_e, bot -= f.pitch_e) {
+        eb[pl][r] = eb[pl][HC + r] = EVec{};
+        if (xin && q0 + r < T) {
+          eb[pl][r] = *reinterpret_cast<const EVec *>(top);
+          eb[pl][HC + r] = *reinterpret_cast<const EVec *>(bot);
         }
-        const uint32_t L = __shfl_up_sync(0xffffffffu, m[FV - 1], 1);
-        const uint32_t R = __shfl_down_sync(0xffffffffu, m[0], 1);
-        uint32_t nm[FV];
-        uint32_t dirs = 0;
-#pragma unroll
-        for (int u = 0; u < FV; ++u) {
-          const uint32_t a = ((u == 0) ? L : m[u - 1]) + dl[u];
-          const uint32_t c = ((u == FV - 1) ? R : m[u + 1]) + dr[u];
-          const uint32_t mn = min3u(a, m[u] + 1u, c + 2u);
-          dirs |= (mn & 3u) << (8 * u);
-          nm[u] = __viaddmax_u32(mn & ~3u, ee[u], oob[u]);
-        }
-#pragma unroll
-        for (int u = 0; u < FV; ++u) m[u] = nm[u];
-        *reinterpret_cast<DirT *>(fd + (i - rs) * FILLW + lane * FV) = (DirT)dirs;
       }
-    };
-    int rb = rs;
-    load_chunk(eb0, rb);
-    while (rb < re) {
-      if (rb + CH < re) load_chunk(eb1, rb + CH);
-      run_chunk(eb0, rb);
-      rb += CH;
-      if (rb >= re) break;
-      if (rb + CH < re) load_chunk(eb0, rb + CH);
-      run_chunk(eb1, rb);
-      rb += CH;
+    }
+  };
+  auto load_row = [&](int i, int pl) {
+    return xin ? *reinterpret_cast<const EVec *>(f.E + pl * f.pstride + (ptrdiff_t)(rs + i) * f.pitch_e + xc) : EVec{};
+  };
+  // the candidates of one chain from its costs: neighbours' values by shuffle; the chain from above
+  // adds the row's own DL and DR, the one from below carries those of the row it comes from
+  auto down_row = [&](const uint32_t (&e)[FV], const uint32_t (&dl)[FV], const uint32_t (&dr)[FV], uint8_t *dst) {
+    const uint32_t L = __shfl_up_sync(0xffffffffu, m[FV - 1], 1), R = __shfl_down_sync(0xffffffffu, m[0], 1);
+    uint32_t l[FV], c[FV], r[FV];
+#pragma unroll
+    for (int u = 0; u < FV; ++u) {
+      l[u] = (u == 0 ? L : m[u > 0 ? u - 1 : 0]) + (FWD ? dl[u] : 0u);
+      c[u] = m[u];
+      r[u] = (u == FV - 1 ? R : m[u < FV - 1 ? u + 1 : u]) + (FWD ? dr[u] : 0u);
+    }
+    step_row(l, c, r, e, m, dst);
+  };
+  auto up_candidates = [&](uint32_t (&l)[FV], uint32_t (&c)[FV], uint32_t (&r)[FV]) {
+    const uint32_t L = __shfl_up_sync(0xffffffffu, FWD ? wr[FV - 1] : w[FV - 1], 1);
+    const uint32_t R = __shfl_down_sync(0xffffffffu, FWD ? wl[0] : w[0], 1);
+#pragma unroll
+    for (int u = 0; u < FV; ++u) {
+      l[u] = u == 0 ? L : (FWD ? wr[u > 0 ? u - 1 : 0] : w[u > 0 ? u - 1 : 0]);
+      c[u] = w[u];
+      r[u] = u == FV - 1 ? R : (FWD ? wl[u < FV - 1 ? u + 1 : u] : w[u < FV - 1 ? u + 1 : u]);
+    }
+  };
+  auto carry = [&](const uint32_t (&dl)[FV], const uint32_t (&dr)[FV]) {
+    if (FWD)
+#pragma unroll
+      for (int u = 0; u < FV; ++u) {
+        wl[u] = w[u] + dl[u];
+        wr[u] = w[u] + dr[u];
+      }
+  };
+  EVec et0[NP], eb0[NP];   // the bottom row and the leading top row
+#pragma unroll
+  for (int pl = 0; pl < NP; ++pl) {
+    eb0[pl] = load_row(n - 1, pl);
+    et0[pl] = lead ? load_row(0, pl) : EVec{};
+  }
+  load_chunk(0);
+  {
+    uint32_t e[FV], dl[FV] = {}, dr[FV] = {};
+    unpack(eb0[0], e);
+    if (FWD) {
+      unpack(eb0[NP > 1 ? 1 : 0], dl);
+      unpack(eb0[NP > 2 ? 2 : 0], dr);
     }
 #pragma unroll
-    for (int u = 0; u < FV; ++u)
-      if (xc + u == jbs) atomicAdd(f.csum, m[u] >> 2);   // the path's cost in this super-tile
-    __syncwarp();
-    // lane 0 follows the directions up the window (relative columns, kept in the direction rows it
-    // has read: a row's entry is not needed again), then the warp writes the seam rows
-    if (lane == 0) {
-      int rel = jbs - x0;
-      bool okp = (unsigned)rel < (unsigned)FILLW;
-      rel = min(max(rel, 0), FILLW - 1);
-      // a step leaving the window is clamped (every read stays in this warp's rows) and recorded as
-      // a failure
-      uint8_t *fb = fd + (re - 1 - rs) * FILLW;
-      for (int i = re - 1; i >= rs; --i, fb -= FILLW) {
-        const int nr = rel + (int)fb[rel] - 1;
-        *reinterpret_cast<uint32_t *>(fb) = (uint32_t)rel;
-        okp &= (unsigned)nr < (unsigned)FILLW;
-        rel = min(max(nr, 0), FILLW - 1);
+    for (int u = 0; u < FV; ++u) w[u] = (xc + u == jbs) ? e[u] : FILL_INF;
+    carry(dl, dr);
+    *reinterpret_cast<DirT *>(fd + (n - 1) * FILLW + lane * FV) = (DirT)0x01010101u;   // no step below it
+    if (lead) {
+      unpack(et0[0], e);
+      if (FWD) {
+        unpack(et0[NP > 1 ? 1 : 0], dl);
+        unpack(et0[NP > 2 ? 2 : 0], dr);
       }
-      if (!okp || x0 + rel != jprev) atomicOr(errw, ERR_FILL_MISMATCH);
+      down_row(e, dl, dr, fd + lane * FV);
     }
-    __syncwarp();
-    for (int i = rs + lane; i < re; i += 32) {
-      const int j = x0 + (int)*reinterpret_cast<const uint32_t *>(fd + (i - rs) * FILLW);
-      seam_out[i * f.step] = j;
-      if (seam_log) seam_log[i * f.step] = j;
+  }
+#pragma unroll 1
+  for (int q0 = 0; q0 < T; q0 += HC) {
+    // each lane reads back only what it stored
+#pragma unroll
+    for (int pl = 0; pl < NP; ++pl)
+#pragma unroll
+      for (int r = 0; r < CR; ++r) est[(pl * CR + r) * 32] = eb[pl][r];
+    if (CR < KSS && q0 + HC < T) load_chunk(q0 + HC);   // in flight during this chunk's rows
+    const int nq = min(HC, T - q0);
+    const EVec *es = est;
+    uint8_t *ft = fd + (lead + q0) * FILLW + lane * FV, *fb = fd + (n - 2 - q0) * FILLW + lane * FV;
+#pragma unroll 1
+    for (int r = 0; r < nq; ++r, ft += FILLW, fb -= FILLW, es += 32) {
+      uint32_t e[FV], g[FV], dl[FV] = {}, dr[FV] = {}, gl[FV] = {}, gr[FV] = {}, l[FV], c[FV], rr[FV];
+      unpack(es[0], e);
+      unpack(es[HC * 32], g);
+      if (FWD) {
+        unpack(es[CR * 32], dl);
+        unpack(es[2 * CR * 32], dr);
+        unpack(es[(CR + HC) * 32], gl);
+        unpack(es[(2 * CR + HC) * 32], gr);
+      }
+      up_candidates(l, c, rr);
+      down_row(e, dl, dr, ft);
+      step_row(l, c, rr, g, w, fb);
+      carry(gl, gr);
     }
-    __syncwarp();
+  }
+  // the join: the leftmost column of row nt - 1 (jprev itself when nt = 0) on a cheapest path, and the
+  // leftmost of its three successors
+  uint32_t best = SENT, where = SENT;   // cost * 256; column in the window << 2 | direction
+  {
+    uint32_t l[FV], c[FV], r[FV];
+    up_candidates(l, c, r);
+#pragma unroll
+    for (int u = 0; u < FV; ++u) {
+      const uint32_t mn = __viaddmin_u32(r[u], 2u, __viaddmin_u32(c[u], 1u, l[u]));
+      const uint32_t sum = m[u] >= FILL_INF || mn >= FILL_INF ? SENT : m[u] + (mn & ~0xFFu);
+      if (sum < best) {
+        best = sum;
+        where = ((uint32_t)(lane * FV + u) << 2) | (mn & 3u);
+      }
+    }
+    const uint32_t b = __reduce_min_sync(0xffffffffu, best);
+    where = __reduce_min_sync(0xffffffffu, best == b ? where : SENT);
+    best = b;
+  }
+  if (lane == 0) atomicAdd(f.csum, (best >> 8) * f.csign);   // the path's cost in this super-tile
+  // lanes 0 and 1 follow the directions up and down (relative columns, kept in the direction rows they
+  // have read: a row's entry is not needed again), then the warp writes the seam rows
+  if (lane < 2) {
+    // a path that leaves the window (it cannot) wraps around inside this warp's rows and ends on the
+    // wrong column
+    int rel = ((int)(where >> 2) + (lane ? (int)(where & 3u) - 1 : 0)) & (FILLW - 1);
+    uint8_t *fb = fd + (lane ? nt : nt - 1) * FILLW;
+    const int stride = lane ? FILLW : -FILLW, steps = lane ? nb : nt;
+#pragma unroll 2
+    for (int q = 0; q < steps; ++q, fb += stride) {
+      const int nr = rel + (int)(fb[rel] & 3u) - 1;
+      *reinterpret_cast<uint32_t *>(fb) = (uint32_t)rel;
+      rel = nr & (FILLW - 1);
+    }
+    if (best == SENT || x0 + rel != (lane ? jbs : jprev)) atomicOr(f.err, ERR_FILL_MISMATCH);
+  }
+  __syncwarp();
+  for (int i = lane; i < n; i += 32) {
+    const int j = x0 + (int)*reinterpret_cast<const uint32_t *>(fd + i * FILLW);
+    f.seam[(rs + i) * f.step] = j;
+    if (f.seam_log) f.seam_log[(rs + i) * f.step] = j;
+  }
+  __syncwarp();
+}
+
+// The super-tiles of one warp, warp*cs + rank, + FW*cs, ... of S; jb: the chain's columns (rank 0's
+// table). The energies of a super-tile's diamond are prefetched into L2 one super-tile ahead: the map
+// may have left L2 since the DP pass read it.
+template <typename G, bool FWD, int KSS, bool DIRECT>
+__device__ __forceinline__ void backtrack_fill(const FillCtx &f, const int *jb, int S, int cs, int rank, int warp,
+                                               int lane) {
+  auto prev = [&](int s) { return s > 0 ? jb[s - 1] : jb[S]; };
+#pragma unroll 1
+  for (int s = warp * cs + rank; s < S; s += G::FW * cs) {
+    const int nx = s + G::FW * cs;
+    if (nx < S) fill_prefetch<KSS, FWD, DIRECT>(f, nx, prev(nx), jb[nx], lane);
+    fill_super_tile<G, FWD, KSS, DIRECT>(f, s, prev(s), jb[s], warp, lane);
   }
 }
 
 // backtrack_fill as a function of its own (not inlined): it gets its own register allocation, so
 // the one-CTA batched kernel, whose 512 threads have at most 128 registers each, can load deeper
 // energy chunks
-template <int NW, int KT, bool CL, int FWM, bool FWD, int KSS, bool DIRECT, int CH>
-static __device__ __noinline__ void backtrack_fill_call(FillCtx f, int s_first, int warp, int lane) {
-  backtrack_fill<NW, KT, CL, FWM, FWD, KSS, DIRECT, CH>(f, s_first, warp, lane);
+template <typename G, bool FWD, int KSS, bool DIRECT>
+static __device__ __noinline__ void backtrack_fill_call(FillCtx f, const int *jb, int S, int cs, int rank, int warp,
+                                                        int lane) {
+  backtrack_fill<G, FWD, KSS, DIRECT>(f, jb, S, cs, rank, warp, lane);
 }
 
 // The row loop: every thread of the CTA (of every CTA of the cluster when CL) calls it with the same
@@ -743,7 +836,6 @@ __device__ void seam_search(const SearchArgs &p, unsigned char *smem, int Smax, 
   int *jb = reinterpret_cast<int *>(smem + plan.jb);
   int *misc = reinterpret_cast<int *>(smem + plan.misc);
   uint32_t *emx = reinterpret_cast<uint32_t *>(smem + plan.emx);   // DIRECT: [NW + 1] per warp, then per CTA
-  uint8_t *fdir = smem + plan.fdir;
   const int gw = plan.gw;
   uint8_t *const gat = smem + plan.gat;
   const int64_t pstride = FWD ? p.pstride : 0;
@@ -822,19 +914,12 @@ __device__ void seam_search(const SearchArgs &p, unsigned char *smem, int Smax, 
   const int *misc0 = CL ? cg::this_cluster().map_shared_rank(misc, 0) : misc;
   const int ok = misc0[0];
   if (ok && warp < G::FW) {
-    const FillCtx f{p.E, jb0, fdir, const_cast<uint32_t *>(reinterpret_cast<const uint32_t *>(misc0 + 1)), p.seam,
-                    p.seam_log, p.err, pstride, p.pitch_e, H, W, Wa, S, cs};
-    // energy chunks: the single-map search (all fill warps, one CTA per SM, latency-bound) has
-    // registers to spare and keeps 32 rows of loads in flight; the multi-map and cluster batched
-    // kernels, whose latency other CTAs hide and whose registers are capped, use 8-row chunks; the
-    // one-CTA batched kernel calls the fill as a function of its own (the same call in the cluster
-    // batched kernel was slower, so that one stays inline).
-    if constexpr (!CL && !FWD) {
-      backtrack_fill_call<NW, KT, CL, FWM, FWD, KSS, DIRECT, 8>(f, warp * cs + rank, warp, lane);
-    } else {
-      constexpr int CH = FWD ? 4 : ((CL && FWM >= FILL_WARPS_MAX) ? 16 : 8);
-      backtrack_fill<NW, KT, CL, FWM, FWD, KSS, DIRECT, CH>(f, warp * cs + rank, warp, lane);
-    }
+    const FillCtx f{p.E, smem + plan.fill, const_cast<uint32_t *>(reinterpret_cast<const uint32_t *>(misc0 + 1)), 1u,
+                    p.seam, p.seam_log, p.err, pstride, p.pitch_e, H, W, Wa};
+    // the one-CTA batched kernel calls the fill as a function of its own (the same call in the
+    // cluster batched kernel was slower, so that one stays inline)
+    if constexpr (!CL && !FWD) backtrack_fill_call<G, FWD, KSS, DIRECT>(f, jb0, S, cs, rank, warp, lane);
+    else backtrack_fill<G, FWD, KSS, DIRECT>(f, jb0, S, cs, rank, warp, lane);
   }
   group_sync<CL>();   // rank 0's shared memory is read above; the seam is complete after this
   // the recomputed path costs must add up to the argmin's
