@@ -49,8 +49,9 @@ __global__ void __launch_bounds__(Geo<NW, KT, true>::THREADS, 1)
   // neighbours push into each other's halo buffers: every CTA's barriers must be initialised first
   cg::this_cluster().sync();
   // the set-up above overlaps the previous kernel of the seam loop; its results are read below
-  pdl_launch_dependents();
   pdl_wait_prerequisites();
+  // only now: the refresh that depends on this launch reads what its predecessors wrote before it waits
+  pdl_launch_dependents();
   SearchArgs a;
   a.E = p.E;
   a.pitch_e = p.pitch_e;
@@ -238,8 +239,9 @@ __global__ void __launch_bounds__(Geo<NW, KT, true>::THREADS, 1)
   // neighbours push into each other's halo buffers: every CTA's barriers must be initialised first
   cl.sync();
   // the set-up above overlaps the previous kernel of the seam loop; its results are read below
-  pdl_launch_dependents();
   pdl_wait_prerequisites();
+  // only now: the refresh that depends on this launch reads what its predecessors wrote before it waits
+  pdl_launch_dependents();
   if (p.gate && (*p.gate & ERR_ENERGY_RANGE)) return;   // left to the wide-cost search
   uint32_t *const end0 = p.scratch, *const end1 = end0 + g.gw;
   uint8_t *const tab = reinterpret_cast<uint8_t *>(end1 + g.gw);

@@ -109,18 +109,84 @@ __global__ void k_unpad_energy(const uint16_t *__restrict__ E, int pe, int H, in
   dst[(int64_t)i * W + j] = E[(int64_t)i * pe + j];
 }
 
-// ---- lazy image compaction: refresh through the pending-removal lists, then add the removal ----
-// one warp per row: refreshed pair (lazy image), list update, energy compaction (refresh_row)
-__global__ void k_refresh(const uint32_t *__restrict__ img, int pitch, uint16_t *__restrict__ E, int pe, int H, int W,
-                          const int32_t *__restrict__ seam, const int16_t *__restrict__ lists_in,
-                          int16_t *__restrict__ lists_out, int m, int *err) {
+// ---- the per-seam refresh, one warp per row: the refreshed energy pair through the pending-removal
+// lists, the removal added to the row's list, the energy row's tail shifted left past the seam ----
+// It sits between one seam's search and the next, so what counts is its chain of memory round trips
+// after the seam is known. Launched as a programmatic dependent it is resident while the search runs,
+// and the search starts its dependents only after it has itself waited for the kernel before it: the
+// energies, lists and image words are then in their final state (nothing writes them until this kernel
+// does). So everything that does not need the seam is loaded before the wait: the whole energy row
+// into registers (R chunks of 8 elements per lane) and the three rows' lists. After the wait: the
+// seam columns, one round trip; the tail goes out of the registers while eight lanes fetch the eight
+// pixels of the refreshed pair, a second one. From the end of the search to the end of the refresh:
+// 1920x1080 5.5 -> 3.2 us (carve 14.6 -> 12.6 ms), 1279x853 4.9 -> 3.1 us (carve 11.6 -> 9.7 ms).
+template <int R>
+__global__ void __launch_bounds__(256) k_refresh(const uint32_t *__restrict__ img, int pitch, uint16_t *E, int pe, int H,
+                                                 int W, const int32_t *__restrict__ seam,
+                                                 const int16_t *__restrict__ lists_in, int16_t *__restrict__ lists_out,
+                                                 int m, int *err) {
   const int lane = threadIdx.x & 31;
-  const int warps = (gridDim.x * blockDim.x) >> 5;
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   pdl_launch_dependents();
+  if (i >= H) return;
+  uint16_t *const er = E + (int64_t)i * pe;
+  const int c_hi = (W - 2) >> 3;   // the chunk holding the new last column
+  uint4 x[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int c = lane + 32 * r;
+    x[r] = make_uint4(0u, 0u, 0u, 0u);
+    if (c <= c_hi + 1) x[r] = __ldcg(reinterpret_cast<const uint4 *>(er + 8 * c));
+  }
+  const RefreshLane f = refresh_lane(lists_in, m, H, i, lane);
   pdl_wait_prerequisites();   // the seam of the search that precedes this launch
-  for (int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < H; i += warps)
-    if (!refresh_row(img, pitch, E, pe, H, W, seam, lists_in, lists_out, m, i, lane) && lane == 0)
-      atomicOr(err, ERR_BAD_SEAM);
+  const int s = __ldcg(seam + i);
+  const int sr = __ldcg(seam + f.row);
+  if (s < 0 || s >= W) {
+    if (lane == 0) atomicOr(err, ERR_BAD_SEAM);
+    return;
+  }
+  const uint32_t px = refresh_pixel(f, img, pitch, W, s, sr, lane);
+  if (lane == 0) list_insert(f.list, lists_out + (int64_t)i * RPEND, s);
+  if (s < W - 1) {
+    const int c_lo = s >> 3;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      // the first element of the next chunk: lane + 1's, or the first lane's next one
+      const uint32_t first = (lane == 0 && r + 1 < R) ? x[r + 1 < R ? r + 1 : r].x : x[r].x;
+      const uint32_t nx = __shfl_sync(0xffffffffu, first, (lane + 1) & 31);
+      const int c = lane + 32 * r;
+      if (c >= c_lo && c <= c_hi) *reinterpret_cast<uint4 *>(er + 8 * c) = shift_chunk(x[r], nx, s - 8 * c);
+    }
+  }
+  __syncwarp();   // the pair goes over the chunk holding s
+  const uint32_t e = refresh_energy(px);
+  if (lane == 0 && s >= 1) er[s - 1] = (uint16_t)e;
+  if (lane == 4 && s <= W - 2) er[s] = (uint16_t)e;
+}
+
+// rows wider than the registers hold: chunk by chunk, everything after the wait
+__global__ void k_refresh_wide(const uint32_t *__restrict__ img, int pitch, uint16_t *__restrict__ E, int pe, int H, int W,
+                               const int32_t *__restrict__ seam, const int16_t *__restrict__ lists_in,
+                               int16_t *__restrict__ lists_out, int m, int *err) {
+  const int lane = threadIdx.x & 31;
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  pdl_launch_dependents();
+  if (i >= H) return;
+  const RefreshLane f = refresh_lane(lists_in, m, H, i, lane);
+  pdl_wait_prerequisites();
+  const int s = seam[i], sr = seam[f.row];
+  if (s < 0 || s >= W) {
+    if (lane == 0) atomicOr(err, ERR_BAD_SEAM);
+    return;
+  }
+  uint16_t *const er = E + (int64_t)i * pe;
+  const uint32_t px = refresh_pixel(f, img, pitch, W, s, sr, lane);
+  if (lane == 0) list_insert(f.list, lists_out + (int64_t)i * RPEND, s);
+  shift_row_u16(er, s, W, lane);
+  const uint32_t e = refresh_energy(px);
+  if (lane == 0 && s >= 1) er[s - 1] = (uint16_t)e;
+  if (lane == 4 && s <= W - 2) er[s] = (uint16_t)e;
 }
 
 __global__ void k_refresh_fwd(const uint32_t *__restrict__ img, int pitch, uint16_t *__restrict__ E, int pe,
@@ -228,11 +294,9 @@ namespace sc {
 
 cudaError_t launch_refresh(const uint32_t *img, int pitch, uint16_t *E, int pe, int H, int W, const int32_t *seam,
                            const int16_t *lists_in, int16_t *lists_out, int m, int *err, cudaStream_t st) {
-  const int warps_per_block = 8;
-  int blocks = (H + warps_per_block - 1) / warps_per_block;
-  if (blocks > 152 * 8) blocks = 152 * 8;
-  return launch_pdl(k_refresh, blocks, warps_per_block * 32, st, img, pitch, E, pe, H, W, seam, lists_in, lists_out, m,
-                    err);
+  // 8 rows per block; registers for rows up to 1024, 2048 or 4096 elements
+  auto *const k = W <= 1024 ? k_refresh<4> : (W <= 2048 ? k_refresh<8> : (W <= 4096 ? k_refresh<16> : k_refresh_wide));
+  return launch_pdl(k, (H + 7) / 8, 256, st, img, pitch, E, pe, H, W, seam, lists_in, lists_out, m, err);
 }
 
 cudaError_t launch_refresh_fwd(const uint32_t *img, int pitch, uint16_t *E, int pe, int64_t pstride, int H, int W,

@@ -22,21 +22,36 @@ __device__ __forceinline__ uint32_t energy_at(const uint32_t *img, int pitch, in
   return sad4(row[jr], row[jl]) + sad4(img[(int64_t)id * pitch + j], img[(int64_t)iu * pitch + j]);
 }
 
+// Eight uint16 elements x moved down one, the first of the next eight (nx, low half) shifted in; the
+// leading `keep` elements (none when keep <= 0) stay where they are.
+__device__ __forceinline__ uint4 shift_chunk(const uint4 &x, uint32_t nx, int keep) {
+  uint4 o;
+  o.x = __funnelshift_r(x.x, x.y, 16);
+  o.y = __funnelshift_r(x.y, x.z, 16);
+  o.z = __funnelshift_r(x.z, x.w, 16);
+  o.w = __funnelshift_r(x.w, nx, 16);
+  if (keep > 0) {
+    auto merge = [keep](uint32_t in, uint32_t sh, int q) {
+      const uint32_t m = (2 * q < keep ? 0x0000FFFFu : 0u) | (2 * q + 1 < keep ? 0xFFFF0000u : 0u);
+      return (in & m) | (sh & ~m);
+    };
+    o.x = merge(x.x, o.x, 0);
+    o.y = merge(x.y, o.y, 1);
+    o.z = merge(x.z, o.z, 2);
+    o.w = merge(x.w, o.w, 3);
+  }
+  return o;
+}
+
 // In-place left shift by one of a 16-byte-aligned uint16 row, row[s+1 .. W-1] -> row[s .. W-2],
 // by one warp, 8 elements (one 16-byte load and store) at a time: chunk c of the result is chunk c of the input moved down one element, with the first
 // element of chunk c+1 shifted in; every lane reads its chunks and the element after each chunk
 // before any lane of the warp writes. The first chunk keeps its elements left of s. Elements from
 // W-1 to the end of the last chunk are left undefined (they lie in the row's padding or in the
 // column that the shift drops).
-// `between` runs once, after the first block of loads is issued and before any store (work that
-// overlaps their latency; it must not touch the row).
-template <typename F>
-__device__ __forceinline__ void shift_row_u16(uint16_t *row, int s, int W, int lane, F &&between) {
+__device__ __forceinline__ void shift_row_u16(uint16_t *row, int s, int W, int lane) {
   constexpr int R = 4;
-  if (s >= W - 1) {
-    between();
-    return;
-  }
+  if (s >= W - 1) return;
   const int c_lo = s >> 3, c_hi = (W - 2) >> 3;
   for (int cb = c_lo; cb <= c_hi; cb += 32 * R) {
     uint4 x[R];
@@ -49,37 +64,16 @@ __device__ __forceinline__ void shift_row_u16(uint16_t *row, int s, int W, int l
         nx[r] = row[8 * c + 8];
       }
     }
-    if (cb == c_lo) between();
     __syncwarp();
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       const int c = cb + r * 32 + lane;
       if (c <= c_hi) {
-        uint4 o;
-        o.x = __funnelshift_r(x[r].x, x[r].y, 16);
-        o.y = __funnelshift_r(x[r].y, x[r].z, 16);
-        o.z = __funnelshift_r(x[r].z, x[r].w, 16);
-        o.w = __funnelshift_r(x[r].w, nx[r], 16);
-        if (c == c_lo) {
-          const int keep = s - 8 * c;   // leading elements of this chunk that stay
-          auto merge = [keep](uint32_t in, uint32_t sh, int q) {
-            const uint32_t m = (2 * q < keep ? 0x0000FFFFu : 0u) | (2 * q + 1 < keep ? 0xFFFF0000u : 0u);
-            return (in & m) | (sh & ~m);
-          };
-          o.x = merge(x[r].x, o.x, 0);
-          o.y = merge(x[r].y, o.y, 1);
-          o.z = merge(x[r].z, o.z, 2);
-          o.w = merge(x[r].w, o.w, 3);
-        }
-        *reinterpret_cast<uint4 *>(row + 8 * c) = o;
+        *reinterpret_cast<uint4 *>(row + 8 * c) = shift_chunk(x[r], nx[r], s - 8 * c);
       }
     }
     __syncwarp();
   }
-}
-
-__device__ __forceinline__ void shift_row_u16(uint16_t *row, int s, int W, int lane) {
-  shift_row_u16(row, s, W, lane, [] {});
 }
 
 __device__ __forceinline__ uint32_t pack_pixel(const uint8_t *s, int C) {
@@ -266,43 +260,34 @@ __device__ __forceinline__ void compact_row_lazy(uint32_t *row, const int16_t *l
 
 namespace sc {
 
-// One warp, row i, after seam `seam` was found in the width-W energy map E (and image words read
-// through the pending-removal lists_in with m entries): the row's refreshed energy pair (lane 0,
-// through the lazy map), the row's list with this removal added (lists_out), then the energy row's
-// tail shifted left past the seam and the pair written at the new columns s-1 and s.
-// Returns false when the seam column is out of range (nothing is changed then).
-__device__ __forceinline__ bool refresh_row(const uint32_t *img, int pitch, uint16_t *E, int pe, int H, int W,
-                                            const int32_t *seam, const int16_t *lists_in, int16_t *lists_out, int m,
-                                            int i, int lane) {
-  // lane 0's pending-removal lists of rows i-1, i, i+1 and the neighbours' seam columns depend on i
-  // alone: loaded beside seam[i], they take a round trip off the refreshed pair's path
-  const int iu = i > 0 ? i - 1 : 0, id = i + 1 < H ? i + 1 : H - 1;
-  LazyRow lu{}, lc{}, ld{};
-  int su = 0, sd = 0;
-  if (lane == 0) {
-    lc = lazy_row(lists_in + (int64_t)i * RPEND, m);
-    lu = lazy_row(lists_in + (int64_t)iu * RPEND, m);
-    ld = lazy_row(lists_in + (int64_t)id * RPEND, m);
-    su = seam[iu];
-    sd = seam[id];
-  }
-  const int s = seam[i];
-  if (s < 0 || s >= W) return false;
-  uint32_t p = 0;
-  uint16_t *er = E + (int64_t)i * pe;
-  // lane 0 computes the refreshed pair (image words through the lists, not the energy row) while
-  // the warp's loads of the energy tail are in flight
-  shift_row_u16(er, s, W, lane, [&] {
-    if (lane == 0) {
-      p = patch_pair(img, pitch, W, i, s, iu, su, lu, lc, id, sd, ld);
-      list_insert(lc, lists_out + (int64_t)i * RPEND, s);
-    }
-  });
-  if (lane == 0) {
-    if (s >= 1) er[s - 1] = (uint16_t)(p & 0xFFFFu);
-    if (s <= W - 2) er[s] = (uint16_t)(p >> 16);
-  }
-  return true;
+// The refreshed pair of row i by one warp, eight lanes fetching one pixel each (see patch_pair for what
+// changes): lanes 0, 1 the new columns s and s-2 of the row itself and lanes 2, 3 column s-1 below and
+// above, which make e(s-1); lanes 4, 5 columns s+1 and s-1 and lanes 6, 7 column s below and above,
+// which make e(s). The other lanes repeat lanes 0..7.
+struct RefreshLane {
+  LazyRow list;   // pending removals of the lane's row
+  int row;        // the row its pixel lies in (i, or a neighbour; edge rows replicated)
+};
+__device__ __forceinline__ RefreshLane refresh_lane(const int16_t *lists, int m, int H, int i, int lane) {
+  RefreshLane f;
+  const int q = lane & 7;
+  f.row = (q & 2) == 0 ? i : ((q & 1) ? max(i - 1, 0) : min(i + 1, H - 1));
+  f.list = lazy_row(lists + (int64_t)f.row * RPEND, m);
+  return f;
+}
+// the lane's pixel; s: row i's seam column, sr: that of the lane's row
+__device__ __forceinline__ uint32_t refresh_pixel(const RefreshLane &f, const uint32_t *img, int pitch, int W, int s,
+                                                  int sr, int lane) {
+  const int q = lane & 7;
+  // new column: s, s-2, s-1, s-1 | s+1, s-1, s, s
+  const int j = clampi(s + ((q & 2) ? ((q & 4) ? 0 : -1) : ((q & 4) ? 1 : 0) - ((q & 1) ? 2 : 0)), 0, W - 2);
+  const int x = j + (j >= sr ? 1 : 0);   // column in the width-W image
+  return img[(int64_t)f.row * pitch + x + lazy_count(f.list, x)];
+}
+// from every lane's pixel: e(s-1) in lanes 0..3, e(s) in lanes 4..7
+__device__ __forceinline__ uint32_t refresh_energy(uint32_t px) {
+  const uint32_t d = sad4(px, __shfl_xor_sync(0xffffffffu, px, 1));
+  return d + __shfl_xor_sync(0xffffffffu, d, 2);
 }
 
 // The energy shift of every row this warp owns (local rows q = warp, warp + nwarps, ... of nq; image
@@ -383,23 +368,7 @@ static __device__ __noinline__ bool shift_rows_bulk(uint16_t *E, int pe, int nq,
       for (int c = c_lo + lane; c <= c_last; c += 32) {
         const uint4 x = *reinterpret_cast<const uint4 *>(b + 8 * (c - c_lo));
         const uint32_t nx = b[8 * (c - c_lo) + 8];
-        uint4 o;
-        o.x = __funnelshift_r(x.x, x.y, 16);
-        o.y = __funnelshift_r(x.y, x.z, 16);
-        o.z = __funnelshift_r(x.z, x.w, 16);
-        o.w = __funnelshift_r(x.w, nx, 16);
-        if (c == c_lo) {
-          const int keep = st - 8 * c;   // leading elements of this chunk that stay
-          auto merge = [keep](uint32_t in, uint32_t sh, int j) {
-            const uint32_t m = (2 * j < keep ? 0x0000FFFFu : 0u) | (2 * j + 1 < keep ? 0xFFFF0000u : 0u);
-            return (in & m) | (sh & ~m);
-          };
-          o.x = merge(x.x, o.x, 0);
-          o.y = merge(x.y, o.y, 1);
-          o.z = merge(x.z, o.z, 2);
-          o.w = merge(x.w, o.w, 3);
-        }
-        *reinterpret_cast<uint4 *>(et + 8 * c) = o;
+        *reinterpret_cast<uint4 *>(et + 8 * c) = shift_chunk(x, nx, st - 8 * c);
         if (c == c_lo) {   // this lane wrote the chunk holding s: the refreshed pair goes over it
           const uint32_t pr = pairs[qt];
           if (st >= 1) et[st - 1] = (uint16_t)(pr & 0xFFFFu);
