@@ -405,16 +405,7 @@ int sc_energy(const uint8_t *img, int H, int W, int C, uint16_t *energy_out, voi
   if (!img || !energy_out) return fail(SC_EINVAL, "null pointer");
   if (H < 1 || W < 1 || !valid_c(C)) return fail(SC_EINVAL, "bad shape %d x %d x %d", H, W, C);
   if ((int64_t)H * W * C >= ((int64_t)1 << 31)) return fail(SC_EINVAL, "H*W*C must be < 2^31");
-  cudaStream_t st = (cudaStream_t)stream;
-  Workspace *wsp;
-  int rc = get_ws(stream, &wsp);
-  if (rc) return rc;
-  Workspace &ws = *wsp;
-  std::lock_guard<std::mutex> lk(ws.mu);
-  const int pitch = round_up(W, 4);
-  SC_CUDA(ws.img.ensure((size_t)H * pitch));
-  SC_CUDA(launch_pack(img, H, W, C, ws.img.p, pitch, st));
-  SC_CUDA(launch_energy(ws.img.p, pitch, H, W, energy_out, W, st));
+  SC_CUDA(launch_energy_bytes(img, H, W, C, energy_out, (cudaStream_t)stream));
   return SC_OK;
 }
 

@@ -70,6 +70,8 @@ cudaError_t launch_unpack(const uint32_t *img, int pitch_img, int H, int W, int 
 cudaError_t launch_transpose(const uint32_t *src, int pitch_src, int H, int W, uint32_t *dst, int pitch_dst,
                              cudaStream_t st);
 cudaError_t launch_energy(const uint32_t *img, int pitch_img, int H, int W, uint16_t *E, int pitch_e, cudaStream_t st);
+// the energy of an HWC byte image into an unpadded H x W map
+cudaError_t launch_energy_bytes(const uint8_t *src, int H, int W, int C, uint16_t *E, cudaStream_t st);
 // caller map -> padded layout; sets *gate (ERR_ENERGY_RANGE) when a seam sum might not fit 24 bits
 cudaError_t launch_copy_energy(const uint16_t *src, int H, int W, uint16_t *E, int pitch_e, int *gate, cudaStream_t st);
 cudaError_t launch_unpad_energy(const uint16_t *E, int pitch_e, int H, int W, uint16_t *dst, cudaStream_t st);
