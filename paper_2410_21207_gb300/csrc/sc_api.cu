@@ -664,7 +664,10 @@ int batch_need_width(const sc_image_desc &d) {
 
 // Scratch of one image in the pool at `off` (pool may be null to size it). `limit` is the widest
 // column range the search stages: the CTA's width, or the cluster's owned columns.
-static BatchItem layout_item(const sc_image_desc &d, int limit, unsigned char *pool, size_t &off, int *S_out) {
+// box_cols x box_rows: the tile that the carving kernel stages through a tensor map of the energies (0: it
+// does not use one; *map_failed is set when the map cannot be encoded).
+static BatchItem layout_item(const sc_image_desc &d, int limit, unsigned char *pool, size_t &off, int *S_out,
+                             int box_cols, int box_rows, bool *map_failed) {
   const int nh = d.H - d.target_h;
   const int R = d.H > d.W ? d.H : d.W;
   const int rows_max = (nh > 0 && d.target_w > d.H) ? d.target_w : d.H;
@@ -686,30 +689,36 @@ static BatchItem layout_item(const sc_image_desc &d, int limit, unsigned char *p
   it.img_w = (uint32_t *)take((size_t)d.H * it.pitch * 4);
   it.img2_w = nh > 0 ? (uint32_t *)take((size_t)d.target_w * it.pitch * 4) : nullptr;
   it.E = (uint16_t *)take((size_t)rows_max * it.pe * 2);
-  it.Mrow = (uint32_t *)take((size_t)(S + 1) * it.pe * 4);
+  it.scratch = (uint32_t *)take((size_t)(S + 1) * it.pe * 4);
   it.seam = (int32_t *)take((size_t)rows_max * 4);
   it.lists = (int16_t *)take((size_t)2 * rows_max * RPEND * 2);
+  it.tmap = CUtensorMap{};
+  if (box_cols > 0 && pool && energy_tensor_map(&it.tmap, it.E, it.pe, rows_max, box_cols, box_rows) != cudaSuccess)
+    *map_failed = true;
   return it;
 }
 
-int batch_cluster_size(const sc_image_desc &d) {
-  const int own = batch_cl_own_cols();
-  return (batch_need_width(d) + own - 1) / own;
-}
+int batch_cluster_size(const sc_image_desc &d) { return batch_cl_ctas(batch_need_width(d)); }
 
 // Estimated carving time, for load balancing: per seam of an h-row, w-column map, c + h (a + b w)
 // microseconds, fitted to measured per-seam times of single images (one GB300, 240..1280 columns,
 // 180..944 rows): the per-row term is the chain of dependent rows, the per-column term the row's
 // work. One CTA of the one-CTA kernel: c 8.3, a 0.0874, b 9.34e-5 (a row costs as much as 936
 // columns: small images cost far more per pixel than large ones). A cluster of cs CTAs of the
-// latency shape: c 11.5, a 0.065, b 1.5e-4 / cs. The 8-row-tile cluster shape is counted as one
-// CTA on a map cs / 2 times narrower.
+// latency shape (240..3900 columns, 180..1332 rows, alone: c 10, a 0.024 + 0.07 / cs, the refresh's rows
+// being dealt over the CTAs, b 9e-5 / cs) is counted 1.2 times slower, as it is beside a GPU full of
+// one-CTA images: three batches of 256 images take 43.4 / 39.0 / 39.6 ms with the split of SMs
+// that the times alone give, 40.2 / 38.6 / 34.8 ms with 1.2 x, 40.2 / 44.6 / 34.8 ms with 1.4 x. The
+// 8-row-tile cluster shape is counted as one CTA on a map cs / 2 times narrower. The one-CTA kernel has
+// become faster than its first fit, which stays the measure of the routing (sc_batch_route reports it);
+// the split uses the later one (c 8.0, a 0.069, b 8.9e-5).
 struct SeamCost {
   double c, a, b;
 };
 static SeamCost cost_one_cta() { return {8.3, 0.0874, 9.34e-5}; }
+static SeamCost cost_one_cta_now() { return {8.0, 0.069, 8.9e-5}; }
 static SeamCost cost_cluster(int shape, int cs) {
-  return shape == CL_LAT ? SeamCost{11.5, 0.065, 1.5e-4 / cs} : SeamCost{8.3, 0.0874, 9.34e-5 * 2.0 / cs};
+  return shape == CL_LAT ? SeamCost{12.0, 0.029 + 0.084 / cs, 1.08e-4 / cs} : SeamCost{8.3, 0.0874, 9.34e-5 * 2.0 / cs};
 }
 // n seams of an h-row map whose width starts at w and drops by one per seam
 static double pass_us(const SeamCost &k, double h, double w, double n) {
@@ -742,7 +751,9 @@ void batch_layout(const sc_image_desc *descs, int n, const BatchCfg &c, unsigned
   // the images that would hold up the batch on one CTA each: carving work above thr_bal x the mean
   // share per SM goes to a latency-shaped cluster (the batch then ends when the average SM does,
   // not when the largest image does)
-  std::vector<char> bal(n, 0);
+  b.map_failed = false;
+  std::vector<char> &bal = b.lat;
+  bal.assign(n, 0);
   if (c.thr_bal > 0.f) {
     const int sms = c.sms > 0 ? c.sms : device_sms();
     double total = 0.0;
@@ -764,15 +775,14 @@ void batch_layout(const sc_image_desc *descs, int n, const BatchCfg &c, unsigned
       continue;
     }
     int S;
-    b.items.push_back(layout_item(d, limit, pool, off, &S));
+    b.items.push_back(layout_item(d, limit, pool, off, &S, limit + 2 * c.kt, c.kt, &b.map_failed));
     if (S > b.Smax) b.Smax = S;
   }
   for (int k : wide) {
     const sc_image_desc &d = descs[k];
     int shape = CL_WIDE, cs = batch_cluster_size(d);
     if (bal[k] || c.wide_lat) {
-      const int own = batch_cl_own_cols(CL_LAT);
-      const int cl = std::max(2, (batch_need_width(d) + own - 1) / own);
+      const int cl = batch_cl_ctas(batch_need_width(d), CL_LAT);
       if (cl <= MAX_CLUSTER) {
         shape = CL_LAT;
         cs = cl;
@@ -792,7 +802,9 @@ void batch_layout(const sc_image_desc *descs, int n, const BatchCfg &c, unsigned
       g->shape = shape;
     }
     int S;
-    g->items.push_back(layout_item(d, cs * batch_cl_own_cols(shape), pool, off, &S));
+    const ClOps o = cl_ops(shape);
+    g->items.push_back(layout_item(d, batch_cl_cols(cs, shape), pool, off, &S, shape == CL_LAT ? o.staged : 0, o.tile_rows,
+                                   &b.map_failed));
     g->index.push_back(k);
     if (S > g->Smax) g->Smax = S;
   }
@@ -883,6 +895,7 @@ static int batch_prepare(BatchRun &r, const sc_image_desc *descs, int n, const B
   batch_layout(descs, n, c, nullptr, r.setup);
   SC_CUDA(r.pool.ensure(r.setup.pool_bytes ? r.setup.pool_bytes : 256));
   batch_layout(descs, n, c, r.pool.p, r.setup);
+  if (r.setup.map_failed) return fail(SC_ECUDA, "cannot encode an energy map's tensor map");
   const int nb = (int)r.setup.items.size();
   const int ng = (int)r.setup.cl.size();
   std::vector<BatchItem> all = r.setup.items;
@@ -904,7 +917,7 @@ static int batch_prepare(BatchRun &r, const sc_image_desc *descs, int n, const B
   // GPU) or than the group has images; the one-CTA launch keeps at least one SM.
   r.cl_clusters.assign(ng, 1);
   std::vector<double> t1;
-  for (const BatchItem &it : r.setup.items) t1.push_back(batch_item_us(it, cost_one_cta()) * per_sm);
+  for (const BatchItem &it : r.setup.items) t1.push_back(batch_item_us(it, cost_one_cta_now()) * per_sm);
   std::vector<std::vector<double>> mk(ng);   // mk[g][c - 1]: group g's end on c clusters
   for (int g = 0; g < ng; ++g) {
     const ClusterGroup &G = r.setup.cl[g];
@@ -1133,12 +1146,17 @@ int sc_batch_route(const sc_image_desc *descs, int n, float thr, int sms, int *c
     shape[k] = CL_WIDE;
     if (one_cta_us) one_cta_us[k] = item_us(descs[k], cost_one_cta());
   }
+  // reported sizes: the CTAs that cover the width, at 768 columns each and at 384 for the latency shape
+  // (whose launch gives the same work to two halves of a cluster, of 640 columns per CTA)
+  auto report = [&](int k) {
+    const int need = batch_need_width(descs[k]), wide = batch_cluster_size(descs[k]), lat = std::max(2, (need + 383) / 384);
+    const bool l = b.lat[k] && lat <= MAX_CLUSTER;
+    shape[k] = l ? CL_LAT : CL_WIDE;
+    cluster_size[k] = l ? lat : (wide <= MAX_CLUSTER ? wide : -1);
+  };
   for (const ClusterGroup &g : b.cl)
-    for (int k : g.index) {
-      cluster_size[k] = g.cs;
-      shape[k] = g.shape;
-    }
-  for (int k : b.fallback) cluster_size[k] = -1;
+    for (int k : g.index) report(k);
+  for (int k : b.fallback) report(k);
   return SC_OK;
 }
 

@@ -15,6 +15,12 @@ namespace sc {
 // up to 64 * (NW + 1) rows); their direction rows share the idle staging ring.
 __host__ __device__ constexpr int batch_fill_warps(int nw, int kt) { return 16; }
 
+// the search's shared memory: its energies arrive by tensor copies of each image's map
+template <int NW, int KT>
+__host__ __device__ inline SearchPlan batch_plan(int Smax) {
+  return search_plan<NW, KT, false, batch_fill_warps(NW, KT), false, KS, false, true>(Smax);
+}
+
 // rows x cols word image -> its transpose (cols x rows), 32x32 tiles staged in shared memory; `tile`
 // holds `ntw` warps' 32x33 tiles.
 __device__ inline void cta_transpose(const uint32_t *src, int ps, int rows, int cols, uint32_t *dst, int pd,
@@ -45,15 +51,15 @@ __device__ inline void cta_transpose(const uint32_t *src, int ps, int rows, int 
 template <int NW, int KT>
 __device__ void batch_seam_pass(const BatchItem &it, uint32_t *words, int rows, int cols, int count,
                                 int32_t *log, int64_t *costs, unsigned char *smem, int Smax, SearchState &st,
-                                int *err) {
+                                int *err, const CUtensorMap *tmap) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
   int16_t *lb[2] = {it.lists, it.lists + (size_t)rows * RPEND};
   // the staging ring is idle between searches: it holds the rows' refreshed pairs
-  const SearchPlan plan = search_plan<NW, KT, false, batch_fill_warps(NW, KT)>(Smax);
+  const SearchPlan plan = batch_plan<NW, KT>(Smax);
   uint32_t *pairs = reinterpret_cast<uint32_t *>(smem + plan.ring);
   const size_t pair_bytes = ((size_t)rows * 4 + 15) & ~(size_t)15;
   uint16_t *sbuf = reinterpret_cast<uint16_t *>(smem + plan.ring + pair_bytes);
-  const int sbuf_elems = (int)(((plan.bars - plan.ring - pair_bytes) / nwarps) & ~(size_t)15) / 2;
+  const int sbuf_elems = (int)(((plan.ring_end - plan.ring - pair_bytes) / nwarps) & ~(size_t)15) / 2;
   uint16_t *const Ecur = it.E + E_PADL;
   int cur = 0, m = 0;
   for (int t = 0; t < count; ++t) {
@@ -68,7 +74,8 @@ __device__ void batch_seam_pass(const BatchItem &it, uint32_t *words, int rows, 
     a.cost = costs ? costs + t : nullptr;
     a.err = err;
     a.gated = false;
-    seam_search<NW, KT, false, batch_fill_warps(NW, KT)>(a, smem, Smax, st);   // ends with a CTA barrier: the seam is complete
+    a.tmap = tmap;
+    seam_search<NW, KT, false, batch_fill_warps(NW, KT), false, KS, false, true>(a, smem, Smax, st);   // ends with a CTA barrier: the seam is complete
     // every row's refreshed pair and list update, one thread per row (into the idle staging ring)
     if (refresh_pairs(words, it.pitch, rows, w, it.seam, lb[cur], lb[cur ^ 1], m, rows, 0, 1, pairs, threadIdx.x,
                       blockDim.x))
@@ -82,6 +89,7 @@ __device__ void batch_seam_pass(const BatchItem &it, uint32_t *words, int rows, 
       atomicOr(err, ERR_TIMEOUT);
     cur ^= 1;
     fence_proxy_async_global();   // the next search stages the compacted energy rows with TMA
+    fence_proxy_async_smem();     // ... into the ring's place, which held this seam's pairs and rows
     __syncthreads();
     if (++m == RPEND) {
       compact_rows_staged(words, it.pitch, rows, 0, 1, lb[cur], m, w - 1, warp, nwarps, lane,
@@ -109,7 +117,8 @@ __device__ void batch_energy(const uint32_t *words, int pitch, int rows, int col
 }
 
 template <int NW, int KT>
-__device__ void batch_carve_item(const BatchItem &it, unsigned char *smem, int Smax, SearchState &st, int *err) {
+__device__ void batch_carve_item(const BatchItem &it, unsigned char *smem, int Smax, SearchState &st, int *err,
+                                 const CUtensorMap *tmap) {
   const int H = it.H, W = it.W, C = it.C, tw = it.tw, th = it.th;
   const int64_t npx = (int64_t)H * W;
   for (int64_t q = threadIdx.x; q < npx; q += blockDim.x) {
@@ -119,18 +128,18 @@ __device__ void batch_carve_item(const BatchItem &it, unsigned char *smem, int S
   __syncthreads();
   batch_energy<NW, KT>(it.img_w, it.pitch, H, W, it.E + E_PADL, it.pe);
   const int nv = W - tw, nh = H - th;
-  batch_seam_pass<NW, KT>(it, it.img_w, H, W, nv, it.seam_log, it.cost_log, smem, Smax, st, err);
+  batch_seam_pass<NW, KT>(it, it.img_w, H, W, nv, it.seam_log, it.cost_log, smem, Smax, st, err, tmap);
   uint32_t *res = it.img_w;
   if (nh > 0) {
-    const SearchPlan plan = search_plan<NW, KT, false, batch_fill_warps(NW, KT)>(Smax);
+    const SearchPlan plan = batch_plan<NW, KT>(Smax);
     uint32_t *tile = reinterpret_cast<uint32_t *>(smem + plan.ring);   // the ring is idle between searches
-    const int ntw_fit = (int)((plan.bars - plan.ring) / (32 * 33 * 4));
+    const int ntw_fit = (int)((plan.ring_end - plan.ring) / (32 * 33 * 4));
     const int ntw = ntw_fit < NW + 1 ? ntw_fit : NW + 1;
     cta_transpose(it.img_w, it.pitch, H, tw, it.img2_w, it.pitch, tile, ntw);   // tw rows x H columns
     __syncthreads();
     batch_energy<NW, KT>(it.img2_w, it.pitch, tw, H, it.E + E_PADL, it.pe);
     batch_seam_pass<NW, KT>(it, it.img2_w, tw, H, nh, it.seam_log ? it.seam_log + (size_t)nv * H : nullptr,
-                            it.cost_log ? it.cost_log + nv : nullptr, smem, Smax, st, err);
+                            it.cost_log ? it.cost_log + nv : nullptr, smem, Smax, st, err, tmap);
     cta_transpose(it.img2_w, it.pitch, tw, th, it.img_w, it.pitch, tile, ntw);  // th rows x tw columns
     __syncthreads();
   }
@@ -147,12 +156,12 @@ __device__ void batch_carve_item(const BatchItem &it, unsigned char *smem, int S
 template <int NW, int KT>
 __global__ void __launch_bounds__(Geo<NW, KT, false>::THREADS, 1)
     k_batch(const BatchItem *__restrict__ items, int n, int Smax, int *queue, int *err) {
-  extern __shared__ __align__(16) unsigned char smem[];
+  extern __shared__ __align__(128) unsigned char smem[];
   __shared__ int next;
   // the current image's descriptor lives in shared memory and its fields are read where they are
   // used, so they do not occupy registers across the seam loop
   __shared__ BatchItem cur;
-  search_init(smem, search_plan<NW, KT, false, batch_fill_warps(NW, KT)>(Smax));
+  search_init(smem, batch_plan<NW, KT>(Smax));
   __syncthreads();
   SearchState st;
   for (;;) {
@@ -164,7 +173,7 @@ __global__ void __launch_bounds__(Geo<NW, KT, false>::THREADS, 1)
     const int k = next;
     __syncthreads();
     if (k >= n) break;
-    batch_carve_item<NW, KT>(cur, smem, Smax, st, err);
+    batch_carve_item<NW, KT>(cur, smem, Smax, st, err, &items[k].tmap);
     __syncthreads();
   }
   // launched as a programmatic dependent of cluster launches (a batch plan starts them first): this
@@ -188,7 +197,7 @@ cudaError_t batch_configure_cfg() {
 template <int NW, int KT>
 cudaError_t launch_batch_cfg(const BatchItem *items, int n, int Smax, int grid, int *queue, int *err,
                              cudaStream_t st, bool pdl) {
-  const size_t smem = search_plan<NW, KT, false, batch_fill_warps(NW, KT)>(Smax).total;
+  const size_t smem = batch_plan<NW, KT>(Smax).total;
   if (smem > BATCH_SMEM_MAX) return cudaErrorInvalidValue;
   cudaError_t e = batch_configure_cfg<NW, KT>();
   if (e != cudaSuccess) return e;

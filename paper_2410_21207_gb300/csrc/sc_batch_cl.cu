@@ -4,6 +4,6 @@
 
 namespace sc {
 
-ClOps cl_ops_wide() { return ClShapeHost<8, 8, 4>::ops(); }
+ClOps cl_ops_wide() { return ClShapeHost<8, 8, 4, false>::ops(); }
 
 }  // namespace sc

@@ -16,25 +16,81 @@
 
 #include "sc_batch_cl.h"
 #include "sc_rowops.cuh"
-#include "sc_search.cuh"
+#include "sc_two.cuh"
 
 namespace sc {
 
-// (count) vertical seams of a rows x cols word image whose energy is in it.E
+// Shared-memory plan of a shape. TWO: the ancestor tables want 128 KB (up to ~1,400 rows of a
+// 2,560-column image); larger ones are followed in global memory.
+template <int NW, int KT, int FWM, bool TWO>
+__host__ __device__ inline TwoPlan clb_plan(int Smax) {
+  using G = Geo<NW, KT, true, FWM>;
+  if (TWO) return two_plan<G, NW, KT, KS>(Smax + 1, 1, (size_t)128 << 10, BATCH_CL_SMEM_MAX);
+  TwoPlan t{};
+  t.plan = search_plan<NW, KT, true, FWM>(Smax);
+  return t;
+}
+
+// The two-ended search (sc_dp.cu describes it) of one cluster: its first half of CTAs sweeps the upper
+// half of the map, the second half the lower one; rank 0 joins them, all of them backtrack.
 template <int NW, int KT, int FWM>
+__device__ __forceinline__ void clb_two_search(SearchArgs a, uint32_t *scratch, const CUtensorMap *tmap, unsigned char *smem,
+                                               const TwoPlan &t, SearchState &st, int rank, int ctas) {
+  using G = Geo<NW, KT, true, FWM>;
+  cg::cluster_group cl = cg::this_cluster();
+  const TwoSplit g = two_split<KT, KS>(a.H);
+  const int cs = ctas / 2, half = rank >= cs ? 1 : 0, gw = cs * G::OWC, H = a.H;
+  const TwoScratch x(scratch, gw);
+  int *misc = reinterpret_cast<int *>(smem + t.plan.misc);
+  a.gtab = x.tab + (half ? (size_t)g.S0 * gw : 0);
+  a.gw = gw;
+  a.endrow = half ? x.end1 : x.end0;
+  a.tmap = tmap;
+  a.rank0 = half * cs;
+  a.ctas = cs;
+  if (half) {
+    a.H = g.H1;
+    a.y0 = H - 1;
+    seam_sweep<NW, KT, true, FWM, false, KS, false, true, true, true>(a, smem, t.plan, st);
+  } else {
+    a.H = g.H0;
+    seam_sweep<NW, KT, true, FWM, false, KS, false, true, true, false>(a, smem, t.plan, st);
+  }
+  fence_proxy_async_global();   // the tables are read by a bulk copy
+  cl.sync();
+  uint32_t cost = SENT;
+  if (rank == 0) {
+    cost = two_join<NW>(g, x, gw, a.W, smem, t, st.joins & 1u, ctas, a.err);
+    if ((size_t)(g.S0 + g.S1) * gw <= t.tab_cap) ++st.joins;
+    if (threadIdx.x == 0 && cost != SENT && a.cost) *a.cost = (int64_t)cost;
+  }
+  cl.sync();
+  if (misc[1]) {
+    const FillCtx f{a.E, nullptr, reinterpret_cast<uint32_t *>(cl.map_shared_rank(misc, 0) + 2), 1u, a.seam, a.seam_log,
+                    a.err, 0, a.pitch_e, 0, a.W, 0};
+    two_fill<G, KS>(g, f, H, t, smem, ctas, rank);
+  }
+  cl.sync();   // the seam is complete
+  // the recomputed path costs must add up to the join's
+  if (rank == 0 && threadIdx.x == 0 && cost != SENT && (uint32_t)misc[2] != cost) atomicOr(a.err, ERR_COST_MISMATCH);
+}
+
+// (count) vertical seams of a rows x cols word image whose energy is in it.E
+template <int NW, int KT, int FWM, bool TWO>
 __device__ void clb_seam_pass(const BatchItem &it, uint32_t *words, int rows, int cols, int count, int32_t *log,
                               int64_t *costs, unsigned char *smem, int Smax, SearchState &st, int *err, int rank,
-                              int cs) {
+                              int cs, const CUtensorMap *tmap) {
   cg::cluster_group cl = cg::this_cluster();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
   int16_t *lb[2] = {it.lists, it.lists + (size_t)rows * RPEND};
   // the staging ring is idle between searches: it holds the owned rows' refreshed pairs
-  const SearchPlan plan = search_plan<NW, KT, true, FWM>(Smax);
+  const TwoPlan tplan = clb_plan<NW, KT, FWM, TWO>(Smax);
+  const SearchPlan &plan = tplan.plan;
   uint32_t *pairs = reinterpret_cast<uint32_t *>(smem + plan.ring);
   const int nq = (rows - rank + cs - 1) / cs;   // rows this CTA owns
   const size_t pair_bytes = ((size_t)(nq > 0 ? nq : 0) * 4 + 15) & ~(size_t)15;
   uint16_t *sbuf = reinterpret_cast<uint16_t *>(smem + plan.ring + pair_bytes);
-  const int sbuf_elems = (int)(((plan.bars - plan.ring - pair_bytes) / nwarps) & ~(size_t)15) / 2;
+  const int sbuf_elems = (int)(((plan.ring_end - plan.ring - pair_bytes) / nwarps) & ~(size_t)15) / 2;
   uint16_t *const Ecur = it.E + E_PADL;
   int cur = 0, m = 0;
   for (int t = 0; t < count; ++t) {
@@ -49,7 +105,9 @@ __device__ void clb_seam_pass(const BatchItem &it, uint32_t *words, int rows, in
     a.cost = costs ? costs + t : nullptr;
     a.err = err;
     a.gated = false;
-    seam_search<NW, KT, true, FWM>(a, smem, Smax, st);   // ends with a cluster barrier
+    // the search ends with a cluster barrier
+    if constexpr (TWO) clb_two_search<NW, KT, FWM>(a, it.scratch, tmap, smem, tplan, st, rank, cs);
+    else seam_search<NW, KT, true, FWM>(a, smem, Smax, st);
     if (refresh_pairs(words, it.pitch, rows, w, it.seam, lb[cur], lb[cur ^ 1], m, nq, rank, cs, pairs, threadIdx.x,
                       blockDim.x))
       atomicOr(err, ERR_BAD_SEAM);
@@ -66,6 +124,7 @@ __device__ void clb_seam_pass(const BatchItem &it, uint32_t *words, int rows, in
       m = 0;
     }
     fence_proxy_async_global();   // the next search stages the compacted energy rows with TMA
+    fence_proxy_async_smem();     // ... into the ring's place, which held this seam's pairs and rows
     cl.sync();
   }
   if (m > 0) {
@@ -109,9 +168,9 @@ __device__ inline void clb_transpose(const uint32_t *src, int ps, int rows, int 
   cg::this_cluster().sync();
 }
 
-template <int NW, int KT, int FWM>
+template <int NW, int KT, int FWM, bool TWO>
 __device__ void clb_carve_item(const BatchItem &it, unsigned char *smem, int Smax, SearchState &st, int *err, int rank,
-                               int cs) {
+                               int cs, const CUtensorMap *tmap) {
   const int H = it.H, W = it.W, C = it.C, tw = it.tw, th = it.th;
   const int64_t tid = (int64_t)rank * blockDim.x + threadIdx.x, nth = (int64_t)cs * blockDim.x;
   const int64_t npx = (int64_t)H * W;
@@ -122,16 +181,16 @@ __device__ void clb_carve_item(const BatchItem &it, unsigned char *smem, int Sma
   cg::this_cluster().sync();
   clb_energy(it.img_w, it.pitch, H, W, it.E + E_PADL, it.pe, rank, cs);
   const int nv = W - tw, nh = H - th;
-  clb_seam_pass<NW, KT, FWM>(it, it.img_w, H, W, nv, it.seam_log, it.cost_log, smem, Smax, st, err, rank, cs);
+  clb_seam_pass<NW, KT, FWM, TWO>(it, it.img_w, H, W, nv, it.seam_log, it.cost_log, smem, Smax, st, err, rank, cs, tmap);
   if (nh > 0) {
-    const SearchPlan plan = search_plan<NW, KT, true, FWM>(Smax);
+    const SearchPlan plan = clb_plan<NW, KT, FWM, TWO>(Smax).plan;
     uint32_t *tile = reinterpret_cast<uint32_t *>(smem + plan.ring);   // the ring is idle between searches
-    const int ntw_fit = (int)((plan.bars - plan.ring) / (32 * 33 * 4));
+    const int ntw_fit = (int)((plan.ring_end - plan.ring) / (32 * 33 * 4));
     const int ntw = ntw_fit < NW + 1 ? ntw_fit : NW + 1;
     clb_transpose(it.img_w, it.pitch, H, tw, it.img2_w, it.pitch, tile, ntw, rank, cs);   // tw rows x H columns
     clb_energy(it.img2_w, it.pitch, tw, H, it.E + E_PADL, it.pe, rank, cs);
-    clb_seam_pass<NW, KT, FWM>(it, it.img2_w, tw, H, nh, it.seam_log ? it.seam_log + (size_t)nv * H : nullptr,
-                  it.cost_log ? it.cost_log + nv : nullptr, smem, Smax, st, err, rank, cs);
+    clb_seam_pass<NW, KT, FWM, TWO>(it, it.img2_w, tw, H, nh, it.seam_log ? it.seam_log + (size_t)nv * H : nullptr,
+                                    it.cost_log ? it.cost_log + nv : nullptr, smem, Smax, st, err, rank, cs, tmap);
     clb_transpose(it.img2_w, it.pitch, tw, th, it.img_w, it.pitch, tile, ntw, rank, cs);   // th rows x tw columns
   }
   const int64_t nout = (int64_t)th * tw;
@@ -144,10 +203,10 @@ __device__ void clb_carve_item(const BatchItem &it, unsigned char *smem, int Sma
   if (it.done && rank == 0 && threadIdx.x == 0) *(volatile int *)it.done = (*(volatile int *)err != 0) ? 2 : 1;
 }
 
-template <int NW, int KT, int FWM>
+template <int NW, int KT, int FWM, bool TWO>
 __global__ void __launch_bounds__(Geo<NW, KT, true, FWM>::THREADS, 1)
     k_batch_cl(const BatchItem *__restrict__ items, int n, int Smax, int *queue, int *err) {
-  extern __shared__ __align__(16) unsigned char smem[];
+  extern __shared__ __align__(128) unsigned char smem[];
   __shared__ int next;
   __shared__ BatchItem cur;   // the current image's descriptor, read where its fields are used
   // a launch chained behind this one (programmatic dependent launch) may start once every CTA of
@@ -156,7 +215,14 @@ __global__ void __launch_bounds__(Geo<NW, KT, true, FWM>::THREADS, 1)
   pdl_launch_dependents();
   cg::cluster_group cl = cg::this_cluster();
   const int rank = (int)cl.block_rank(), cs = (int)cl.num_blocks();
-  search_init(smem, search_plan<NW, KT, true, FWM>(Smax));
+  {
+    const TwoPlan t = clb_plan<NW, KT, FWM, TWO>(Smax);
+    search_init(smem, t.plan);
+    if (TWO && threadIdx.x == 0) {
+      mbar_init(reinterpret_cast<uint64_t *>(smem + t.tbar), 1);
+      fence_mbar_init();
+    }
+  }
   cl.sync();
   SearchState st;
   for (;;) {
@@ -167,21 +233,21 @@ __global__ void __launch_bounds__(Geo<NW, KT, true, FWM>::THREADS, 1)
     if (k >= n) break;
     if (threadIdx.x == 0) cur = items[k];
     __syncthreads();
-    clb_carve_item<NW, KT, FWM>(cur, smem, Smax, st, err, rank, cs);
+    clb_carve_item<NW, KT, FWM, TWO>(cur, smem, Smax, st, err, rank, cs, &items[k].tmap);
   }
   // chained behind another launch: do not end before it does (no-op otherwise)
   pdl_wait_prerequisites();
 }
 
 // The host side of one shape: shared memory, capacity and launch (instantiated once per shape).
-template <int NW, int KT, int FWM>
+template <int NW, int KT, int FWM, bool TWO>
 struct ClShapeHost {
   using G = Geo<NW, KT, true, FWM>;
-  static size_t smem_bytes(int Smax) { return search_plan<NW, KT, true, FWM>(Smax).total; }
+  static size_t smem_bytes(int Smax) { return clb_plan<NW, KT, FWM, TWO>(Smax).plan.total; }
   static cudaError_t configure() {
     static std::atomic<bool> done{false};
     if (done.load()) return cudaSuccess;
-    auto k = k_batch_cl<NW, KT, FWM>;
+    auto k = k_batch_cl<NW, KT, FWM, TWO>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BATCH_CL_SMEM_MAX);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -212,7 +278,7 @@ struct ClShapeHost {
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute at[2];
     cfg_for(cfg, at, 1, cs, Smax, nullptr);
-    return cudaOccupancyMaxActiveClusters(clusters, k_batch_cl<NW, KT, FWM>, &cfg);
+    return cudaOccupancyMaxActiveClusters(clusters, k_batch_cl<NW, KT, FWM, TWO>, &cfg);
   }
   static cudaError_t launch(const BatchItem *items, int n, int cs, int Smax, int clusters, int *queue, int *err,
                             cudaStream_t st, bool pdl) {
@@ -222,9 +288,9 @@ struct ClShapeHost {
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute at[2];
     cfg_for(cfg, at, clusters, cs, Smax, st, pdl);
-    return cudaLaunchKernelEx(&cfg, k_batch_cl<NW, KT, FWM>, items, n, Smax, queue, err);
+    return cudaLaunchKernelEx(&cfg, k_batch_cl<NW, KT, FWM, TWO>, items, n, Smax, queue, err);
   }
-  static ClOps ops() { return ClOps{G::OWC, &smem_bytes, &capacity, &launch}; }
+  static ClOps ops() { return ClOps{G::OWC, TWO ? 2 : 1, KT, G::BW, &smem_bytes, &capacity, &launch}; }
 };
 
 }  // namespace sc

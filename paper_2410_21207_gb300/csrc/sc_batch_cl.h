@@ -9,14 +9,17 @@ constexpr size_t BATCH_CL_SMEM_MAX = 232448 - 1024;   // the opt-in limit minus 
 // Two cluster shapes of the persistent kernel:
 //   CL_WIDE: 8 compute warps, 8-row tiles, 768 own columns per CTA. Images wider than one CTA of the
 //            one-CTA kernel: few CTAs per image, little redundant halo work (throughput).
-//   CL_LAT:  8 compute warps, 32-row tiles, 384 own columns per CTA. The heaviest images of a
-//            batch, and the serving form's wide and heavy requests: a quarter of the tile boundaries
-//            per seam and twice the CTAs, so one image's seams finish sooner (latency), at more SM
+//   CL_LAT:  8 compute warps, 16-row tiles, 640 own columns per CTA, two-ended: one half of the
+//            cluster's CTAs sweeps the upper half of the map, the other the lower half. The heaviest
+//            images of a batch, and the serving form's wide and heavy requests: half the chain of
+//            dependent rows per seam, so one image's seams finish sooner (latency), at more SM
 //            time per seam.
 enum ClShape { CL_WIDE = 0, CL_LAT = 1 };
 
 struct ClOps {
   int own;                                                     // columns each CTA of a cluster owns
+  int parts;                                                   // parts of the map a cluster sweeps at once (1 or 2)
+  int tile_rows, staged;                                       // rows and columns of a staged tile
   size_t (*smem)(int Smax);                                    // dynamic shared memory per CTA
   cudaError_t (*capacity)(int cs, int Smax, int *clusters);    // clusters of cs CTAs resident at once
   // `clusters` persistent clusters of cs CTAs carve items[0..n) (a queue counter at *queue, zeroed);
@@ -30,8 +33,15 @@ ClOps cl_ops_wide();
 ClOps cl_ops_lat();
 inline ClOps cl_ops(int shape) { return shape == CL_LAT ? cl_ops_lat() : cl_ops_wide(); }
 
-// columns each CTA of the cluster owns: an image of searched width w needs ceil(w / own) CTAs
-inline int batch_cl_own_cols(int shape = CL_WIDE) { return cl_ops(shape).own; }
+// CTAs of the cluster for an image of searched width w, and the columns such a cluster covers
+inline int batch_cl_ctas(int w, int shape = CL_WIDE) {
+  const ClOps o = cl_ops(shape);
+  return o.parts * ((w + o.own - 1) / o.own);
+}
+inline int batch_cl_cols(int ctas, int shape) {
+  const ClOps o = cl_ops(shape);
+  return ctas / o.parts * o.own;
+}
 inline size_t batch_cl_smem_bytes(int Smax, int shape = CL_WIDE) { return cl_ops(shape).smem(Smax); }
 inline cudaError_t batch_cl_capacity(int cs, int Smax, int *clusters, int shape = CL_WIDE) {
   return cl_ops(shape).capacity(cs, Smax, clusters);

@@ -1,11 +1,13 @@
 // One image of a batched carve, as the persistent kernel reads it (device pointers).
 #pragma once
 #include <cstdint>
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 namespace sc {
 
 struct BatchItem {
+  CUtensorMap tmap;     // the energy buffer, in the boxes of the kernel that carves the image (64-byte aligned)
   const uint8_t *img;   // H x W x C uint8 (caller's)
   uint8_t *out;         // th x tw x C uint8 (caller's)
   int32_t *seam_log;    // nullable (caller's)
@@ -17,7 +19,7 @@ struct BatchItem {
   uint32_t *img_w;      // max(H,W) x pitch words: the image being carved
   uint32_t *img2_w;     // max(H,W) x pitch words: its transpose for the horizontal pass
   uint16_t *E;          // rows x pe energies (column 0 at E + E_PADL)
-  uint32_t *Mrow;       // (ceil(rows/KS) + 1) x pe saved cost rows (column 0 at Mrow + E_PADL)
+  uint32_t *scratch;    // two-ended search: cost rows and ancestor tables, (ceil(rows/KS) + 1) * pe words
   int32_t *seam;        // rows
   int16_t *lists;       // two generations of pending-removal lists, rows x RPEND each
   // nullable: set to 1 (or 2 if the device error word was non-zero) once `out` is complete and

@@ -6,7 +6,7 @@
 namespace sc {
 
 #define SC_BATCH_CASES(X) X(8, 8) X(8, 16) X(8, 32)
-#define SC_SMEM(N, K) case K: return search_plan<N, K, false, batch_fill_warps(N, K)>(Smax).total;
+#define SC_SMEM(N, K) case K: return batch_plan<N, K>(Smax).total;
 #define SC_OCC(N, K) case K: batch_configure_cfg<N, K>(); \
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_batch<N, K>, Geo<N, K, false>::THREADS, smem); break;
 #define SC_LAUNCH(N, K) case K: return launch_batch_cfg<N, K>(items, n, Smax, grid, queue, err, st, pdl);

@@ -3,10 +3,9 @@
 // energy by one cluster (k_dp, seam_search in sc_search.cuh).
 #include <atomic>
 
-#include <cuda.h>
 #include <cudaTypedefs.h>
 
-#include "sc_search.cuh"
+#include "sc_two.cuh"
 
 namespace sc {
 
@@ -45,7 +44,7 @@ __global__ void __launch_bounds__(Geo<NW, KT, true>::THREADS, 1)
   extern __shared__ __align__(128) unsigned char smem[];
   constexpr int KSS = dp_super_rows<NW, KT, FWD>();
   const int S = (p.H + KSS - 1) / KSS;
-  search_init(smem, search_plan<NW, KT, true, FILL_WARPS_MAX, FWD, KSS>(S));
+  search_init(smem, search_plan<NW, KT, true, FILL_WARPS_MAX, FWD, KSS, false, true>(S));
   // neighbours push into each other's halo buffers: every CTA's barriers must be initialised first
   cg::this_cluster().sync();
   // the set-up above overlaps the previous kernel of the seam loop; its results are read below
@@ -90,9 +89,8 @@ static cudaError_t launch_dp_cluster(void (*kernel)(KArgs...), int grid, int cs,
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-// Tensor map of `rows` rows of pitch elements (base: 16-byte aligned), copied in boxes of KT rows, BW
-// columns split into equal parts of at most 256. The driver's encoder is looked up once.
-static cudaError_t energy_tensor_map(CUtensorMap *m, const uint16_t *base, int pitch, int rows, int BW, int KT) {
+// The driver's encoder is looked up once.
+cudaError_t energy_tensor_map(CUtensorMap *m, const uint16_t *base, int pitch, int rows, int BW, int KT) {
   static std::atomic<PFN_cuTensorMapEncodeTiled_v12000> encode{nullptr};
   PFN_cuTensorMapEncodeTiled_v12000 fn = encode.load();
   if (!fn) {
@@ -105,7 +103,7 @@ static cudaError_t energy_tensor_map(CUtensorMap *m, const uint16_t *base, int p
     encode.store(fn);
   }
   const cuuint64_t dims[2] = {(cuuint64_t)pitch, (cuuint64_t)rows}, strides[1] = {(cuuint64_t)pitch * 2};
-  const cuuint32_t box[2] = {(cuuint32_t)(BW / ((BW + 255) / 256)), (cuuint32_t)KT}, es[2] = {1, 1};
+  const cuuint32_t box[2] = {(cuuint32_t)tensor_box_cols(BW), (cuuint32_t)KT}, es[2] = {1, 1};
   const CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_UINT16, 2, const_cast<uint16_t *>(base), dims, strides, box, es,
                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
@@ -115,7 +113,7 @@ static cudaError_t energy_tensor_map(CUtensorMap *m, const uint16_t *base, int p
 template <int NW, int KT, bool FWD = false>
 static cudaError_t launch_dp_shape(const DpArgs &a, int cs, cudaStream_t st) {
   constexpr int KSS = dp_super_rows<NW, KT, FWD>();
-  const size_t smem = search_plan<NW, KT, true, FILL_WARPS_MAX, FWD, KSS>((a.H + KSS - 1) / KSS).total;
+  const size_t smem = search_plan<NW, KT, true, FILL_WARPS_MAX, FWD, KSS, false, true>((a.H + KSS - 1) / KSS).total;
   static bool configured = false;
   if (!configured) {
     cudaError_t e = cudaFuncSetAttribute(k_dp<NW, KT, FWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
@@ -170,46 +168,9 @@ template <int NW, int KT>
 struct Two {
   static constexpr int KSS = dp_super_rows<NW, KT, false>();
   using G = Geo<NW, KT, true, FILL_WARPS_MAX, KSS>;
-  int H0, H1, S0, S1, cs, gw;
-  size_t tab_bytes;      // both tables
-  bool tab_smem;         // rank 0 of the finishing cluster copies them into its staging ring's place
-  SearchPlan plan;       // jb holds both halves' columns: S0 + 1, then S1 + 1
-  size_t tbar;           // mbarrier of that copy
-
-  __host__ __device__ Two(int H, int ctas) : cs(ctas) {
-    // a whole number of tiles in the upper half where there is a choice: only one half then ends on a
-    // ragged tile
-    H0 = ((H + 1) / 2 + KT - 1) / KT * KT;
-    H1 = H - H0;
-    S0 = (H0 + KSS - 1) / KSS;
-    S1 = (H1 + KSS - 1) / KSS;
-    gw = cs * G::OWC;
-    tab_bytes = (size_t)(S0 + S1) * gw;
-    layout(true);
-    if (plan.total > SEARCH_SMEM_LIMIT) layout(false);
-  }
-  __host__ __device__ void layout(bool tab) {
-    tab_smem = tab;
-    size_t o = 0;
-    auto take = [&](size_t bytes) { const size_t at = o; o = (o + bytes + 15) & ~(size_t)15; return at; };
-    plan.bnd = take((size_t)2 * G::BW * 4);
-    plan.hbuf = take((size_t)2 * 2 * K2 * 4);
-    plan.wmin = 0;
-    plan.cmin = take((size_t)(NW + 1 + (S0 + S1 + cs - 1) / cs) * 8);   // warps' minima, then super-tiles' ends
-    plan.jb = take((size_t)(S0 + S1 + 2) * 4);
-    plan.misc = take(16);   // [0] this CTA arrived last, [1] its cluster goes on with the ends in cmin
-    plan.anc = plan.emx = plan.gat = 0;
-    plan.gw = 0;
-    plan.bars = take((size_t)(NSLOT + 3) * 8);
-    tbar = plan.bars + (size_t)(NSLOT + 2) * 8;
-    // the staging ring; after the sweep its place holds the tables, then the fills' rows
-    size_t r = (size_t)NSLOT * KT * G::BW * 2;
-    const size_t fb = (size_t)G::FW * G::fill_bytes(false);
-    r = r > fb ? r : fb;
-    if (tab && tab_bytes > r) r = tab_bytes;
-    o = (o + 127) & ~(size_t)127;
-    plan.ring = plan.fill = take(r);
-    plan.total = o;
+  static __host__ __device__ TwoPlan plan(const TwoSplit &s, int cs) {
+    const size_t tab = (size_t)(s.S0 + s.S1) * cs * G::OWC;
+    return two_plan<G, NW, KT, KSS>(s.S0 + s.S1, cs, tab, SEARCH_SMEM_LIMIT);
   }
 };
 
@@ -223,15 +184,13 @@ __global__ void __launch_bounds__(Geo<NW, KT, true>::THREADS, 1)
   cg::cluster_group cl = cg::this_cluster();
   const int cs = (int)cl.num_blocks(), rank = (int)cl.block_rank();
   const int half = (int)blockIdx.x / cs;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const T g(p.H, cs);
-  const SearchPlan &plan = g.plan;
-  int *jb = reinterpret_cast<int *>(smem + plan.jb);
-  int *misc = reinterpret_cast<int *>(smem + plan.misc);
-  uint64_t *tbar = reinterpret_cast<uint64_t *>(smem + g.tbar);
-  search_init(smem, plan);
+  const TwoSplit g = two_split<KT, KSS>(p.H);
+  const TwoPlan t = T::plan(g, cs);
+  const int gw = cs * G::OWC;
+  int *misc = reinterpret_cast<int *>(smem + t.plan.misc);
+  search_init(smem, t.plan);
   if (threadIdx.x == 0) {
-    mbar_init(tbar, 1);
+    mbar_init(reinterpret_cast<uint64_t *>(smem + t.tbar), 1);
     fence_mbar_init();
     misc[0] = misc[1] = 0;
     prefetch_tensormap(&tmap);
@@ -243,29 +202,27 @@ __global__ void __launch_bounds__(Geo<NW, KT, true>::THREADS, 1)
   // only now: the refresh that depends on this launch reads what its predecessors wrote before it waits
   pdl_launch_dependents();
   if (p.gate && (*p.gate & ERR_ENERGY_RANGE)) return;   // left to the wide-cost search
-  uint32_t *const end0 = p.scratch, *const end1 = end0 + g.gw;
-  uint8_t *const tab = reinterpret_cast<uint8_t *>(end1 + g.gw);
-  const uint16_t *const E1 = p.E + (ptrdiff_t)(p.H - 1) * p.pitch_e;
+  const TwoScratch x(p.scratch, gw);
   {
     SearchArgs a;
-    a.E = half ? E1 : p.E;
-    a.pitch_e = half ? -p.pitch_e : p.pitch_e;
+    a.E = p.E;
+    a.pitch_e = p.pitch_e;
     a.H = half ? g.H1 : g.H0;
     a.W = p.W;
     a.err = p.err;
     a.gated = false;
     a.pstride = 0;
-    a.gtab = tab + (half ? (size_t)g.S0 * g.gw : 0);
-    a.gw = g.gw;
-    a.endrow = half ? end1 : end0;
+    a.gtab = x.tab + (half ? (size_t)g.S0 * gw : 0);
+    a.gw = gw;
+    a.endrow = half ? x.end1 : x.end0;
     a.tmap = &tmap;
     a.y0 = half ? p.H - 1 : 0;
     SearchState st;
-    if (half) seam_sweep<NW, KT, true, FILL_WARPS_MAX, false, KSS, false, true, true, true>(a, smem, plan, st);
-    else seam_sweep<NW, KT, true, FILL_WARPS_MAX, false, KSS, false, true, true, false>(a, smem, plan, st);
+    if (half) seam_sweep<NW, KT, true, FILL_WARPS_MAX, false, KSS, false, true, true, true>(a, smem, t.plan, st);
+    else seam_sweep<NW, KT, true, FILL_WARPS_MAX, false, KSS, false, true, true, false>(a, smem, t.plan, st);
   }
-  // ---- count this CTA in ----
-  fence_proxy_async_global();   // the tables are read by a bulk copy below
+  // ---- count this CTA in; the last one joins the halves ----
+  fence_proxy_async_global();   // the tables are read by a bulk copy
   __syncthreads();
   if (threadIdx.x == 0 && atomic_add_acq_rel(p.sync, 1) == 2 * cs - 1) {
     *p.sync = 0;   // for the next launch
@@ -273,105 +230,22 @@ __global__ void __launch_bounds__(Geo<NW, KT, true>::THREADS, 1)
   }
   __syncthreads();
   if (misc[0]) {
-    // ---- the last CTA: the seam's cost and its columns in the two middle rows ----
-    unsigned char *const stab = smem + plan.ring;
-    if (warp == NW && g.tab_smem) {
-      // both ancestor tables arrive meanwhile, in a few large copies
-      fence_proxy_async_global();
-      fence_proxy_async_smem();   // the ring's last reads come first
-      if (lane == 0) mbar_arrive_expect_tx(tbar, (uint32_t)g.tab_bytes);
-      __syncwarp();
-      constexpr uint32_t PIECE = 8192;
-      for (uint32_t o = lane * PIECE; o < (uint32_t)g.tab_bytes; o += 32 * PIECE)
-        bulk_g2s(stab + o, tab + o, min(PIECE, (uint32_t)g.tab_bytes - o), tbar);
-    }
-    uint32_t best = SENT, where = SENT;   // cost; upper column << 2 | step to the lower column
-#pragma unroll 4
-    for (int q = threadIdx.x; q < (p.W + 3) / 4; q += G::THREADS) {
-      const int j0 = 4 * q;
-      const uint4 d = __ldcg(reinterpret_cast<const uint4 *>(end0) + q), u = __ldcg(reinterpret_cast<const uint4 *>(end1) + q);
-      const uint32_t ul = j0 > 0 ? __ldcg(end1 + j0 - 1) : SENT, ur = j0 + 4 < p.W ? __ldcg(end1 + j0 + 4) : SENT;
-      const uint32_t dv[4] = {d.x, d.y, d.z, d.w}, uv[6] = {ul, u.x, u.y, u.z, u.w, ur};
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const int j = j0 + c;
-        const uint32_t right = j + 1 < p.W ? uv[c + 2] : SENT;
-        const uint32_t m = min3u(uv[c], uv[c + 1], right), sum = dv[c] + m;
-        if (j < p.W && sum < best) {   // columns come in ascending order: ties keep the left one
-          best = sum;
-          where = ((uint32_t)j << 2) | (m == uv[c] ? 0u : (m == uv[c + 1] ? 1u : 2u));
-        }
-      }
-    }
-    const uint32_t wb = __reduce_min_sync(0xffffffffu, best);
-    const uint32_t ww = __reduce_min_sync(0xffffffffu, best == wb ? where : SENT);
-    uint2 *const cmin = reinterpret_cast<uint2 *>(smem + plan.cmin);
-    if (lane == 0) cmin[warp] = make_uint2(wb, ww);
-    __syncthreads();
-    if (warp == 0) {
-      const uint2 v = lane <= NW ? cmin[lane] : make_uint2(SENT, SENT);
-      best = __reduce_min_sync(0xffffffffu, v.x);
-      where = __reduce_min_sync(0xffffffffu, v.x == best ? v.y : SENT);
-      // ---- ancestor chains: lane 0 towards the top, lane 1 towards the bottom ----
-      bool bad = false;
-      if (g.tab_smem && !mbar_wait_bounded(tbar, 0u, WAIT_TIMEOUT_NS)) {
-        if (lane == 0) atomicOr(p.err, ERR_TIMEOUT);
-        bad = true;
-      }
-      if (lane < 2) {
-        const int Sh = lane ? g.S1 : g.S0;
-        int *jh = jb + (lane ? g.S0 + 1 : 0);
-        int j = (int)(where >> 2) + (lane ? (int)(where & 3u) - 1 : 0);
-        // a column outside the map is clamped (every read stays inside the table) and recorded
-        auto keep = [&](int c) { bad |= (unsigned)c >= (unsigned)p.W; return min(max(c, 0), p.W - 1); };
-        j = keep(j);
-        size_t at = (size_t)(Sh - 1 + (lane ? g.S0 : 0)) * g.gw;
-        for (int s = Sh - 1; s >= 0; --s, at -= g.gw) {
-          jh[s] = j;
-          j = keep(j + (g.tab_smem ? (int)stab[at + j] : (int)__ldcg(tab + at + j)) - 128);
-        }
-        jh[Sh] = j;
-        if (bad) atomicOr(p.err, ERR_BAD_SEAM);
-      }
-      bad = __any_sync(0xffffffffu, bad);
-      if (lane == 0 && !bad) {
-        if (p.cost) *p.cost = (int64_t)best;
-        atomicAdd(reinterpret_cast<uint32_t *>(p.sync + 1), best);
-      }
-      __syncwarp();
-      // CTA r of the cluster gets the ends of super-tiles r, r + cs, ... (the upper half's first)
-      for (int r = lane; r < cs; r += 32) {
-        int2 *dst = reinterpret_cast<int2 *>(cl.map_shared_rank(smem + plan.cmin, r));
-        for (int q = r; q < g.S0 + g.S1; q += cs) {
-          const int *jh = q < g.S0 ? jb : jb + g.S0 + 1;
-          const int s = q < g.S0 ? q : q - g.S0, Sh = q < g.S0 ? g.S0 : g.S1;
-          *dst++ = make_int2(s > 0 ? jh[s - 1] : jh[Sh], jh[s]);
-        }
-        cl.map_shared_rank(misc, r)[1] = bad ? 0 : 1;
-      }
+    const uint32_t cost = two_join<NW>(g, x, gw, p.W, smem, t, 0u, cs, p.err);
+    if (threadIdx.x == 0 && cost != SENT) {
+      if (p.cost) *p.cost = (int64_t)cost;
+      atomicAdd(reinterpret_cast<uint32_t *>(p.sync + 1), cost);
     }
   }
   cl.sync();
-
-  // ---- the super-tiles of both halves ----
   if (misc[1] == 0) return;   // the other cluster goes on (or a recorded failure)
-  const int2 *const ends = reinterpret_cast<const int2 *>(smem + plan.cmin);
-#pragma unroll 1
-  for (int k = warp; k * cs + rank < g.S0 + g.S1; k += G::FW) {
-    if (warp >= G::FW) break;
-    const int q = k * cs + rank;
-    const bool low = q >= g.S0;
-    const int last = low ? p.H - 1 : 0;
-    const FillCtx f{low ? E1 : p.E, smem + plan.fill, reinterpret_cast<uint32_t *>(p.sync + 1), 0xFFFFFFFFu, p.seam + last,
-                    p.seam_log ? p.seam_log + last : nullptr, p.err, 0, low ? -p.pitch_e : p.pitch_e,
-                    low ? g.H1 : g.H0, p.W, 0, low ? -1 : 1};
-    fill_super_tile<G, false, KSS, false>(f, low ? q - g.S0 : q, ends[k].x, ends[k].y, warp, lane);
-  }
+  const FillCtx f{p.E, nullptr, reinterpret_cast<uint32_t *>(p.sync + 1), 0xFFFFFFFFu, p.seam, p.seam_log, p.err, 0,
+                  p.pitch_e, 0, p.W, 0};
+  two_fill<G, KSS>(g, f, p.H, t, smem, cs, rank);
 }
 
 template <int NW, int KT>
 static cudaError_t launch_dp_two(const DpArgs &a, int cs, cudaStream_t st) {
-  const size_t smem = Two<NW, KT>(a.H, cs).plan.total;
+  const size_t smem = Two<NW, KT>::plan(two_split<KT, Two<NW, KT>::KSS>(a.H), cs).plan.total;
   static bool configured = false;
   if (!configured) {
     cudaError_t e = cudaFuncSetAttribute(k_dp_two<NW, KT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);

@@ -40,7 +40,7 @@ struct BatchCfg {
 // shape) and the heaviest ones of a balanced plan (CL_LAT); one group per shape and cluster size
 struct ClusterGroup {
   int shape = 0;   // ClShape
-  int cs = 1;
+  int cs = 1;      // CTAs of a cluster
   int Smax = 1;
   std::vector<BatchItem> items;
   std::vector<int> index;         // descriptor index of each item
@@ -49,8 +49,10 @@ struct BatchSetup {
   std::vector<BatchItem> items;   // images carved by one CTA each (device pointers filled in)
   std::vector<ClusterGroup> cl;   // images carved by one cluster each
   std::vector<int> fallback;      // descriptor indices carved by the per-seam cluster path
+  std::vector<char> lat;          // per descriptor: the latency shape was asked for
   size_t pool_bytes = 0;
   int Smax = 1;
+  bool map_failed = false;        // a tensor map could not be encoded
   int cluster_images() const {
     int n = 0;
     for (const ClusterGroup &g : cl) n += (int)g.items.size();

@@ -10,6 +10,7 @@
 //   seam  : int32[H]; patch: uint32[H] (the two refreshed energies of a row, low/high half).
 #pragma once
 #include <cstdint>
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 namespace sc {
@@ -90,6 +91,11 @@ cudaError_t launch_dp(const DpArgs &a, cudaStream_t st);   // forward energy whe
 // direction words and wide_anc_elems(H, W) uint16 ancestors. Forward energy when a.pstride > 0
 // (W <= 4096); the multi-map form takes a device array of n DpArgs of one size (e1 only).
 cudaError_t launch_dp_wide(const DpArgs &a, uint32_t *dirs, uint16_t *anc, cudaStream_t st);
+// Tensor map of `rows` rows of pitch elements (base: 16-byte aligned, pitch a multiple of 8), copied in
+// boxes of KT rows; BW columns go in tensor_boxes(BW) boxes of tensor_box_cols(BW) <= 256 columns.
+constexpr int tensor_boxes(int BW) { return (BW + 255) / 256; }
+constexpr int tensor_box_cols(int BW) { return ((BW + tensor_boxes(BW) - 1) / tensor_boxes(BW) + 7) / 8 * 8; }
+cudaError_t energy_tensor_map(CUtensorMap *m, const uint16_t *base, int pitch, int rows, int BW, int KT);
 struct MultiArgs;
 cudaError_t launch_dp_wide_multi(const DpArgs *dargs_dev, const MultiArgs *inl, int n, int H, int W, uint32_t *dirs,
                                  uint16_t *anc, cudaStream_t st);

@@ -410,19 +410,26 @@ static __device__ __noinline__ void compact_rows_staged(uint32_t *img, int pitch
       for (int x = a + 4 * lane; x < b; x += 128) cp_async16(buf + (x - a), row + x);
       cp_async_wait_all();
       __syncwarp();
-      for (int jb = j0; jb < j1; jb += 32) {
-        const int j = jb + lane;
-        int c = __popc(__ballot_sync(0xffffffffu, lq <= jb));
-        unsigned in = __ballot_sync(0xffffffffu, lq > jb && lq < jb + 32);
-        while (in) {
-          const int bq = __ffs(in) - 1;
-          in &= in - 1;
-          const int lv = __shfl_sync(0xffffffffu, lq, bq);
-          c += (j >= lv) ? 1 : 0;
+      // 4 x 32 outputs at a time, their gathers in flight together
+#pragma unroll 1
+      for (int jb = j0; jb < j1; jb += 128) {
+        uint32_t v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int b0 = jb + 32 * u, j = b0 + lane;
+          int c = __popc(__ballot_sync(0xffffffffu, lq <= b0));
+          unsigned in = __ballot_sync(0xffffffffu, lq > b0 && lq < b0 + 32);
+          while (in) {
+            const int bq = __ffs(in) - 1;
+            in &= in - 1;
+            const int lv = __shfl_sync(0xffffffffu, lq, bq);
+            c += (j >= lv) ? 1 : 0;
+          }
+          v[u] = (j < j1) ? buf[j + c - a] : 0u;
         }
-        const uint32_t v = (j < j1) ? buf[j + c - a] : 0u;
-        __syncwarp();
-        if (j < j1) row[j] = v;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (jb + 32 * u + lane < j1) row[jb + 32 * u + lane] = v[u];
       }
       __syncwarp();   // the buffer is reused by the next piece
     }

@@ -81,11 +81,12 @@ struct Geo {
 
 // offsets of the dynamic shared-memory regions used by seam_search
 struct SearchPlan {
-  size_t bnd, hbuf, anc, wmin, cmin, jb, misc, emx, fill, ring, bars, gat, total;
+  size_t bnd, hbuf, anc, wmin, cmin, jb, misc, emx, fill, ring, ring_end, bars, gat, total;
   int gw;   // row stride (bytes) of the gathered ancestor table in rank 0; 0: not gathered
 };
 
-template <int NW, int KT, bool CL, int FWM = FILL_WARPS_MAX, bool FWD = false, int KSS = KS, bool DIRECT = false>
+template <int NW, int KT, bool CL, int FWM = FILL_WARPS_MAX, bool FWD = false, int KSS = KS, bool DIRECT = false,
+          bool TM = false>
 __host__ __device__ inline SearchPlan search_plan(int S) {
   using G = Geo<NW, KT, CL, FWM, KSS>;
   SearchPlan p;
@@ -101,9 +102,11 @@ __host__ __device__ inline SearchPlan search_plan(int S) {
   o = (o + 15) & ~(size_t)15;
   // the backtrack fill works in the staging ring's place, which is idle by then (every staged tile
   // has been consumed before the argmin)
-  const size_t fill_sz = (size_t)G::FW * G::fill_bytes(FWD), ring_sz = (size_t)NSLOT * (FWD ? 3 : 1) * KT * G::BW * 2;
+  const size_t fill_sz = (size_t)G::FW * G::fill_bytes(FWD), 
+               ring_sz = (size_t)NSLOT * (FWD ? 3 : 1) * KT * (TM ? tensor_boxes(G::BW) * tensor_box_cols(G::BW) : G::BW) * 2;
   o = (o + 127) & ~(size_t)127;   // (tensor copies: 128-byte aligned)
   p.ring = p.fill = o; o += fill_sz > ring_sz ? fill_sz : ring_sz;  o = (o + 15) & ~(size_t)15;
+  p.ring_end = o;
   p.bars = o; o += (size_t)(NSLOT + 2) * 8;   // full[NSLOT], halo[2]
   o = (o + 15) & ~(size_t)15;
   // single-map cluster search: every CTA writes its super-tile ancestors straight into rank 0's
@@ -138,12 +141,14 @@ struct SearchArgs {
   uint32_t *endrow = nullptr;
   const void *tmap = nullptr;   // tensor map of the energy buffer (rows of pitch_e elements)
   int y0 = 0, plane_rows = 0;   // its row of this half's row 0; rows from one cost plane to the next
+  int rank0 = 0, ctas = 0;      // the cluster's CTAs that sweep this map: ctas from rank0 on (0: all of them)
 };
 
 // Running counters of the mbarrier phases, identical in every thread of the CTA.
 struct SearchState {
   uint32_t tiles = 0;  // tiles staged so far (ring slot and phase)
   uint32_t exch = 0;   // inter-CTA exchanges so far (halo buffer and phase)
+  uint32_t joins = 0;  // two-ended searches of one cluster: table copies so far (rank 0)
 };
 
 __device__ __forceinline__ uint32_t min3u(uint32_t a, uint32_t b, uint32_t c) { return __vimin3_u32(a, b, c); }
@@ -599,8 +604,9 @@ __device__ __forceinline__ unsigned long long seam_sweep(const SearchArgs &p, un
   constexpr bool LAT = CL && FWM >= FILL_WARPS_MAX && NW == 4;
   using G = Geo<NW, KT, CL, FWM, KSS>;
   constexpr int Q = G::Q, BW = G::BW, OWC = G::OWC, K2E = G::K2E;
-  const int rank = CL ? (int)cg::this_cluster().block_rank() : 0;
-  const int cs = CL ? (int)cg::this_cluster().num_blocks() : 1;
+  const int rank0 = TWO ? p.rank0 : 0;
+  const int rank = CL ? (int)cg::this_cluster().block_rank() - rank0 : 0;
+  const int cs = CL ? (TWO && p.ctas ? p.ctas : (int)cg::this_cluster().num_blocks()) : 1;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const bool producer = (warp == NW);
   const int H = p.H, W = p.W;
@@ -627,9 +633,10 @@ __device__ __forceinline__ unsigned long long seam_sweep(const SearchArgs &p, un
   for (int u = 0; u < V; ++u) oobm[u] = (c0 + u < 0 || c0 + u >= W) ? SENT : 0u;
   const bool edge = __any_sync(0xffffffffu, (oobm[0] | oobm[V - 1]) != 0u);
   const int bidx0 = c0 - (ext0 - KT);           // index of c0 in bnd and in a staged energy row
-  constexpr int NBOX = TM ? (BW + 255) / 256 : 1;   // a tensor copy's rows hold at most 256 elements
-  constexpr int BWB = BW / NBOX;                     // staged row stride
-  static_assert(BWB * NBOX == BW && BWB % 8 == 0 && (KT * BWB * 2) % 128 == 0, "tensor box");
+  constexpr int NBOX = TM ? tensor_boxes(BW) : 1;
+  constexpr int BWB = TM ? tensor_box_cols(BW) : BW;  // staged row stride
+  constexpr int SLOT = KT * NBOX * BWB;              // elements of a staged tile (one plane)
+  static_assert(BWB % 4 == 0 && (!TM || (KT * BWB * 2) % 128 == 0), "tensor box");
   unsigned long long lastmin = ~0ull;
   const int nt = p.gated ? 0 : (H + KT - 1) / KT;
   // single CTA: only the warps whose strips reach into [0, W) compute, and only their columns are
@@ -656,13 +663,15 @@ __device__ __forceinline__ unsigned long long seam_sweep(const SearchArgs &p, un
       const int rbeg = tt * KT;
       if constexpr (TM) {
         if (lane == 0) {
-          mbar_arrive_expect_tx(&full[slot], (uint32_t)(NP * KT * BW * 2));
+          // (a single CTA stages only the boxes its active warps read)
+          const int nbox = CL ? NBOX : min(NBOX, (nwa * Q + 2 * KT + BWB - 1) / BWB);
+          mbar_arrive_expect_tx(&full[slot], (uint32_t)(NP * nbox * KT * BWB * 2));
           const int y = REV ? p.y0 - rbeg - (KT - 1) : p.y0 + rbeg;
 #pragma unroll
           for (int pl = 0; pl < NP; ++pl)
-#pragma unroll
-            for (int b = 0; b < NBOX; ++b)
-              tensor_g2s_2d(ring + (size_t)((slot * NP + pl) * NBOX + b) * KT * BWB, p.tmap, E_PADL + cbeg + b * BWB,
+#pragma unroll (CL ? NBOX : 1)
+            for (int b = 0; b < nbox; ++b)
+              tensor_g2s_2d(ring + (size_t)(slot * NP + pl) * SLOT + b * KT * BWB, p.tmap, E_PADL + cbeg + b * BWB,
                             y + pl * p.plane_rows, &full[slot]);
         }
         return;
@@ -673,7 +682,7 @@ __device__ __forceinline__ unsigned long long seam_sweep(const SearchArgs &p, un
       if (lane < nrows) {
 #pragma unroll
         for (int pl = 0; pl < NP; ++pl)
-          bulk_g2s(ring + (size_t)((slot * NP + pl) * KT + lane) * BW + (clo - cbeg),
+          bulk_g2s(ring + (size_t)(slot * NP + pl) * SLOT + lane * BW + (clo - cbeg),
                    Estage + pl * pstride + (ptrdiff_t)(rbeg + lane) * pitch_e + (clo - cbeg), COPY_BYTES, &full[slot]);
       }
     };
@@ -705,8 +714,8 @@ __device__ __forceinline__ unsigned long long seam_sweep(const SearchArgs &p, un
     if constexpr (CL) {
       const bool tl = cta_own && rank > 0 && c0 < A + K2, tr = cta_own && rank < cs - 1 && c0 >= B - K2;
       if (tl || tr) {
-        push = mapa_u32(hbuf + (tl ? K2 + (c0 - A) : c0 - (B - K2)), tl ? rank - 1 : rank + 1);
-        push_bar = mapa_u32(hbar, tl ? rank - 1 : rank + 1);
+        push = mapa_u32(hbuf + (tl ? K2 + (c0 - A) : c0 - (B - K2)), rank0 + (tl ? rank - 1 : rank + 1));
+        push_bar = mapa_u32(hbar, rank0 + (tl ? rank - 1 : rank + 1));
       }
     }
     uint8_t *anc_out = TWO ? gat0 + c0 : nullptr;   // where this lane's ancestors of the current super-tile go
@@ -736,7 +745,7 @@ __device__ __forceinline__ unsigned long long seam_sweep(const SearchArgs &p, un
         const int n = (H - r0 < KT) ? H - r0 : KT;
         const bool more = t + 1 < nt;
         const uint32_t g = st.tiles + t;
-        const uint16_t *er = ring + (size_t)(g % NSLOT) * NP * KT * BW + er0;
+        const uint16_t *er = ring + (size_t)(g % NSLOT) * NP * SLOT + er0;
         if (t > 0) {
           // window of the previous row from the boundary buffer, or from the halo buffer for a
           // neighbour's columns after an exchange (relative ancestors -> warp frame). At a new
@@ -760,10 +769,10 @@ __device__ __forceinline__ unsigned long long seam_sweep(const SearchArgs &p, un
           if (EDGE) { k[0] |= oobm[0]; k[1] |= oobm[1]; k[2] |= oobm[2]; k[3] |= oobm[3]; }
         }
         if (FWD) {
-          if (n == KT) dp_rows_fwd<KT, BWB, KT * BW, EDGE>(k, er, oobm);
-          else dp_rows_n_fwd<BWB, KT * BW, EDGE>(k, er, oobm, n);
+          if (n == KT) dp_rows_fwd<KT, BWB, SLOT, EDGE>(k, er, oobm);
+          else dp_rows_n_fwd<BWB, SLOT, EDGE>(k, er, oobm, n);
         } else {
-          dp_rows<(TM ? KT : 8), BWB, EDGE, LAT, DIRECT, REV>(k, er, oobm, n, emax, cm);
+          dp_rows<(CL && FWM >= FILL_WARPS_MAX ? KT : 8), BWB, EDGE, LAT, DIRECT, REV>(k, er, oobm, n, emax, cm);
         }
         // bookkeeping on the tile's last row, the only one where a super-tile (KSS is a multiple
         // of KT) or the image can end: the ancestors of the CTA-own columns (in rank 0's gathered
@@ -829,7 +838,7 @@ __device__ void seam_search(const SearchArgs &p, unsigned char *smem, int Smax, 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int H = p.H, W = p.W, Wa = (W + 7) & ~7;
   const int S = (H + KSS - 1) / KSS;
-  const SearchPlan plan = search_plan<NW, KT, CL, FWM, FWD, KSS, DIRECT>(Smax);
+  const SearchPlan plan = search_plan<NW, KT, CL, FWM, FWD, KSS, DIRECT, TM>(Smax);
   uint8_t *ancT = reinterpret_cast<uint8_t *>(smem + plan.anc);
   unsigned long long *wmin = reinterpret_cast<unsigned long long *>(smem + plan.wmin);
   unsigned long long *cmin = reinterpret_cast<unsigned long long *>(smem + plan.cmin);

@@ -304,10 +304,12 @@ bool admit(sc_server *s) {
   }
   // per-image scratch layouts, each placed in its own arena block
   std::vector<BatchItem> items(n);
+  bool map_failed = false;
   for (int k = 0; k < n; ++k) {
     BatchSetup b;
     batch_layout(&descs[k], 1, s->cfg, s->arena.base + allocs[2 * k + 1].first, b);
     items[k] = kind ? b.cl[0].items[0] : b.items[0];
+    map_failed |= b.map_failed;
     items[k].done = s->flags + s->reqs[take[k]].flag;   // page-locked, mapped: the same address on the device
   }
   allocs.clear();
@@ -338,7 +340,9 @@ bool admit(sc_server *s) {
     r.status = 1;
   }
   cudaError_t le;
-  if (kind) {
+  if (map_failed) {
+    le = cudaErrorInvalidValue;   // nothing is launched: the requests fail
+  } else if (kind) {
     auto key = std::make_pair(kind, Smax);
     auto it = s->cl_capacity.find(key);
     if (it == s->cl_capacity.end()) {
