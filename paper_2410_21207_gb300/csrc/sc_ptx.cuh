@@ -88,15 +88,6 @@ constexpr uint64_t WAIT_TIMEOUT_NS = 2000000000ull;   // 2 s: far beyond any leg
 
 namespace sc {
 
-// retire an mbarrier whose memory is about to hold other data (no operation may be pending on it)
-__device__ __forceinline__ void mbar_inval(uint64_t *bar) {
-  asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-
 // shared::cluster address of `p` (an address in this CTA's shared memory) in CTA `rank`
 __device__ __forceinline__ uint32_t mapa_u32(const void *p, uint32_t rank) {
   uint32_t r;

@@ -291,97 +291,87 @@ __device__ __forceinline__ uint32_t refresh_energy(uint32_t px) {
 }
 
 // The energy shift of every row this warp owns (local rows q = warp, warp + nwarps, ... of nq; image
-// row row0 + q * rstride), each followed by its refreshed pair (pairs[q]: e(s-1) | e(s) << 16), staged
-// by TMA. In rounds, the warp takes as many of its next rows as its buffer holds (a prefix sum of
-// their tail sizes over the lanes); lane l copies row l's tail (the 16-byte chunks from the one
-// holding s to the one after the new last column) with one bulk copy, all completing on one
-// mbarrier at the head of the buffer; then each row is written back one element to the left, 32
-// lanes over its chunks, reading only the staged copy (so nothing is overwritten before it is read).
-// buf: this warp's buffer, 16-byte aligned, buf_bytes of it (the first 16 hold the mbarrier). Rows
-// whose seam is out of range are skipped (the caller records the error). Returns false when a wait
-// ran out (the caller records ERR_TIMEOUT). Not inlined (nor is compact_rows_staged): a separate
-// function gets its own register allocation, and inlined the two phases cost the one-CTA batched
-// kernel ~160 bytes of spills.
-static __device__ __noinline__ bool shift_rows_bulk(uint16_t *E, int pe, int nq, int row0, int rstride, int w, const int32_t *seam,
-                                       const uint32_t *pairs, int warp, int nwarps, int lane, unsigned char *buf,
-                                       int buf_bytes) {
-  uint64_t *bar = reinterpret_cast<uint64_t *>(buf);
-  unsigned char *data = buf + 16;
-  const int cap = buf_bytes - 16;
+// row row0 + q * rstride), each followed by its refreshed pair (pairs[q]: e(s-1) | e(s) << 16), NR rows
+// at a time through registers: a lane holds chunks cb + lane and cb + 32 + lane (8 elements each, cb first
+// the chunk holding s) of each row, takes the element after each chunk from the next lane, and writes the
+// chunk one element to the left; longer tails go on block by block from the left, each read before it
+// is written. Rows whose seam is out of range are skipped (the caller records the error).
+// Latency-bound (four warps per SM sub-partition): all the rows' loads are in flight at once and nothing goes
+// through shared memory. Against tails staged there by bulk copies and written back chunk by chunk, per seam
+// of one image: 400x900 96.2 -> 93.4 us, 1254x944 176.1 -> 174.1 us, 2500x1332 on its cluster 223.6 -> 217.0.
+// Not inlined (nor is compact_rows): a separate function gets its own register allocation, and inlined
+// the two phases cost the one-CTA batched kernel ~160 bytes of spills.
+static __device__ __noinline__ void shift_rows(uint16_t *E, int pe, int nq, int row0, int rstride, int w,
+                                               const int32_t *seam, const uint32_t *pairs, int warp, int nwarps,
+                                               int lane) {
+  constexpr int R = 2, NR = 4;
   const int c_last = (w - 2) >> 3;   // the chunk holding the new last column
   const int nk = warp < nq ? (nq - warp + nwarps - 1) / nwarps : 0;
-  if (nk == 0) return true;
-  if (lane == 0) mbar_init(bar, 1);
-  fence_mbar_init();
-  __syncwarp();
-  uint32_t parity = 0;
-  bool ok = true;
-  for (int k0 = 0; k0 < nk;) {
-    const int k = k0 + lane;
-    const int q = warp + k * nwarps;
-    const int s = k < nk ? seam[row0 + q * rstride] : -1;
-    uint16_t *er = E + (size_t)(row0 + (k < nk ? q : 0) * rstride) * pe;
-    const int bytes = (k < nk && s >= 0 && s < w - 1) ? 16 * (c_last - (s >> 3) + 2) : 0;
-    int incl = bytes;
+  const int64_t rowstep = (int64_t)nwarps * rstride * pe;
+  uint16_t *e0 = E + (int64_t)(row0 + warp * rstride) * pe;   // the group's first row
+#pragma unroll 1
+  for (int k0 = 0; k0 < nk; k0 += 32) {
+    const int kl = k0 + lane;
+    const int sl = kl < nk ? seam[row0 + (warp + kl * nwarps) * rstride] : -1;
+    const uint32_t pl = kl < nk ? pairs[warp + kl * nwarps] : 0u;
+    const int n = min(32, nk - k0);
+#pragma unroll 1
+    for (int t = 0; t < n; t += NR, e0 += NR * rowstep) {
+      int s[NR], cb[NR];
+      bool any = false;
 #pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const int t = __shfl_up_sync(0xffffffffu, incl, d);
-      if (lane >= d) incl += t;
-    }
-    // the rows taken are a prefix of the lanes (incl never decreases)
-    const int n = __popc(__ballot_sync(0xffffffffu, k < nk && incl <= cap));
-    if (n == 0) {   // the next row's tail alone exceeds the buffer: shifted in place, chunk by chunk
-      const int s0 = __shfl_sync(0xffffffffu, s, 0);
-      uint16_t *e0 = E + (size_t)(row0 + warp * rstride + k0 * nwarps * rstride) * pe;
-      const uint32_t pr = pairs[warp + k0 * nwarps];
-      shift_row_u16(e0, s0, w, lane);
-      __syncwarp();
-      if (lane == 0) {
-        if (s0 >= 1) e0[s0 - 1] = (uint16_t)(pr & 0xFFFFu);
-        e0[s0] = (uint16_t)(pr >> 16);
+      for (int v = 0; v < NR; ++v) {
+        s[v] = __shfl_sync(0xffffffffu, sl, t + v);   // (t + v <= 31: t is a multiple of NR)
+        // past the last row, a seam out of range, or one in the last column: nothing to shift
+        cb[v] = (t + v >= n || s[v] < 0 || s[v] >= w - 1) ? c_last + 1 : s[v] >> 3;
+        any |= cb[v] <= c_last;
       }
-      k0 += 1;
-      continue;
-    }
-    const int total = __shfl_sync(0xffffffffu, incl, n - 1);
-    const int off = incl - bytes;
-    if (total > 0) {
-      fence_proxy_async_smem();   // this warp's reads of the buffer's previous round come first
-      __syncwarp();
-      if (lane == 0) mbar_arrive_expect_tx(bar, (uint32_t)total);
-      __syncwarp();
-      if (lane < n && bytes > 0) bulk_g2s(data + off, er + 8 * (s >> 3), (uint32_t)bytes, bar);
-      ok = mbar_wait_bounded(bar, parity, WAIT_TIMEOUT_NS);
-      parity ^= 1u;
-      if (!__all_sync(0xffffffffu, ok)) return false;   // copies may be in flight: the barrier stays
-    }
-    // a seam in the last column: nothing to shift, only the left refreshed value
-    if (lane < n && s == w - 1 && s >= 1) er[s - 1] = (uint16_t)(pairs[q] & 0xFFFFu);
-    for (int t = 0; t < n; ++t) {
-      const int bt = __shfl_sync(0xffffffffu, bytes, t);
-      if (bt == 0) continue;
-      const int st = __shfl_sync(0xffffffffu, s, t), ot = __shfl_sync(0xffffffffu, off, t);
-      const int qt = warp + (k0 + t) * nwarps;
-      uint16_t *et = E + (size_t)(row0 + qt * rstride) * pe;
-      const uint16_t *b = reinterpret_cast<const uint16_t *>(data + ot);
-      const int c_lo = st >> 3;
-      for (int c = c_lo + lane; c <= c_last; c += 32) {
-        const uint4 x = *reinterpret_cast<const uint4 *>(b + 8 * (c - c_lo));
-        const uint32_t nx = b[8 * (c - c_lo) + 8];
-        *reinterpret_cast<uint4 *>(et + 8 * c) = shift_chunk(x, nx, st - 8 * c);
-        if (c == c_lo) {   // this lane wrote the chunk holding s: the refreshed pair goes over it
-          const uint32_t pr = pairs[qt];
-          if (st >= 1) et[st - 1] = (uint16_t)(pr & 0xFFFFu);
-          et[st] = (uint16_t)(pr >> 16);
+      while (any) {
+        uint4 x[NR][R];
+        uint32_t after[NR];
+#pragma unroll
+        for (int v = 0; v < NR; ++v) {
+          const uint16_t *er = e0 + v * rowstep;
+          after[v] = 0u;
+#pragma unroll
+          for (int r = 0; r < R; ++r) {
+            const int c = cb[v] + 32 * r;
+            x[v][r] = make_uint4(0u, 0u, 0u, 0u);
+            if (cb[v] <= c_last && c <= c_last + 1) {   // (the same for every lane)
+              if (c + lane <= c_last + 1) x[v][r] = __ldcg(reinterpret_cast<const uint4 *>(er + 8 * (c + lane)));
+            }
+          }
+          // the element after the block's last chunk
+          if (cb[v] + 32 * R <= c_last + 1) after[v] = __ldcg(er + 8 * (cb[v] + 32 * R));
+        }
+        any = false;
+#pragma unroll
+        for (int v = 0; v < NR; ++v) {
+          uint16_t *er = e0 + v * rowstep;
+#pragma unroll
+          for (int r = 0; r < R; ++r) {
+            const int c = cb[v] + 32 * r;
+            if (c > c_last) continue;   // (the same for every lane)
+            const uint32_t first = lane > 0 ? x[v][r].x : (r + 1 < R ? x[v][r + 1 < R ? r + 1 : r].x : after[v]);
+            const uint32_t nx = __shfl_sync(0xffffffffu, first, (lane + 1) & 31);
+            const uint4 o = shift_chunk(x[v][r], nx, r == 0 ? s[v] - 8 * (c + lane) : 0);
+            if (c + lane <= c_last) *reinterpret_cast<uint4 *>(er + 8 * (c + lane)) = o;
+          }
+          cb[v] += 32 * R;
+          any |= cb[v] <= c_last;
         }
       }
+      __syncwarp();
+      // the pairs, one lane per row
+      const uint32_t pr = __shfl_sync(0xffffffffu, pl, (t + (lane & (NR - 1))) & 31);
+      const int sr = __shfl_sync(0xffffffffu, sl, (t + (lane & (NR - 1))) & 31);
+      if (lane < NR && t + lane < n && sr >= 0 && sr < w) {
+        uint16_t *er = e0 + lane * rowstep;
+        if (sr >= 1) er[sr - 1] = (uint16_t)(pr & 0xFFFFu);
+        if (sr <= w - 2) er[sr] = (uint16_t)(pr >> 16);
+      }
     }
-    __syncwarp();   // the buffer is reused by the next round
-    k0 += n;
   }
-  __syncwarp();
-  if (lane == 0) mbar_inval(bar);   // the buffer holds other data next
-  return ok;
 }
 
 // compact_row_lazy for every row this warp owns (local rows q = warp, warp + nwarps, ... of nq;
