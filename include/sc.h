@@ -104,7 +104,8 @@ int sc_energy(const uint8_t *img, int H, int W, int C, uint16_t *energy_out, voi
  * seam_out: device, int32[H]; seam_out[i] in [0, W), |seam_out[i] - seam_out[i-1]| <= 1.
  * cost_out: device, int64[1] or NULL: the seam's total energy (the minimum of M's last row).
  * The fast search packs each cost with its backtrack ancestor into 32 bits, which holds costs
- * below 2^24; while copying the map the library checks H * max(e) < 2^24 on the device, and a map
+ * below 2^24; the library checks H * max(e) < 2^24 on the device (in the search itself for a map it
+ * reads in place: W a multiple of 8 and a 16-byte aligned base; while copying any other), and a map
  * that fails it is searched instead by a slower kernel with exact 32-bit costs (one CTA, about
  * 0.1 ms per 1080 x 1920 map). Both give the same seam and cost; nothing is refused.
  * Errors: SC_EINVAL for NULL energy/seam_out, H < 1, W < 1, H > SC_MAX_ROWS, W > SC_MAX_COLS;

@@ -38,13 +38,13 @@ DpShape dp_shape_for(int W) {
 template <int NW, int KT, bool FWD>
 __host__ __device__ constexpr int dp_super_rows() { return (NW == 4 && KT == 32 && !FWD) ? KS : KS_WIDE; }
 
-template <int NW, int KT, bool FWD = false>
+template <int NW, int KT, bool FWD = false, bool DIRECT = false>
 __global__ void __launch_bounds__(Geo<NW, KT, true>::THREADS, 1)
     k_dp(DpArgs p, const __grid_constant__ CUtensorMap tmap) {
   extern __shared__ __align__(128) unsigned char smem[];
   constexpr int KSS = dp_super_rows<NW, KT, FWD>();
   const int S = (p.H + KSS - 1) / KSS;
-  search_init(smem, search_plan<NW, KT, true, FILL_WARPS_MAX, FWD, KSS, false, true>(S));
+  search_init(smem, search_plan<NW, KT, true, FILL_WARPS_MAX, FWD, KSS, DIRECT, true>(S));
   // neighbours push into each other's halo buffers: every CTA's barriers must be initialised first
   cg::this_cluster().sync();
   // the set-up above overlaps the previous kernel of the seam loop; its results are read below
@@ -60,12 +60,14 @@ __global__ void __launch_bounds__(Geo<NW, KT, true>::THREADS, 1)
   a.seam_log = p.seam_log;
   a.cost = p.cost;
   a.err = p.err;
-  a.gated = (p.gate != nullptr) && (*p.gate & ERR_ENERGY_RANGE);
+  a.gated = !DIRECT && (p.gate != nullptr) && (*p.gate & ERR_ENERGY_RANGE);
+  a.gate = p.gate;
   a.pstride = p.pstride;
   a.tmap = &tmap;
+  a.x0 = DIRECT ? 0 : E_PADL;
   a.plane_rows = FWD ? (int)(p.pstride / p.pitch_e) : 0;
   SearchState st;
-  seam_search<NW, KT, true, FILL_WARPS_MAX, FWD, KSS, false, true>(a, smem, S, st);
+  seam_search<NW, KT, true, FILL_WARPS_MAX, FWD, KSS, DIRECT, true>(a, smem, S, st);
 }
 
 // one or two clusters of cs CTAs; a programmatic dependent (may start before its predecessor ends)
@@ -110,24 +112,24 @@ cudaError_t energy_tensor_map(CUtensorMap *m, const uint16_t *base, int pitch, i
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-template <int NW, int KT, bool FWD = false>
+template <int NW, int KT, bool FWD = false, bool DIRECT = false>
 static cudaError_t launch_dp_shape(const DpArgs &a, int cs, cudaStream_t st) {
   constexpr int KSS = dp_super_rows<NW, KT, FWD>();
-  const size_t smem = search_plan<NW, KT, true, FILL_WARPS_MAX, FWD, KSS, false, true>((a.H + KSS - 1) / KSS).total;
+  const size_t smem = search_plan<NW, KT, true, FILL_WARPS_MAX, FWD, KSS, DIRECT, true>((a.H + KSS - 1) / KSS).total;
   static bool configured = false;
   if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(k_dp<NW, KT, FWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
+    cudaError_t e = cudaFuncSetAttribute(k_dp<NW, KT, FWD, DIRECT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_dp<NW, KT, FWD>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    e = cudaFuncSetAttribute(k_dp<NW, KT, FWD, DIRECT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     configured = true;
   }
   if (smem > 232448) return cudaErrorInvalidValue;
   CUtensorMap tmap;
   const int rows = a.H + (FWD ? (int)(2 * a.pstride / a.pitch_e) : 0);   // the three planes in a row
-  const cudaError_t e = energy_tensor_map(&tmap, a.E - E_PADL, a.pitch_e, rows, Geo<NW, KT, true>::BW, KT);
+  const cudaError_t e = energy_tensor_map(&tmap, DIRECT ? a.E : a.E - E_PADL, a.pitch_e, rows, Geo<NW, KT, true>::BW, KT);
   if (e != cudaSuccess) return e;
-  return launch_dp_cluster(k_dp<NW, KT, FWD>, cs, cs, Geo<NW, KT, true>::THREADS, smem, st, a, tmap);
+  return launch_dp_cluster(k_dp<NW, KT, FWD, DIRECT>, cs, cs, Geo<NW, KT, true>::THREADS, smem, st, a, tmap);
 }
 
 // ---- the two-ended search ----
@@ -174,7 +176,7 @@ struct Two {
   }
 };
 
-template <int NW, int KT>
+template <int NW, int KT, bool DIRECT>
 __global__ void __launch_bounds__(Geo<NW, KT, true>::THREADS, 1)
     k_dp_two(DpArgs p, const __grid_constant__ CUtensorMap tmap) {
   extern __shared__ __align__(128) unsigned char smem[];
@@ -201,7 +203,7 @@ __global__ void __launch_bounds__(Geo<NW, KT, true>::THREADS, 1)
   pdl_wait_prerequisites();
   // only now: the refresh that depends on this launch reads what its predecessors wrote before it waits
   pdl_launch_dependents();
-  if (p.gate && (*p.gate & ERR_ENERGY_RANGE)) return;   // left to the wide-cost search
+  if (!DIRECT && p.gate && (*p.gate & ERR_ENERGY_RANGE)) return;   // left to the wide-cost search
   const TwoScratch x(p.scratch, gw);
   {
     SearchArgs a;
@@ -216,10 +218,12 @@ __global__ void __launch_bounds__(Geo<NW, KT, true>::THREADS, 1)
     a.gw = gw;
     a.endrow = half ? x.end1 : x.end0;
     a.tmap = &tmap;
+    a.x0 = DIRECT ? 0 : E_PADL;
     a.y0 = half ? p.H - 1 : 0;
+    a.gmax = reinterpret_cast<uint32_t *>(p.sync + 2);
     SearchState st;
-    if (half) seam_sweep<NW, KT, true, FILL_WARPS_MAX, false, KSS, false, true, true, true>(a, smem, t.plan, st);
-    else seam_sweep<NW, KT, true, FILL_WARPS_MAX, false, KSS, false, true, true, false>(a, smem, t.plan, st);
+    if (half) seam_sweep<NW, KT, true, FILL_WARPS_MAX, false, KSS, DIRECT, true, true, true>(a, smem, t.plan, st);
+    else seam_sweep<NW, KT, true, FILL_WARPS_MAX, false, KSS, DIRECT, true, true, false>(a, smem, t.plan, st);
   }
   // ---- count this CTA in; the last one joins the halves ----
   fence_proxy_async_global();   // the tables are read by a bulk copy
@@ -227,6 +231,16 @@ __global__ void __launch_bounds__(Geo<NW, KT, true>::THREADS, 1)
   if (threadIdx.x == 0 && atomic_add_acq_rel(p.sync, 1) == 2 * cs - 1) {
     *p.sync = 0;   // for the next launch
     misc[0] = 1;
+    if (DIRECT) {
+      // the 24-bit keys hold the seam sums only while H * max(e) < 2^24; otherwise this result is void and
+      // the wide-cost search, launched next, takes the map
+      const uint32_t e = (uint32_t)__ldcg(p.sync + 2);
+      p.sync[2] = 0;
+      if ((uint64_t)e * (uint64_t)p.H >= ((uint64_t)1 << 24)) {
+        misc[0] = 0;
+        if (p.gate) atomicOr(p.gate, ERR_ENERGY_RANGE);
+      }
+    }
   }
   __syncthreads();
   if (misc[0]) {
@@ -239,26 +253,38 @@ __global__ void __launch_bounds__(Geo<NW, KT, true>::THREADS, 1)
   cl.sync();
   if (misc[1] == 0) return;   // the other cluster goes on (or a recorded failure)
   const FillCtx f{p.E, nullptr, reinterpret_cast<uint32_t *>(p.sync + 1), 0xFFFFFFFFu, p.seam, p.seam_log, p.err, 0,
-                  p.pitch_e, 0, p.W, 0};
-  two_fill<G, KSS>(g, f, p.H, t, smem, cs, rank);
+                  p.pitch_e, 0, p.W, (p.W + 7) & ~7};
+  two_fill<G, KSS, DIRECT>(g, f, p.H, t, smem, cs, rank);
 }
 
-template <int NW, int KT>
+template <int NW, int KT, bool DIRECT>
 static cudaError_t launch_dp_two(const DpArgs &a, int cs, cudaStream_t st) {
   const size_t smem = Two<NW, KT>::plan(two_split<KT, Two<NW, KT>::KSS>(a.H), cs).plan.total;
   static bool configured = false;
   if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(k_dp_two<NW, KT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
+    cudaError_t e = cudaFuncSetAttribute(k_dp_two<NW, KT, DIRECT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_dp_two<NW, KT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    e = cudaFuncSetAttribute(k_dp_two<NW, KT, DIRECT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     configured = true;
   }
   if (smem > SEARCH_SMEM_LIMIT) return cudaErrorInvalidValue;
   CUtensorMap tmap;
-  const cudaError_t e = energy_tensor_map(&tmap, a.E - E_PADL, a.pitch_e, a.H, Geo<NW, KT, true>::BW, KT);
+  const cudaError_t e = energy_tensor_map(&tmap, DIRECT ? a.E : a.E - E_PADL, a.pitch_e, a.H, Geo<NW, KT, true>::BW, KT);
   if (e != cudaSuccess) return e;
-  return launch_dp_cluster(k_dp_two<NW, KT>, 2 * cs, cs, Geo<NW, KT, true>::THREADS, smem, st, a, tmap);
+  return launch_dp_cluster(k_dp_two<NW, KT, DIRECT>, 2 * cs, cs, Geo<NW, KT, true>::THREADS, smem, st, a, tmap);
+}
+
+template <bool DIRECT>
+static cudaError_t launch_dp_e1(const DpArgs &a, const DpShape &s, cudaStream_t st) {
+  if (a.H >= TWO_MIN_ROWS) {
+    if (s.nw == 4 && s.kt == 32) return launch_dp_two<4, 32, DIRECT>(a, s.cs, st);
+    if (s.nw == 8 && s.kt == 32) return launch_dp_two<8, 32, DIRECT>(a, s.cs, st);
+    return launch_dp_two<8, 16, DIRECT>(a, s.cs, st);
+  }
+  if (s.nw == 4 && s.kt == 32) return launch_dp_shape<4, 32, false, DIRECT>(a, s.cs, st);
+  if (s.nw == 8 && s.kt == 32) return launch_dp_shape<8, 32, false, DIRECT>(a, s.cs, st);
+  return launch_dp_shape<8, 16, false, DIRECT>(a, s.cs, st);
 }
 
 // forward energy stages three planes per row: one shape, 4 warps x 16-row tiles (W <= 4096)
@@ -272,14 +298,7 @@ cudaError_t launch_dp(const DpArgs &a, cudaStream_t st) {
   }
   const DpShape s = dp_shape_for(a.W);
   if (s.cs > MAX_CLUSTER) return cudaErrorInvalidValue;
-  if (a.H >= TWO_MIN_ROWS) {
-    if (s.nw == 4 && s.kt == 32) return launch_dp_two<4, 32>(a, s.cs, st);
-    if (s.nw == 8 && s.kt == 32) return launch_dp_two<8, 32>(a, s.cs, st);
-    return launch_dp_two<8, 16>(a, s.cs, st);
-  }
-  if (s.nw == 4 && s.kt == 32) return launch_dp_shape<4, 32>(a, s.cs, st);
-  if (s.nw == 8 && s.kt == 32) return launch_dp_shape<8, 32>(a, s.cs, st);
-  return launch_dp_shape<8, 16>(a, s.cs, st);
+  return a.direct ? launch_dp_e1<true>(a, s, st) : launch_dp_e1<false>(a, s, st);
 }
 
 }  // namespace sc

@@ -249,7 +249,10 @@ __device__ void wide_search(const DpArgs &p, uint32_t *__restrict__ dirs, uint16
     atomicAdd(&red[32], sum);
   }
   __syncthreads();
-  if (t == 0 && red[32] != (red[0] >> 32)) atomicOr(p.err, ERR_COST_MISMATCH);
+  if (t == 0) {
+    if (red[32] != (red[0] >> 32)) atomicOr(p.err, ERR_COST_MISMATCH);
+    *p.gate = 0;   // for the next call (every thread has read it)
+  }
 }
 
 template <bool FWD>

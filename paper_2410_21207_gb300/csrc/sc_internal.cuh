@@ -54,13 +54,16 @@ struct DpArgs {
   int pitch_e;
   int H, W;
   uint32_t *scratch;   // two-ended search: cost rows and ancestor tables, (ceil(H/KS) + 1) * pitch_e words
-  int *sync;           // two-ended search: [0] arrival counter, [1] cost check sum; 0 between launches
+  int *sync;           // two-ended search: [0] arrival counter, [1] cost check sum, [2] energy maximum; 0
+                       // between launches
   int32_t *seam;       // out [H]
   int32_t *seam_log;   // nullable, out [H]
   int64_t *cost;       // nullable, out [1]
   int *err;            // device error word
   int *gate;           // nullable: with ERR_ENERGY_RANGE set the 24-bit search skips the map and the
                        // wide-cost search takes it (the multi-map search also sets it itself)
+  bool direct = false; // E is the caller's unpadded map (16-byte aligned, pitch_e = W a multiple of 8): read
+                       // in place, its 24-bit range checked by the search itself, which sets the gate
   int64_t pstride = 0; // forward energy: elements between the CU, DL, DR planes (0: the e1 map)
 };
 

@@ -139,7 +139,9 @@ struct SearchArgs {
   uint8_t *gtab = nullptr;
   int gw = 0;
   uint32_t *endrow = nullptr;
+  uint32_t *gmax = nullptr;     // DIRECT: the maximum of the map's energies, over both halves
   const void *tmap = nullptr;   // tensor map of the energy buffer (rows of pitch_e elements)
+  int x0 = E_PADL;              // its column of the map's column 0
   int y0 = 0, plane_rows = 0;   // its row of this half's row 0; rows from one cost plane to the next
   int rank0 = 0, ctas = 0;      // the cluster's CTAs that sweep this map: ctas from rank0 on (0: all of them)
 };
@@ -671,7 +673,7 @@ __device__ __forceinline__ unsigned long long seam_sweep(const SearchArgs &p, un
           for (int pl = 0; pl < NP; ++pl)
 #pragma unroll (CL ? NBOX : 1)
             for (int b = 0; b < nbox; ++b)
-              tensor_g2s_2d(ring + (size_t)(slot * NP + pl) * SLOT + b * KT * BWB, p.tmap, E_PADL + cbeg + b * BWB,
+              tensor_g2s_2d(ring + (size_t)(slot * NP + pl) * SLOT + b * KT * BWB, p.tmap, p.x0 + cbeg + b * BWB,
                             y + pl * p.plane_rows, &full[slot]);
         }
         return;
@@ -817,10 +819,13 @@ __device__ __forceinline__ unsigned long long seam_sweep(const SearchArgs &p, un
     else tiles(std::integral_constant<bool, false>());
     if (DIRECT) {
       const uint32_t m = __reduce_max_sync(0xffffffffu, max(emax & 0xFFFFu, emax >> 16));
-      if (lane == 0) emx[warp] = m;
+      if (lane == 0) {
+        if (TWO) atomicMax(p.gmax, m);
+        else emx[warp] = m;
+      }
     }
   }
-  if (DIRECT && lane == 0 && (producer || !active)) emx[warp] = 0u;
+  if (DIRECT && !TWO && lane == 0 && (producer || !active)) emx[warp] = 0u;
   st.tiles += (uint32_t)nt;
   if (CL && nt > 0) st.exch += (uint32_t)((cs > 1) ? ((H - 1) / K2) : 0);
   return lastmin;

@@ -168,7 +168,7 @@ __device__ __forceinline__ uint32_t two_join(const TwoSplit &g, const TwoScratch
 
 // The calling CTA's share of the super-tiles of both halves of an H-row map (rank r of `ctas`), from the
 // ends two_join left in its cmin.
-template <typename G, int KSS>
+template <typename G, int KSS, bool DIRECT = false>
 __device__ __forceinline__ void two_fill(const TwoSplit &g, FillCtx f, int H, const TwoPlan &t, unsigned char *smem,
                                          int ctas, int rank) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -188,7 +188,7 @@ __device__ __forceinline__ void two_fill(const TwoSplit &g, FillCtx f, int H, co
     const bool low = q >= g.S0;
     FillCtx c = low ? dn : up;
     c.H = low ? g.H1 : g.H0;
-    fill_super_tile<G, false, KSS, false>(c, low ? q - g.S0 : q, ends[k].x, ends[k].y, warp, lane);
+    fill_super_tile<G, false, KSS, DIRECT>(c, low ? q - g.S0 : q, ends[k].x, ends[k].y, warp, lane);
   }
 }
 

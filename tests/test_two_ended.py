@@ -68,3 +68,27 @@ def test_two_ended_search_parity(H, W):
             sc.check()
             assert int(c.cpu()[0]) == cost, kind
             np.testing.assert_array_equal(seam.cpu().numpy(), ref, err_msg=f"{H}x{W} {kind}")
+
+
+# maps read in place (rows of a multiple of 8 columns from a 16-byte boundary) and the same maps 2 bytes off
+# it (copied first), at both sides of the 24-bit range: H * max(e) = 2^24 - H (fast) and 2^24 (wide-cost);
+# 128 rows: one cluster, 512: both ends; then an ordinary map on the same workspace
+@pytest.mark.gpu
+@pytest.mark.parametrize("H,W,emax", [(512, 64, 32767), (512, 64, 32768), (512, 2056, 32768), (128, 264, 65535),
+                                      (256, 8, 65535), (264, 136, 65535)])
+def test_maps_in_place_at_the_range_limit(H, W, emax):
+    from paper_2410_21207_gb300 import binding as sc
+    rng = np.random.default_rng(H + W + emax)
+    near = rng.integers(emax - 3, emax, size=(H, W), endpoint=True).astype(np.uint16)
+    near[H // 2, W // 2] = emax
+    plain = rng.integers(0, 2041, size=(H, W)).astype(np.uint16)
+    for e in (near, plain, near, plain):
+        ref, cost = oracle.dp_seam(e)
+        buf = torch.zeros(H * W + 8, dtype=torch.uint16, device="cuda")
+        for off in (0, 1):
+            view = buf[off:off + H * W].view(H, W)
+            view.copy_(torch.from_numpy(e))
+            seam, c = sc.find_seam(view)
+            sc.check()
+            assert int(c.cpu()[0]) == cost
+            np.testing.assert_array_equal(seam.cpu().numpy(), ref)
