@@ -1,6 +1,6 @@
 // One seam search per launch (the per-seam path of the carve and sc_find_seam): maps of at least
-// TWO_MIN_ROWS rows from both ends by two thread-block clusters (k_dp_two), shorter ones and forward
-// energy by one cluster (k_dp, seam_search in sc_search.cuh).
+// TWO_MIN_ROWS rows from both ends by two thread-block clusters (k_dp_two), shorter ones by one cluster
+// (k_dp, seam_search in sc_search.cuh).
 #include <atomic>
 
 #include <cudaTypedefs.h>
@@ -166,21 +166,21 @@ static cudaError_t launch_dp_shape(const DpArgs &a, int cs, cudaStream_t st) {
 // 3840 columns).
 constexpr int TWO_MIN_ROWS = 192;
 
-template <int NW, int KT>
+template <int NW, int KT, bool FWD>
 struct Two {
-  static constexpr int KSS = dp_super_rows<NW, KT, false>();
+  static constexpr int KSS = FWD ? KS : dp_super_rows<NW, KT, false>();
   using G = Geo<NW, KT, true, FILL_WARPS_MAX, KSS>;
   static __host__ __device__ TwoPlan plan(const TwoSplit &s, int cs) {
     const size_t tab = (size_t)(s.S0 + s.S1) * cs * G::OWC;
-    return two_plan<G, NW, KT, KSS>(s.S0 + s.S1, cs, tab, SEARCH_SMEM_LIMIT);
+    return two_plan<G, NW, KT, KSS, FWD>(s.S0 + s.S1, cs, tab, SEARCH_SMEM_LIMIT);
   }
 };
 
-template <int NW, int KT, bool DIRECT>
+template <int NW, int KT, bool DIRECT, bool FWD>
 __global__ void __launch_bounds__(Geo<NW, KT, true>::THREADS, 1)
     k_dp_two(DpArgs p, const __grid_constant__ CUtensorMap tmap) {
   extern __shared__ __align__(128) unsigned char smem[];
-  using T = Two<NW, KT>;
+  using T = Two<NW, KT, FWD>;
   using G = typename T::G;
   constexpr int KSS = T::KSS;
   cg::cluster_group cl = cg::this_cluster();
@@ -204,7 +204,11 @@ __global__ void __launch_bounds__(Geo<NW, KT, true>::THREADS, 1)
   // only now: the refresh that depends on this launch reads what its predecessors wrote before it waits
   pdl_launch_dependents();
   if (!DIRECT && p.gate && (*p.gate & ERR_ENERGY_RANGE)) return;   // left to the wide-cost search
-  const TwoScratch x(p.scratch, gw);
+  TwoScratch x(p.scratch, gw);
+  if (FWD) {
+    x.dl = p.E + p.pstride + (ptrdiff_t)g.H0 * p.pitch_e;
+    x.dr = p.E + 2 * p.pstride + (ptrdiff_t)g.H0 * p.pitch_e;
+  }
   {
     SearchArgs a;
     a.E = p.E;
@@ -213,7 +217,8 @@ __global__ void __launch_bounds__(Geo<NW, KT, true>::THREADS, 1)
     a.W = p.W;
     a.err = p.err;
     a.gated = false;
-    a.pstride = 0;
+    a.pstride = FWD ? p.pstride : 0;
+    a.plane_rows = FWD ? (int)(p.pstride / p.pitch_e) : 0;
     a.gtab = x.tab + (half ? (size_t)g.S0 * gw : 0);
     a.gw = gw;
     a.endrow = half ? x.end1 : x.end0;
@@ -222,8 +227,8 @@ __global__ void __launch_bounds__(Geo<NW, KT, true>::THREADS, 1)
     a.y0 = half ? p.H - 1 : 0;
     a.gmax = reinterpret_cast<uint32_t *>(p.sync + 2);
     SearchState st;
-    if (half) seam_sweep<NW, KT, true, FILL_WARPS_MAX, false, KSS, DIRECT, true, true, true>(a, smem, t.plan, st);
-    else seam_sweep<NW, KT, true, FILL_WARPS_MAX, false, KSS, DIRECT, true, true, false>(a, smem, t.plan, st);
+    if (half) seam_sweep<NW, KT, true, FILL_WARPS_MAX, FWD, KSS, DIRECT, true, true, true>(a, smem, t.plan, st);
+    else seam_sweep<NW, KT, true, FILL_WARPS_MAX, FWD, KSS, DIRECT, true, true, false>(a, smem, t.plan, st);
   }
   // ---- count this CTA in; the last one joins the halves ----
   fence_proxy_async_global();   // the tables are read by a bulk copy
@@ -244,35 +249,36 @@ __global__ void __launch_bounds__(Geo<NW, KT, true>::THREADS, 1)
   }
   __syncthreads();
   if (misc[0]) {
-    const uint32_t cost = two_join<NW>(g, x, gw, p.W, smem, t, 0u, cs, p.err);
+    const uint32_t cost = two_join<NW, FWD>(g, x, gw, p.W, smem, t, 0u, cs, p.err);
     if (threadIdx.x == 0 && cost != SENT) {
       if (p.cost) *p.cost = (int64_t)cost;
-      atomicAdd(reinterpret_cast<uint32_t *>(p.sync + 1), cost);
+      atomicAdd(reinterpret_cast<uint32_t *>(p.sync + 1), cost - (FWD ? (uint32_t)misc[3] : 0u));
     }
   }
   cl.sync();
   if (misc[1] == 0) return;   // the other cluster goes on (or a recorded failure)
-  const FillCtx f{p.E, nullptr, reinterpret_cast<uint32_t *>(p.sync + 1), 0xFFFFFFFFu, p.seam, p.seam_log, p.err, 0,
-                  p.pitch_e, 0, p.W, (p.W + 7) & ~7};
-  two_fill<G, KSS, DIRECT>(g, f, p.H, t, smem, cs, rank);
+  const FillCtx f{p.E, nullptr, reinterpret_cast<uint32_t *>(p.sync + 1), 0xFFFFFFFFu, p.seam, p.seam_log, p.err,
+                  FWD ? p.pstride : 0, p.pitch_e, 0, p.W, (p.W + 7) & ~7};
+  two_fill<G, KSS, DIRECT, FWD>(g, f, p.H, t, smem, cs, rank);
 }
 
-template <int NW, int KT, bool DIRECT>
+template <int NW, int KT, bool DIRECT, bool FWD = false>
 static cudaError_t launch_dp_two(const DpArgs &a, int cs, cudaStream_t st) {
-  const size_t smem = Two<NW, KT>::plan(two_split<KT, Two<NW, KT>::KSS>(a.H), cs).plan.total;
+  const size_t smem = Two<NW, KT, FWD>::plan(two_split<KT, Two<NW, KT, FWD>::KSS>(a.H), cs).plan.total;
   static bool configured = false;
   if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(k_dp_two<NW, KT, DIRECT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
+    cudaError_t e = cudaFuncSetAttribute(k_dp_two<NW, KT, DIRECT, FWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_dp_two<NW, KT, DIRECT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    e = cudaFuncSetAttribute(k_dp_two<NW, KT, DIRECT, FWD>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     configured = true;
   }
   if (smem > SEARCH_SMEM_LIMIT) return cudaErrorInvalidValue;
   CUtensorMap tmap;
-  const cudaError_t e = energy_tensor_map(&tmap, DIRECT ? a.E : a.E - E_PADL, a.pitch_e, a.H, Geo<NW, KT, true>::BW, KT);
+  const int rows = a.H + (FWD ? (int)(2 * a.pstride / a.pitch_e) : 0);   // the three planes in a row
+  const cudaError_t e = energy_tensor_map(&tmap, DIRECT ? a.E : a.E - E_PADL, a.pitch_e, rows, Geo<NW, KT, true>::BW, KT);
   if (e != cudaSuccess) return e;
-  return launch_dp_cluster(k_dp_two<NW, KT, DIRECT>, 2 * cs, cs, Geo<NW, KT, true>::THREADS, smem, st, a, tmap);
+  return launch_dp_cluster(k_dp_two<NW, KT, DIRECT, FWD>, 2 * cs, cs, Geo<NW, KT, true>::THREADS, smem, st, a, tmap);
 }
 
 template <bool DIRECT>
@@ -294,6 +300,7 @@ cudaError_t launch_dp(const DpArgs &a, cudaStream_t st) {
   if (a.pstride > 0) {
     const int cs = (a.W + Geo<4, 16, true>::OWC - 1) / Geo<4, 16, true>::OWC;
     if (cs > MAX_CLUSTER) return cudaErrorInvalidValue;
+    if (a.H >= TWO_MIN_ROWS) return launch_dp_two<4, 16, false, true>(a, cs, st);
     return launch_dp_shape<4, 16, true>(a, cs < 1 ? 1 : cs, st);
   }
   const DpShape s = dp_shape_for(a.W);

@@ -143,6 +143,9 @@ __global__ void k_forward(const uint32_t *__restrict__ img, int pitch, int H, in
   E[(int64_t)i * pe + j] = (uint16_t)cu;
   E[pstride + (int64_t)i * pe + j] = (uint16_t)dl;
   E[2 * pstride + (int64_t)i * pe + j] = (uint16_t)dr;
+  // the search from the bottom steps out of the row below the last one, which has no costs (where the planes
+  // have no such row, the next plane's row 0 holds zeros, or a tensor copy reads them)
+  if (i == H - 1 && (int64_t)H * pe < pstride) E[pstride + (int64_t)H * pe + j] = 0;
 }
 
 // ---- caller forward planes -> padded layout. DL in row 0 and column 0 and DR in row 0 and the
@@ -270,7 +273,67 @@ __global__ void k_refresh_wide(const uint32_t *__restrict__ img, int pitch, uint
   if (lane == 4 && s <= W - 2) er[s] = (uint16_t)e;
 }
 
-__global__ void k_refresh_fwd(const uint32_t *__restrict__ img, int pitch, uint16_t *__restrict__ E, int pe,
+// The same for the three forward-energy planes (plane p at E + p * pstride; R chunks per lane and plane): lanes
+// 0..2 fetch the pixels left and right of and above the new column s-1, lanes 4..6 those of column s.
+template <int R>
+__global__ void __launch_bounds__(128) k_refresh_fwd(const uint32_t *__restrict__ img, int pitch, uint16_t *E, int pe,
+                                                     int64_t pstride, int H, int W, const int32_t *__restrict__ seam,
+                                                     const int16_t *__restrict__ lists_in,
+                                                     int16_t *__restrict__ lists_out, int m, int *err) {
+  const int lane = threadIdx.x & 31;
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  pdl_launch_dependents();
+  if (i >= H) return;
+  uint16_t *const er = E + (int64_t)i * pe;
+  const int c_hi = (W - 2) >> 3;   // the chunk holding the new last column
+  uint4 x[3][R];
+#pragma unroll
+  for (int pl = 0; pl < 3; ++pl)
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int c = lane + 32 * r;
+      x[pl][r] = make_uint4(0u, 0u, 0u, 0u);
+      if (c <= c_hi + 1) x[pl][r] = __ldcg(reinterpret_cast<const uint4 *>(er + pl * pstride + 8 * c));
+    }
+  const int row = (lane & 2) ? max(i - 1, 0) : i;
+  const LazyRow list = lazy_row(lists_in + (int64_t)row * RPEND, m);
+  pdl_wait_prerequisites();   // the seam of the search that precedes this launch
+  const int s = __ldcg(seam + i);
+  const int sr = __ldcg(seam + row);
+  if (s < 0 || s >= W) {
+    if (lane == 0) atomicOr(err, ERR_BAD_SEAM);
+    return;
+  }
+  const int col = (lane & 4) ? s : s - 1;   // the new column this lane works for
+  const int j = clampi((lane & 2) ? col : ((lane & 1) ? col + 1 : col - 1), 0, W - 2);
+  const int xs = j + (j >= sr ? 1 : 0);     // column in the width-W image
+  const uint32_t px = img[(int64_t)row * pitch + xs + lazy_count(list, xs)];
+  if (lane == 0) list_insert(list, lists_out + (int64_t)i * RPEND, s);
+  if (s < W - 1) {
+    const int c_lo = s >> 3;
+#pragma unroll
+    for (int pl = 0; pl < 3; ++pl)
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const uint32_t first = (lane == 0 && r + 1 < R) ? x[pl][r + 1 < R ? r + 1 : r].x : x[pl][r].x;
+        const uint32_t nx = __shfl_sync(0xffffffffu, first, (lane + 1) & 31);
+        const int c = lane + 32 * r;
+        if (c >= c_lo && c <= c_hi)
+          *reinterpret_cast<uint4 *>(er + pl * pstride + 8 * c) = shift_chunk(x[pl][r], nx, s - 8 * c);
+      }
+  }
+  __syncwarp();   // the refreshed values go over the chunk holding s
+  const uint32_t pl = __shfl_sync(0xffffffffu, px, lane & 4), pr = __shfl_sync(0xffffffffu, px, (lane & 4) | 1),
+                 up = __shfl_sync(0xffffffffu, px, (lane & 4) | 2);
+  const bool left = col >= 1, right = col + 1 < W - 1;
+  const uint32_t cu = left && right ? sad4(pr, pl) : 0u, dl = i >= 1 && left ? sad4(up, pl) : 0u,
+                 dr = i >= 1 && right ? sad4(up, pr) : 0u;
+  const int plane = lane & 3;
+  if (lane < 8 && plane < 3 && col >= 0 && col <= W - 2)
+    er[plane * pstride + col] = (uint16_t)(plane == 0 ? cu : (plane == 1 ? dl : dr));
+}
+
+__global__ void k_refresh_fwd_wide(const uint32_t *__restrict__ img, int pitch, uint16_t *__restrict__ E, int pe,
                               int64_t pstride, int H, int W, const int32_t *__restrict__ seam,
                               const int16_t *__restrict__ lists_in, int16_t *__restrict__ lists_out, int m, int *err) {
   const int lane = threadIdx.x & 31;
@@ -393,10 +456,17 @@ cudaError_t launch_refresh(const uint32_t *img, int pitch, uint16_t *E, int pe, 
 cudaError_t launch_refresh_fwd(const uint32_t *img, int pitch, uint16_t *E, int pe, int64_t pstride, int H, int W,
                                const int32_t *seam, const int16_t *lists_in, int16_t *lists_out, int m, int *err,
                                cudaStream_t st) {
+  if (W <= 1024)
+    return launch_pdl(k_refresh_fwd<4>, (H + 3) / 4, 128, st, img, pitch, E, pe, pstride, H, W, seam, lists_in, lists_out,
+                      m, err);
+  if (W <= 2048)
+    return launch_pdl(k_refresh_fwd<8>, (H + 3) / 4, 128, st, img, pitch, E, pe, pstride, H, W, seam, lists_in, lists_out,
+                      m, err);
+  // three planes of wider rows do not fit the registers: everything after the wait
   const int warps_per_block = 8;
   int blocks = (H + warps_per_block - 1) / warps_per_block;
   if (blocks > 152 * 8) blocks = 152 * 8;
-  return launch_pdl(k_refresh_fwd, blocks, warps_per_block * 32, st, img, pitch, E, pe, pstride, H, W, seam, lists_in,
+  return launch_pdl(k_refresh_fwd_wide, blocks, warps_per_block * 32, st, img, pitch, E, pe, pstride, H, W, seam, lists_in,
                     lists_out, m, err);
 }
 

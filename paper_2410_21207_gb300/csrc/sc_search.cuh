@@ -41,7 +41,8 @@
 // With FWD (forward energy) the map has three planes, CU, DL and DR, and a cell's cost depends on
 // the direction it is reached from: M(i,j) = CU(i,j) + min(M(i-1,j-1) + DL(i,j), M(i-1,j),
 // M(i-1,j+1) + DR(i,j)). Optimal predecessors still never cross (a crossing pair would need
-// DL + DR < 0), so the ancestor keys keep their meaning; the planes are staged side by side.
+// DL + DR < 0), so the ancestor keys keep their meaning; the planes are staged side by side. Swept
+// upwards, a step costs the DL or DR of the row it leaves (dp_row_fwd_rev).
 #pragma once
 #include <cooperative_groups.h>
 #include <type_traits>
@@ -266,31 +267,57 @@ __device__ __forceinline__ void dp_row_fwd(uint32_t (&k)[V], uint2 cu, uint2 dl,
   k[0] = n0; k[1] = n1; k[2] = n2; k[3] = n3;
 }
 
+// The same for a sweep upwards: a path that leaves column j of the row below (previous row, keys k) costs that
+// row's DR towards column j + 1 and its DL towards column j - 1, so dl and dr are the previous row's and are
+// added before the neighbours take the sums.
+template <bool MASK>
+__device__ __forceinline__ void dp_row_fwd_rev(uint32_t (&k)[V], uint2 cu, uint2 dl, uint2 dr, const uint32_t (&oobm)[V]) {
+  uint32_t l[V] = {k[0] + lo8(dl.x), k[1] + hi8(dl.x), k[2] + lo8(dl.y), k[3] + hi8(dl.y)};   // towards j - 1
+  uint32_t g[V] = {k[0] + lo8(dr.x), k[1] + hi8(dr.x), k[2] + lo8(dr.y), k[3] + hi8(dr.y)};   // towards j + 1
+  if (MASK)
+#pragma unroll
+    for (int u = 0; u < V; ++u) {
+      l[u] |= oobm[u];   // (an excluded cell's key plus a padding value would wrap)
+      g[u] |= oobm[u];
+    }
+  const uint32_t L = __shfl_up_sync(0xffffffffu, g[V - 1], 1);
+  const uint32_t R = __shfl_down_sync(0xffffffffu, l[0], 1);
+  const uint32_t n0 = add_mask<MASK>(min3u(L, k[0], l[1]), lo8(cu.x), oobm[0]);
+  const uint32_t n1 = add_mask<MASK>(min3u(g[0], k[1], l[2]), hi8(cu.x), oobm[1]);
+  const uint32_t n2 = add_mask<MASK>(min3u(g[1], k[2], l[3]), lo8(cu.y), oobm[2]);
+  const uint32_t n3 = add_mask<MASK>(min3u(g[2], k[3], R), hi8(cu.y), oobm[3]);
+  k[0] = n0; k[1] = n1; k[2] = n2; k[3] = n3;
+}
+
 // KT forward-energy rows of a full tile (row stride BW); the three planes are PL elements apart in
 // the staging ring.
-template <int KT, int BW, int PL, bool MASK>
+template <int KT, int BW, int PL, bool MASK, bool REV>
 __device__ __forceinline__ void dp_rows_fwd(uint32_t (&k)[V], const uint16_t *er, const uint32_t (&oobm)[V]) {
-  uint2 a0 = *reinterpret_cast<const uint2 *>(er), a1 = *reinterpret_cast<const uint2 *>(er + PL),
-        a2 = *reinterpret_cast<const uint2 *>(er + 2 * PL);
+  constexpr int RS = REV ? -BW : BW;
+  auto row = [&](int pl, int r) { return *reinterpret_cast<const uint2 *>(er + pl * PL + r * RS); };
+  uint2 a0 = row(0, 0), a1 = row(1, 0), a2 = row(2, 0);
 #pragma unroll
   for (int r = 0; r < KT; ++r) {
     const uint2 c0 = a0, c1 = a1, c2 = a2;
     if (r + 1 < KT) {
-      a0 = *reinterpret_cast<const uint2 *>(er + (r + 1) * BW);
-      a1 = *reinterpret_cast<const uint2 *>(er + PL + (r + 1) * BW);
-      a2 = *reinterpret_cast<const uint2 *>(er + 2 * PL + (r + 1) * BW);
+      a0 = row(0, r + 1);
+      a1 = row(1, r + 1);
+      a2 = row(2, r + 1);
     }
-    dp_row_fwd<MASK>(k, c0, c1, c2, oobm);
+    if (REV) dp_row_fwd_rev<MASK>(k, c0, c1, c2, oobm);
+    else dp_row_fwd<MASK>(k, c0, c1, c2, oobm);
   }
 }
 
 // n (n < KT) forward-energy rows of a ragged last tile.
-template <int BW, int PL, bool MASK>
+template <int BW, int PL, bool MASK, bool REV>
 __device__ __forceinline__ void dp_rows_n_fwd(uint32_t (&k)[V], const uint16_t *er, const uint32_t (&oobm)[V], int n) {
-  for (int r = 0; r < n; ++r)
-    dp_row_fwd<MASK>(k, *reinterpret_cast<const uint2 *>(er + r * BW),
-                     *reinterpret_cast<const uint2 *>(er + PL + r * BW),
-                     *reinterpret_cast<const uint2 *>(er + 2 * PL + r * BW), oobm);
+  constexpr int RS = REV ? -BW : BW;
+  auto row = [&](int pl, int r) { return *reinterpret_cast<const uint2 *>(er + pl * PL + r * RS); };
+  for (int r = 0; r < n; ++r) {
+    if (REV) dp_row_fwd_rev<MASK>(k, row(0, r), row(1, r), row(2, r), oobm);
+    else dp_row_fwd<MASK>(k, row(0, r), row(1, r), row(2, r), oobm);
+  }
 }
 
 // Initialise the staging and halo mbarriers (thread 0; the caller then synchronises the CTA, and
@@ -364,7 +391,10 @@ __device__ __forceinline__ void fill_prefetch(const FillCtx &f, int s, int jprev
 }
 
 // super-tile s between columns jprev and jbs, by one warp
-template <typename G, bool FWD, int KSS, bool DIRECT>
+// Forward energy: a step costs the DL or DR of the lower (image) of its two rows. In a map swept downwards
+// the chain from above enters that row and adds its own DL and DR, the chain from below leaves it and
+// carries them to the neighbours; FLIP (a map swept upwards) exchanges the two.
+template <typename G, bool FWD, int KSS, bool DIRECT, bool FLIP = false>
 __device__ __forceinline__ void fill_super_tile(const FillCtx &f, int s, int jprev, int jbs, int warp, int lane) {
   constexpr int NP = FWD ? 3 : 1;   // cost planes per row
   constexpr int FV = G::FV, FILLW = G::FILLW, CR = G::fill_rows(FWD), HC = CR / 2;
@@ -379,7 +409,8 @@ __device__ __forceinline__ void fill_super_tile(const FillCtx &f, int s, int jpr
   // the upper nt rows and the lower nb; after the bottom row, which only holds the path's end, and the
   // top row where nt = nb, both chains have T more rows to run together
   const int nt = n >> 1, nb = n - nt, T = nb - 1, lead = nt - T;   // lead: 0 or 1
-  uint32_t m[FV], w[FV], wl[FV], wr[FV], oob[FV];   // costs from above, from below (FWD: plus DL, DR of their row)
+  // costs from above and from below (FWD: the carrying chain's plus DL, DR of their row; FLIP: the other one's)
+  uint32_t m[FV], w[FV], cl[FV], cr[FV], oob[FV];
 #pragma unroll
   for (int u = 0; u < FV; ++u) {
     oob[u] = (xc + u < 0 || xc + u >= f.W) ? FILL_INF : 0u;
@@ -402,6 +433,9 @@ __device__ __forceinline__ void fill_super_tile(const FillCtx &f, int s, int jpr
 #pragma unroll
     for (int u = 0; u < FV; ++u) {
       mn[u] = __viaddmin_u32(r[u], 2u, __viaddmin_u32(c[u], 1u, l[u]));
+    }
+#pragma unroll
+    for (int u = 0; u < FV; ++u) {
       out[u] = __viaddmax_u32(mn[u] & ~0xFFu, e[u], oob[u]);
     }
     uint32_t d = __byte_perm(mn[0], mn[1], 0x0040);
@@ -430,36 +464,45 @@ __device__ __forceinline__ void fill_super_tile(const FillCtx &f, int s, int jpr
   auto load_row = [&](int i, int pl) {
     return xin ? *reinterpret_cast<const EVec *>(f.E + pl * f.pstride + (ptrdiff_t)(rs + i) * f.pitch_e + xc) : EVec{};
   };
-  // the candidates of one chain from its costs: neighbours' values by shuffle; the chain from above
-  // adds the row's own DL and DR, the one from below carries those of the row it comes from
-  auto down_row = [&](const uint32_t (&e)[FV], const uint32_t (&dl)[FV], const uint32_t (&dr)[FV], uint8_t *dst) {
-    const uint32_t L = __shfl_up_sync(0xffffffffu, m[FV - 1], 1), R = __shfl_down_sync(0xffffffffu, m[0], 1);
-    uint32_t l[FV], c[FV], r[FV];
+  // the candidates of a chain from its costs x: neighbours' values by shuffle
+  auto entering = [&](const uint32_t (&x)[FV], const uint32_t (&dl)[FV], const uint32_t (&dr)[FV], uint32_t (&l)[FV],
+                      uint32_t (&r)[FV]) {
+    const uint32_t L = __shfl_up_sync(0xffffffffu, x[FV - 1], 1), R = __shfl_down_sync(0xffffffffu, x[0], 1);
 #pragma unroll
     for (int u = 0; u < FV; ++u) {
-      l[u] = (u == 0 ? L : m[u > 0 ? u - 1 : 0]) + (FWD ? dl[u] : 0u);
-      c[u] = m[u];
-      r[u] = (u == FV - 1 ? R : m[u < FV - 1 ? u + 1 : u]) + (FWD ? dr[u] : 0u);
+      l[u] = (u == 0 ? L : x[u > 0 ? u - 1 : 0]) + (FWD ? dl[u] : 0u);
+      r[u] = (u == FV - 1 ? R : x[u < FV - 1 ? u + 1 : u]) + (FWD ? dr[u] : 0u);
     }
-    step_row(l, c, r, e, m, dst);
   };
-  auto up_candidates = [&](uint32_t (&l)[FV], uint32_t (&c)[FV], uint32_t (&r)[FV]) {
-    const uint32_t L = __shfl_up_sync(0xffffffffu, FWD ? wr[FV - 1] : w[FV - 1], 1);
-    const uint32_t R = __shfl_down_sync(0xffffffffu, FWD ? wl[0] : w[0], 1);
+  auto leaving = [&](uint32_t (&l)[FV], uint32_t (&r)[FV]) {
+    const uint32_t L = __shfl_up_sync(0xffffffffu, cr[FV - 1], 1), R = __shfl_down_sync(0xffffffffu, cl[0], 1);
 #pragma unroll
     for (int u = 0; u < FV; ++u) {
-      l[u] = u == 0 ? L : (FWD ? wr[u > 0 ? u - 1 : 0] : w[u > 0 ? u - 1 : 0]);
-      c[u] = w[u];
-      r[u] = u == FV - 1 ? R : (FWD ? wl[u < FV - 1 ? u + 1 : u] : w[u < FV - 1 ? u + 1 : u]);
+      l[u] = u == 0 ? L : cr[u > 0 ? u - 1 : 0];
+      r[u] = u == FV - 1 ? R : cl[u < FV - 1 ? u + 1 : u];
     }
   };
-  auto carry = [&](const uint32_t (&dl)[FV], const uint32_t (&dr)[FV]) {
+  auto carry = [&](const uint32_t (&x)[FV], const uint32_t (&dl)[FV], const uint32_t (&dr)[FV]) {
     if (FWD)
 #pragma unroll
       for (int u = 0; u < FV; ++u) {
-        wl[u] = w[u] + dl[u];
-        wr[u] = w[u] + dr[u];
+        cl[u] = x[u] + dl[u];
+        cr[u] = x[u] + dr[u];
       }
+  };
+  auto down_row = [&](const uint32_t (&e)[FV], const uint32_t (&dl)[FV], const uint32_t (&dr)[FV], uint8_t *dst) {
+    uint32_t l[FV], r[FV];
+    if (FWD && FLIP) leaving(l, r);
+    else entering(m, dl, dr, l, r);
+    step_row(l, m, r, e, m, dst);
+    if (FLIP) carry(m, dl, dr);
+  };
+  auto up_row = [&](const uint32_t (&e)[FV], const uint32_t (&dl)[FV], const uint32_t (&dr)[FV], uint8_t *dst) {
+    uint32_t l[FV], r[FV];
+    if (FWD && !FLIP) leaving(l, r);
+    else entering(w, dl, dr, l, r);
+    step_row(l, w, r, e, w, dst);
+    if (!FLIP) carry(w, dl, dr);
   };
   EVec et0[NP], eb0[NP];   // the bottom row and the leading top row
 #pragma unroll
@@ -477,7 +520,16 @@ __device__ __forceinline__ void fill_super_tile(const FillCtx &f, int s, int jpr
     }
 #pragma unroll
     for (int u = 0; u < FV; ++u) w[u] = (xc + u == jbs) ? e[u] : FILL_INF;
-    carry(dl, dr);
+    if (!FLIP) carry(w, dl, dr);
+    if (FWD && FLIP) {
+      // the chain from above leaves row rs - 1 (the added row, without costs, for s = 0)
+      uint32_t pl[FV] = {}, pr[FV] = {};
+      if (rs > 0) {
+        unpack(load_row(-1, NP > 1 ? 1 : 0), pl);
+        unpack(load_row(-1, NP > 2 ? 2 : 0), pr);
+      }
+      carry(m, pl, pr);
+    }
     *reinterpret_cast<DirT *>(fd + (n - 1) * FILLW + lane * FV) = (DirT)0x01010101u;   // no step below it
     if (lead) {
       unpack(et0[0], e);
@@ -501,7 +553,7 @@ __device__ __forceinline__ void fill_super_tile(const FillCtx &f, int s, int jpr
     uint8_t *ft = fd + (lead + q0) * FILLW + lane * FV, *fb = fd + (n - 2 - q0) * FILLW + lane * FV;
 #pragma unroll 1
     for (int r = 0; r < nq; ++r, ft += FILLW, fb -= FILLW, es += 32) {
-      uint32_t e[FV], g[FV], dl[FV] = {}, dr[FV] = {}, gl[FV] = {}, gr[FV] = {}, l[FV], c[FV], rr[FV];
+      uint32_t e[FV], g[FV], dl[FV] = {}, dr[FV] = {}, gl[FV] = {}, gr[FV] = {};
       unpack(es[0], e);
       unpack(es[HC * 32], g);
       if (FWD) {
@@ -510,24 +562,29 @@ __device__ __forceinline__ void fill_super_tile(const FillCtx &f, int s, int jpr
         unpack(es[(CR + HC) * 32], gl);
         unpack(es[(2 * CR + HC) * 32], gr);
       }
-      up_candidates(l, c, rr);
+      up_row(g, gl, gr, fb);
       down_row(e, dl, dr, ft);
-      step_row(l, c, rr, g, w, fb);
-      carry(gl, gr);
     }
   }
   // the join: the leftmost column of row nt - 1 (jprev itself when nt = 0) on a cheapest path, and the
   // leftmost of its three successors
   uint32_t best = SENT, where = SENT;   // cost * 256; column in the window << 2 | direction
   {
-    uint32_t l[FV], c[FV], r[FV];
-    up_candidates(l, c, r);
+    // the cost up to column j and on to j - 1, j, j + 1 of the next row
+    uint32_t l[FV], r[FV];
+    const uint32_t zero[FV] = {};
+    if (FWD && !FLIP) leaving(l, r);
+    else entering(w, zero, zero, l, r);
 #pragma unroll
     for (int u = 0; u < FV; ++u) {
-      const uint32_t mn = __viaddmin_u32(r[u], 2u, __viaddmin_u32(c[u], 1u, l[u]));
-      const uint32_t sum = m[u] >= FILL_INF || mn >= FILL_INF ? SENT : m[u] + (mn & ~0xFFu);
-      if (sum < best) {
-        best = sum;
+      const uint32_t a = (FWD && FLIP ? cl[u] : m[u]), c = (FWD && FLIP ? cr[u] : m[u]);
+      // (a sum with an excluded term stays above FILL_INF, or wraps when both are: tested first)
+      const uint32_t sl = m[u] >= FILL_INF || l[u] >= FILL_INF ? SENT - 2u : a + l[u];
+      const uint32_t sc = m[u] >= FILL_INF || w[u] >= FILL_INF ? SENT - 2u : m[u] + w[u];
+      const uint32_t sr = m[u] >= FILL_INF || r[u] >= FILL_INF ? SENT - 2u : c + r[u];
+      const uint32_t mn = __viaddmin_u32(sr, 2u, __viaddmin_u32(sc, 1u, sl));
+      if (mn < SENT - 2u && (mn & ~0xFFu) < best) {
+        best = mn & ~0xFFu;
         where = ((uint32_t)(lane * FV + u) << 2) | (mn & 3u);
       }
     }
@@ -674,7 +731,7 @@ __device__ __forceinline__ unsigned long long seam_sweep(const SearchArgs &p, un
 #pragma unroll (CL ? NBOX : 1)
             for (int b = 0; b < nbox; ++b)
               tensor_g2s_2d(ring + (size_t)(slot * NP + pl) * SLOT + b * KT * BWB, p.tmap, p.x0 + cbeg + b * BWB,
-                            y + pl * p.plane_rows, &full[slot]);
+                            y + pl * p.plane_rows + (REV && pl > 0 ? 1 : 0), &full[slot]);   // (REV: DL, DR of the row below)
         }
         return;
       }
@@ -771,8 +828,8 @@ __device__ __forceinline__ unsigned long long seam_sweep(const SearchArgs &p, un
           if (EDGE) { k[0] |= oobm[0]; k[1] |= oobm[1]; k[2] |= oobm[2]; k[3] |= oobm[3]; }
         }
         if (FWD) {
-          if (n == KT) dp_rows_fwd<KT, BWB, SLOT, EDGE>(k, er, oobm);
-          else dp_rows_n_fwd<BWB, SLOT, EDGE>(k, er, oobm, n);
+          if (n == KT) dp_rows_fwd<KT, BWB, SLOT, EDGE, REV>(k, er, oobm);
+          else dp_rows_n_fwd<BWB, SLOT, EDGE, REV>(k, er, oobm, n);
         } else {
           dp_rows<(CL && FWM >= FILL_WARPS_MAX ? KT : 8), BWB, EDGE, LAT, DIRECT, REV>(k, er, oobm, n, emax, cm);
         }

@@ -31,7 +31,7 @@ struct TwoPlan {
   size_t tbar;       // mbarrier of the tables' copy
   size_t tab_cap;
 };
-template <typename G, int NW, int KT, int KSS>
+template <typename G, int NW, int KT, int KSS, bool FWD = false>
 __host__ __device__ inline TwoPlan two_plan(int S, int ctas, size_t want_tab, size_t limit) {
   TwoPlan t;
   SearchPlan &p = t.plan;
@@ -41,14 +41,15 @@ __host__ __device__ inline TwoPlan two_plan(int S, int ctas, size_t want_tab, si
   p.hbuf = take((size_t)2 * 2 * K2 * 4);
   p.cmin = take((size_t)(NW + 1 + (S + ctas - 1) / ctas) * 8);
   p.jb = take((size_t)(S + 2) * 4);
-  p.misc = take(16);   // [0] this CTA arrived last (two clusters), [1] go on with the ends in cmin, [2] cost sum
+  p.misc = take(16);   // [0] this CTA arrived last (two clusters), [1] go on with the ends in cmin, [2] cost sum,
+                       // [3] forward energy: the cost of the step between the halves
   p.wmin = p.anc = p.emx = p.gat = 0;
   p.gw = 0;
   p.bars = take((size_t)(NSLOT + 3) * 8);
   t.tbar = p.bars + (size_t)(NSLOT + 2) * 8;
   o = (o + 127) & ~(size_t)127;   // (tensor copies: 128-byte aligned)
-  size_t r = (size_t)NSLOT * KT * tensor_boxes(G::BW) * tensor_box_cols(G::BW) * 2;
-  const size_t fb = (size_t)G::FW * G::fill_bytes(false);
+  size_t r = (size_t)NSLOT * (FWD ? 3 : 1) * KT * tensor_boxes(G::BW) * tensor_box_cols(G::BW) * 2;
+  const size_t fb = (size_t)G::FW * G::fill_bytes(FWD);
   r = r > fb ? r : fb;
   if (want_tab > r && o < limit) {
     const size_t room = (limit - o) & ~(size_t)127;
@@ -66,6 +67,7 @@ __host__ __device__ inline TwoPlan two_plan(int S, int ctas, size_t want_tab, si
 struct TwoScratch {
   uint32_t *end0, *end1;
   uint8_t *tab;
+  const uint16_t *dl = nullptr, *dr = nullptr;   // forward energy: DL and DR of the lower half's first row
   __device__ TwoScratch(uint32_t *scratch, int gw)
       : end0(scratch), end1(scratch + gw), tab(reinterpret_cast<uint8_t *>(scratch + 2 * gw)) {}
 };
@@ -75,7 +77,7 @@ struct TwoScratch {
 // cluster rank 0 on the ends (column above, column at the bottom) of super-tiles r, r + ctas, ... (the
 // upper half's first) in its cmin, and in its misc[1] whether to go on. tphase: parity of this use of the
 // tables' barrier. Returns to thread 0 the seam's cost (SENT after a recorded failure).
-template <int NW>
+template <int NW, bool FWD = false>
 __device__ __forceinline__ uint32_t two_join(const TwoSplit &g, const TwoScratch &x, int gw, int W, unsigned char *smem,
                                              const TwoPlan &t, uint32_t tphase, int ctas, int *err) {
   cg::cluster_group cl = cg::this_cluster();
@@ -114,11 +116,15 @@ __device__ __forceinline__ uint32_t two_join(const TwoSplit &g, const TwoScratch
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
       const int j = j0 + c;
-      const uint32_t right = j + 1 < W ? uv[c + 2] : SENT;
-      const uint32_t m = min3u(uv[c], uv[c + 1], right), sum = dv[c] + m;
+      uint32_t left = uv[c], right = j + 1 < W ? uv[c + 2] : SENT;
+      if (FWD && g.H1 > 0) {   // stepping to column j - 1 costs that cell's DR, to column j + 1 its DL
+        if (j > 0) left += (uint32_t)__ldcg(x.dr + j - 1);
+        if (j + 1 < W) right += (uint32_t)__ldcg(x.dl + j + 1);
+      }
+      const uint32_t m = min3u(left, uv[c + 1], right), sum = dv[c] + m;
       if (j < W && sum < best) {   // columns come in ascending order: ties keep the left one
         best = sum;
-        where = ((uint32_t)j << 2) | (m == uv[c] ? 0u : (m == uv[c + 1] ? 1u : 2u));
+        where = ((uint32_t)j << 2) | (m == left ? 0u : (m == uv[c + 1] ? 1u : 2u));
       }
     }
   }
@@ -152,7 +158,14 @@ __device__ __forceinline__ uint32_t two_join(const TwoSplit &g, const TwoScratch
     if (bad) atomicOr(err, ERR_BAD_SEAM);
   }
   bad = __any_sync(0xffffffffu, bad);
-  if (lane == 0) misc[2] = 0;
+  if (lane == 0) {
+    misc[2] = 0;
+    if (FWD) {
+      // the step between the halves belongs to no super-tile
+      const int j = (int)(where >> 2), d = (int)(where & 3u);
+      misc[3] = (bad || g.H1 == 0 || d == 1) ? 0 : (int)__ldcg(d == 0 ? x.dr + j - 1 : x.dl + j + 1);
+    }
+  }
   __syncwarp();
   for (int r = lane; r < ctas; r += 32) {
     int2 *dst = reinterpret_cast<int2 *>(cl.map_shared_rank(smem + t.plan.cmin, r));
@@ -168,7 +181,7 @@ __device__ __forceinline__ uint32_t two_join(const TwoSplit &g, const TwoScratch
 
 // The calling CTA's share of the super-tiles of both halves of an H-row map (rank r of `ctas`), from the
 // ends two_join left in its cmin.
-template <typename G, int KSS, bool DIRECT = false>
+template <typename G, int KSS, bool DIRECT = false, bool FWD = false>
 __device__ __forceinline__ void two_fill(const TwoSplit &g, FillCtx f, int H, const TwoPlan &t, unsigned char *smem,
                                          int ctas, int rank) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -188,7 +201,8 @@ __device__ __forceinline__ void two_fill(const TwoSplit &g, FillCtx f, int H, co
     const bool low = q >= g.S0;
     FillCtx c = low ? dn : up;
     c.H = low ? g.H1 : g.H0;
-    fill_super_tile<G, false, KSS, DIRECT>(c, low ? q - g.S0 : q, ends[k].x, ends[k].y, warp, lane);
+    if (FWD && low) fill_super_tile<G, FWD, KSS, DIRECT, true>(c, q - g.S0, ends[k].x, ends[k].y, warp, lane);
+    else fill_super_tile<G, FWD, KSS, DIRECT>(c, low ? q - g.S0 : q, ends[k].x, ends[k].y, warp, lane);
   }
 }
 

@@ -92,3 +92,41 @@ def test_maps_in_place_at_the_range_limit(H, W, emax):
             sc.check()
             assert int(c.cpu()[0]) == cost
             np.testing.assert_array_equal(seam.cpu().numpy(), ref)
+
+
+# forward energy from both ends: 256 columns a CTA, 16-row tiles, 32-row super-tiles; planes of one row count
+# only (the lower half's first step reads the row below the last one)
+@pytest.mark.gpu
+@pytest.mark.parametrize("H,W", [(191, 40), (192, 1), (193, 2), (207, 255), (223, 256), (225, 257), (255, 2049),
+                                 (320, 4096), (1079, 515)])
+def test_forward_from_both_ends(H, W):
+    from paper_2410_21207_gb300 import binding as sc
+    rng = np.random.default_rng(H * 4099 + W)
+    for kind, hi in (("image", 256), ("ties", 2), ("planes", 0)):
+        if hi:
+            planes = oracle.forward_costs(rng.integers(0, hi, size=(H, W, 3)).astype(np.uint8))
+        else:   # any values, entries without a predecessor included
+            planes = tuple(rng.integers(0, 4000, size=(H, W)).astype(np.uint16) for _ in range(3))
+        ref, cost = oracle.dp_seam_forward(*planes)
+        seam, c = sc.find_seam_forward(*[torch.from_numpy(p).cuda() for p in planes])
+        sc.check()
+        assert int(c.cpu()[0]) == cost, kind
+        np.testing.assert_array_equal(seam.cpu().numpy(), ref, err_msg=f"{H}x{W} {kind}")
+
+
+# both passes; wider than tall, square and taller than wide (rows below the planes' last one exist or not), and
+# rows wider than the refresh keeps in registers
+@pytest.mark.gpu
+@pytest.mark.parametrize("H,W,tw,th", [(200, 260, 240, 194), (230, 230, 210, 215), (300, 210, 200, 280),
+                                       (193, 2070, 2040, 193)])
+def test_forward_carve_from_both_ends(H, W, tw, th):
+    from paper_2410_21207_gb300 import binding as sc
+    rng = np.random.default_rng(H + W)
+    for hi in (256, 2):
+        img = rng.integers(0, hi, size=(H, W, 3)).astype(np.uint8)
+        out, log, cost = sc.carve_forward(torch.from_numpy(img).cuda(), tw, th, with_log=True)
+        sc.check()
+        r_out, r_log, r_cost = oracle.carve_forward(img, tw, th, with_log=True)
+        np.testing.assert_array_equal(log.cpu().numpy(), r_log)
+        np.testing.assert_array_equal(cost.cpu().numpy(), r_cost)
+        np.testing.assert_array_equal(out.cpu().numpy(), r_out)
