@@ -30,16 +30,15 @@ __device__ __forceinline__ uint4 shift_chunk(const uint4 &x, uint32_t nx, int ke
   o.y = __funnelshift_r(x.y, x.z, 16);
   o.z = __funnelshift_r(x.z, x.w, 16);
   o.w = __funnelshift_r(x.w, nx, 16);
-  if (keep > 0) {
-    auto merge = [keep](uint32_t in, uint32_t sh, int q) {
-      const uint32_t m = (2 * q < keep ? 0x0000FFFFu : 0u) | (2 * q + 1 < keep ? 0xFFFF0000u : 0u);
-      return (in & m) | (sh & ~m);
-    };
-    o.x = merge(x.x, o.x, 0);
-    o.y = merge(x.y, o.y, 1);
-    o.z = merge(x.z, o.z, 2);
-    o.w = merge(x.w, o.w, 3);
-  }
+  // (branch-free: a warp whose lane 0 took a branch here would wait for it on every row)
+  auto merge = [keep](uint32_t in, uint32_t sh, int q) {
+    const uint32_t m = keep > 2 * q + 1 ? 0xFFFFFFFFu : (keep > 2 * q ? 0x0000FFFFu : 0u);
+    return (in & m) | (sh & ~m);
+  };
+  o.x = merge(x.x, o.x, 0);
+  o.y = merge(x.y, o.y, 1);
+  o.z = merge(x.z, o.z, 2);
+  o.w = merge(x.w, o.w, 3);
   return o;
 }
 
@@ -296,10 +295,13 @@ __device__ __forceinline__ uint32_t refresh_energy(uint32_t px) {
 // the chunk holding s) of each row, takes the element after each chunk from the next lane, and writes the
 // chunk one element to the left; longer tails go on block by block from the left, each read before it
 // is written. Rows whose seam is out of range are skipped (the caller records the error).
-// Latency-bound (four warps per SM sub-partition): all the rows' loads are in flight at once and nothing goes
-// through shared memory. Against tails staged there by bulk copies and written back chunk by chunk, per seam
-// of one image: 400x900 96.2 -> 93.4 us, 1254x944 176.1 -> 174.1 us, 2500x1332 on its cluster 223.6 -> 217.0.
-// Not inlined (nor is compact_rows): a separate function gets its own register allocation, and inlined
+// Bound by the latency of its instruction stream: no branch depends on a row's tail length (a branch and
+// its reconvergence per load and store cost as much as the loads: 1254x944 173.2 -> 170.9 us a seam,
+// 2500x1332 98.2 -> 94.5 on its cluster), and nothing goes through shared memory. Against tails staged there
+// by bulk copies and written back chunk by chunk, per seam of one image: 400x900 96.2 -> 90.8 us, 1254x944
+// 176.1 -> 170.9 us, 2500x1332 on a cluster of 8-row tiles 223.6 -> 207.9. Slower: two rows of 6 chunks per
+// lane, eight rows of one, four of four.
+// Not inlined (nor is compact_rows_staged): a separate function gets its own register allocation, and inlined
 // the two phases cost the one-CTA batched kernel ~160 bytes of spills.
 static __device__ __noinline__ void shift_rows(uint16_t *E, int pe, int nq, int row0, int rstride, int w,
                                                const int32_t *seam, const uint32_t *pairs, int warp, int nwarps,
@@ -318,44 +320,38 @@ static __device__ __noinline__ void shift_rows(uint16_t *E, int pe, int nq, int 
 #pragma unroll 1
     for (int t = 0; t < n; t += NR, e0 += NR * rowstep) {
       int s[NR], cb[NR];
+      uint16_t *er[NR];
       bool any = false;
 #pragma unroll
       for (int v = 0; v < NR; ++v) {
         s[v] = __shfl_sync(0xffffffffu, sl, t + v);   // (t + v <= 31: t is a multiple of NR)
+        er[v] = e0 + (t + v < n ? v : 0) * rowstep;
         // past the last row, a seam out of range, or one in the last column: nothing to shift
         cb[v] = (t + v >= n || s[v] < 0 || s[v] >= w - 1) ? c_last + 1 : s[v] >> 3;
         any |= cb[v] <= c_last;
       }
       while (any) {
+        // no branches: lanes past the tail load its last chunk again, and only the stores are predicated
         uint4 x[NR][R];
         uint32_t after[NR];
 #pragma unroll
         for (int v = 0; v < NR; ++v) {
-          const uint16_t *er = e0 + v * rowstep;
-          after[v] = 0u;
 #pragma unroll
-          for (int r = 0; r < R; ++r) {
-            const int c = cb[v] + 32 * r;
-            x[v][r] = make_uint4(0u, 0u, 0u, 0u);
-            if (cb[v] <= c_last && c <= c_last + 1) {   // (the same for every lane)
-              if (c + lane <= c_last + 1) x[v][r] = __ldcg(reinterpret_cast<const uint4 *>(er + 8 * (c + lane)));
-            }
-          }
+          for (int r = 0; r < R; ++r)
+            x[v][r] = __ldcg(reinterpret_cast<const uint4 *>(er[v] + 8 * min(cb[v] + 32 * r + lane, c_last + 1)));
           // the element after the block's last chunk
-          if (cb[v] + 32 * R <= c_last + 1) after[v] = __ldcg(er + 8 * (cb[v] + 32 * R));
+          after[v] = __ldcg(er[v] + 8 * min(cb[v] + 32 * R, c_last + 1));
         }
         any = false;
 #pragma unroll
         for (int v = 0; v < NR; ++v) {
-          uint16_t *er = e0 + v * rowstep;
 #pragma unroll
           for (int r = 0; r < R; ++r) {
-            const int c = cb[v] + 32 * r;
-            if (c > c_last) continue;   // (the same for every lane)
             const uint32_t first = lane > 0 ? x[v][r].x : (r + 1 < R ? x[v][r + 1 < R ? r + 1 : r].x : after[v]);
             const uint32_t nx = __shfl_sync(0xffffffffu, first, (lane + 1) & 31);
-            const uint4 o = shift_chunk(x[v][r], nx, r == 0 ? s[v] - 8 * (c + lane) : 0);
-            if (c + lane <= c_last) *reinterpret_cast<uint4 *>(er + 8 * (c + lane)) = o;
+            const int c = cb[v] + 32 * r + lane;
+            const uint4 o = shift_chunk(x[v][r], nx, r == 0 ? s[v] - 8 * c : 0);
+            if (c <= c_last) *reinterpret_cast<uint4 *>(er[v] + 8 * c) = o;
           }
           cb[v] += 32 * R;
           any |= cb[v] <= c_last;
