@@ -799,77 +799,86 @@ __device__ __forceinline__ unsigned long long seam_sweep(const SearchArgs &p, un
       if (nt > 0 && !mbar_wait_bounded(&full[st.tiles % NSLOT], (st.tiles / NSLOT) & 1u, WAIT_TIMEOUT_NS)) {
         if (lane == 0) atomicOr(p.err, ERR_TIMEOUT);
       }
+      // few branches: a branch and its reconvergence cost about as much as a row in these short chains, so
+      // the conditions are uniform ones, lanes are told apart by predicated stores, and the window of the
+      // next tile is loaded behind the barrier of this one (per seam: 1920x1080 26.1 -> 24.3 us, 3840x2160
+      // 61.1 -> 57.2, forward energy at 1920x1080 48.3 -> 41.5, 1254x944 on one CTA 170.9 -> 165.6; 58 concurrent
+      // 3840x2160 maps 258 -> 242 us; fixed row counts before that: 26.4 -> 26.1, 62.3 -> 61.1, 264 -> 258)
       for (int t = 0; t < nt; ++t) {
         const int r0 = t * KT;
         const int n = (H - r0 < KT) ? H - r0 : KT;
-        const bool more = t + 1 < nt;
-        const uint32_t g = st.tiles + t;
-        const uint16_t *er = ring + (size_t)(g % NSLOT) * NP * SLOT + er0;
-        if (t > 0) {
-          // window of the previous row from the boundary buffer, or from the halo buffer for a
-          // neighbour's columns after an exchange (relative ancestors -> warp frame). At a new
-          // super-tile every cell becomes its own ancestor; the old ancestor field is dropped
-          // without arithmetic (it may lie outside this warp's frame).
-          const uint32_t *src = bnd + ((t - 1) & 1) * BW + bidx0;
-          if (CL && hneed && cs > 1 && (r0 % K2) == 0) {
-            const uint32_t xg = st.exch + (uint32_t)(r0 / K2 - 1);
-            if (!mbar_wait_bounded(&hbar[xg & 1], (xg >> 1) & 1u, WAIT_TIMEOUT_NS)) {
-              if (lane == 0) atomicOr(p.err, ERR_TIMEOUT);
-            }
-            if (hoff >= 0) src = hbuf + (int)(xg & 1) * 2 * K2 + hoff;
-          }
-          const uint4 v = *reinterpret_cast<const uint4 *>(src);
-          const bool fresh = FRESH || (r0 % KSS) == 0;
-          const uint32_t d = own_a - 128u;
-          k[0] = fresh ? ((v.x & ~0xFFu) | own_a) : (v.x + d);
-          k[1] = fresh ? ((v.y & ~0xFFu) | (own_a + 1u)) : (v.y + d + 1u);
-          k[2] = fresh ? ((v.z & ~0xFFu) | (own_a + 2u)) : (v.z + d + 2u);
-          k[3] = fresh ? ((v.w & ~0xFFu) | (own_a + 3u)) : (v.w + d + 3u);
-          if (EDGE) { k[0] |= oobm[0]; k[1] |= oobm[1]; k[2] |= oobm[2]; k[3] |= oobm[3]; }
-        }
+        const uint16_t *er = ring + (size_t)((st.tiles + t) % NSLOT) * NP * SLOT + er0;
         if (FWD) {
           if (n == KT) dp_rows_fwd<KT, BWB, SLOT, EDGE, REV>(k, er, oobm);
           else dp_rows_n_fwd<BWB, SLOT, EDGE, REV>(k, er, oobm, n);
         } else {
-          dp_rows<(CL && FWM >= FILL_WARPS_MAX ? KT : 8), BWB, EDGE, LAT, DIRECT, REV>(k, er, oobm, n, emax, cm);
+          constexpr int U = CL && FWM >= FILL_WARPS_MAX ? KT : 8;
+          if (n == KT) dp_rows<U, BWB, EDGE, LAT, DIRECT, REV>(k, er, oobm, KT, emax, cm);   // (a fixed count)
+          else dp_rows<8, BWB, EDGE, LAT, DIRECT, REV>(k, er, oobm, n, emax, cm);
         }
+        const bool more = t + 1 < nt;
         // bookkeeping on the tile's last row, the only one where a super-tile (KSS is a multiple
         // of KT) or the image can end: the ancestors of the CTA-own columns (in rank 0's gathered
         // table, the global one or this CTA's), and below the last row its costs
-        if (cta_own && (FRESH || ((r0 + n) % KSS) == 0 || !more)) {
+        if (FRESH || ((r0 + n) % KSS) == 0 || !more) {
           const uint32_t anc = pack_ancestors(k, c0, frame_base);
-          const size_t sup = (size_t)((r0 + n - 1) / KSS);
           if (TWO) {
-            *reinterpret_cast<uint32_t *>(anc_out) = anc;
+            if (cta_own) *reinterpret_cast<uint32_t *>(anc_out) = anc;
             anc_out += gw;
-            if (!more) *reinterpret_cast<uint4 *>(p.endrow + c0) = make_uint4(k[0] >> 8, k[1] >> 8, k[2] >> 8, k[3] >> 8);
           } else {
-            *reinterpret_cast<uint32_t *>(gw ? gat0 + sup * gw + c0 : ancT + sup * OWC + (c0 - A)) = anc;
+            const size_t sup = (size_t)((r0 + n - 1) / KSS);
+            uint8_t *const dst = gw ? gat0 + sup * gw + c0 : ancT + sup * OWC + (c0 - A);
+            if (cta_own) *reinterpret_cast<uint32_t *>(dst) = anc;
+          }
+        }
+        if (!more) {
+          if (TWO) {
+            if (cta_own)
+              *reinterpret_cast<uint4 *>(p.endrow + c0) = make_uint4(k[0] >> 8, k[1] >> 8, k[2] >> 8, k[3] >> 8);
+          } else if (cta_own) {
 #pragma unroll
             for (int u = 0; u < V; ++u) {
-              if (!more && c0 + u < W) {
+              if (c0 + u < W) {
                 const unsigned long long c = ((unsigned long long)(k[u] >> 8) << 32) | (unsigned)(c0 + u);
                 lastmin = c < lastmin ? c : lastmin;
               }
             }
           }
+          break;
         }
-        if (more) {
-          const bool exch = CL && ((r0 + KT) % K2 == 0) && cs > 1;
-          // publish this warp's strip (relative ancestor encoding)
-          const uint32_t d = FRESH ? 0u : own_a - 128u, du = FRESH ? 0u : 1u;
-          uint4 v;
-          v.x = k[0] - d; v.y = k[1] - d - du; v.z = k[2] - d - 2 * du; v.w = k[3] - d - 3 * du;
-          if constexpr (CL) if (exch) {
-            // read there at the start of the next tile
-            const uint32_t par = (st.exch + (uint32_t)((r0 + KT) / K2 - 1)) & 1u;
-            if (push) st_async_v4(push + par * (2 * K2 * 4), v, push_bar + par * 8);
-            if (threadIdx.x == 0)
-              mbar_arrive_expect_tx(&hbar[par], (uint32_t)(((rank > 0) + (rank < cs - 1)) * K2 * 4));
+        // publish this warp's strip (relative ancestor encoding)
+        const uint32_t d = own_a - 128u, dp = FRESH ? 0u : d, du = FRESH ? 0u : 1u;
+        uint4 v;
+        v.x = k[0] - dp; v.y = k[1] - dp - du; v.z = k[2] - dp - 2 * du; v.w = k[3] - dp - 3 * du;
+        const bool exch = CL && ((r0 + KT) % K2 == 0) && cs > 1;
+        const uint32_t xg = st.exch + (uint32_t)((r0 + KT) / K2 - 1);
+        if constexpr (CL) if (exch) {
+          // read there at the start of the next tile
+          if (push) st_async_v4(push + (xg & 1u) * (2 * K2 * 4), v, push_bar + (xg & 1u) * 8);
+          if (threadIdx.x == 0)
+            mbar_arrive_expect_tx(&hbar[xg & 1u], (uint32_t)(((rank > 0) + (rank < cs - 1)) * K2 * 4));
+        }
+        uint32_t *const bt = bnd + (t & 1) * BW + bidx0;
+        if (strip_lane) *reinterpret_cast<uint4 *>(bt) = v;
+        named_bar_sync(G::THREADS);
+        // the next tile's window from the boundary buffer, or from the halo buffer for a neighbour's columns
+        // after an exchange (relative ancestors -> warp frame). At a new super-tile every cell becomes its
+        // own ancestor; the old ancestor field is dropped without arithmetic (it may lie outside this
+        // warp's frame).
+        const uint32_t *src = bt;
+        if (CL && hneed && exch) {
+          if (!mbar_wait_bounded(&hbar[xg & 1u], (xg >> 1) & 1u, WAIT_TIMEOUT_NS)) {
+            if (lane == 0) atomicOr(p.err, ERR_TIMEOUT);
           }
-          if (strip_lane) *reinterpret_cast<uint4 *>(bnd + (t & 1) * BW + bidx0) = v;
-          named_bar_sync(G::THREADS);
+          if (hoff >= 0) src = hbuf + (int)(xg & 1u) * 2 * K2 + hoff;
         }
+        const uint4 y = *reinterpret_cast<const uint4 *>(src);
+        const bool fresh = FRESH || ((r0 + KT) % KSS) == 0;
+        k[0] = fresh ? ((y.x & ~0xFFu) | own_a) : (y.x + d);
+        k[1] = fresh ? ((y.y & ~0xFFu) | (own_a + 1u)) : (y.y + d + 1u);
+        k[2] = fresh ? ((y.z & ~0xFFu) | (own_a + 2u)) : (y.z + d + 2u);
+        k[3] = fresh ? ((y.w & ~0xFFu) | (own_a + 3u)) : (y.w + d + 3u);
+        if (EDGE) { k[0] |= oobm[0]; k[1] |= oobm[1]; k[2] |= oobm[2]; k[3] |= oobm[3]; }
       }
     };
     if (edge) tiles(std::integral_constant<bool, true>());
