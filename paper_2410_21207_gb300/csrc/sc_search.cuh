@@ -356,10 +356,11 @@ __device__ __forceinline__ void group_sync() {
 // Energies are read in chunks of fill_rows() rows, half of them from either end, every load of a chunk
 // in flight at once, and held in shared memory, so that the row loop stays a loop: the code runs
 // once per search and warp, from a cold instruction cache, where unrolled rows cost more to fetch
-// than to execute.
-// Latency-bound: loads ~1,100 cycles, rows and walk of half a super-tile each. Steps (1920x1080 carve):
-// full costs recomputed in a 4*KSS window from saved cost rows 25.0 ms, between the two ends 24.5 ms (a
-// batch of 256 images 44.5 -> 40.7 ms).
+// than to execute (three rows at a time are the best of 1, 3 and 5: 3840x2160 57.2 / 55.8 / 56.1 us a seam).
+// Latency-bound: the energies' round trip, then rows and walk of half a super-tile each (about 500, 1,900 and
+// 1,300 cycles). Against full costs recomputed in a 4*KSS window from saved cost rows (25.0 ms a 1920x1080
+// carve): between the two ends 24.5 ms (a batch of 256 images 44.5 -> 40.7 ms); from both ends, with the
+// energies in shared memory and the fused minima, 3.8 -> 2.1 us of a 1920x1080 seam.
 constexpr uint32_t FILL_INF = 0x80000000u;   // above every path's 256 * cost (64 rows * 2 * 65535 * 256 < 2^31)
 
 struct FillCtx {
@@ -551,7 +552,7 @@ __device__ __forceinline__ void fill_super_tile(const FillCtx &f, int s, int jpr
     const int nq = min(HC, T - q0);
     const EVec *es = est;
     uint8_t *ft = fd + (lead + q0) * FILLW + lane * FV, *fb = fd + (n - 2 - q0) * FILLW + lane * FV;
-#pragma unroll 1
+#pragma unroll (FWD ? 1 : 3)
     for (int r = 0; r < nq; ++r, ft += FILLW, fb -= FILLW, es += 32) {
       uint32_t e[FV], g[FV], dl[FV] = {}, dr[FV] = {}, gl[FV] = {}, gr[FV] = {};
       unpack(es[0], e);
@@ -601,7 +602,7 @@ __device__ __forceinline__ void fill_super_tile(const FillCtx &f, int s, int jpr
     int rel = ((int)(where >> 2) + (lane ? (int)(where & 3u) - 1 : 0)) & (FILLW - 1);
     uint8_t *fb = fd + (lane ? nt : nt - 1) * FILLW;
     const int stride = lane ? FILLW : -FILLW, steps = lane ? nb : nt;
-#pragma unroll 2
+#pragma unroll 4
     for (int q = 0; q < steps; ++q, fb += stride) {
       const int nr = rel + (int)(fb[rel] & 3u) - 1;
       *reinterpret_cast<uint32_t *>(fb) = (uint32_t)rel;
