@@ -185,7 +185,7 @@ int sc_find_seam_multi_shape(int warps, int tile_rows);
  * synchronise the device and take unpredictable time inside a latency-critical loop, and hosts
  * that budget every device byte through their own allocator forbid allocations they do not
  * control. Same arguments and result as sc_find_seam (any uint16 map, exact seam and cost), but
- * every scratch byte (a padded copy of the energy map, the saved cost rows, the wide-cost search's
+ * every scratch byte (a padded copy of the energy map, the search's cost rows, the wide-cost search's
  * directions and ancestors, three status words) lives in one fixed array of 32 MiB inside the
  * library's device image, held by every GPU that loads the library until the process exits; the
  * call never calls cudaMalloc or cudaFree. Differences from sc_find_seam:
@@ -270,7 +270,7 @@ int sc_carve_batch(const sc_image_desc *descs, int n, void *stream);
  * autotune = 1 times every one-CTA configuration (8, 12 or 15 compute warps per CTA; DP tile
  * height 8, 16 or 32 rows) on the real batch, then load-balancing variants of the fastest (images
  * whose estimated carving time exceeds 0.8, 1.0, 1.2, 1.4, 1.7 or 2.0 x the batch's mean share
- * per SM carved by clusters of 32-row tiles, at least 2 CTAs, 384 columns per CTA), and keeps the
+ * per SM carved by clusters of the latency shape, which sweep an image from both ends), and keeps the
  * fastest; autotune = 2 takes the default configuration with that balancing at 1.4 x the mean share;
  * 0 takes the default configuration. The images' contents may
  * change between runs; their pointers and sizes may not. sc_batch_plan_run enqueues one replay on
@@ -280,11 +280,12 @@ int sc_carve_batch(const sc_image_desc *descs, int n, void *stream);
  * counterpart: this is the batched form's scheduler, exposed so that callers can see where their
  * images go). descs: HOST array of n descriptors (only H, W, C, target_w and target_h are read;
  * the pointers may be NULL); thr: the balancing threshold (images whose estimated one-CTA carve
- * exceeds thr x the batch's mean share per SM go to clusters of the 32-row-tile shape; 0: no
+ * exceeds thr x the batch's mean share per SM go to clusters of the latency shape; 0: no
  * balancing; autotune = 2 uses 1.4); sms: the SM count the share is computed over (152 on a
  * GB300). Outputs, HOST arrays of n: cluster_size[k] 0 when one CTA carves image k, the cluster's
  * CTA count otherwise, -1 when no cluster covers it (the per-seam path carves it); shape[k] 0 for
- * clusters of 8-row tiles (images wider than one CTA), 1 for clusters of 32-row tiles; one_cta_us
+ * clusters of 8-row tiles (images wider than one CTA), 1 for clusters of the latency shape (counted at
+ * 384 columns per CTA; the launch gives as many CTAs to the two halves of the image); one_cta_us
  * (nullable): the carving-time model's estimate of image k's carve on one CTA, in microseconds.
  * Errors: SC_EINVAL for a NULL array, n < 1, thr < 0, sms < 1 or a descriptor that fails the
  * sc_carve size checks. */
@@ -303,7 +304,7 @@ int sc_batch_plan_destroy(sc_batch_plan *plan);
  * micro-batches of up to max_batch requests of one kind, in arrival order within the kind:
  * requests that fit one CTA (searched width <= 1440) go to one persistent one-CTA-per-image
  * launch, wider ones, and those whose carve on one CTA would take over an estimated 50 ms, to one
- * persistent cluster-per-image launch per cluster size (clusters of 32-row tiles, 384 columns per
+ * persistent cluster-per-image launch per cluster size (clusters of the latency shape, 640 columns per
  * CTA: the heaviest requests set the tail latency). Micro-batches
  * on different streams run concurrently, so requests submitted while others are on the GPU start
  * as soon as memory and a stream free up. Every result equals sc_carve of that image alone.

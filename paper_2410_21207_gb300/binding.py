@@ -386,7 +386,7 @@ class BatchPlan:
     def __init__(self, imgs: Sequence, targets: Sequence[Tuple[int, int]], autotune=False,
                  with_log: bool = False):
         """autotune: False/0 default configuration, True/1 time the configurations and balancing
-        variants, 2 default configuration with the heaviest images on 32-row-tile clusters."""
+        variants, 2 default configuration with the heaviest images on latency-shaped clusters."""
         torch = _torch()
         self.imgs = list(imgs)
         self.descs, self.outs, self.logs = _batch_descs(self.imgs, targets, with_log)
@@ -422,7 +422,7 @@ def batch_route(sizes, thr: float = 1.4, sms: int = 152):
     """sc_batch_route: where a batch plan carves each image, computed on the host (no device call).
     sizes: (H, W, C, target_w, target_h) per image -> (cluster_size, shape, one_cta_us) lists:
     cluster_size 0 for one CTA, the cluster's CTA count, or -1 for the per-seam path; shape 0 for
-    8-row-tile clusters, 1 for 32-row-tile clusters; one_cta_us the model's one-CTA carve time."""
+    8-row-tile clusters, 1 for latency-shaped clusters; one_cta_us the model's one-CTA carve time."""
     n = len(sizes)
     descs = (ImageDesc * max(n, 1))()
     for k, (H, W, C, tw, th) in enumerate(sizes):

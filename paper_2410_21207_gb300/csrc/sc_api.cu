@@ -407,11 +407,28 @@ int sc_release_workspaces(void) {
   return SC_OK;
 }
 
+// whether [a, a + na) and [b, b + nb) share a byte: such calls take the form that copies its input first
+static bool overlap(const void *a, size_t na, const void *b, size_t nb) {
+  return b && (uintptr_t)a < (uintptr_t)b + nb && (uintptr_t)b < (uintptr_t)a + na;
+}
+
 int sc_energy(const uint8_t *img, int H, int W, int C, uint16_t *energy_out, void *stream) {
   if (!img || !energy_out) return fail(SC_EINVAL, "null pointer");
   if (H < 1 || W < 1 || !valid_c(C)) return fail(SC_EINVAL, "bad shape %d x %d x %d", H, W, C);
   if ((int64_t)H * W * C >= ((int64_t)1 << 31)) return fail(SC_EINVAL, "H*W*C must be < 2^31");
-  SC_CUDA(launch_energy_bytes(img, H, W, C, energy_out, (cudaStream_t)stream));
+  cudaStream_t st = (cudaStream_t)stream;
+  if (overlap(img, (size_t)H * W * C, energy_out, (size_t)H * W * 2)) {
+    Workspace *wsp;
+    int rc = get_ws(stream, &wsp);
+    if (rc) return rc;
+    std::lock_guard<std::mutex> lk(wsp->mu);
+    const int pitch = round_up(W, 4);
+    SC_CUDA(wsp->img.ensure((size_t)H * pitch));
+    SC_CUDA(launch_pack(img, H, W, C, wsp->img.p, pitch, st));
+    SC_CUDA(launch_energy(wsp->img.p, pitch, H, W, energy_out, W, st));
+    return SC_OK;
+  }
+  SC_CUDA(launch_energy_bytes(img, H, W, C, energy_out, st));
   return SC_OK;
 }
 
@@ -432,7 +449,8 @@ int sc_find_seam(const uint16_t *energy, int H, int W, int32_t *seam_out, int64_
   if (gate && (rc = ensure_wide(ws, H, W, 1))) return rc;
   // a map whose rows are 16-byte aligned is read in place (no copy of 2 bytes a pixel there and back before
   // the search, and no launch: 1920x1080 39.9 -> 28.7 us a call, 64x48 25 -> 19); any other is first copied
-  if ((W % 8) == 0 && ((uintptr_t)energy & 15u) == 0)
+  if ((W % 8) == 0 && ((uintptr_t)energy & 15u) == 0 && !overlap(energy, (size_t)H * W * 2, seam_out, (size_t)H * 4) &&
+      !overlap(energy, (size_t)H * W * 2, cost_out, 8))
     return launch_search(ws, energy, W, H, W, seam_out, nullptr, cost_out, gate, st, 0, true);
   SC_CUDA(ws.E.ensure((size_t)H * pe));
   SC_CUDA(launch_copy_energy(energy, H, W, ws.E.p + E_PADL, pe, ws.flags.p + 1, st));

@@ -3,12 +3,13 @@
 // rows KT and backtrack-fill warps FWM; sc_batch_cl.cu and sc_batch_cl_lat.cu instantiate the two
 // shapes of sc_batch_cl.h.
 // Each cluster repeatedly takes the next image from a queue and carves it completely, like the
-// one-CTA batched kernel (sc_batch.cuh), with the cluster-wide seam search (seam_search with CL)
+// one-CTA batched kernel (sc_batch.cuh), with the cluster-wide seam search (seam_search with CL, or the
+// two-ended clb_two_search)
 // and the per-seam row work split over the cluster's CTAs: CTA r owns rows r, r + cs, r + 2cs, ...
 // Per seam: the search (ends with a cluster barrier); every owned row's refreshed energy pair and
 // pending-removal list update, one thread per row; a cluster barrier (the pairs read neighbouring
-// rows' words, which the compaction below rewrites); the energy row shifted past the seam with the
-// pair written in, one warp per row, and every RPEND seams the image words compacted; a cluster
+// rows' words, which the compaction below rewrites); the energy rows shifted past the seam with the
+// pair written in, four per warp at a time, and every RPEND seams the image words compacted; a cluster
 // barrier. Several clusters run side by side, so a batch of wide images keeps the GPU busy where
 // the per-seam cluster path would run one image's latency-bound chain at a time.
 #pragma once

@@ -10,7 +10,7 @@
 namespace sc {
 
 // The search of one map is a chain of H dependent rows, so its shape is chosen for latency: tall
-// 32-row tiles cross a tile boundary (strip exchange, staging barrier, bookkeeping) half as often
+// 32-row tiles cross a tile boundary (strip exchange, barrier, bookkeeping) half as often
 // as 16-row ones, at the price of more redundant halo columns, which only costs idle SMs. Shapes
 // in order of preference; the first whose cluster covers W is used.
 struct DpShapeDef {
@@ -32,9 +32,9 @@ DpShape dp_shape_for(int W) {
   return s;
 }
 
-// Super-tile height: KS (32) rows for the 4-warp shape, whose ancestor chain is local (the table is
-// gathered in rank 0) and whose serial backtrack fill halves against 64; KS_WIDE (64) for the wide
-// shapes and forward energy, whose chain hops cross CTAs through DSMEM and would double.
+// Super-tile height: KS (32) rows for the 4-warp shape, whose ancestor chain is local and whose serial
+// backtrack fill halves against 64; KS_WIDE (64) for the wide shapes, whose ancestor tables would not
+// fit shared memory, and for the one-ended forward search, whose chain hops cross CTAs.
 template <int NW, int KT, bool FWD>
 __host__ __device__ constexpr int dp_super_rows() { return (NW == 4 && KT == 32 && !FWD) ? KS : KS_WIDE; }
 
@@ -158,8 +158,8 @@ static cudaError_t launch_dp_shape(const DpArgs &a, int cs, cudaStream_t st) {
 // super-tile, upper half first), gw = the columns the cluster covers. It fits (S + 1) rows of pitch_e
 // words, S = ceil(H / 32), for H >= 64: 8 gw + (S + 1) gw <= 4 (S + 1) pitch_e.
 //
-// Bound by latency: the chain of H / 2 rows (about 54 cycles a row with the tile boundaries), then
-// the hand-over, chain and fill. 1920x1080 carve 24.5 -> 17.7 ms, 3840x2160 carve 183.9 -> 106.8 ms,
+// Bound by latency: the chain of H / 2 rows, then the hand-over, chains and fill. Against the one-ended
+// search, both with the kernels of that time: 1920x1080 carve 24.5 -> 17.7 ms, 3840x2160 carve 183.9 -> 106.8 ms,
 // 1279x853 -> 1021x701 18.5 -> 13.5 ms. The hand-over costs a few microseconds, so short maps keep the
 // one-ended search: one launch takes 16.5 / 16.6 us (two-ended / one-ended) at 128 rows, 18.5 / 17.2 at
 // 160, 18.5 / 18.7 at 192, 18.7 / 20.8 at 256, 22.8 / 28.9 at 512 (1000 columns; the same line at 64 to

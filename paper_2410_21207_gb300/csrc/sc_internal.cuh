@@ -23,7 +23,7 @@ constexpr int E_PADR = 1024;   // right pad (elements)
 // rows inside a CTA (shared memory) and every K2 rows between the CTAs of a cluster (DSMEM).
 // Ancestors are tracked over super-tiles of KS rows; the single-map search of maps wider than a
 // 4-warp cluster covers uses KS_WIDE (its ancestor chain reads other CTAs through DSMEM, one load per
-// super-tile). Buffers of saved cost rows are sized for KS, the shorter. KT is a template
+// super-tile). The two-ended search's scratch is sized for KS, the shorter. KT is a template
 // parameter of each kernel.
 constexpr int V = 4;
 constexpr int KS = 32;
