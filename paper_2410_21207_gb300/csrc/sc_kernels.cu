@@ -448,9 +448,12 @@ namespace sc {
 
 cudaError_t launch_refresh(const uint32_t *img, int pitch, uint16_t *E, int pe, int H, int W, const int32_t *seam,
                            const int16_t *lists_in, int16_t *lists_out, int m, int *err, cudaStream_t st) {
-  // 8 rows per block; registers for rows up to 1024, 2048 or 4096 elements
+  // registers for rows up to 1024, 2048 or 4096 elements
   auto *const k = W <= 1024 ? k_refresh<4> : (W <= 2048 ? k_refresh<8> : (W <= 4096 ? k_refresh<16> : k_refresh_wide));
-  return launch_pdl(k, (H + 7) / 8, 256, st, img, pitch, E, pe, H, W, seam, lists_in, lists_out, m, err);
+  // rows per block: small blocks start and end sooner (per seam, blocks of 8 / 4 / 2 / 1 rows: 1920x1080 24.25 /
+  // 23.9 / 24.1 / 24.1 us, 700x500 15.1 / 14.6 / 14.6 / 14.7; 3840x2160 makes no difference)
+  const int rows = W <= 2048 ? 4 : 8;
+  return launch_pdl(k, (H + rows - 1) / rows, 32 * rows, st, img, pitch, E, pe, H, W, seam, lists_in, lists_out, m, err);
 }
 
 cudaError_t launch_refresh_fwd(const uint32_t *img, int pitch, uint16_t *E, int pe, int64_t pstride, int H, int W,
