@@ -595,7 +595,9 @@ __device__ __forceinline__ void fill_super_tile(const FillCtx &f, int s, int jpr
   }
   if (lane == 0) atomicAdd(f.csum, (best >> 8) * f.csign);   // the path's cost in this super-tile
   // lanes 0 and 1 follow the directions up and down (relative columns, kept in the direction rows they
-  // have read: a row's entry is not needed again), then the warp writes the seam rows
+  // have read: a row's entry is not needed again), then the warp writes the seam rows. The barrier
+  // orders every lane's direction stores before the walk: shuffles and reductions order no memory.
+  __syncwarp();
   if (lane < 2) {
     // a path that leaves the window (it cannot) wraps around inside this warp's rows and ends on the
     // wrong column

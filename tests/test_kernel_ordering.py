@@ -1,0 +1,32 @@
+"""Memory order inside the kernels that no result can show reliably: each check reads the source for the
+barrier, fence or load that orders what one thread or kernel writes and another one reads."""
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2410_21207_gb300", "csrc")
+
+
+def _code(name):
+    """A source file without its comments."""
+    with open(os.path.join(CSRC, name)) as f:
+        return re.sub(r"//[^\n]*|/\*.*?\*/", "", f.read(), flags=re.S)
+
+
+def _function(code, start):
+    """From `start` to the closing brace of the function whose head it begins."""
+    at = code.index(start)
+    depth = 0
+    for i in range(code.index("{", at), len(code)):
+        depth += {"{": 1, "}": -1}.get(code[i], 0)
+        if depth == 0:
+            return code[at:i + 1]
+    raise AssertionError("unbalanced braces after " + start)
+
+
+def test_the_walk_follows_a_barrier_after_the_direction_stores():
+    """Every lane of a fill warp stores directions; lanes 0 and 1 read other lanes' and write over them."""
+    fill = _function(_code("sc_search.cuh"), "void fill_super_tile(")
+    stores = [m.end() for m in re.finditer(r"\b(?:down_row|up_row)\(e|\bup_row\(g|\bdown_row\(e", fill)]
+    walk = fill.index("fb[rel]")
+    assert stores and max(stores) < walk
+    assert "__syncwarp();" in fill[max(stores):walk]
