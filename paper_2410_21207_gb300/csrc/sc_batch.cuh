@@ -115,6 +115,8 @@ __device__ void batch_energy(const uint32_t *words, int pitch, int rows, int col
 template <int NW, int KT>
 __device__ void batch_carve_item(const BatchItem &it, unsigned char *smem, int Smax, SearchState &st, int *err,
                                  const CUtensorMap *tmap) {
+  // the thread that issues this image's tensor copies
+  if (threadIdx.x == NW * 32) fence_tensormap_acquire(tmap);
   const int H = it.H, W = it.W, C = it.C, tw = it.tw, th = it.th;
   const int64_t npx = (int64_t)H * W;
   for (int64_t q = threadIdx.x; q < npx; q += blockDim.x) {

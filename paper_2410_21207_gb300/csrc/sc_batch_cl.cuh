@@ -169,6 +169,8 @@ __device__ inline void clb_transpose(const uint32_t *src, int ps, int rows, int 
 template <int NW, int KT, int FWM, bool TWO>
 __device__ void clb_carve_item(const BatchItem &it, unsigned char *smem, int Smax, SearchState &st, int *err, int rank,
                                int cs, const CUtensorMap *tmap) {
+  // the thread that issues this image's tensor copies
+  if (TWO && threadIdx.x == NW * 32) fence_tensormap_acquire(tmap);
   const int H = it.H, W = it.W, C = it.C, tw = it.tw, th = it.th;
   const int64_t tid = (int64_t)rank * blockDim.x + threadIdx.x, nth = (int64_t)cs * blockDim.x;
   const int64_t npx = (int64_t)H * W;

@@ -44,6 +44,12 @@ __device__ __forceinline__ void tensor_g2s_2d(void *dst_smem, const void *tmap, 
       "l"(tmap), "r"(x), "r"(y), "r"(smem_u32(bar))
       : "memory");
 }
+// order the host's writes of a tensor map in global memory before this thread's later tensor copies of it
+// (a map in a kernel parameter needs none): the copies read it through a proxy of their own, which may
+// still hold what an earlier map at the same address said
+__device__ __forceinline__ void fence_tensormap_acquire(const void *tmap) {
+  asm volatile("fence.proxy.tensormap::generic.acquire.sys [%0], 128;" ::"l"(tmap) : "memory");
+}
 __device__ __forceinline__ void prefetch_tensormap(const void *tmap) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(tmap) : "memory");
 }

@@ -30,3 +30,15 @@ def test_the_walk_follows_a_barrier_after_the_direction_stores():
     walk = fill.index("fb[rel]")
     assert stores and max(stores) < walk
     assert "__syncwarp();" in fill[max(stores):walk]
+
+
+def test_tensor_maps_in_global_memory_are_acquired():
+    """The batched kernels copy through maps the host wrote into global memory: the thread that issues the
+    copies (the producer warp's first) acquires each image's map before its first search."""
+    for name, item, search in (("sc_batch.cuh", "void batch_carve_item(", "batch_seam_pass<"),
+                               ("sc_batch_cl.cuh", "void clb_carve_item(", "clb_seam_pass<")):
+        body = _function(_code(name), item)
+        fence = re.search(r"if \((?:TWO && )?threadIdx\.x == NW \* 32\) fence_tensormap_acquire\(tmap\);", body)
+        assert fence and fence.start() < body.index(search), name
+    fence = _function(_code("sc_ptx.cuh"), "void fence_tensormap_acquire(")
+    assert "fence.proxy.tensormap::generic.acquire.sys" in fence
