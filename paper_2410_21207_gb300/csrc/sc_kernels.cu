@@ -199,8 +199,10 @@ __global__ void k_unpad_energy(const uint16_t *__restrict__ E, int pe, int H, in
 // after the seam is known. Launched as a programmatic dependent it is resident while the search runs,
 // and the search starts its dependents only after it has itself waited for the kernel before it: the
 // energies, lists and image words are then in their final state (nothing writes them until this kernel
-// does). So everything that does not need the seam is loaded before the wait: the whole energy row
-// into registers (R chunks of 8 elements per lane) and the three rows' lists. After the wait: the
+// does), complete in L2, where the search's wait left them; only this kernel's own wait would say
+// anything of an SM's L1, so these loads go past it. So everything that does not need the seam is loaded
+// before the wait: the whole energy row into registers (R chunks of 8 elements per lane) and the three
+// rows' lists. After the wait: the
 // seam columns, one round trip; the tail goes out of the registers while eight lanes fetch the eight
 // pixels of the refreshed pair, a second one. From the end of the search to the end of the refresh:
 // 1920x1080 5.5 -> 3.2 us (carve 14.6 -> 12.6 ms), 1279x853 4.9 -> 3.1 us (carve 11.6 -> 9.7 ms).
@@ -296,7 +298,7 @@ __global__ void __launch_bounds__(128) k_refresh_fwd(const uint32_t *__restrict_
       if (c <= c_hi + 1) x[pl][r] = __ldcg(reinterpret_cast<const uint4 *>(er + pl * pstride + 8 * c));
     }
   const int row = (lane & 2) ? max(i - 1, 0) : i;
-  const LazyRow list = lazy_row(lists_in + (int64_t)row * RPEND, m);
+  const LazyRow list = lazy_row_l2(lists_in + (int64_t)row * RPEND, m);
   pdl_wait_prerequisites();   // the seam of the search that precedes this launch
   const int s = __ldcg(seam + i);
   const int sr = __ldcg(seam + row);

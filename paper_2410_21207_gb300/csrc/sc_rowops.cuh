@@ -112,9 +112,7 @@ struct LazyRow {
   uint32_t t[RPEND / 2];
 };
 
-__device__ __forceinline__ LazyRow lazy_row(const int16_t *list, int m) {
-  const uint4 a = *reinterpret_cast<const uint4 *>(list);
-  const uint4 b = *reinterpret_cast<const uint4 *>(list + 8);
+__device__ __forceinline__ LazyRow lazy_row_of(const uint4 a, const uint4 b, int m) {
   const uint32_t w[RPEND / 2] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
   LazyRow r;
 #pragma unroll
@@ -125,6 +123,16 @@ __device__ __forceinline__ LazyRow lazy_row(const int16_t *list, int m) {
     r.t[k] = (lo | (hi << 16)) - ((uint32_t)(2 * k) | ((uint32_t)(2 * k + 1) << 16));
   }
   return r;
+}
+
+__device__ __forceinline__ LazyRow lazy_row(const int16_t *list, int m) {
+  const uint4 *const p = reinterpret_cast<const uint4 *>(list);
+  return lazy_row_of(p[0], p[1], m);
+}
+// past L1: for the loads a kernel makes ahead of its griddepcontrol.wait
+__device__ __forceinline__ LazyRow lazy_row_l2(const int16_t *list, int m) {
+  const uint4 *const p = reinterpret_cast<const uint4 *>(list);
+  return lazy_row_of(__ldcg(p), __ldcg(p + 1), m);
 }
 
 // removals passed by current column j (0 <= j < 2^15)
@@ -271,7 +279,7 @@ __device__ __forceinline__ RefreshLane refresh_lane(const int16_t *lists, int m,
   RefreshLane f;
   const int q = lane & 7;
   f.row = (q & 2) == 0 ? i : ((q & 1) ? max(i - 1, 0) : min(i + 1, H - 1));
-  f.list = lazy_row(lists + (int64_t)f.row * RPEND, m);
+  f.list = lazy_row_l2(lists + (int64_t)f.row * RPEND, m);
   return f;
 }
 // the lane's pixel; s: row i's seam column, sr: that of the lane's row

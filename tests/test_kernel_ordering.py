@@ -42,3 +42,19 @@ def test_tensor_maps_in_global_memory_are_acquired():
         assert fence and fence.start() < body.index(search), name
     fence = _function(_code("sc_ptx.cuh"), "void fence_tensormap_acquire(")
     assert "fence.proxy.tensormap::generic.acquire.sys" in fence
+
+
+def test_loads_ahead_of_the_wait_go_past_l1():
+    """The refresh kernels read energies and lists of the kernel before last ahead of their
+    griddepcontrol.wait, which alone would make an SM's L1 current: every such load is an L2 one."""
+    kernels, rows = _code("sc_kernels.cu"), _code("sc_rowops.cuh")
+    for name in ("k_refresh(", "k_refresh_wide(", "k_refresh_fwd("):
+        body = _function(kernels, name)
+        ahead = body[body.index("{"):body.index("pdl_wait_prerequisites();")]
+        assert not re.search(r"\b(?:seam|img|lists_in|lists_out|E|er)\s*\[", ahead), name
+        assert "lazy_row(" not in ahead and "refresh_pixel(" not in ahead, name
+        for cast in re.findall(r"[\w:(]*\(?\s*reinterpret_cast<const \w+ \*>\([^;]*;", ahead):
+            assert cast.startswith("__ldcg("), (name, cast)
+    lane = _function(rows, "RefreshLane refresh_lane(")
+    assert "lazy_row_l2(" in lane and "lazy_row(" not in lane
+    assert _function(rows, "LazyRow lazy_row_l2(").count("__ldcg(") == 2
