@@ -99,6 +99,8 @@ struct DevBuf {
   }
 };
 
+constexpr int FLAG_WORDS = 8;
+
 struct Workspace {
   std::mutex mu;
   DevBuf<uint32_t> img, img2, scratch;
@@ -106,7 +108,7 @@ struct Workspace {
   DevBuf<int32_t> seam;
   DevBuf<int16_t> lists;          // two generations of pending-removal lists
   DevBuf<uint8_t> hin, hout;     // staging for the host-pointer entry point
-  DevBuf<int> flags;             // [0] error word, [1] energy-range gate, [2..4] the search's sync words
+  DevBuf<int> flags;             // FLAG_WORDS: [0] error word, [1] energy-range gate, [2..4] the search's sync words
   DevBuf<int> gates;             // one energy-range gate per map of sc_find_seam_multi
   DevBuf<uint32_t> wdirs;        // wide-cost search: directions and ancestors (per map)
   DevBuf<uint16_t> wanc;
@@ -156,9 +158,9 @@ static int get_ws(void *stream, Workspace **out) {
 }
 
 static int ensure_flags(Workspace &ws, cudaStream_t st) {
-  SC_CUDA(ws.flags.ensure(8));
+  SC_CUDA(ws.flags.ensure(FLAG_WORDS));
   if (!ws.flags_zeroed) {
-    SC_CUDA(cudaMemsetAsync(ws.flags.p, 0, 8 * sizeof(int), st));
+    SC_CUDA(cudaMemsetAsync(ws.flags.p, 0, FLAG_WORDS * sizeof(int), st));
     ws.flags_zeroed = true;
   }
   return SC_OK;
@@ -332,10 +334,12 @@ int sc_check(void *stream) {
   std::lock_guard<std::mutex> lk(ws.mu);
   // a stream with no earlier work has fresh (uninitialised) flag words: they start at zero
   if ((rc = ensure_flags(ws, st))) return rc;
+  // read and cleared in the stream's order: the words hold the searches' sync words too, and a search
+  // launched right after this call must not find them cleared while it runs
+  int h[FLAG_WORDS] = {};
+  SC_CUDA(cudaMemcpyAsync(h, ws.flags.p, sizeof(h), cudaMemcpyDeviceToHost, st));
+  SC_CUDA(cudaMemsetAsync(ws.flags.p, 0, sizeof(h), st));
   SC_CUDA(cudaStreamSynchronize(st));
-  int h[4] = {0, 0, 0, 0};
-  SC_CUDA(cudaMemcpy(h, ws.flags.p, 4 * sizeof(int), cudaMemcpyDeviceToHost));
-  SC_CUDA(cudaMemset(ws.flags.p, 0, 4 * sizeof(int)));
   int e = h[0];
   if (h[3] != 0) e |= ERR_COST_MISMATCH;   // some search's path costs did not add up to its cost
   if (int *ge = device_error_word()) {

@@ -58,3 +58,12 @@ def test_loads_ahead_of_the_wait_go_past_l1():
     lane = _function(rows, "RefreshLane refresh_lane(")
     assert "lazy_row_l2(" in lane and "lazy_row(" not in lane
     assert _function(rows, "LazyRow lazy_row_l2(").count("__ldcg(") == 2
+
+
+def test_check_clears_the_search_words_in_stream_order():
+    """sc_check clears words that a running search counts in; the caller's stream may not be ordered with
+    the default stream, so the clearing goes on the caller's."""
+    body = _function(_code("sc_api.cu"), "int sc_check(")
+    clears = re.findall(r"cudaMemset(?:Async)?\(ws\.flags[^;]*;", body)
+    assert len(clears) == 1 and clears[0].startswith("cudaMemsetAsync(") and ", st)" in clears[0]
+    assert body.index(clears[0]) < body.index("cudaStreamSynchronize(st)")
