@@ -117,13 +117,11 @@ struct Workspace {
   DevBuf<uint8_t> enl_tmp;
   DevBuf<uint32_t> enl_bits;
   DevBuf<DpArgs> dargs;
-  bool flags_zeroed = false;
   void release_all() {
     img.release(); img2.release(); scratch.release();
     E.release(); seam.release(); lists.release(); hin.release(); hout.release(); flags.release();
     Emulti.release(); dargs.release(); gates.release(); wdirs.release(); wanc.release();
     enl_log.release(); enl_tmp.release(); enl_bits.release();
-    flags_zeroed = false;
   }
 };
 
@@ -157,14 +155,25 @@ static int get_ws(void *stream, Workspace **out) {
   return SC_OK;
 }
 
-static int ensure_flags(Workspace &ws, cudaStream_t st) {
-  SC_CUDA(ws.flags.ensure(FLAG_WORDS));
-  if (!ws.flags_zeroed) {
-    SC_CUDA(cudaMemsetAsync(ws.flags.p, 0, FLAG_WORDS * sizeof(int), st));
-    ws.flags_zeroed = true;
+// At least n words that are 0 when they are new. The kernels leave them 0 from one call to the next, so
+// they are cleared here, complete before the call goes on: cleared on the caller's stream they would be
+// cleared at a replay only, when that stream is being captured.
+static int ensure_zeroed(DevBuf<int> &b, size_t n) {
+  if (n <= b.cap) return SC_OK;
+  SC_CUDA(b.ensure(n));
+  cudaStream_t z;
+  cudaError_t e = cudaStreamCreateWithFlags(&z, cudaStreamNonBlocking);
+  if (e == cudaSuccess) {
+    e = cudaMemsetAsync(b.p, 0, n * sizeof(int), z);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(z);
+    cudaStreamDestroy(z);
   }
+  if (e != cudaSuccess) b.release();
+  SC_CUDA(e);
   return SC_OK;
 }
+
+static int ensure_flags(Workspace &ws) { return ensure_zeroed(ws.flags, FLAG_WORDS); }
 
 static bool valid_c(int C) { return C == 1 || C == 3 || C == 4; }
 
@@ -189,7 +198,7 @@ int workspace_reserve(cudaStream_t st, int H, int W) {
   int rc = get_ws((void *)st, &wsp);
   if (rc) return rc;
   std::lock_guard<std::mutex> lk(wsp->mu);
-  if ((rc = ensure_flags(*wsp, st))) return rc;
+  if ((rc = ensure_flags(*wsp))) return rc;
   return ensure_carve_buffers(*wsp, H, W);
 }
 
@@ -286,7 +295,7 @@ int carve_impl(const uint8_t *img, int H, int W, int C, int tw, int th, uint8_t 
   if (rc) return rc;
   Workspace &ws = *wsp;
   std::lock_guard<std::mutex> lk(ws.mu);
-  if ((rc = ensure_flags(ws, st))) return rc;
+  if ((rc = ensure_flags(ws))) return rc;
   if ((rc = ensure_carve_buffers(ws, H, W))) return rc;
   const int R = H > W ? H : W;
   const int pitch = round_up(R, 4);
@@ -333,7 +342,7 @@ int sc_check(void *stream) {
   Workspace &ws = *wsp;
   std::lock_guard<std::mutex> lk(ws.mu);
   // a stream with no earlier work has fresh (uninitialised) flag words: they start at zero
-  if ((rc = ensure_flags(ws, st))) return rc;
+  if ((rc = ensure_flags(ws))) return rc;
   // read and cleared in the stream's order: the words hold the searches' sync words too, and a search
   // launched right after this call must not find them cleared while it runs
   int h[FLAG_WORDS] = {};
@@ -445,7 +454,7 @@ int sc_find_seam(const uint16_t *energy, int H, int W, int32_t *seam_out, int64_
   if (rc) return rc;
   Workspace &ws = *wsp;
   std::lock_guard<std::mutex> lk(ws.mu);
-  if ((rc = ensure_flags(ws, st))) return rc;
+  if ((rc = ensure_flags(ws))) return rc;
   const int pe = pitch_e_for(W);
   SC_CUDA(ws.scratch.ensure((size_t)((H + KS - 1) / KS + 1) * pe));
   // any map of so few rows fits the 24-bit search: no range check, no wide-cost search
@@ -473,7 +482,7 @@ int sc_find_seam_multi(const uint16_t *const *energies, int n, int H, int W, int
   if (rc) return rc;
   Workspace &ws = *wsp;
   std::lock_guard<std::mutex> lk(ws.mu);
-  if ((rc = ensure_flags(ws, st))) return rc;
+  if ((rc = ensure_flags(ws))) return rc;
   const int pe = pitch_e_for(W);
   const size_t e_per = (size_t)H * pe;
   // a map is read in place when its rows are 16-byte aligned (W a multiple of 8, aligned base);
@@ -483,10 +492,7 @@ int sc_find_seam_multi(const uint16_t *const *energies, int n, int H, int W, int
   for (int k = 0; k < n; ++k) ncopy += !in_place(k);
   if (ncopy) SC_CUDA(ws.Emulti.ensure(e_per * ncopy));
   SC_CUDA(ws.dargs.ensure((size_t)n));
-  if (ws.gates.cap < (size_t)n) {   // (0 between calls: the wide-cost search clears the ones that were set)
-    SC_CUDA(ws.gates.ensure((size_t)n));
-    SC_CUDA(cudaMemsetAsync(ws.gates.p, 0, (size_t)n * sizeof(int), st));
-  }
+  if ((rc = ensure_zeroed(ws.gates, (size_t)n))) return rc;   // (the wide-cost search clears the ones that were set)
   const bool gated = range_gated(H, 65535);
   if (gated && (rc = ensure_wide(ws, H, W, n))) return rc;
   std::vector<DpArgs> h(n);
@@ -573,7 +579,7 @@ int sc_find_seam_forward(const uint16_t *cu, const uint16_t *dl, const uint16_t 
   if (rc) return rc;
   Workspace &ws = *wsp;
   std::lock_guard<std::mutex> lk(ws.mu);
-  if ((rc = ensure_flags(ws, st))) return rc;
+  if ((rc = ensure_flags(ws))) return rc;
   const int pe = pitch_e_for(W);
   const int64_t pstride = (int64_t)H * pe;
   SC_CUDA(ws.E.ensure((size_t)3 * H * pe));
@@ -597,7 +603,7 @@ int sc_enlarge(const uint8_t *img, int H, int W, int C, int target_w, uint8_t *o
   const int nwords = (W + 31) / 32;
   {
     std::lock_guard<std::mutex> lk(ws.mu);
-    if ((rc = ensure_flags(ws, st))) return rc;
+    if ((rc = ensure_flags(ws))) return rc;
     SC_CUDA(ws.enl_log.ensure((size_t)k * H));
     SC_CUDA(ws.enl_tmp.ensure((size_t)H * (W - k) * C));
     SC_CUDA(ws.enl_bits.ensure((size_t)H * nwords));
@@ -619,7 +625,7 @@ int sc_selftest_wait_timeout(int limit_us, void *stream) {
   int rc = get_ws(stream, &wsp);
   if (rc) return rc;
   std::lock_guard<std::mutex> lk(wsp->mu);
-  if ((rc = ensure_flags(*wsp, st))) return rc;
+  if ((rc = ensure_flags(*wsp))) return rc;
   SC_CUDA(launch_wait_selftest((uint64_t)limit_us * 1000u, wsp->flags.p, st));
   return SC_OK;
 }
