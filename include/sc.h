@@ -284,7 +284,7 @@ int sc_carve_batch(const sc_image_desc *descs, int n, void *stream);
  * balancing; autotune = 2 uses 1.4); sms: the SM count the share is computed over (152 on a
  * GB300). Outputs, HOST arrays of n: cluster_size[k] 0 when one CTA carves image k, the cluster's
  * CTA count otherwise, -1 when no cluster covers it (the per-seam path carves it); shape[k] 0 for
- * clusters of 8-row tiles (images wider than one CTA), 1 for clusters of the latency shape (counted at
+ * clusters of 8-row tiles (images wider or taller than one CTA has room for), 1 for clusters of the latency shape (counted at
  * 384 columns per CTA; the launch gives as many CTAs to the two halves of the image); one_cta_us
  * (nullable): the carving-time model's estimate of image k's carve on one CTA, in microseconds.
  * Errors: SC_EINVAL for a NULL array, n < 1, thr < 0, sms < 1 or a descriptor that fails the
@@ -302,8 +302,9 @@ int sc_batch_plan_destroy(sc_batch_plan *plan);
  * A server owns one device arena of budget_bytes (the memory ledger) and `streams` CUDA streams.
  * A worker thread admits queued requests whenever the arena and a stream have room, as
  * micro-batches of up to max_batch requests of one kind, in arrival order within the kind:
- * requests that fit one CTA (searched width <= 1440) go to one persistent one-CTA-per-image
- * launch, wider ones, and those whose carve on one CTA would take over an estimated 50 ms, to one
+ * requests that fit one CTA (searched width <= 1440, no more rows than its shared memory has room
+ * for) go to one persistent one-CTA-per-image
+ * launch, wider and taller ones, and those whose carve on one CTA would take over an estimated 50 ms, to one
  * persistent cluster-per-image launch per cluster size (clusters of the latency shape, 640 columns per
  * CTA: the heaviest requests set the tail latency). Micro-batches
  * on different streams run concurrently, so requests submitted while others are on the GPU start

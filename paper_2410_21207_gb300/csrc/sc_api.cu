@@ -782,7 +782,7 @@ static int device_sms() {
 }
 
 // Lays out every batched image's scratch in one pool (offsets; `pool` may be null to size it):
-// images that one CTA of configuration c covers first, then the wider ones by cluster size.
+// images that one CTA of configuration c covers first, then the wider and taller ones by cluster size.
 void batch_layout(const sc_image_desc *descs, int n, const BatchCfg &c, unsigned char *pool, BatchSetup &b) {
   b.items.clear();
   b.cl.clear();
@@ -794,7 +794,7 @@ void batch_layout(const sc_image_desc *descs, int n, const BatchCfg &c, unsigned
   // the images that would hold up the batch on one CTA each: carving work above thr_bal x the mean
   // share per SM goes to a latency-shaped cluster (the batch then ends when the average SM does,
   // not when the largest image does)
-  b.map_failed = false;
+  b.map_failed = b.tall = false;
   std::vector<char> &bal = b.lat;
   bal.assign(n, 0);
   if (c.thr_bal > 0.f) {
@@ -817,6 +817,11 @@ void batch_layout(const sc_image_desc *descs, int n, const BatchCfg &c, unsigned
       wide.push_back(k);
       continue;
     }
+    if (!batch_rows_fit(c.nw, c.kt, rows0)) {   // more rows than the CTA has shared memory for
+      wide.push_back(k);
+      b.tall = true;
+      continue;
+    }
     int S;
     b.items.push_back(layout_item(d, limit, pool, off, &S, limit + 2 * c.kt, c.kt, &b.map_failed));
     if (S > b.Smax) b.Smax = S;
@@ -831,7 +836,8 @@ void batch_layout(const sc_image_desc *descs, int n, const BatchCfg &c, unsigned
         cs = cl;
       }
     }
-    if (cs > MAX_CLUSTER) {
+    const int rows0 = (d.H > d.target_h && d.target_w > d.H) ? d.target_w : d.H;
+    if (cs > MAX_CLUSTER || batch_cl_smem_bytes((rows0 + KS - 1) / KS, shape) > BATCH_CL_SMEM_MAX) {
       b.fallback.push_back(k);
       continue;
     }
@@ -886,16 +892,20 @@ static int check_batch_descs(const sc_image_desc *descs, int n) {
   return SC_OK;
 }
 
-// the widest configuration whose shared memory fits this batch and that covers the most images
+// the configuration that covers the most images, the first of those whose CTAs have room for the rows of
+// every image narrow enough for them; only when there is none (images of over 7,168 rows), of all of them
 static BatchCfg default_batch_cfg(const sc_image_desc *descs, int n) {
   BatchCfg best = kBatchCfgs[0];
   int best_cover = -1;
-  for (const BatchCfg &c : kBatchCfgs) {
-    BatchSetup b;
-    batch_layout(descs, n, c, nullptr, b);
-    if (batch_smem_bytes(c.nw, c.kt, b.Smax) > 232448 - 1024) continue;
-    const int cover = (int)b.items.size();
-    if (cover > best_cover) { best_cover = cover; best = c; }
+  for (const bool tall : {false, true}) {
+    for (const BatchCfg &c : kBatchCfgs) {
+      BatchSetup b;
+      batch_layout(descs, n, c, nullptr, b);
+      if (b.tall != tall) continue;
+      const int cover = (int)b.items.size();
+      if (cover > best_cover) { best_cover = cover; best = c; }
+    }
+    if (best_cover >= 0) break;
   }
   return best;
 }
@@ -1116,8 +1126,7 @@ int sc_batch_plan_create(const sc_image_desc *descs, int n, int autotune, void *
     for (const BatchCfg &c : kBatchCfgs) {
       BatchSetup b;
       batch_layout(descs, n, c, nullptr, b);
-      if (b.items.size() < b0.items.size()) continue;
-      if (batch_smem_bytes(c.nw, c.kt, b.Smax) > 232448 - 1024) continue;
+      if (b.items.size() < b0.items.size() || (b.tall && !b0.tall)) continue;
       float ms = 0.f;
       if ((rc = trial_ms(c, &ms))) { delete p; return rc; }
       if (ms < best_ms) { best_ms = ms; best = c; }
@@ -1199,7 +1208,7 @@ int sc_batch_route(const sc_image_desc *descs, int n, float thr, int sms, int *c
   };
   for (const ClusterGroup &g : b.cl)
     for (int k : g.index) report(k);
-  for (int k : b.fallback) report(k);
+  for (int k : b.fallback) cluster_size[k] = -1;
   return SC_OK;
 }
 

@@ -179,8 +179,6 @@ __global__ void __launch_bounds__(Geo<NW, KT, false>::THREADS, 1)
   pdl_wait_prerequisites();
 }
 
-constexpr size_t BATCH_SMEM_MAX = 232448 - 1024;   // the opt-in limit minus room for static shared memory
-
 template <int NW, int KT>
 cudaError_t batch_configure_cfg() {
   static bool configured = false;

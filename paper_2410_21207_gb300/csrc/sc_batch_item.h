@@ -4,6 +4,8 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include "sc_internal.cuh"
+
 namespace sc {
 
 struct BatchItem {
@@ -35,6 +37,11 @@ inline int batch_width_limit(int nw, int kt) { return nw * (128 - 2 * kt); }
 cudaError_t launch_batch(int nw, int kt, const BatchItem *items, int n, int Smax, int grid, int *queue, int *err,
                          cudaStream_t st, bool pdl = false);
 size_t batch_smem_bytes(int nw, int kt, int Smax);
+constexpr size_t BATCH_SMEM_MAX = 232448 - 1024;     // the opt-in limit minus room for static shared memory
+// whether a CTA of the configuration has room for a map of `rows` rows (its ancestor table grows with them)
+inline bool batch_rows_fit(int nw, int kt, int rows) {
+  return batch_smem_bytes(nw, kt, (rows + KS - 1) / KS) <= BATCH_SMEM_MAX;
+}
 int batch_blocks_per_sm(int nw, int kt, int Smax);   // after the kernel's smem attribute is set
 
 }  // namespace sc

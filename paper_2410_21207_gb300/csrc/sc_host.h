@@ -52,6 +52,7 @@ struct BatchSetup {
   std::vector<char> lat;          // per descriptor: the latency shape was asked for
   size_t pool_bytes = 0;
   int Smax = 1;
+  bool tall = false;              // an image left the one-CTA kernel for its height alone
   bool map_failed = false;        // a tensor map could not be encoded
   int cluster_images() const {
     int n = 0;

@@ -258,9 +258,7 @@ bool admit(sc_server *s) {
     sc_image_desc d = desc_of(r);
     int S = 1;
     const size_t scratch = item_bytes(s, d, &S);
-    const int sm = std::max(Smax, S);
-    const size_t smem = kind ? batch_cl_smem_bytes(sm, kind_shape(kind)) : batch_smem_bytes(s->cfg.nw, s->cfg.kt, sm);
-    if (smem > 232448 - 1024) break;
+    const int sm = std::max(Smax, S);   // (batch_layout gave the request a kernel with room for its rows)
     const size_t nin = (size_t)r.H * r.W * r.C, nout = (size_t)r.th * r.tw * r.C;
     if (s->free_flags.size() < 2) break;   // one word stays for the launch's error word
     if (r.staged && !s->staging.base && !s->staging.init_host(std::min(s->budget, (size_t)2 << 30))) break;
