@@ -49,7 +49,7 @@ __device__ inline void cta_transpose(const uint32_t *src, int ps, int rows, int 
 // lists, adds the removal to the row's list and compacts the energy row; the words are compacted
 // every RPEND seams and at the end of the pass.
 template <int NW, int KT>
-__device__ void batch_seam_pass(const BatchItem &it, uint32_t *words, int rows, int cols, int count,
+__device__ void batch_seam_pass(const BatchJob &it, uint32_t *words, int rows, int cols, int count,
                                 int32_t *log, int64_t *costs, unsigned char *smem, int Smax, SearchState &st,
                                 int *err, const CUtensorMap *tmap) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
@@ -113,7 +113,7 @@ __device__ void batch_energy(const uint32_t *words, int pitch, int rows, int col
 }
 
 template <int NW, int KT>
-__device__ void batch_carve_item(const BatchItem &it, unsigned char *smem, int Smax, SearchState &st, int *err,
+__device__ void batch_carve_item(const BatchJob &it, unsigned char *smem, int Smax, SearchState &st, int *err,
                                  const CUtensorMap *tmap) {
   // the thread that issues this image's tensor copies
   if (threadIdx.x == NW * 32) fence_tensormap_acquire(tmap);
@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(Geo<NW, KT, false>::THREADS, 1)
   __shared__ int next;
   // the current image's descriptor lives in shared memory and its fields are read where they are
   // used, so they do not occupy registers across the seam loop
-  __shared__ BatchItem cur;
+  __shared__ BatchJob cur;
   search_init(smem, batch_plan<NW, KT>(Smax));
   __syncthreads();
   SearchState st;

@@ -78,7 +78,7 @@ __device__ __forceinline__ void clb_two_search(SearchArgs a, uint32_t *scratch, 
 
 // (count) vertical seams of a rows x cols word image whose energy is in it.E
 template <int NW, int KT, int FWM, bool TWO>
-__device__ void clb_seam_pass(const BatchItem &it, uint32_t *words, int rows, int cols, int count, int32_t *log,
+__device__ void clb_seam_pass(const BatchJob &it, uint32_t *words, int rows, int cols, int count, int32_t *log,
                               int64_t *costs, unsigned char *smem, int Smax, SearchState &st, int *err, int rank,
                               int cs, const CUtensorMap *tmap) {
   cg::cluster_group cl = cg::this_cluster();
@@ -167,7 +167,7 @@ __device__ inline void clb_transpose(const uint32_t *src, int ps, int rows, int 
 }
 
 template <int NW, int KT, int FWM, bool TWO>
-__device__ void clb_carve_item(const BatchItem &it, unsigned char *smem, int Smax, SearchState &st, int *err, int rank,
+__device__ void clb_carve_item(const BatchJob &it, unsigned char *smem, int Smax, SearchState &st, int *err, int rank,
                                int cs, const CUtensorMap *tmap) {
   // the thread that issues this image's tensor copies
   if (TWO && threadIdx.x == NW * 32) fence_tensormap_acquire(tmap);
@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(Geo<NW, KT, true, FWM>::THREADS, 1)
     k_batch_cl(const BatchItem *__restrict__ items, int n, int Smax, int *queue, int *err) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ int next;
-  __shared__ BatchItem cur;   // the current image's descriptor, read where its fields are used
+  __shared__ BatchJob cur;   // the current image's descriptor, read where its fields are used
   // a launch chained behind this one (programmatic dependent launch) may start once every CTA of
   // this launch is resident: a batch plan places its clusters before the one-CTA launch fills the
   // remaining SMs

@@ -8,8 +8,7 @@
 
 namespace sc {
 
-struct BatchItem {
-  CUtensorMap tmap;     // the energy buffer, in the boxes of the kernel that carves the image (64-byte aligned)
+struct BatchJob {
   const uint8_t *img;   // H x W x C uint8 (caller's)
   uint8_t *out;         // th x tw x C uint8 (caller's)
   int32_t *seam_log;    // nullable (caller's)
@@ -28,6 +27,9 @@ struct BatchItem {
   // visible to the host; `out` may then be host-mapped memory (the serving form)
   int *done;
 };
+struct BatchItem : BatchJob {
+  CUtensorMap tmap;     // the energy buffer, in the boxes of the kernel that carves the image (64-byte aligned)
+};
 
 // width a CTA of nw compute warps with tile height kt covers
 inline int batch_width_limit(int nw, int kt) { return nw * (128 - 2 * kt); }
@@ -37,7 +39,9 @@ inline int batch_width_limit(int nw, int kt) { return nw * (128 - 2 * kt); }
 cudaError_t launch_batch(int nw, int kt, const BatchItem *items, int n, int Smax, int grid, int *queue, int *err,
                          cudaStream_t st, bool pdl = false);
 size_t batch_smem_bytes(int nw, int kt, int Smax);
-constexpr size_t BATCH_SMEM_MAX = 232448 - 1024;     // the opt-in limit minus room for static shared memory
+// the opt-in limit minus the kernel's static shared memory (the current image's BatchJob and a queue index)
+constexpr size_t BATCH_SMEM_MAX = 232448 - 192;
+static_assert(sizeof(BatchJob) + 16 <= 192, "static shared memory of the one-CTA kernel");
 // whether a CTA of the configuration has room for a map of `rows` rows (its ancestor table grows with them)
 inline bool batch_rows_fit(int nw, int kt, int rows) {
   return batch_smem_bytes(nw, kt, (rows + KS - 1) / KS) <= BATCH_SMEM_MAX;

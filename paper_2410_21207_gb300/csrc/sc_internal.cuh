@@ -95,9 +95,18 @@ cudaError_t launch_dp(const DpArgs &a, cudaStream_t st);   // forward energy whe
 // (W <= 4096); the multi-map form takes a device array of n DpArgs of one size (e1 only).
 cudaError_t launch_dp_wide(const DpArgs &a, uint32_t *dirs, uint16_t *anc, cudaStream_t st);
 // Tensor map of `rows` rows of pitch elements (base: 16-byte aligned, pitch a multiple of 8), copied in
-// boxes of KT rows; BW columns go in tensor_boxes(BW) boxes of tensor_box_cols(BW) <= 256 columns.
-constexpr int tensor_boxes(int BW) { return (BW + 255) / 256; }
-constexpr int tensor_box_cols(int BW) { return ((BW + tensor_boxes(BW) - 1) / tensor_boxes(BW) + 7) / 8 * 8; }
+// boxes of KT rows; BW columns go in tensor_boxes(BW) boxes of tensor_box_cols(BW) <= 256 columns: as few
+// boxes as can be of those, up to twice the fewest, that together stage the fewest columns more than BW (each
+// takes 6 KT bytes of the staging ring, which the ancestor tables of tall images need)
+constexpr int tensor_box_width(int BW, int boxes) { return ((BW + boxes - 1) / boxes + 7) / 8 * 8; }
+constexpr int tensor_boxes(int BW) {
+  const int least = (BW + 255) / 256;
+  int best = least;
+  for (int n = least; n <= 2 * least; ++n)
+    if (n * tensor_box_width(BW, n) < best * tensor_box_width(BW, best)) best = n;
+  return best;
+}
+constexpr int tensor_box_cols(int BW) { return tensor_box_width(BW, tensor_boxes(BW)); }
 cudaError_t energy_tensor_map(CUtensorMap *m, const uint16_t *base, int pitch, int rows, int BW, int KT);
 struct MultiArgs;
 cudaError_t launch_dp_wide_multi(const DpArgs *dargs_dev, const MultiArgs *inl, int n, int H, int W, uint32_t *dirs,

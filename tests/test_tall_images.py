@@ -8,10 +8,10 @@ from paper_2410_21207_gb300 import binding as sc
 
 
 def test_route_of_images_taller_than_any_configuration():
-    """7,168 rows are the most a one-CTA configuration has room for; clusters of 8-row tiles 7,392."""
-    cs, shape, _ = sc.batch_route([(7168, 20, 1, 18, 7168)], 0.0, 152)
+    """7,232 rows are the most a one-CTA configuration has room for; clusters of 8-row tiles 7,392."""
+    cs, shape, _ = sc.batch_route([(7232, 20, 1, 18, 7232)], 0.0, 152)
     assert cs == [0]
-    cs, shape, _ = sc.batch_route([(7169, 20, 1, 18, 7169), (7392, 20, 1, 18, 7392), (7393, 20, 1, 18, 7393),
+    cs, shape, _ = sc.batch_route([(7233, 20, 1, 18, 7233), (7392, 20, 1, 18, 7392), (7393, 20, 1, 18, 7393),
                                    (8192, 20, 1, 18, 8192), (100, 20, 1, 18, 100)], 0.0, 152)
     assert cs == [1, 1, -1, -1, 0] and shape[:2] == [0, 0]
     # with both passes as well: 11 CTAs would cover the second pass's columns, but not the first one's rows
@@ -19,8 +19,24 @@ def test_route_of_images_taller_than_any_configuration():
     assert cs == [-1]
 
 
+# the most rows each configuration has room for, and one row more (which the next one in the list takes)
 @pytest.mark.gpu
-@pytest.mark.parametrize("W,H", [(8, 8192), (9, 7393), (9, 7169)])
+@pytest.mark.parametrize("H,cfg", [(1728, (15, 16)), (1729, (15, 8)), (2560, (15, 8)), (2561, (12, 8)), (3680, (12, 8)),
+                                   (3681, (8, 16))])
+def test_default_configuration_by_height(H, cfg):
+    torch = pytest.importorskip("torch")
+    img = np.random.default_rng(H).integers(0, 256, size=(H, 24, 3), dtype=np.uint8)
+    plan = sc.BatchPlan([torch.from_numpy(img).cuda()], [(22, H)])
+    info = plan.info()
+    assert (info["compute_warps"], info["tile_rows"], info["batched"]) == (*cfg, 1)
+    out = plan.run()[0]
+    sc.check()
+    np.testing.assert_array_equal(out.cpu().numpy(), oracle.carve(img, 22, H))
+    plan.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("W,H", [(8, 8192), (9, 7393), (9, 7233)])
 def test_tall_images_in_a_batch(W, H):
     torch = pytest.importorskip("torch")
     rng = np.random.default_rng(H)
