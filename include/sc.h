@@ -270,7 +270,7 @@ int sc_carve_batch(const sc_image_desc *descs, int n, void *stream);
  * autotune = 1 times every one-CTA configuration (8, 12 or 15 compute warps per CTA; DP tile
  * height 8, 16 or 32 rows) on the real batch, then load-balancing variants of the fastest (images
  * whose estimated carving time exceeds 0.8, 1.0, 1.2, 1.4, 1.7 or 2.0 x the batch's mean share
- * per SM carved by clusters of the latency shape, which sweep an image from both ends), and keeps the
+ * per SM carved by clusters of a latency shape), and keeps the
  * fastest; autotune = 2 takes the default configuration with that balancing at 1.4 x the mean share;
  * 0 takes the default configuration. The images' contents may
  * change between runs; their pointers and sizes may not. sc_batch_plan_run enqueues one replay on
@@ -280,12 +280,13 @@ int sc_carve_batch(const sc_image_desc *descs, int n, void *stream);
  * counterpart: this is the batched form's scheduler, exposed so that callers can see where their
  * images go). descs: HOST array of n descriptors (only H, W, C, target_w and target_h are read;
  * the pointers may be NULL); thr: the balancing threshold (images whose estimated one-CTA carve
- * exceeds thr x the batch's mean share per SM go to clusters of the latency shape; 0: no
+ * exceeds thr x the batch's mean share per SM go to clusters of a latency shape; 0: no
  * balancing; autotune = 2 uses 1.4); sms: the SM count the share is computed over (152 on a
  * GB300). Outputs, HOST arrays of n: cluster_size[k] 0 when one CTA carves image k, the cluster's
  * CTA count otherwise, -1 when no cluster covers it (the per-seam path carves it); shape[k] 0 for
- * clusters of 8-row tiles (images wider or taller than one CTA has room for), 1 for clusters of the latency shape (counted at
- * 384 columns per CTA; the launch gives as many CTAs to the two halves of the image); one_cta_us
+ * clusters of 8-row tiles (images wider or taller than one CTA has room for), 1 for clusters of a latency
+ * shape, which sweeps the image from both ends (2 ceil(width / 640) CTAs, up to 16, while the plan's
+ * images take at most 1.5 x the SMs so, else max(2, ceil(width / 384)) CTAs); one_cta_us
  * (nullable): the carving-time model's estimate of image k's carve on one CTA, in microseconds.
  * Errors: SC_EINVAL for a NULL array, n < 1, thr < 0, sms < 1 or a descriptor that fails the
  * sc_carve size checks. */

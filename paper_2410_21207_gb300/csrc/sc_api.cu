@@ -732,7 +732,9 @@ static BatchItem layout_item(const sc_image_desc &d, int limit, unsigned char *p
   it.img_w = (uint32_t *)take((size_t)d.H * it.pitch * 4);
   it.img2_w = nh > 0 ? (uint32_t *)take((size_t)d.target_w * it.pitch * 4) : nullptr;
   it.E = (uint16_t *)take((size_t)rows_max * it.pe * 2);
-  it.scratch = (uint32_t *)take((size_t)(S + 1) * it.pe * 4);
+  // cost rows and ancestor tables of a two-ended search: limit columns wide, one super-tile more than S where
+  // both halves end on a part of one
+  it.scratch = (uint32_t *)take(std::max((size_t)(S + 1) * it.pe * 4, (size_t)(8 + S + 1) * limit));
   it.seam = (int32_t *)take((size_t)rows_max * 4);
   it.lists = (int16_t *)take((size_t)2 * rows_max * RPEND * 2);
   it.tmap = CUtensorMap{};
@@ -751,7 +753,8 @@ int batch_cluster_size(const sc_image_desc &d) { return batch_cl_ctas(batch_need
 // latency shape (240..3900 columns, 180..1332 rows, alone: c 10, a 0.024 + 0.07 / cs, the refresh's rows
 // being dealt over the CTAs, b 9e-5 / cs) is counted 1.2 times slower, as it is beside a GPU full of
 // one-CTA images: three batches of 256 images take 43.4 / 39.0 / 39.6 ms with the split of SMs
-// that the times alone give, 40.2 / 38.6 / 34.8 ms with 1.2 x, 40.2 / 44.6 / 34.8 ms with 1.4 x. The
+// that the times alone give, 40.2 / 38.6 / 34.8 ms with 1.2 x, 40.2 / 44.6 / 34.8 ms with 1.4 x (CL_LAT; CL_LAT_12 counts
+// alike: 3 CTAs of it take 900x600 47.2, 1000x700 57.1, 1152x944 78.0 us a seam, 4 of CL_LAT 43.9, 50.5, 68.8). The
 // 8-row-tile cluster shape is counted as one CTA on a map cs / 2 times narrower. The one-CTA kernel has
 // become faster than its first fit, which stays the measure of the routing (sc_batch_route reports it);
 // the split uses the later one (c 8.0, a 0.069, b 8.9e-5).
@@ -761,7 +764,8 @@ struct SeamCost {
 static SeamCost cost_one_cta() { return {8.3, 0.0874, 9.34e-5}; }
 static SeamCost cost_one_cta_now() { return {8.0, 0.069, 8.9e-5}; }
 static SeamCost cost_cluster(int shape, int cs) {
-  return shape == CL_LAT ? SeamCost{12.0, 0.029 + 0.084 / cs, 1.08e-4 / cs} : SeamCost{8.3, 0.0874, 9.34e-5 * 2.0 / cs};
+  if (shape != CL_WIDE) return {12.0, 0.029 + 0.084 / cs, 1.08e-4 / cs};
+  return {8.3, 0.0874, 9.34e-5 * 2.0 / cs};
 }
 // n seams of an h-row map whose width starts at w and drops by one per seam
 static double pass_us(const SeamCost &k, double h, double w, double n) {
@@ -795,10 +799,9 @@ void batch_layout(const sc_image_desc *descs, int n, const BatchCfg &c, unsigned
   // share per SM goes to a latency-shaped cluster (the batch then ends when the average SM does,
   // not when the largest image does)
   b.map_failed = b.tall = false;
-  std::vector<char> &bal = b.lat;
-  bal.assign(n, 0);
+  std::vector<char> bal(n, 0);
+  const int sms = c.thr_bal > 0.f ? (c.sms > 0 ? c.sms : device_sms()) : 0;
   if (c.thr_bal > 0.f) {
-    const int sms = c.sms > 0 ? c.sms : device_sms();
     double total = 0.0;
     for (int k = 0; k < n; ++k) total += item_us(descs[k], cost_one_cta());
     const double share = sms > 0 ? total / sms : 0.0;
@@ -826,14 +829,30 @@ void batch_layout(const sc_image_desc *descs, int n, const BatchCfg &c, unsigned
     b.items.push_back(layout_item(d, limit, pool, off, &S, limit + 2 * c.kt, c.kt, &b.map_failed));
     if (S > b.Smax) b.Smax = S;
   }
+  // A balanced image's cluster: 2 ceil(w / 640) CTAs, the most that shorten its seams, or max(2, ceil(w / 384)),
+  // which take fewer of the SMs that others wait for. The line is where they are equal: plans of 8 to 96 images
+  // of the benchmark's sizes (up to 208 CTAs) take 1.02 to 1.20 x as long with the smaller clusters, of 128
+  // images (238 and 244 CTAs) 1.04 and 0.96 x, of 192 (261) 0.92 x, of 256 (295 to 322) 0.92 to 1.00 x.
+  bool larger = c.wide_lat;
+  if (c.thr_bal > 0.f) {
+    int ctas = (int)b.items.size();
+    for (int k : wide) {
+      const int w = batch_need_width(descs[k]);
+      ctas += bal[k] ? batch_cl_ctas(w, CL_LAT) : batch_cl_ctas(w);
+    }
+    larger = 2 * ctas <= 3 * sms;
+  }
   for (int k : wide) {
     const sc_image_desc &d = descs[k];
     int shape = CL_WIDE, cs = batch_cluster_size(d);
     if (bal[k] || c.wide_lat) {
-      const int cl = batch_cl_ctas(batch_need_width(d), CL_LAT);
-      if (cl <= MAX_CLUSTER) {
+      const int w = batch_need_width(d);
+      if (larger && batch_cl_ctas(w, CL_LAT) <= MAX_CLUSTER) {
         shape = CL_LAT;
-        cs = cl;
+        cs = batch_cl_ctas(w, CL_LAT);
+      } else if (bal[k] && batch_lat_ctas(w) <= MAX_CLUSTER) {
+        shape = batch_lat_shape(w);
+        cs = batch_lat_ctas(w);
       }
     }
     const int rows0 = (d.H > d.target_h && d.target_w > d.H) ? d.target_w : d.H;
@@ -852,8 +871,7 @@ void batch_layout(const sc_image_desc *descs, int n, const BatchCfg &c, unsigned
     }
     int S;
     const ClOps o = cl_ops(shape);
-    g->items.push_back(layout_item(d, batch_cl_cols(cs, shape), pool, off, &S, shape == CL_LAT ? o.staged : 0, o.tile_rows,
-                                   &b.map_failed));
+    g->items.push_back(layout_item(d, batch_cl_cols(cs, shape), pool, off, &S, o.staged, o.tile_rows, &b.map_failed));
     g->index.push_back(k);
     if (S > g->Smax) g->Smax = S;
   }
@@ -1198,16 +1216,11 @@ int sc_batch_route(const sc_image_desc *descs, int n, float thr, int sms, int *c
     shape[k] = CL_WIDE;
     if (one_cta_us) one_cta_us[k] = item_us(descs[k], cost_one_cta());
   }
-  // reported sizes: the CTAs that cover the width, at 768 columns each and at 384 for the latency shape
-  // (whose launch gives the same work to two halves of a cluster, of 640 columns per CTA)
-  auto report = [&](int k) {
-    const int need = batch_need_width(descs[k]), wide = batch_cluster_size(descs[k]), lat = std::max(2, (need + 383) / 384);
-    const bool l = b.lat[k] && lat <= MAX_CLUSTER;
-    shape[k] = l ? CL_LAT : CL_WIDE;
-    cluster_size[k] = l ? lat : (wide <= MAX_CLUSTER ? wide : -1);
-  };
   for (const ClusterGroup &g : b.cl)
-    for (int k : g.index) report(k);
+    for (int k : g.index) {
+      cluster_size[k] = g.cs;
+      shape[k] = g.shape == CL_WIDE ? 0 : 1;   // (both latency shapes)
+    }
   for (int k : b.fallback) cluster_size[k] = -1;
   return SC_OK;
 }

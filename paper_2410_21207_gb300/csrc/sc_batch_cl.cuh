@@ -1,7 +1,7 @@
 // Batched persistent carving with one thread-block cluster per image (images wider than one CTA,
 // and the heaviest images of a batch), templated on the cluster's shape: compute warps NW, tile
-// rows KT and backtrack-fill warps FWM; sc_batch_cl.cu and sc_batch_cl_lat.cu instantiate the two
-// shapes of sc_batch_cl.h.
+// rows KT and backtrack-fill warps FWM; sc_batch_cl.cu, sc_batch_cl_lat.cu and sc_batch_cl_lat12.cu instantiate
+// the shapes of sc_batch_cl.h.
 // Each cluster repeatedly takes the next image from a queue and carves it completely, like the
 // one-CTA batched kernel (sc_batch.cuh), with the cluster-wide seam search (seam_search with CL, or the
 // two-ended clb_two_search)
@@ -33,14 +33,15 @@ __host__ __device__ inline TwoPlan clb_plan(int Smax) {
 }
 
 // The two-ended search (sc_dp.cu describes it) of one cluster: its first half of CTAs sweeps the upper
-// half of the map, the second half the lower one; rank 0 joins them, all of them backtrack.
+// half of the map, the second half the lower one (of an odd number the last CTA waits); rank 0 joins them,
+// all of them backtrack.
 template <int NW, int KT, int FWM>
 __device__ __forceinline__ void clb_two_search(SearchArgs a, uint32_t *scratch, const CUtensorMap *tmap, unsigned char *smem,
                                                const TwoPlan &t, SearchState &st, int rank, int ctas) {
   using G = Geo<NW, KT, true, FWM>;
   cg::cluster_group cl = cg::this_cluster();
   const TwoSplit g = two_split<KT, KS>(a.H);
-  const int cs = ctas / 2, half = rank >= cs ? 1 : 0, gw = cs * G::OWC, H = a.H;
+  const int cs = ctas / 2, half = rank >= cs ? 1 : 0, gw = cs * G::OWC + 2 * G::K2E, H = a.H;
   const TwoScratch x(scratch, gw);
   int *misc = reinterpret_cast<int *>(smem + t.plan.misc);
   a.gtab = x.tab + (half ? (size_t)g.S0 * gw : 0);
@@ -52,7 +53,7 @@ __device__ __forceinline__ void clb_two_search(SearchArgs a, uint32_t *scratch, 
   if (half) {
     a.H = g.H1;
     a.y0 = H - 1;
-    seam_sweep<NW, KT, true, FWM, false, KS, false, true, true, true>(a, smem, t.plan, st);
+    if (rank < 2 * cs) seam_sweep<NW, KT, true, FWM, false, KS, false, true, true, true>(a, smem, t.plan, st);
   } else {
     a.H = g.H0;
     seam_sweep<NW, KT, true, FWM, false, KS, false, true, true, false>(a, smem, t.plan, st);
@@ -290,7 +291,7 @@ struct ClShapeHost {
     cfg_for(cfg, at, clusters, cs, Smax, st, pdl);
     return cudaLaunchKernelEx(&cfg, k_batch_cl<NW, KT, FWM, TWO>, items, n, Smax, queue, err);
   }
-  static ClOps ops() { return ClOps{G::OWC, TWO ? 2 : 1, KT, G::BW, &smem_bytes, &capacity, &launch}; }
+  static ClOps ops() { return ClOps{G::OWC, TWO ? 2 : 1, TWO ? 2 * G::K2E : 0, KT, TWO ? G::BW : 0, &smem_bytes, &capacity, &launch}; }
 };
 
 }  // namespace sc

@@ -24,7 +24,7 @@ int static_pending_errors(int *bits);
 struct BatchCfg {
   int nw, kt;
   // load balance: an image whose estimated carving time on one CTA exceeds thr_bal x the whole
-  // batch's mean share per SM is carved by a cluster of the latency shape (CL_LAT, at least 2 CTAs)
+  // batch's mean share per SM is carved by a cluster of a latency shape (at least 2 CTAs)
   // instead of one CTA, so that it does not hold up the batch (0: off)
   float thr_bal = 0.f;
   // images wider than one CTA take the latency shape too (where 16 CTAs of it cover them): the
@@ -37,7 +37,7 @@ struct BatchCfg {
   int sms = 0;
 };
 // images carved by the cluster-per-image batched kernel: those wider than one CTA (CL_WIDE
-// shape) and the heaviest ones of a balanced plan (CL_LAT); one group per shape and cluster size
+// shape) and the heaviest ones of a balanced plan (CL_LAT, CL_LAT_12); one group per shape and cluster size
 struct ClusterGroup {
   int shape = 0;   // ClShape
   int cs = 1;      // CTAs of a cluster
@@ -49,7 +49,6 @@ struct BatchSetup {
   std::vector<BatchItem> items;   // images carved by one CTA each (device pointers filled in)
   std::vector<ClusterGroup> cl;   // images carved by one cluster each
   std::vector<int> fallback;      // descriptor indices carved by the per-seam cluster path
-  std::vector<char> lat;          // per descriptor: the latency shape was asked for
   size_t pool_bytes = 0;
   int Smax = 1;
   bool tall = false;              // an image left the one-CTA kernel for its height alone

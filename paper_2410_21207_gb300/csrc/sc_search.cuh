@@ -144,7 +144,7 @@ struct SearchArgs {
   const void *tmap = nullptr;   // tensor map of the energy buffer (rows of pitch_e elements)
   int x0 = E_PADL;              // its column of the map's column 0
   int y0 = 0, plane_rows = 0;   // its row of this half's row 0; rows from one cost plane to the next
-  int rank0 = 0, ctas = 0;      // the cluster's CTAs that sweep this map: ctas from rank0 on (0: all of them)
+  int rank0 = 0, ctas = 0;      // the cluster's CTAs that sweep this half: ctas from rank0 on (0: all of them)
 };
 
 // Running counters of the mbarrier phases, identical in every thread of the CTA.
@@ -683,13 +683,16 @@ __device__ __forceinline__ unsigned long long seam_sweep(const SearchArgs &p, un
   uint8_t *const gat0 = TWO ? p.gtab : ((CL && gw) ? cg::this_cluster().map_shared_rank(smem + plan.gat, 0) : smem + plan.gat);
 
   // geometry
-  const int A = rank * OWC, B = A + OWC;
-  const int ext0 = A - K2E;                     // extended range start
+  // (a cluster of a batch: no CTA lies beyond the map's edges, and the columns it would own there are the
+  // outermost CTAs' own)
+  const int edge_cols = TWO && p.ctas ? K2E : 0;
+  const int ext0 = rank * OWC - K2E + edge_cols;   // extended range start
+  const int A = rank == 0 ? 0 : ext0 + K2E, B = ext0 + K2E + OWC + (rank == cs - 1 ? edge_cols : 0);
   const int own0 = ext0 + warp * Q;             // warp strip start
   const int c0 = own0 - KT + lane * V;          // this lane's first column
   const int frame_base = own0 - KSS;            // ancestor frame of this warp
   const bool strip_lane = !producer && (lane * V >= KT) && (lane * V < KT + Q);
-  const bool cta_own = strip_lane && c0 >= A && c0 < B;   // A, B, c0 are multiples of 4
+  const bool cta_own = strip_lane && c0 >= A && c0 < B;   // own columns; A, B, c0 are multiples of 4
   uint32_t oobm[V];
 #pragma unroll
   for (int u = 0; u < V; ++u) oobm[u] = (c0 + u < 0 || c0 + u >= W) ? SENT : 0u;

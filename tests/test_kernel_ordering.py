@@ -38,7 +38,7 @@ def test_tensor_maps_in_global_memory_are_acquired():
     for name, item, search in (("sc_batch.cuh", "void batch_carve_item(", "batch_seam_pass<"),
                                ("sc_batch_cl.cuh", "void clb_carve_item(", "clb_seam_pass<")):
         body = _function(_code(name), item)
-        fence = re.search(r"if \((?:TWO && )?threadIdx\.x == NW \* 32\) fence_tensormap_acquire\(tmap\);", body)
+        fence = re.search(r"if \((?:T\w+ && )?threadIdx\.x == NW \* 32\) fence_tensormap_acquire\(tmap\);", body)
         assert fence and fence.start() < body.index(search), name
     fence = _function(_code("sc_ptx.cuh"), "void fence_tensormap_acquire(")
     assert "fence.proxy.tensormap::generic.acquire.sys" in fence
