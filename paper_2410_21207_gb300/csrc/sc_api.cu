@@ -350,7 +350,7 @@ int sc_check(void *stream) {
   SC_CUDA(cudaMemsetAsync(ws.flags.p, 0, sizeof(h), st));
   SC_CUDA(cudaStreamSynchronize(st));
   int e = h[0];
-  if (h[3] != 0) e |= ERR_COST_MISMATCH;   // some search's path costs did not add up to its cost
+  if (h[3] != 0) e |= ERR_COST_MISMATCH;   // the last search's path costs did not add up to its cost
   if (int *ge = device_error_word()) {
     int g = 0;
     SC_CUDA(cudaMemcpy(&g, ge, sizeof(int), cudaMemcpyDeviceToHost));

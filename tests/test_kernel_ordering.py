@@ -67,3 +67,14 @@ def test_check_clears_the_search_words_in_stream_order():
     clears = re.findall(r"cudaMemset(?:Async)?\(ws\.flags[^;]*;", body)
     assert len(clears) == 1 and clears[0].startswith("cudaMemsetAsync(") and ", st)" in clears[0]
     assert body.index(clears[0]) < body.index("cudaStreamSynchronize(st)")
+
+
+def test_a_search_checks_the_cost_of_the_one_before():
+    """A two-ended search leaves 0 in its cost word when its super-tiles' costs add up to its own; the next
+    one looks at what it finds there and takes it away, so that two differences cannot cancel."""
+    kernel = _function(_code("sc_dp.cu"), "k_dp_two(DpArgs p")
+    assert kernel.index("__ldcg(p.sync + 1)") < kernel.index("two_join<") < kernel.index("atomicAdd(")
+    found = kernel[kernel.index("if (left != 0u)"):]
+    assert "atomicSub(reinterpret_cast<uint32_t *>(p.sync + 1), left);" in found
+    assert "atomicOr(p.err, ERR_COST_MISMATCH);" in found
+    assert re.search(r"if \(h\[3\] != 0\) e \|= ERR_COST_MISMATCH", _function(_code("sc_api.cu"), "int sc_check("))
