@@ -186,7 +186,7 @@ int sc_find_seam_multi_shape(int warps, int tile_rows);
  * that budget every device byte through their own allocator forbid allocations they do not
  * control. Same arguments and result as sc_find_seam (any uint16 map, exact seam and cost), but
  * every scratch byte (a padded copy of the energy map, the search's cost rows, the wide-cost search's
- * directions and ancestors, three status words) lives in one fixed array of 32 MiB inside the
+ * directions and ancestors, status and sync words) lives in one fixed array of 32 MiB inside the
  * library's device image, held by every GPU that loads the library until the process exits; the
  * call never calls cudaMalloc or cudaFree. Differences from sc_find_seam:
  *   - Size limit: the map must fit the array, roughly H * (W + 1280) * 2.3 bytes plus one row of

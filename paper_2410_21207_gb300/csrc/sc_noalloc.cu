@@ -6,7 +6,7 @@
 // a latency-critical frame loop cannot afford, and hosts that account for every device byte through
 // their own allocator or a fixed memory budget forbid allocations they do not control. Such callers
 // pass their own input and output buffers; the scratch (a padded copy of the energy map, the
-// search's cost rows and ancestor tables, the wide-cost search's directions and ancestors, three status
+// search's cost rows and ancestor tables, the wide-cost search's directions and ancestors, status and sync
 // words) comes from the array below.
 #include <cstdio>
 #include <mutex>

@@ -25,19 +25,20 @@
 //     super-tile boundary, and then the super-tiles are backtracked in parallel, each by a search
 //     between its two boundary columns in a 2*KSS-column window (KSS/16 columns per lane) with
 //     explicit directions.
-//   * Energies are staged in shared memory by TMA: a producer warp issues one bulk copy per row
-//     (one row per lane) into an NSLOT-slot ring, waits for the next tile to land and joins the CTA
-//     barrier that ends the current one, which also frees its slot; a lane reads its 4 energies of a
-//     row with one 8-byte shared-memory load.
+//   * Energies are staged in shared memory by TMA: a producer warp issues a tile's copies (tensor copies
+//     of a few boxes, or in the multi-map and CL_WIDE kernels one bulk copy per row, a row per lane) into
+//     an NSLOT-slot ring, waits for the next tile to land and joins the CTA barrier that ends the current
+//     one, which also frees its slot; a lane reads its 4 energies of a row with one 8-byte shared-memory
+//     load.
 //   * The rows of a tile are branch-free (the map has an added row of cost 0 above row 0), and
 //     per-super-tile bookkeeping runs after the tile, on its last row (the only row of a tile where
 //     it can occur, since KSS is a multiple of KT).
 // The result is Algorithm 3's seam exactly (leftmost ties, leftmost last-row minimum).
 // With DIRECT the map is the caller's own H x W array (any row pitch that is a multiple of 8
-// elements, 16-byte aligned rows), read in place: the row copies are clipped to the map's columns,
-// the backtrack's loads outside it are skipped, and the 24-bit cost range is checked here instead
-// of by a copy kernel (a per-row maximum of the staged energies, reduced over the cluster; a map
-// that fails it is left to the wide-cost search through its gate).
+// elements, 16-byte aligned rows), read in place: row copies are clipped to its columns (tensor copies
+// read 0 beyond them), the backtrack's loads outside it are skipped, and the 24-bit cost range is checked
+// here instead of by a copy kernel (a per-row maximum of the staged energies, reduced over the cluster; a
+// map that fails it is left to the wide-cost search through its gate).
 // With FWD (forward energy) the map has three planes, CU, DL and DR, and a cell's cost depends on
 // the direction it is reached from: M(i,j) = CU(i,j) + min(M(i-1,j-1) + DL(i,j), M(i-1,j),
 // M(i-1,j+1) + DR(i,j)). Optimal predecessors still never cross (a crossing pair would need
@@ -653,9 +654,9 @@ static __device__ __noinline__ void backtrack_fill_call(FillCtx f, const int *jb
 // row-by-row copy costs its warp about 65 cycles, 2,100 per 32-row tile: more than the tile's rows
 // take, so the producer paced the sweep); the box rows of the half swept upwards (REV) lie in reverse
 // order. Half a 1920x1080 map: 40,000 -> 29,700 cycles; 3840x2160: 88,500 -> 73,500; a forward-energy
-// carve at 1920x1080 (three planes: 48 row copies per 16-row tile) 60.3 -> 34.9 ms. The batched and
-// multi-map kernels keep the row copies: their maps have no tensor maps (a caller's, or one of a
-// batch's many), and several warps per SM sub-partition need longer for a tile than its copies.
+// carve at 1920x1080 (three planes: 48 row copies per 16-row tile) 60.3 -> 34.9 ms. The one-CTA batched
+// kernel and the two-ended clusters copy through the tensor map of the image's own energies. The multi-map
+// kernel, whose maps are the callers', and the 8-row-tile clusters keep the row copies: 8 copies a tile.
 template <int NW, int KT, bool CL, int FWM, bool FWD, int KSS, bool DIRECT, bool TM, bool TWO = false, bool REV = false>
 __device__ __forceinline__ unsigned long long seam_sweep(const SearchArgs &p, unsigned char *smem, const SearchPlan &plan,
                                                          SearchState &st) {
@@ -721,7 +722,8 @@ __device__ __forceinline__ unsigned long long seam_sweep(const SearchArgs &p, un
   const uint32_t COPY_BYTES = (uint32_t)(chi - clo) * 2;
 
   if (producer) {
-    // ---- energy staging: rows of columns [ext0 - KT, ext0 - KT + BW), one bulk copy per lane ----
+    // ---- energy staging: rows of columns [ext0 - KT, ext0 - KT + BW), by the first lane's tensor copies
+    // or one bulk copy per lane ----
     const uint16_t *Estage = p.E + (ext0 - KT);
     auto issue = [&](int tt) {
       const int slot = (int)((st.tiles + tt) % NSLOT);
