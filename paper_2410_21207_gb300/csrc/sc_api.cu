@@ -343,6 +343,7 @@ int sc_check(void *stream) {
   std::lock_guard<std::mutex> lk(ws.mu);
   // a stream with no earlier work has fresh (uninitialised) flag words: they start at zero
   if ((rc = ensure_flags(ws))) return rc;
+  SC_CUDA(cudaStreamSynchronize(st));   // (refused under capture, before anything is enqueued)
   // read and cleared in the stream's order: the words hold the searches' sync words too, and a search
   // launched right after this call must not find them cleared while it runs
   int h[FLAG_WORDS] = {};

@@ -66,7 +66,10 @@ def test_check_clears_the_search_words_in_stream_order():
     body = _function(_code("sc_api.cu"), "int sc_check(")
     clears = re.findall(r"cudaMemset(?:Async)?\(ws\.flags[^;]*;", body)
     assert len(clears) == 1 and clears[0].startswith("cudaMemsetAsync(") and ", st)" in clears[0]
-    assert body.index(clears[0]) < body.index("cudaStreamSynchronize(st)")
+    enqueued = [m.start() for m in re.finditer(r"Async\(", body)]
+    waits = [m.start() for m in re.finditer(r"cudaStreamSynchronize\(st\)", body)]
+    # the first wait refuses a stream that is being captured, the last one completes the copy and the clearing
+    assert waits[0] < min(enqueued) and body.index(clears[0]) < waits[-1]
 
 
 def test_a_search_checks_the_cost_of_the_one_before():
