@@ -286,7 +286,8 @@ int sc_carve_batch(const sc_image_desc *descs, int n, void *stream);
  * CTA count otherwise, -1 when no cluster covers it (the per-seam path carves it); shape[k] 0 for
  * clusters of 8-row tiles (images wider or taller than one CTA has room for), 1 for clusters of a latency
  * shape, which sweeps the image from both ends (2 ceil(width / 640) CTAs, up to 16, while the plan's
- * images take at most 1.5 x the SMs so, else max(2, ceil(width / 384)) CTAs); one_cta_us
+ * images take at most 1.8 x the SMs so and at most 0.9 x the SMs images are not routed for their time;
+ * else max(2, ceil(width / 384)) CTAs); one_cta_us
  * (nullable): the carving-time model's estimate of image k's carve on one CTA, in microseconds.
  * Errors: SC_EINVAL for a NULL array, n < 1, thr < 0, sms < 1 or a descriptor that fails the
  * sc_carve size checks. */

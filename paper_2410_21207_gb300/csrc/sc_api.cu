@@ -831,17 +831,18 @@ void batch_layout(const sc_image_desc *descs, int n, const BatchCfg &c, unsigned
     if (S > b.Smax) b.Smax = S;
   }
   // A balanced image's cluster: 2 ceil(w / 640) CTAs, the most that shorten its seams, or max(2, ceil(w / 384)),
-  // which take fewer of the SMs that others wait for. The line is where they are equal: plans of 8 to 96 images
-  // of the benchmark's sizes (up to 208 CTAs) take 1.02 to 1.20 x as long with the smaller clusters, of 128
-  // images (238 and 244 CTAs) 1.04 and 0.96 x, of 192 (261) 0.92 x, of 256 (295 to 322) 0.92 to 1.00 x.
+  // which take fewer of the SMs that others wait for. The larger ones while at most 0.9 x the SMs images are not
+  // balanced and all images' CTAs are at most 1.8 x the SMs. 49 plans of the benchmark's sizes, their time with
+  // the smaller clusters against the larger ones: of 72 to 100 images 0.99 to 1.22 (mean 1.10), of 112 to 153
+  // (up to 121 others) 0.91 to 1.15 (1.06), of 168 (133 to 135 others) 0.94 to 1.06 (1.00), of 184 (151 to
+  // 157) 0.90 to 0.98 (0.94), of 200 to 256 0.86 to 1.04 (0.97).
   bool larger = c.wide_lat;
   if (c.thr_bal > 0.f) {
-    int ctas = (int)b.items.size();
-    for (int k : wide) {
-      const int w = batch_need_width(descs[k]);
-      ctas += bal[k] ? batch_cl_ctas(w, CL_LAT) : batch_cl_ctas(w);
-    }
-    larger = 2 * ctas <= 3 * sms;
+    int ctas = 0, others = 0;
+    for (int k = 0; k < n; ++k) others += !bal[k];
+    for (int k : wide) ctas += batch_cl_ctas(batch_need_width(descs[k]), bal[k] ? CL_LAT : CL_WIDE);
+    ctas += (int)b.items.size();
+    larger = 10 * others <= 9 * sms && 10 * ctas <= 18 * sms;
   }
   for (int k : wide) {
     const sc_image_desc &d = descs[k];
