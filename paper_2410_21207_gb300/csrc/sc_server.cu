@@ -6,8 +6,8 @@
 //   2. admits queued requests while the device-memory ledger (one arena of the configured budget,
 //      first-fit) has room, as micro-batches of up to max_batch requests of one kind, in arrival
 //      order within the kind: requests that fit one CTA go to the one-CTA persistent kernel
-//      (k_batch), wider ones and those whose one-CTA carve would take over an estimated 50 ms to
-//      the cluster-per-image persistent kernel in its latency shape (k_batch_cl), one micro-batch
+//      (k_batch), wider and taller ones and those whose one-CTA carve would take over an estimated
+//      50 ms to the cluster-per-image persistent kernel in its latency shape (k_batch_cl), one micro-batch
 //      per cluster size,
 //   3. enqueues each micro-batch on a free stream: host->device copies of the inputs, the launch,
 //      a completion event.
@@ -136,7 +136,7 @@ struct sc_server {
   size_t budget = 0;
   int max_batch = 64;
   int dev = 0;
-  // wide requests, and those whose one-CTA carve would take over 50 ms, on latency-shaped clusters
+  // wide and tall requests, and those whose one-CTA carve would take over 50 ms, on latency-shaped clusters
   sc::BatchCfg cfg{15, 16, 0.f, true, 50000.f};
   int sms = 1, occ = 1;
   sc::Arena arena;
